@@ -186,10 +186,11 @@ extern "C" int sd_entropy(sd_store* s, int32_t tree, double* h_entropy, void* st
     if (live <= 0) return SD_OK;
     int *fa = nullptr, *fb = nullptr;
     unsigned char* small = nullptr;                              // total, acc, wsum, counters
-    if (cudaMalloc(&fa, sizeof(int) * (size_t)live) != cudaSuccess || cudaMalloc(&fb, sizeof(int) * (size_t)live) != cudaSuccess ||
-        cudaMalloc(&small, 64) != cudaSuccess) {
+    if (sd_device_malloc((void**)&fa, sizeof(int) * (size_t)live, st) != cudaSuccess ||
+        sd_device_malloc((void**)&fb, sizeof(int) * (size_t)live, st) != cudaSuccess ||
+        sd_device_malloc((void**)&small, 64, st) != cudaSuccess) {
         cudaGetLastError();
-        cudaFree(fa); cudaFree(fb); cudaFree(small);
+        sd_device_free(fa, st); sd_device_free(fb, st); sd_device_free(small, st);
         return SD_ERR_NOMEM;
     }
     unsigned long long* total = (unsigned long long*)small;
@@ -216,7 +217,7 @@ extern "C" int sd_entropy(sd_store* s, int32_t tree, double* h_entropy, void* st
     if (ce == cudaSuccess) ce = cudaMemcpyAsync(&h_acc, acc, sizeof(double), cudaMemcpyDeviceToHost, st);
     if (ce == cudaSuccess) ce = cudaMemcpyAsync(&h_w, wsum, sizeof(h_w), cudaMemcpyDeviceToHost, st);
     if (ce == cudaSuccess) ce = cudaStreamSynchronize(st);
-    cudaFree(fa); cudaFree(fb); cudaFree(small);
+    sd_device_free(fa, st); sd_device_free(fb, st); sd_device_free(small, st);
     if (ce != cudaSuccess) return SD_ERR_CUDA;
     *h_entropy = h_w ? h_acc / (double)h_w : 0.0;
     return SD_OK;
@@ -276,10 +277,14 @@ extern "C" int sd_enumerate(sd_store* s, int32_t tree, int64_t max_nodes, int32_
     const long long room = max_nodes > 0 ? max_nodes : 1;        // nodes with children among the records written
     int *fe[2] = {nullptr, nullptr}, *fr[2] = {nullptr, nullptr};
     unsigned char* small = nullptr;                              // n_out, frontier sizes
-    bool okm = cudaMalloc(&small, 64) == cudaSuccess;
+    bool okm = sd_device_malloc((void**)&small, 64, st) == cudaSuccess;
     for (int b = 0; b < 2 && okm; ++b)
-        okm = cudaMalloc(&fe[b], sizeof(int) * (size_t)room) == cudaSuccess && cudaMalloc(&fr[b], sizeof(int) * (size_t)room) == cudaSuccess;
-    auto release = [&]() { cudaFree(small); for (int b = 0; b < 2; ++b) { cudaFree(fe[b]); cudaFree(fr[b]); } };
+        okm = sd_device_malloc((void**)&fe[b], sizeof(int) * (size_t)room, st) == cudaSuccess &&
+              sd_device_malloc((void**)&fr[b], sizeof(int) * (size_t)room, st) == cudaSuccess;
+    auto release = [&]() {
+        sd_device_free(small, st);
+        for (int b = 0; b < 2; ++b) { sd_device_free(fe[b], st); sd_device_free(fr[b], st); }
+    };
     if (!okm) { cudaGetLastError(); release(); return SD_ERR_NOMEM; }
     unsigned long long* n_out = (unsigned long long*)small;
     int* cnt = (int*)(small + 8);                                // cnt[0], cnt[1]: frontier sizes
