@@ -367,45 +367,52 @@ global_insert_kernel(sd_store sv, int n, const int32_t* d_slot, const int64_t* d
     }
 }
 
-// Warp i + 1 of the grid appends item i to its request slot (items for the global tree are
-// taken by global_insert_kernel).
-__global__ void append_kernel(sd_store sv, int n, const int32_t* d_slot, const int64_t* d_offsets,
-                              const int32_t* d_tokens, const uint8_t* d_reset) {
-    const int lane = threadIdx.x & 31;
-    const int warp = (int)((blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5);
-    if (warp > n || warp == 0) return;
-    const int i = warp - 1;
+// Block i appends item i to its request slot (items for the global tree are taken by
+// global_insert_kernel): APP_AHEAD tokens at a time, looked up ahead by all warps and appended by the first.
+constexpr int APPEND_THREADS = 256;
+
+__global__ void __launch_bounds__(APPEND_THREADS)
+append_kernel(sd_store sv, const int32_t* d_slot, const int64_t* d_offsets, const int32_t* d_tokens, const uint8_t* d_reset) {
+    __shared__ AppendShared sh;
+    __shared__ int sh_len, sh_status;
+    const int i = blockIdx.x, tid = threadIdx.x, lane = tid & 31, wib = tid >> 5;
     const int slot = d_slot[i];
     if (slot < 0 || slot >= sv.R) return;
     SlotState* ss = sv.s_state + slot;
-    int32_t* text = sv.s_text + (long long)slot * sv.T;
-    TreeRef tr{sv.s_ent + (long long)slot * sv.spn, sv.s_root + (long long)slot * sv.V, (int)sv.spn};
+    int32_t* const text = sv.s_text + (long long)slot * sv.T;
+    int32_t* const root = sv.s_root + (long long)slot * sv.V;
     int len = ss->len, used = ss->used, live = ss->live, status = ss->status;
-    int act = ss->active[lane], room = ss->room[lane], run_cb = ss->run_cb[lane];
-    unsigned run_w = ss->run_w[lane];
+    int act = ss->active[lane], cb = ss->run_cb[lane];
+    unsigned w = append_pack(ss->run_w[lane], ss->room[lane]);
     if (d_reset && d_reset[i]) {
         // forget the old tree: only root-table cells of tokens that occur can be set
-        for (int k = lane; k < len; k += 32) tr.root[text[k]] = -1;
-        __syncwarp();
-        len = 0; used = 0; live = 0; status = 0; act = -1; room = 0; run_cb = 0; run_w = 0;
-        if (lane == 0) ss->gen += 1;
+        for (int k = tid; k < len; k += APPEND_THREADS) root[text[k]] = -1;
+        len = 0; used = 0; live = 0; status = 0; act = -1; cb = 0; w = 0;
+        __syncthreads();
+        if (tid == 0) ss->gen += 1;
     }
-    const long long b = d_offsets[i], e = d_offsets[i + 1];
-    for (long long k = b; k < e && !(status & (SD_STATUS_POOL_FULL | SD_STATUS_BAD_TOKEN)); ++k) {
-        const int x = d_tokens[k];
-        if (x < 0 || x >= sv.V) { status |= SD_STATUS_BAD_TOKEN; break; }
-        if (len >= sv.T || !append_token(tr, sv.D, x, len, lane, act, room, run_cb, run_w, used, live)) {
-            status |= SD_STATUS_POOL_FULL;
-            break;
+    const int32_t* const tok = d_tokens + d_offsets[i];
+    const int n_new = (int)(d_offsets[i + 1] - d_offsets[i]);
+    for (int k = 0; k < n_new && !(status & (SD_STATUS_POOL_FULL | SD_STATUS_BAD_TOKEN)); k += APP_AHEAD) {
+        const int m = min(APP_AHEAD, n_new - k);
+        append_stage_tokens(sh, text, len, tok + k, n_new - k, tid, APPEND_THREADS);
+        if (tid == 0) sh.ahead = m >= 3 ? 1 : 0;
+        __syncthreads();
+        if (m >= 3) {                                            // (one or two tokens are as soon searched for in their turn)
+            search_ahead(sh, sv, sv.s_ent + (long long)slot * sv.spn, root, len, m, tid / APP_LANES, APPEND_THREADS / APP_LANES, lane);
+            __syncthreads();
         }
-        if (lane == 0) text[len] = x;
-        ++len;
+        if (wib == 0) {
+            append_tokens(sh, sv, slot, tok + k, m, 1, lane, act, cb, w, len, used, live, status);
+            if (lane == 0) { sh_len = len; sh_status = status; }
+        }
+        __syncthreads();
+        len = sh_len; status = sh_status;
     }
-    ss->active[lane] = act;
-    ss->room[lane] = room;
-    ss->run_cb[lane] = run_cb;
-    ss->run_w[lane] = run_w;
-    if (lane == 0) { ss->len = len; ss->used = used; ss->live = live; ss->status = status; }
+    if (wib == 0) {
+        append_store(ss, lane, act, cb, w);
+        if (lane == 0) { ss->len = len; ss->used = used; ss->live = live; ss->status = status; }
+    }
 }
 
 }  // namespace
@@ -416,8 +423,6 @@ extern "C" int sd_append(sd_store* s, int32_t n, const int32_t* d_slot, const in
     SD_CHECK_DEVICE(s);
     if (n == 0) return SD_OK;
     if (!d_slot || !d_offsets) return SD_ERR_INVALID_ARG;
-    const int warps_per_block = 4;
-    const unsigned blocks = (unsigned)((n + 1 + warps_per_block - 1) / warps_per_block);
     // The global tree and the request trees share nothing: the insert into the global tree runs
     // beside the appends, on the store's own stream, which starts behind everything the caller's
     // stream holds so far and which the caller's stream waits for before it goes on.
@@ -427,7 +432,7 @@ extern "C" int sd_append(sd_store* s, int32_t n, const int32_t* d_slot, const in
     global_insert_kernel<<<GI_CTAS, GI_THREADS, 0, s->aux>>>(*s, n, d_slot, d_offsets, d_tokens);
     SD_CUDA_OK(cudaGetLastError());
     SD_CUDA_OK(cudaEventRecord(s->ev_join, s->aux));
-    append_kernel<<<blocks, warps_per_block * 32, 0, st>>>(*s, n, d_slot, d_offsets, d_tokens, d_reset);
+    append_kernel<<<(unsigned)n, APPEND_THREADS, 0, st>>>(*s, d_slot, d_offsets, d_tokens, d_reset);
     SD_CUDA_OK(cudaGetLastError());
     SD_CUDA_OK(cudaStreamWaitEvent(st, s->ev_join, 0));
     SD_CUDA_OK(cudaGetLastError());

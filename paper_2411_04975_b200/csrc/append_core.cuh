@@ -22,12 +22,6 @@
 
 namespace {
 
-struct TreeRef {
-    int4* ent;
-    int32_t* root;
-    int cap;                 // entries in the pool
-};
-
 __device__ __forceinline__ int* word(int4* e, int k) { return reinterpret_cast<int*>(e) + k; }
 
 // Loads of tree entries.  CG: read through L2 only, for a kernel whose blocks run on several SMs
@@ -38,8 +32,7 @@ template <bool CG> __device__ __forceinline__ int ld_tok(const int4* p) { return
 // Inserts child x at sorted position `pos` into the child run of `parent`
 // (cb, n children, flags in w).  `fresh` > 0: the run is full and moves to
 // ent[fresh ...).  Returns the new child's entry index.
-// G: entries moved (or, in the look-up, read) per round.  Eight where registers are plentiful;
-// the decode-step kernel, which has to share its registers with the speculation code, uses four.
+// G: entries moved (or, in the look-up, read) per round.
 template <int G, bool CG = false>
 __device__ int insert_child(int4* ent, int parent, int cb, int n, int pos, int x, int fresh, bool moves) {
     const int4 ne = make_int4(x, 1, 0, 0);
@@ -153,130 +146,282 @@ __device__ int lookup_child(const int4* ent, int cb, int n, int x, int& pos, int
     return found;
 }
 
-// All 32 lanes call.  `act` is this lane's active node of depth lane + 1 (-1: none);
-// on return it is the active node after x was appended.  `t` is the context length
-// before the append.  `used` / `live` are warp-uniform pool counters.
-// Returns false, changing nothing, if the pool cannot hold the new nodes.
-// (run_cb, run_w) travel with `act`: the active node's child run as of now, so that the
-// next token's look-up starts at the run itself instead of first reading the node.
-template <int G = 8>
-__device__ bool append_token(const TreeRef& tr, int D, int x, int t, int lane, int& act, int& room, int& run_cb,
-                             unsigned& run_w, int& used, int& live) {
+// ---------------------------------------------------------------------------------------------
+// Append to a request's tree: one warp, a lane per active node.
+//
+// Tokens follow one another strictly (the next one starts at the nodes this one found or made), so a
+// request with 16 accepted tokens waits for 16 steps in a row, and that is what most decode steps wait
+// for.  A warp gets about one instruction per seven cycles on such a chain, so what counts is how few
+// there are.  Nearly all runs below the first levels have at most four children: four loads per lane, all at
+// once, and no search.  The first levels' runs are long; where a token belongs in them is looked up ahead by
+// other warps, for many tokens at once (search_ahead: eight lanes per search), and the lane then reads four
+// entries around that place.  What is left (a place that is not known, an insert into a run) is done by
+// the whole warp for one lane at a time.  (A search of up to eight entries per lane and round for every
+// lane, four rounds for a long run, took 2.3 us per token with the SM to itself and 3.8 with four
+// blocks on it.)
+constexpr int APP_AHEAD = 28;                 // tokens looked up ahead
+constexpr int APP_SHALLOW = 4;                // depths looked up ahead
+constexpr int APP_LANES = 8;                  // lanes per search
+constexpr unsigned ROOM_SHIFT = 24, ROOM_MASK = 31u;            // room behind a node, kept in the spare bits of its w field while appending
+
+struct AppendShared {
+    int tok[APP_AHEAD + APP_SHALLOW + 2];     // the first new tokens, the few before and the two behind them (-1: none)
+    int hint[APP_AHEAD][APP_SHALLOW];         // by token and parent depth: where it belonged in that run before the append (-1: unknown)
+    int ahead;                                // warps that have left their hints
+};
+
+// One range of a sorted run being searched by eight lanes.
+struct RunSearch {
+    const int4* run;
+    int lo, hi;
+};
+
+__device__ __forceinline__ int search_probe(const RunSearch& r, int k) { return r.lo + ((r.hi - r.lo) * (k + 1)) / 9; }
+
+// All lanes of the warp call; the eight lanes of a group search for x in their run (an empty range is allowed).
+// Returns its place or -1, with the child run of the entry found; `place` is where it belongs.
+__device__ __forceinline__ int group_lookup(RunSearch a, int x, int lane, int& place, int2& zw) {
     const unsigned FULL = 0xffffffffu;
-    const int parent = __shfl_up_sync(FULL, act, 1);            // node of depth `lane`
-    const int parent_room = __shfl_up_sync(FULL, room, 1);      // free entries reserved behind it
-    const int parent_cb = __shfl_up_sync(FULL, run_cb, 1);
-    const unsigned parent_w = __shfl_up_sync(FULL, run_w, 1);
-    const bool valid = lane <= min(t, D - 1);
-    int found = -1, pos = 0, cb = 0, n = 0;
-    unsigned w = 0;
-    int4 fe = make_int4(0, 0, 0, 0);                             // the child's entry when found
-    if (valid) {
-        if (lane == 0) {
-            found = tr.root[x];
-            if (found >= 0) fe = tr.ent[found];
-        } else {
-            cb = parent_cb; w = parent_w;
-            if (w == RUN_UNKNOWN) { const int4 pe = tr.ent[parent]; cb = pe.z; w = (unsigned)pe.w; }
-            n = (int)(w & RUN_COUNT_MASK);
-            found = lookup_child<G>(tr.ent, cb, n, x, pos, fe);
+    const int l = lane & (APP_LANES - 1), gb = lane & ~(APP_LANES - 1);
+    while (true) {
+        const bool on = a.hi - a.lo > APP_LANES;
+        if (!__any_sync(FULL, on)) break;
+        int t = 0;
+        if (on) t = a.run[search_probe(a, l)].x;
+        const int c = __popc((__ballot_sync(FULL, on && t < x) >> gb) & 0xffu);          // probes below x
+        if (on) {
+            const int lo = c > 0 ? search_probe(a, c - 1) + 1 : a.lo;
+            const int hi = c < APP_LANES ? search_probe(a, c) + 1 : a.hi;                // keep the pivot: it may be x itself
+            a.lo = lo; a.hi = hi;
         }
     }
-    const bool need = valid && found < 0;
-    int asz = 0;                                                 // fresh entries this lane needs
-    bool behind_parent = false;                                  // the new leaf goes to parent + 1
-    int new_room = 0;
-    if (need) {
-        if (lane == 0 || n == 0) {
-            // first child of a leaf (or a new depth-1 node): start or continue a chain block
-            if (lane > 0 && parent_room > 0) { behind_parent = true; new_room = parent_room - 1; }
-            else { asz = D - lane; new_room = asz - 1; }
-        } else if ((uint32_t)n == sd_run_capacity(w)) {
-            asz = (int)sd_pow2ceil((uint32_t)n + 1u);
+    int4 e = make_int4(-1, 0, 0, 0);
+    const bool v = a.lo + l < a.hi;
+    if (v) e = a.run[a.lo + l];
+    const unsigned lt = (__ballot_sync(FULL, v && e.x < x) >> gb) & 0xffu;
+    const unsigned eq = (__ballot_sync(FULL, v && e.x == x) >> gb) & 0xffu;
+    place = a.lo + __popc(lt);
+    const int k = eq ? __ffs(eq) - 1 : 0;
+    zw.x = __shfl_sync(FULL, e.z, k, APP_LANES);
+    zw.y = __shfl_sync(FULL, e.w, k, APP_LANES);
+    return eq ? a.lo + k : -1;
+}
+
+// The tokens sh.tok holds: token 0 of the append is sh.tok[APP_SHALLOW - 1].
+__device__ __forceinline__ void append_stage_tokens(AppendShared& sh, const int32_t* text, int t_old, const int32_t* newtok, int n_new,
+                                                    int tid, int nthreads) {
+    for (int i = tid; i < APP_AHEAD + APP_SHALLOW + 2; i += nthreads) {
+        const int k = i - (APP_SHALLOW - 1);
+        sh.tok[i] = k < 0 ? (t_old + k >= 0 ? text[t_old + k] : -1) : (k < n_new ? newtok[k] : -1);
+    }
+}
+
+// Whole warps call, `group` of `groups` groups of eight lanes: a group per start position walks APP_SHALLOW
+// levels from the root and notes where each token belongs in the run it meets.  Reads the tree only (the
+// appending warp may be at work: a place it has changed meanwhile is recognised when the hint is used).
+__device__ __forceinline__ void search_ahead(AppendShared& sh, const sd_store& sv, const int4* ent, const int32_t* root, int t_old,
+                                             int n_new, int group, int groups, int lane) {
+    const int n = min(n_new, APP_AHEAD);
+    for (int g0 = 0; g0 < n + APP_SHALLOW - 1; g0 += groups) {
+        const int g = g0 + group, k0 = g - (APP_SHALLOW - 1);    // the path starts at token k0 of the append
+        const bool on = k0 < n && t_old + k0 >= 0;
+        int x = on ? sh.tok[g] : -1;
+        int2 zw = make_int2(0, 0);
+        bool node = false;
+        if (x >= 0 && x < sv.V) {
+            const int at = root[x];
+            node = at >= 0;
+            if (node) zw = *reinterpret_cast<const int2*>(&ent[at].z);
+        }
+        if ((lane & (APP_LANES - 1)) == 0 && on && k0 >= 0) sh.hint[k0][0] = -1;
+#pragma unroll 1
+        for (int d = 2; d <= APP_SHALLOW; ++d) {
+            const int k = k0 + d - 1;                            // the token that takes the path to depth d
+            const bool q = on && k < n;
+            x = q ? sh.tok[g + d - 1] : -1;
+            // (an entry being written may be read half old, half new: never beyond the pool)
+            const bool good = q && node && zw.x >= 0 && (long long)zw.x + ((unsigned)zw.y & RUN_COUNT_MASK) <= sv.spn;
+            const RunSearch r{ent + (good ? zw.x : 0), 0, good ? (int)((unsigned)zw.y & RUN_COUNT_MASK) : 0};
+            int place;
+            int2 next;
+            const int at = group_lookup(r, x, lane, place, next);
+            if ((lane & (APP_LANES - 1)) == 0 && q && k >= 0) sh.hint[k][d - 1] = node ? place : -1;
+            node = at >= 0;
+            zw = next;
         }
     }
-    int inc = asz;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const int y = __shfl_up_sync(FULL, inc, o);
-        if (lane >= o) inc += y;
+}
+
+// Place of x in the sorted run ent[cb .. cb + n), and whether it is there.  Whole warp, arguments warp-uniform.
+__device__ __forceinline__ int warp_place(const int4* ent, int cb, int n, int x, int lane, bool& there) {
+    const unsigned FULL = 0xffffffffu;
+    int lo = 0, hi = n;
+    while (hi - lo > 32) {
+        const int q = lo + (int)(((long long)(hi - lo) * (lane + 1)) / 33);
+        const int c = __popc(__ballot_sync(FULL, ent[cb + q].x < x));
+        const int below = __shfl_sync(FULL, q, max(c - 1, 0)), at = __shfl_sync(FULL, q, min(c, 31));
+        if (c > 0) lo = below + 1;
+        if (c < 32) hi = at + 1;                                 // keep the pivot: it may be x itself
     }
-    const int total = __shfl_sync(FULL, inc, 31);
-    if ((long long)used + total > (long long)tr.cap) return false;
-    const int fresh = behind_parent ? parent + 1 : used + inc - asz;
-    const bool moves = behind_parent || asz > 0;
-    used += total;
+    const int t = lo + lane < hi ? ent[cb + lo + lane].x : 0x7fffffff;
+    there = __any_sync(FULL, t == x);
+    return lo + __popc(__ballot_sync(FULL, t < x));
+}
 
-    // A lane that moves entries of its run must not do so while the next lane edits the
-    // header of an entry inside that run (only possible when the last tokens repeat one
-    // token): it then waits for that lane, see the rounds below.
-    const int next_parent = __shfl_down_sync(FULL, parent, 1);
-    const int next_need = __shfl_down_sync(FULL, need ? 1 : 0, 1);
-    const bool clash = need && lane >= 1 && lane < 31 && next_need && next_parent >= cb && next_parent < cb + n;
-
-    if (valid && found >= 0) {
-        // a count changes: the copies in the run's top block (if any) are stale from now on
-        if (lane > 0 && (w & RUN_HAS_TOP)) *word(&tr.ent[parent], 3) = (int)(w & ~RUN_HAS_TOP);
-        *word(&tr.ent[found], 1) = fe.y + 1;
-        act = found;
-        run_cb = fe.z;
-        run_w = (unsigned)fe.w;
-        // the next lane works on this very node's run (new child, or flag dropped): what was read may be stale
-        if (lane < 31 && next_parent == found) run_w = RUN_UNKNOWN;
-        else if (run_w & RUN_COUNT_MASK) {
-            // The next token's look-up starts in this run: ask L2 for what its first round will
-            // read (the whole run if it is short, else the seven probes of an eight-way split).
-            const int nn = (int)(run_w & RUN_COUNT_MASK);
-            asm volatile("prefetch.global.L2 [%0];" ::"l"(tr.ent + run_cb));
-            if (nn > G) {
-                const int step = G == 8 ? (nn >> 3) : ((nn + 7) >> 3);
+// All 32 lanes of a warp call: appends newtok[0 .. n_new) to the slot's tree and text.  Lane d - 1 holds the
+// active node of depth d (act, -1: none) with its child run (cb, w as RUN_UNKNOWN or count | flags | room);
+// len / used / live / status are warp-uniform.  A token outside the vocabulary or one the pool or the text buffer
+// has no room for ends the append in front of it.  sh.tok is staged; hints are used once
+// ahead_warps warps have left theirs.
+__device__ __forceinline__ void append_tokens(AppendShared& sh, const sd_store& sv, int slot, const int32_t* newtok, int n_new, int ahead_warps,
+                                              int lane, int& act, int& cb, unsigned& w, int& len, int& used, int& live, int& status) {
+    const unsigned FULL = 0xffffffffu;
+    int4* const ent = sv.s_ent + (long long)slot * sv.spn;
+    int32_t* const root = sv.s_root + (long long)slot * sv.V;
+    int32_t* const text = sv.s_text + (long long)slot * sv.T;
+    const int D = sv.D;
+    auto token = [&](int k) { return k < APP_AHEAD + 2 ? sh.tok[k + APP_SHALLOW - 1] : (k < n_new ? newtok[k] : -1); };
+    auto root_of = [&](int x) { return x >= 0 && x < sv.V ? root[x] : -1; };
+    int x1 = len >= 1 ? text[len - 1] : -1, x2 = len >= 2 ? text[len - 2] : -2;
+    int x = token(0), xn = token(1);
+    // the depth-1 node of the token at hand is read while the tokens before it are being taken
+    int r = root_of(x), rn = root_of(xn);
+    int4 re = r >= 0 ? ent[r] : make_int4(0, 0, 0, 0);
+    bool hints = false;
+    for (int k = 0; k < n_new; ++k) {
+        if (x < 0 || x >= sv.V) { status |= SD_STATUS_BAD_TOKEN; return; }
+        if (len >= sv.T) { status |= SD_STATUS_POOL_FULL; return; }
+        const int parent = __shfl_up_sync(FULL, act, 1);         // node of depth `lane`
+        int pcb = __shfl_up_sync(FULL, cb, 1);
+        unsigned pw = __shfl_up_sync(FULL, w, 1);
+        const bool valid = lane <= min(len, D - 1);
+        if (!hints && k < APP_AHEAD) hints = *(volatile int*)&sh.ahead == ahead_warps;
+        if (r < 0 && (x == x1 || x == x2)) { r = root[x]; if (r >= 0) re = ent[r]; }          // (made by one of the last two tokens)
+        else if (r >= 0 && (x == x1 || x == x2)) re = ent[r];    // (its count and run may have changed since it was read)
+        int found = -1, place = 0, n = 0, fy = 0, fz = 0;
+        unsigned fw = 0;
+        if (lane == 0) { found = r; fy = re.y; fz = re.z; fw = (unsigned)re.w; pw = 0; pcb = 0; }
+        else if (valid) {
+            if (pw == RUN_UNKNOWN) { const int2 zw = *reinterpret_cast<const int2*>(&ent[parent].z); pcb = zw.x; pw = (unsigned)zw.y; }
+            n = (int)(pw & RUN_COUNT_MASK);
+        }
+        int lo = 0, m = n;                                       // the entries to look at
+        bool known = true;
+        if (n > 4) {
+            known = false;
+            m = 0;
+            if (hints && lane < APP_SHALLOW && k < APP_AHEAD) {
+                const int h = sh.hint[k][lane];
+                if (h >= 0) { lo = min(max(h - 1, 0), n - 4); m = 4; }
+            }
+        }
+        if (m > 0) {
+            int t[4];
 #pragma unroll
-                for (int k = 0; k < 7; ++k) {
-                    const int q = G == 8 ? (k + 1) * step : (k + 1) * step - 1;
-                    if (q < nn) asm volatile("prefetch.global.L2 [%0];" ::"l"(tr.ent + run_cb + q));
+            for (int u = 0; u < 4; ++u) t[u] = u < m ? ent[pcb + lo + u].x : 0x7fffffff;
+            int below = 0;
+#pragma unroll
+            for (int u = 0; u < 4; ++u) below += t[u] < x ? 1 : 0;
+            place = lo + below;
+#pragma unroll
+            for (int u = 0; u < 4; ++u) if (t[u] == x) found = pcb + lo + u;
+            // (a hint: the run may have grown since, or be another one by now)
+            if (n > 4) known = found >= 0 || ((lo == 0 || below > 0) && (lo + 4 == n || below < 4));
+        }
+        unsigned open = __ballot_sync(FULL, !known);
+        while (open) {                                           // long runs: the whole warp, one after the other
+            const int src = __ffs(open) - 1;
+            open &= open - 1;
+            const int scb = __shfl_sync(FULL, pcb, src);
+            bool there;
+            const int at = warp_place(ent, scb, __shfl_sync(FULL, n, src), x, lane, there);
+            if (lane == src) { place = at; found = there ? scb + at : -1; }
+        }
+        if (lane > 0 && found >= 0) { const int4 fe = ent[found]; fy = fe.y; fz = fe.z; fw = (unsigned)fe.w; }
+        const int next_parent = __shfl_down_sync(FULL, parent, 1);
+        // on to the next token's depth-1 node
+        const int xnn = token(k + 2);
+        const int rnn = root_of(xnn);
+        const int4 ren = rn >= 0 ? ent[rn] : make_int4(0, 0, 0, 0);
+
+        const bool need = valid && found < 0;
+        const unsigned needs = __ballot_sync(FULL, need);
+        int new_act = found, new_cb = fz;
+        unsigned new_w = fw;
+        if (found >= 0) {
+            *word(&ent[found], 1) = fy + 1;
+            if (lane < 31 && next_parent == found) new_w = RUN_UNKNOWN;      // the next lane may be editing this very node's run
+        } else { new_cb = 0; new_w = 0; }
+        if (needs) {
+            const unsigned room = lane == 0 ? 0u : (pw >> ROOM_SHIFT) & ROOM_MASK;
+            const unsigned rw = pw & ~(ROOM_MASK << ROOM_SHIFT);
+            const bool leaf = need && n == 0;                    // first child of a leaf, or a new depth-1 node
+            int asz = 0;                                         // fresh entries this lane needs
+            if (leaf) asz = room > 0u ? 0 : D - lane;            // continue the chain block behind the parent, or start one
+            else if (need && (uint32_t)n == sd_run_capacity(rw)) asz = (int)sd_pow2ceil((uint32_t)n + 1u);
+            int fresh = parent + 1;
+            if (__any_sync(FULL, asz > 0)) {
+                int inc = asz;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const int y = __shfl_up_sync(FULL, inc, o);
+                    if (lane >= o) inc += y;
+                }
+                const int total = __shfl_sync(FULL, inc, 31);
+                if ((long long)used + total > (long long)sv.spn) {
+                    // nothing of this token stays: the counts raised above go back
+                    if (found >= 0) *word(&ent[found], 1) = fy;
+                    status |= SD_STATUS_POOL_FULL;
+                    return;
+                }
+                if (asz > 0) fresh = used + inc - asz;
+                used += total;
+            }
+            if (leaf) new_w = (asz > 0 ? (unsigned)(asz - 1) : room - 1u) << ROOM_SHIFT;
+            // a tail that repeats one token is the only case in which a run to be edited holds the parent of the
+            // next lane: then everything goes lane by lane, deepest first
+            const bool repeats = len >= 2 && x1 == x2;
+            if (leaf && !repeats) {
+                ent[fresh] = make_int4(x, 1, 0, 0);
+                if (lane == 0) root[x] = fresh;
+                else *reinterpret_cast<int2*>(&ent[parent].z) = make_int2(fresh, 1);
+                new_act = fresh;
+            }
+            unsigned runs = __ballot_sync(FULL, need && (repeats || !leaf));
+            if (runs) {
+                __syncwarp();
+                while (runs) {
+                    const int src = 31 - __clz((int)runs);
+                    runs &= ~(1u << src);
+                    const int sn = __shfl_sync(FULL, n, src), sfresh = __shfl_sync(FULL, fresh, src);
+                    const bool moves = __shfl_sync(FULL, (leaf || asz > 0) ? 1 : 0, src) != 0;
+                    int idx = sfresh;
+                    if (src == 0) { if (lane == 0) { ent[sfresh] = make_int4(x, 1, 0, 0); root[x] = sfresh; } }
+                    else
+                        idx = insert_child_warp(ent, __shfl_sync(FULL, parent, src), __shfl_sync(FULL, pcb, src), sn,
+                                                __shfl_sync(FULL, place, src), x, sfresh, moves, lane);
+                    if (lane == src) new_act = idx;
                 }
             }
-        }
-    } else {
-        run_cb = 0;
-        run_w = 0;                                               // a new leaf (or no node at all)
-    }
-    room = new_room;
-    // Inserts run in rounds: a lane whose insert would move an entry that the next lane still has
-    // to edit waits for that lane (deepest first); everybody else goes at once.  Almost always
-    // there is one round; a tail of k equal tokens needs up to k.
-    unsigned pend = __ballot_sync(FULL, need);
-    for (int round = 0; round < 33 && pend; ++round) {
-        const bool next_pending = lane < 31 && ((pend >> (lane + 1)) & 1u);
-        const bool ready = need && ((pend >> lane) & 1u) && !(clash && next_pending);
-        // inserts that move many entries are done by the whole warp, one after the other
-        const bool big = ready && lane > 0 && (moves ? n : n - pos) > 48;
-        if (ready && !big) {
-            if (lane == 0) {
-                tr.ent[fresh] = make_int4(x, 1, 0, 0);
-                tr.root[x] = fresh;
-                act = fresh;
-            } else {
-                act = insert_child<G>(tr.ent, parent, cb, n, pos, x, fresh, moves);
-            }
+            live += __popc(needs);
         }
         __syncwarp();
-        unsigned bm = __ballot_sync(FULL, big);
-        while (bm) {
-            const int src = __ffs(bm) - 1;
-            bm &= bm - 1;
-            const int idx = insert_child_warp(tr.ent, __shfl_sync(FULL, parent, src), __shfl_sync(FULL, cb, src),
-                                              __shfl_sync(FULL, n, src), __shfl_sync(FULL, pos, src), x,
-                                              __shfl_sync(FULL, fresh, src), __shfl_sync(FULL, moves ? 1 : 0, src) != 0,
-                                              lane);
-            if (lane == src) act = idx;
-        }
-        pend &= ~__ballot_sync(FULL, ready);
-        __syncwarp();
+        act = valid ? new_act : -1;
+        cb = valid ? new_cb : 0;
+        w = valid ? new_w : 0u;
+        if (lane == 0) text[len] = x;
+        ++len;
+        x2 = x1; x1 = x; x = xn; xn = xnn;
+        r = rn; re = ren; rn = rnn;
     }
-    if (!valid) { act = -1; room = 0; run_cb = 0; run_w = 0; }
-    live += __popc(__ballot_sync(FULL, need));
-    return true;
+}
+
+// SlotState's fields to and from the registers of append_tokens.
+__device__ __forceinline__ unsigned append_pack(unsigned run_w, int room) { return run_w == RUN_UNKNOWN ? run_w : run_w | ((unsigned)room << ROOM_SHIFT); }
+__device__ __forceinline__ void append_store(SlotState* ss, int lane, int act, int cb, unsigned w) {
+    ss->active[lane] = act; ss->run_cb[lane] = cb;
+    ss->room[lane] = w == RUN_UNKNOWN ? 0 : (int)((w >> ROOM_SHIFT) & ROOM_MASK);
+    ss->run_w[lane] = w == RUN_UNKNOWN ? w : w & ~(ROOM_MASK << ROOM_SHIFT);
 }
 
 }  // namespace

@@ -32,7 +32,6 @@
 #define RUN_HAS_TOP 0x40000000u
 #define SD_TOP_MIN 128            // runs longer than this get a top block
 #define SD_TOP_BLOCK 65           // entries of a top block
-#define SD_OCC_LANES 32           // a per-request match node with at most this many occurrences is expanded a lane per occurrence
 
 struct GlobalState {          // device-resident bookkeeping of the global tree
     int32_t used;             // entries handed out

@@ -2,13 +2,8 @@
 //
 // sd_speculate / sd_step: ONE launch, one thread block per request (speculate_fused_kernel):
 //   - sd_step: warp 0 appends the request's accepted tokens to its tree (exactly what sd_append
-//     does) while the other warps match and expand; only jobs through the request's tree wait;
-//   - sd_step, blocks with many tokens to append: the other warps copy the request's text into
-//     shared memory and scan it for the earlier occurrences of the last token: how many tokens before each one agree with the context says
-//     which patterns it is an occurrence of.  A per-request match node with at most 32
-//     occurrences needs no tree at all: a lane per occurrence, the node's sub-tree is read off
-//     the text behind the occurrences (expand_occ).  Otherwise the per-request match nodes are
-//     the slot's active nodes (sd_step: a job that needs them waits for the append);
+//     does) while the other warps look ahead for it, match and expand; the per-request match
+//     nodes are the slot's active nodes, so only jobs through the request's tree wait for it;
 //   - the global match nodes are advanced from the nodes cached at the previous call by
 //     descending only the tokens appended since;
 //   - the (tree, p) jobs go into a queue, costliest first, a warp per job; a job is dropped,
@@ -281,17 +276,11 @@ __global__ void select_emit_kernel(sd_store sv, int n, const int32_t* __restrict
 // of at most one request per SM gets bigger blocks (W = 24 / 16), a batch of more than two
 // requests per SM smaller ones (W = 8 / 5, four per SM) to stay in one wave.
 constexpr int CTA_WARPS = 10;                  // the usual block (96 registers; 16 warps x 64 registers spill: 87 us against 83.5)
-constexpr int CTA_WARPS_STEP = 10;             // the usual block of sd_step: 10 warps with 96 registers each and
-constexpr int STEP_G = 4;                      // an append that moves four entries per round, so that the
-                                               // append in front does not spill.  Measured per step: 92.7 us;
-                                               // 9 warps 92.8, 11 (80 registers) 95, 8 (128) 96; with eight
-                                               // entries per round: 8 warps x 128 registers 95, 10 x 96 100,
-                                               // 12 x 80 100, 16 x 64 104, 6 x 168 110
+constexpr int CTA_WARPS_STEP = 10;             // the usual block of sd_step
 constexpr int CTA_WARPS_WIDE = 24;             // small batches (one block per SM at most): the block has the SM's
 constexpr int CTA_WARPS_WIDE_STEP = 16;        // registers to itself (80 per thread; sd_step: 128)
 constexpr int CTA_WARPS_NARROW = 8;            // batches of more than two requests per SM: four blocks per SM
-constexpr int CTA_WARPS_NARROW_STEP = 5;       // (sd_step: 96 registers and the four-entry append; 512 requests:
-                                               // 82 us per step, 88 with 4 warps x 128 registers, 100 with 8 x 64)
+constexpr int CTA_WARPS_NARROW_STEP = 5;       // (sd_step: 96 registers)
 
 struct WarpWork {
     Frontier F;
@@ -317,52 +306,16 @@ struct BlockSharedT {
     int njobs, next, nwide, nwide_kept;
     long long slice_sum[WARPS];
     int slice_fs[WARPS];
-    // per-request tree, read off the text: earlier occurrences of the last token by the number of
-    // tokens before them that agree with the context
-    int r_hist[SD_MAX_DEPTH + 2];
-    int r_cum[SD_MAX_DEPTH + 2];              // r_cum[p]: occurrences of the pattern of length p
-    int r_fill[SD_MAX_DEPTH + 2];
-    int r_list[SD_OCC_LANES];                 // the occurrences of the patterns that have at most 32, longest matches first
-    int r_pn;                                 // shortest such pattern
+    AppendShared app;
+    int src_node[SD_MAX_DEPTH];               // where the walk to a global match node starts: node (-1: nowhere) ...
+    int src_from[SD_MAX_DEPTH];               // ... and the first token to take
     int app_done;                             // sd_step: warp 0 has appended the new tokens
     int nlate, late[SD_MAX_DEPTH];            // per-request jobs whose wait for the append ran out
-    int scan_next[2];
     unsigned best_hi;                         // high word of the largest SCORE reached so far: a lower
                                               // bound of it (scores are non-negative doubles), which is
                                               // all the pruning needs; 32 bits keep the atomic native
     int win_warp;
 };
-
-// find_child that also hands back the matched entry (valid when the result is >= 0)
-__device__ int find_child_entry(const int4* __restrict__ ent, int cb, int n, int x, int lane, int4& out) {
-    int lo = 0, hi = n;
-    for (int it = 0; it < 6 && hi - lo > 32; ++it) {
-        const int q = lo + (int)(((long long)(hi - lo) * (lane + 1)) / 33);
-        const int tk = ent[cb + q].x;
-        const unsigned ge = __ballot_sync(FULL, tk >= x);
-        const int f = ge ? __ffs(ge) - 1 : 32;
-        const int q_prev = __shfl_sync(FULL, q, f > 0 ? f - 1 : 0);
-        const int q_at = __shfl_sync(FULL, q, f < 32 ? f : 31);
-        if (f > 0) lo = q_prev + 1;
-        if (f < 32) hi = q_at + 1;
-    }
-    int found = -1;
-    for (int base = lo; base < hi && found < 0; base += 32) {
-        const int idx = base + lane;
-        int4 e = make_int4(-1, 0, 0, 0);
-        if (idx < hi) e = ent[cb + idx];
-        const unsigned eq = __ballot_sync(FULL, idx < hi && e.x == x);
-        if (eq) {
-            const int src = __ffs(eq) - 1;
-            found = cb + base + src;
-            out.x = __shfl_sync(FULL, e.x, src); out.y = __shfl_sync(FULL, e.y, src);
-            out.z = __shfl_sync(FULL, e.z, src); out.w = __shfl_sync(FULL, e.w, src);
-        }
-    }
-    return found;
-}
-
-
 
 __device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
 
@@ -559,44 +512,6 @@ __device__ void push_children_w(const int4* __restrict__ ent, int cb, int n, int
         }
     }
 }
-
-// MatchPattern from a known node: descend text[from .. to).  Levels whose child run lies inside
-// the window already in registers cost no memory access.  Returns the node reached (-1: no
-// match) and its child run in (cb, n).
-// The context is `text` up to position t_old and `newtok` from there on (tokens that are
-// being appended in the same launch).
-__device__ int walk_from(const int4* __restrict__ ent, int limit, int node, const int32_t* __restrict__ text, int t_old,
-                         const int32_t* __restrict__ newtok, int from, int to, int lane, int& cb, unsigned& wfull) {
-    if (node < 0) return -1;
-    int wb = node;
-    int4 w = load_window(ent, wb, limit, lane);
-    cb = __shfl_sync(FULL, w.z, 0);
-    wfull = (unsigned)__shfl_sync(FULL, w.w, 0);
-    int n = (int)(wfull & RUN_COUNT_MASK);
-    for (int pos = from; pos < to; ++pos) {
-        const int x = pos < t_old ? text[pos] : newtok[pos - t_old];
-        if (n == 0) return -1;
-        if (n > 32) {                                           // wide run: 32-way search
-            int4 e;
-            node = find_child_entry(ent, cb, n, x, lane, e);
-            if (node < 0) return -1;
-            cb = e.z; wfull = (unsigned)e.w; n = (int)(wfull & RUN_COUNT_MASK);
-            wb = -64;                                           // no usable window
-            continue;
-        }
-        if (!(cb >= wb && cb + n <= wb + 32)) { wb = cb; w = load_window(ent, wb, limit, lane); }
-        const int rel = wb + lane - cb;
-        const unsigned hit = __ballot_sync(FULL, rel >= 0 && rel < n && w.x == x);
-        if (!hit) return -1;
-        const int src = __ffs(hit) - 1;
-        node = wb + src;
-        cb = __shfl_sync(FULL, w.z, src);
-        wfull = (unsigned)__shfl_sync(FULL, w.w, src);
-        n = (int)(wfull & RUN_COUNT_MASK);
-    }
-    return node;
-}
-
 
 // Children of a node whose run has a top block (see RUN_HAS_TOP): the 64 best by count are
 // listed, best first, right before the run, together with the sum of all counts.
@@ -830,121 +745,6 @@ __device__ void expand_job(BlockShared& sh, WarpWork& W, const int4* __restrict_
     __syncwarp();
 }
 
-// ---------------------------------------------------------------------------------------------
-// Occurrence mode: ExpandSpeculationTree + SCORE for one (tree, p) job whose match node has at
-// most 32 occurrences, a lane per occurrence.  cptr[k] (k >= 1) is the k-th token behind the
-// lane's occurrence of the pattern and kmax says how many of them count (end of the text or
-// sequence, depth cap; 0: the lane holds no occurrence of this job).
-// A node below N_p is the set of lanes that agree on the tokens so far.  Every lane knows the
-// deepest node on its own path that is already in the speculation tree (k levels down, index
-// par_idx, D value d_par); the candidate it stands for is the next node on its path:
-//   COUNT = lanes that agree on the next token too, sibling sum = lanes that have a next token.
-// The candidates of all lanes together are exactly the frontier of Algorithm 1's expansion.
-template <class BlockShared>
-__device__ void expand_occ(BlockShared& sh, WarpWork& W, const int* cptr, int kmax, int tree, int p, int budget,
-                           unsigned flags, int lane) {
-    const int order = tree * SD_MAX_DEPTH + p;                  // loop order of Algorithm 1
-    const int buf = W.best_buf ^ 1;
-    int cnt = 0;
-    double score = 0.0;
-    bool dropped = false;
-    int k = 0, par_idx = -1;
-    double d_par = 1.0;                                         // D(N_p) = 1
-    bool cv = false;                                            // this lane stands for a candidate
-    int ctok = 0;
-    double cd = 0.0;
-    unsigned cmask = 0;                                         // lanes of the candidate node
-    // candidates of the lanes in `grp`, which share (k, par_idx, d_par); returns the lanes with a next token
-    auto refresh = [&](unsigned grp) -> unsigned {
-        const bool in = (grp >> lane) & 1u;
-        const bool valid = in && k + 1 <= kmax;
-        const unsigned vm = __ballot_sync(FULL, valid);
-        if (in) cv = false;
-        if (valid) {
-            ctok = cptr[k + 1];
-            cmask = __match_any_sync(vm, ctok);
-            const int c = __popc(cmask), s = __popc(vm);
-            cd = c == s ? d_par : __dmul_rn(d_par, __ddiv_rn((double)c, (double)s));   // Eq. 2 with Eq. 1
-            cv = true;
-        }
-        return vm;
-    };
-    refresh(__ballot_sync(FULL, kmax > 0));
-    while (cnt < budget) {
-        // ---- the best candidate: larger D, then smaller token, then smaller parent index
-        const unsigned hi = cv ? (unsigned)__double2hiint(cd) : 0u;     // D > 0, so hi > 0 for a candidate
-        const unsigned mx = __reduce_max_sync(FULL, hi);
-        if (mx == 0u) break;                                    // the frontier is empty
-        unsigned b = __ballot_sync(FULL, hi == mx);
-        int leader = __ffs(b) - 1;
-        unsigned lm = __shfl_sync(FULL, cmask, leader);
-        if (b & ~lm) {                                          // several nodes share the high word: full comparison
-            const bool in1 = hi == mx;
-            const unsigned lo = in1 ? (unsigned)__double2loint(cd) : 0u;
-            const unsigned mlo = __reduce_max_sync(FULL, lo);
-            const bool in2 = in1 && lo == mlo;
-            const unsigned mtk = __reduce_min_sync(FULL, in2 ? (unsigned)ctok : 0xffffffffu);
-            const bool in3 = in2 && (unsigned)ctok == mtk;
-            const unsigned mpk = __reduce_min_sync(FULL, in3 ? (unsigned)(par_idx + 1) : 0xffffffffu);
-            b = __ballot_sync(FULL, in3 && (unsigned)(par_idx + 1) == mpk);
-            leader = __ffs(b) - 1;
-            lm = __shfl_sync(FULL, cmask, leader);
-        }
-        const double wd = __shfl_sync(FULL, cd, leader);
-        const int wt = __shfl_sync(FULL, ctok, leader), wp = __shfl_sync(FULL, par_idx, leader);
-        // everything still to come is at most wd each
-        if ((score + (double)(budget - cnt) * wd) * 1.000000001 < best_so_far(sh)) { dropped = true; break; }
-        if (lane == 0) { W.tok[buf][cnt] = wt; W.par[buf][cnt] = (unsigned char)(wp + 1); }
-        score = __dadd_rn(score, wd);                           // Eq. 4, insertion order
-        int idx = cnt++;
-        const bool in = (lm >> lane) & 1u;
-        if (in) { ++k; par_idx = idx; d_par = wd; }
-        if ((flags & SD_FLAG_LINEAR) && !in) cv = false;        // chain variant: only the new node's children go on
-        // the best of the other candidates: while the new node has one child that all its lanes
-        // continue with, that child has the same D; if that is strictly above every other
-        // candidate it is the next node whatever else there is, and no arg-max is needed
-        const unsigned oth = __reduce_max_sync(FULL, (!in && cv) ? (unsigned)__double2hiint(cd) : 0u);
-        const bool chain_ok = (unsigned)__double2hiint(wd) > oth;
-        const int first = __ffs(lm) - 1;
-        while (true) {
-            const unsigned vm = refresh(lm);
-            if (cnt >= budget || !chain_ok || vm != lm || __shfl_sync(FULL, cmask, first) != lm) break;
-            if ((score + (double)(budget - cnt) * wd) * 1.000000001 < best_so_far(sh)) { dropped = true; break; }
-            if ((lm & (lm - 1u)) == 0u) {
-                // one occurrence: the rest of its text, as far as it counts and the budget goes
-                const int k0 = __shfl_sync(FULL, k, first);
-                const int len = min(__shfl_sync(FULL, kmax, first) - k0, budget - cnt);
-                const int* src = (const int*)(unsigned long long)__shfl_sync(FULL, (unsigned long long)cptr, first);
-                for (int j = lane; j < len; j += 32) {
-                    W.tok[buf][cnt + j] = src[k0 + 1 + j];
-                    W.par[buf][cnt + j] = (unsigned char)((j == 0 ? idx : cnt + j - 1) + 1);
-                }
-                for (int j = 0; j < len; ++j) score = __dadd_rn(score, wd);
-                cnt += len;
-                idx = cnt - 1;
-                if (in) { k += len; par_idx = idx; }
-            } else {
-                const int ct = __shfl_sync(FULL, ctok, first);
-                if (lane == 0) { W.tok[buf][cnt] = ct; W.par[buf][cnt] = (unsigned char)(idx + 1); }
-                score = __dadd_rn(score, wd);
-                idx = cnt++;
-                if (in) { ++k; par_idx = idx; }
-            }
-        }
-        if (dropped) break;
-        // the final SCORE of this job is at least its running value: let the others prune on it
-        if (lane == 0) atomicMax(&sh.best_hi, (unsigned)__double2hiint(score));
-    }
-    __syncwarp();
-    if (!dropped && (score > W.best_score || (score == W.best_score && score > 0.0 && order < W.best_order))) {
-        if (lane == 0) {
-            W.best_score = score; W.best_order = order; W.best_n = cnt; W.best_buf = buf;
-            atomicMax(&sh.best_hi, (unsigned)__double2hiint(score));
-        }
-    }
-    __syncwarp();
-}
-
 // A per-request job that goes through the tree's entries: the match node of pattern length p is
 // the slot's active node of depth p (kept current by the append).  Whole warp.
 template <class BlockShared>
@@ -977,15 +777,9 @@ __device__ void request_tree_job(BlockShared& sh, WarpWork& W, const sd_store& s
 //   1. match.  Global tree: the match nodes are advanced from the nodes cached at the previous
 //      call by descending only the tokens appended since (full walks when the cache is stale).
 //      Per-request tree: the slot's active nodes are the match nodes (sd_step: once the append
-//      is done).  A block of sd_step that appends many tokens does not wait for that: it copies
-//      the request's text (with the tokens being appended) into shared memory and scans it for the
-//      earlier occurrences of its last token; the number of tokens before an occurrence that
-//      agree with the context says which patterns it belongs to.
+//      is done).
 //   2. expand: the (tree, p) jobs that matched go into a queue, costliest first; a warp per job.
-//      Global jobs go through the tree's entries.  Per-request jobs whose match node has at most
-//      32 occurrences in a scanned text are read off the text (expand_occ: a lane per
-//      occurrence, no tree) and come first; the others go through the request's tree from the
-//      slot's active nodes.  sd_step: warp 0 appends the accepted tokens to the request's tree
+//      sd_step: warp 0 appends the accepted tokens to the request's tree
 //      meanwhile, exactly as sd_append would, and joins the queue when it is done; the other
 //      warps meet at a barrier of their own until then, and only a warp that has taken a job
 //      through the request's tree waits for the append (a bounded wait on a flag).
@@ -996,13 +790,13 @@ __device__ void request_tree_job(BlockShared& sh, WarpWork& W, const sd_store& s
 // score another job of the request has already reached (the running scores are published).
 constexpr int BAR_GROUP = 1, BAR_JOIN = 2;    // hardware barriers beside the block-wide one
 
-template <bool STEP, int WARPS, int MINB, int APPEND_G = 8>
+template <bool STEP, int WARPS, int MINB>
 __global__ void __launch_bounds__(WARPS * 32, MINB)
 speculate_fused_kernel(sd_store sv, int n, const int32_t* __restrict__ d_slot, int Pe, double alpha, int max_spec,
                        unsigned flags, double tau, const int32_t* __restrict__ d_budget_cap, int32_t* d_n_draft,
                        int32_t* d_tokens, int32_t* d_parents, int32_t* d_positions, uint32_t* d_mask, int32_t* d_chosen_tree,
                        int32_t* d_chosen_p, double* d_score, int32_t* d_status, const int64_t* __restrict__ d_app_off,
-                       const int32_t* __restrict__ d_app_tok, int stage_tokens) {
+                       const int32_t* __restrict__ d_app_tok) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     using BlockShared = BlockSharedT<WARPS>;
     constexpr int CTA_WARPS = WARPS;
@@ -1010,10 +804,6 @@ speculate_fused_kernel(sd_store sv, int n, const int32_t* __restrict__ d_slot, i
     // the warps that do everything but the append: all of them, or all but warp 0
     constexpr int GW0 = STEP ? 1 : 0, GWARPS = WARPS - GW0, GT = GWARPS * 32;
     BlockShared& sh = *reinterpret_cast<BlockShared*>(smem_raw);
-    int* const stx = reinterpret_cast<int*>(smem_raw + ((sizeof(BlockShared) + 15) & ~(size_t)15));
-    // new tokens from which a block reads its text off shared memory: 6 with two blocks per SM
-    // (9 warps scan), 12 with four (4 warps scan); measured, see the staging decision below
-    constexpr int STAGE_MIN_NEW = MINB >= 4 ? 12 : 6;
     const int tid = threadIdx.x, lane = tid & 31, wib = tid >> 5;
     const int gtid = tid - GW0 * 32, gw = wib - GW0;             // index inside that group (negative: warp 0 of sd_step)
     auto group_sync = [&]() {
@@ -1042,22 +832,14 @@ speculate_fused_kernel(sd_store sv, int n, const int32_t* __restrict__ d_slot, i
         t = t_old + n_new;
     }
     bool usable = ok && !(status & (SD_STATUS_POOL_FULL | SD_STATUS_BAD_TOKEN)) && t > 0;
-    // the stored text starts its way into shared memory now (asynchronous copies, nothing waits
-    // for them here): it arrives while the cached match nodes and the append list are read
     const int32_t* text = ok ? sv.s_text + (long long)slot * sv.T : nullptr;
-    const bool prefetched = STEP && MINB > 1 && n_new >= STAGE_MIN_NEW && ok && gtid >= 0 && t_old <= stage_tokens && !(flags & SD_FLAG_GLOBAL_ONLY);
-    if (prefetched) {
-        const unsigned dst0 = (unsigned)__cvta_generic_to_shared(stx);
-        for (int q = gtid; q < t_old; q += GT)
-            asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst0 + 4u * q), "l"(text + q) : "memory");
-    }
+    if (STEP && ok) append_stage_tokens(sh.app, text, t_old, newtok, n_new, tid, NT);
     int cap = max_spec;
     if (d_budget_cap && d_budget_cap[i] >= 0) cap = min(cap, d_budget_cap[i]);
     if (tid < 2 * SD_MAX_DEPTH) { (&sh.node[0][0])[tid] = -1; (&sh.nc[0][0])[tid] = 0; }
-    if (tid < SD_MAX_DEPTH + 2) { sh.r_hist[tid] = 0; sh.r_cum[tid] = 0; sh.r_fill[tid] = 0; }
     if (tid == 0) {
         sh.njobs = 0; sh.next = 0; sh.nwide = 0; sh.nwide_kept = 0; sh.best_hi = 0u; sh.win_warp = -1;
-        sh.r_pn = SD_MAX_DEPTH + 1; sh.scan_next[0] = 0; sh.scan_next[1] = 0; sh.app_done = 0; sh.nlate = 0;
+        sh.app_done = 0; sh.nlate = 0; sh.app.ahead = 0;
     }
     WarpWork& W = sh.w[wib];
     if (lane == 0) { W.best_score = 0.0; W.best_order = 1 << 30; W.best_n = 0; W.best_buf = 0; }
@@ -1065,61 +847,38 @@ speculate_fused_kernel(sd_store sv, int n, const int32_t* __restrict__ d_slot, i
     // ---------------- 1. match
     bool want_g = usable && !(flags & SD_FLAG_REQUEST_ONLY);
     bool want_r = usable && !(flags & SD_FLAG_GLOBAL_ONLY);
-    // warps that advance the global match nodes, and this warp's rank among them
-    const int mwarps = GWARPS;
-    const int mrank = gw;
-    constexpr int MROUNDS = (SD_MAX_DEPTH + GWARPS - 1) / GWARPS;   // pattern lengths per warp
-    int src_node[MROUNDS], src_from[MROUNDS];                   // per target: start node and first text index
-#pragma unroll
-    for (int h = 0; h < MROUNDS; ++h) { src_node[h] = -1; src_from[h] = 0; }
-    if (want_g && mrank >= 0) {
+    if (want_g && gtid >= 0 && gtid < Pe) {
+        // the walk to the match node of the last d tokens starts at the node kept from the call before, or at the root
         const bool cache_ok = ss->g_gen == ss->gen && ss->g_epoch == sv.g_state->epoch && ss->g_len <= t;
         const int k = t - ss->g_len;                            // tokens appended since the cache was taken
-        const int depths = ss->g_depths;
-#pragma unroll
-        for (int h = 0; h < MROUNDS; ++h) {
-            const int d = mrank + 1 + h * mwarps;               // target pattern length
-            if (d > Pe || d > t) continue;
-            if (cache_ok && d > k && d - k <= depths) {
-                src_node[h] = ss->g_node[d - k - 1];            // node of the tokens before the new ones
-                src_from[h] = t - k;
+        const int d = gtid + 1;
+        int node = -1, from = t;
+        if (d <= t) {
+            if (cache_ok && d > k && d - k <= ss->g_depths) {
+                node = ss->g_node[d - k - 1];                   // node of the tokens before the new ones
+                from = t - k;
             } else {
                 const int x0 = t - d < t_old ? text[t - d] : newtok[t - d - t_old];
-                src_node[h] = (x0 >= 0 && x0 < sv.V) ? sv.g_root[x0] : -1;
-                src_from[h] = t - d + 1;
+                node = (x0 >= 0 && x0 < sv.V) ? sv.g_root[x0] : -1;
+                from = t - d + 1;
             }
         }
+        sh.src_node[gtid] = node; sh.src_from[gtid] = from;
     }
     // all cached nodes read before any is replaced; and: is this a second block for the same slot?
     const bool refused = __syncthreads_or(dup) != 0;
     if (refused) { usable = false; want_g = false; want_r = false; status = SD_STATUS_BAD_SLOT; }
-    // The text can be read off only if it fits the shared memory left for it, and it is only
-    // worth the copy and the scan (about 16 us for 4,096 tokens) where a long append would
-    // otherwise hold the per-request jobs up: from STAGE_MIN_NEW new tokens on.  sd_speculate
-    // does not read it at all: with no append going on, the slot's active nodes are the
-    // per-request match nodes, at no cost.  Nor do blocks that have an SM to themselves (small
-    // batches: measured on 64 requests with 8,192-token texts, 112 us per step without, 141 with).
-    const bool staged = STEP && MINB > 1 && n_new >= STAGE_MIN_NEW && want_r && t >= 2 && t <= stage_tokens;
-    const int Lcap = min(Pe, D - 1);                            // a match node at depth D has no children
+    const bool look_ahead = STEP && n_new >= 3 && usable;         // (one or two tokens are as soon searched for in their turn)
     if (STEP && wib == 0) {
         if (ok && n_new > 0 && !refused) {
             // ---- the request's accepted tokens go into its tree and text (as sd_append does)
-            int32_t* wtext = sv.s_text + (long long)slot * sv.T;
-            TreeRef tr{sv.s_ent + (long long)slot * sv.spn, sv.s_root + (long long)slot * sv.V, (int)sv.spn};
             int len = ss->len, used = ss->used, live = ss->live, st = ss->status;
-            int act = ss->active[lane], room = ss->room[lane], run_cb = ss->run_cb[lane];
-            unsigned run_w = ss->run_w[lane];
-            for (int k = 0; k < n_new && !(st & (SD_STATUS_POOL_FULL | SD_STATUS_BAD_TOKEN)); ++k) {
-                const int x = newtok[k];
-                if (x < 0 || x >= sv.V) { st |= SD_STATUS_BAD_TOKEN; break; }
-                if (len >= sv.T || !append_token<APPEND_G>(tr, sv.D, x, len, lane, act, room, run_cb, run_w, used, live)) {
-                    st |= SD_STATUS_POOL_FULL;
-                    break;
-                }
-                if (lane == 0) wtext[len] = x;
-                ++len;
+            if (!(st & (SD_STATUS_POOL_FULL | SD_STATUS_BAD_TOKEN))) {
+                int act = ss->active[lane], cb = ss->run_cb[lane];
+                unsigned w = append_pack(ss->run_w[lane], ss->room[lane]);
+                append_tokens(sh.app, sv, slot, newtok, n_new, GWARPS, lane, act, cb, w, len, used, live, st);
+                append_store(ss, lane, act, cb, w);
             }
-            ss->active[lane] = act; ss->room[lane] = room; ss->run_cb[lane] = run_cb; ss->run_w[lane] = run_w;
             if (lane == 0) { ss->len = len; ss->used = used; ss->live = live; ss->status = st; }
         }
         __threadfence_block();
@@ -1127,87 +886,60 @@ speculate_fused_kernel(sd_store sv, int n, const int32_t* __restrict__ d_slot, i
         // join the others once their queue is ready
         asm volatile("bar.sync %0, %1;" ::"r"(BAR_JOIN), "r"(NT) : "memory");
     } else {
-        // ---- the tokens being appended join the text in shared memory
-        if (staged)
-            for (int q = t_old + gtid; q < t; q += GT) stx[q] = newtok[q - t_old];
-        // ---- global match nodes
+        if (look_ahead) {
+            search_ahead(sh.app, sv, sv.s_ent + (long long)slot * sv.spn, sv.s_root + (long long)slot * sv.V, t_old, n_new, gtid / APP_LANES,
+                         GT / APP_LANES, lane);
+            __threadfence_block();
+            __syncwarp();
+            if (lane == 0) atomicAdd(&sh.app.ahead, 1);
+        }
+        // ---- global match nodes: eight lanes per pattern length
         if (want_g) {
-#pragma unroll
-            for (int h = 0; h < MROUNDS; ++h) {
-                const int d = mrank + 1 + h * mwarps;
-                if (d > Pe) continue;
-                int cb = 0;
-                unsigned wf = 0;
-                const int node = (d > t) ? -1 : walk_from(sv.g_ent, (int)sv.g_cap, src_node[h], text, t_old, newtok, src_from[h], t,
-                                                          lane, cb, wf);
-                if (lane == 0) {
+            for (int p0 = 0; p0 < Pe; p0 += GT / APP_LANES) {
+                const int d = p0 + gtid / APP_LANES + 1;
+                int node = d <= Pe ? sh.src_node[d - 1] : -1;
+                int pos = d <= Pe ? sh.src_from[d - 1] : t;
+                int2 zw = make_int2(0, 0);
+                if (node >= 0) zw = *reinterpret_cast<const int2*>(&sv.g_ent[node].z);
+                // The eight entries at hand hold the next levels, too, where they are only children (most of them
+                // are): a token then costs no load.
+                int wb = -64;
+                int4 e = make_int4(-1, 0, 0, 0);
+                const int l = lane & (APP_LANES - 1), gb = lane & ~(APP_LANES - 1);
+                while (true) {
+                    bool on = node >= 0 && pos < t;
+                    if (!__any_sync(FULL, on)) break;
+                    const int x = on ? (pos < t_old ? text[pos] : newtok[pos - t_old]) : -1;
+                    const int n = on ? (int)((unsigned)zw.y & RUN_COUNT_MASK) : 0;
+                    const bool far = n > APP_LANES;
+                    if (__any_sync(FULL, far)) {                // long runs are searched
+                        int place;
+                        int2 next;
+                        const int at = group_lookup(RunSearch{sv.g_ent + zw.x, 0, far ? n : 0}, x, lane, place, next);
+                        if (far) { node = at >= 0 ? zw.x + at : -1; zw = next; ++pos; on = false; }
+                    }
+                    if (!__any_sync(FULL, on)) continue;
+                    if (on && (zw.x < wb || zw.x + n > wb + APP_LANES)) {
+                        wb = zw.x;
+                        if (wb + l < (int)sv.g_cap) e = sv.g_ent[wb + l];
+                    }
+                    const int off = zw.x - wb;
+                    const unsigned eq = (__ballot_sync(FULL, on && l >= off && l < off + n && e.x == x) >> gb) & 0xffu;
+                    const int k = eq ? __ffs(eq) - 1 : 0;
+                    const int nz = __shfl_sync(FULL, e.z, k, APP_LANES), nw = __shfl_sync(FULL, e.w, k, APP_LANES);
+                    if (on) { node = eq ? wb + k : -1; zw = make_int2(nz, nw); ++pos; }
+                }
+                if ((lane & (APP_LANES - 1)) == 0 && d <= Pe) {
                     ss->g_node[d - 1] = node;
                     sh.node[0][d - 1] = node;
-                    if (node >= 0) { sh.cb[0][d - 1] = cb; sh.nc[0][d - 1] = wf; }
+                    if (node >= 0) { sh.cb[0][d - 1] = zw.x; sh.nc[0][d - 1] = (unsigned)zw.y; }
                 }
             }
             if (gtid == 0) { ss->g_gen = ss->gen; ss->g_epoch = sv.g_state->epoch; ss->g_len = t; ss->g_depths = Pe; }
         }
-        if (prefetched) asm volatile("cp.async.wait_all;" ::: "memory");
-        group_sync();                                           // the text is in shared memory
-        // ---- per-request occurrences: a chunk of 256 positions at a time, handed out by a counter
-        // (warps that come late from their walks take fewer).  Pass 0 finds the occurrences of the
-        // last token, notes their match lengths and counts them by length; pass 1 collects those
-        // of the patterns that have at most 32 of them.
-        const int last = staged ? stx[t - 1] : 0;
-        const int nchunks = staged ? (t - 1 + 255) / 256 : 0;
-        unsigned char* const sell = reinterpret_cast<unsigned char*>(stx + stage_tokens);   // match length per position (0: none)
-        auto scan_pass = [&](int pass) {
-            const int pn = sh.r_pn;
-            while (true) {
-                int c = 0;
-                if (lane == 0) c = atomicAdd(&sh.scan_next[pass], 1);
-                c = __shfl_sync(FULL, c, 0);
-                if (c >= nchunks) break;
-#pragma unroll 1
-                for (int u = 0; u < 8; ++u) {
-                    const int e = c * 256 + u * 32 + lane;
-                    if (e >= t - 1) continue;
-                    if (pass == 0) {
-                        int l = 0;
-                        if (stx[e] == last) {
-                            l = 1;
-                            while (l < Lcap && e - l >= 0 && stx[e - l] == stx[t - 1 - l]) ++l;
-                            // equal lengths of the 32 positions are counted once (frequent last tokens
-                            // would otherwise all queue up at one counter)
-                            const unsigned grp = __match_any_sync(__activemask(), l);
-                            if (lane == __ffs(grp) - 1) atomicAdd(&sh.r_hist[l], __popc(grp));
-                        }
-                        sell[e] = (unsigned char)l;
-                    } else {
-                        const int l = sell[e];
-                        if (l >= pn) sh.r_list[sh.r_cum[l + 1] + atomicAdd(&sh.r_fill[l], 1)] = e;
-                    }
-                }
-            }
-        };
-        scan_pass(0);
-        group_sync();
-        if (gw == 0) {
-            int h = (lane + 1 <= Lcap) ? sh.r_hist[lane + 1] : 0;   // lane L: matches of exactly L + 1 tokens
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {                  // suffix sums: matches of at least L + 1 tokens
-                const int y = __shfl_down_sync(FULL, h, o);
-                if (lane + o < 32) h += y;
-            }
-            sh.r_cum[lane + 1] = h;
-            const unsigned few = __ballot_sync(FULL, h <= SD_OCC_LANES);
-            if (lane == 0) sh.r_pn = __ffs(few);                // (the counts fall with the length: lane 31 always qualifies)
-        }
-        group_sync();
-        if (staged && sh.r_cum[sh.r_pn] > 0) scan_pass(1);
         group_sync();
 
-        // ---------------- 2. the job queue, costliest first.  Per-request jobs that have to go through
-        // the tree (more than 32 occurrences, or no text in shared memory) come last: in sd_step
-        // they have to wait for the append.
-        // (order: the jobs that are read off the text first: they are quick and a long match there
-        // sets a score that rules out most of the others; then by the nodes a job can add at most)
+        // ---------------- 2. the job queue, by the number of nodes a job can add at most
         if (gtid < 2 * SD_MAX_DEPTH) {
             const int tree = gtid / SD_MAX_DEPTH, p = gtid % SD_MAX_DEPTH + 1;
             int c = 0;
@@ -1225,9 +957,7 @@ speculate_fused_kernel(sd_store sv, int n, const int32_t* __restrict__ d_slot, i
                 }
             } else if (want_r && p <= Pe && p <= t) {
                 c = min(budget_for(alpha, p, cap), 2 * (D - p));
-                if (staged && !(p <= Lcap && sh.r_cum[p] > 0)) c = 0;      // no earlier occurrence: nothing to speculate
-                else if (c > 0 && staged && p >= sh.r_pn) c += 2000;       // read off the text
-                else if (c > 0) c += 1000;                                  // through the request's tree: by cost among the global jobs
+                if (c > 0) c += 1000;
             }
             sh.cost[gtid] = c;
         }
@@ -1240,7 +970,7 @@ speculate_fused_kernel(sd_store sv, int n, const int32_t* __restrict__ d_slot, i
                     const int cq = sh.cost[q];
                     rank += (cq > c || (cq == c && q < gtid)) ? 1 : 0;
                 }
-                sh.job[rank] = gtid | ((c < 2000 && gtid >= SD_MAX_DEPTH) ? 128 : 0);   // bit 7: through the request's tree (sd_step: once the append is done)
+                sh.job[rank] = gtid;
                 atomicAdd(&sh.njobs, 1);
             }
         }
@@ -1256,7 +986,7 @@ speculate_fused_kernel(sd_store sv, int n, const int32_t* __restrict__ d_slot, i
             j = __shfl_sync(FULL, j, 0);
             if (j >= njobs) break;
             const int code = sh.job[j];
-            const int tree = (code & 127) / SD_MAX_DEPTH, p = (code & 127) % SD_MAX_DEPTH + 1;
+            const int tree = code / SD_MAX_DEPTH, p = code % SD_MAX_DEPTH + 1;
             const int budget = budget_for(alpha, p, cap);
             // SCORE <= number of draft nodes (every D <= 1), and SCORE <= number of levels below the
             // match node: the D values of one level of a tree add up to at most 1 (Eq. 1 shares out
@@ -1264,11 +994,6 @@ speculate_fused_kernel(sd_store sv, int n, const int32_t* __restrict__ d_slot, i
             if ((double)min(budget, D - p) * 1.000000001 < best_so_far(sh)) continue;
             if (tree == 0) {
                 expand_job(sh, W, sv.g_ent, (int)sv.g_cap, 0, p, budget, flags, false, 0, lane);
-            } else if (!(code & 128)) {
-                const int m = sh.r_cum[p];
-                const int e = lane < m ? sh.r_list[lane] : 0;
-                const int kmax = lane < m ? min(t - 1 - e, D - p) : 0;
-                expand_occ(sh, W, stx + e, kmax, 1, p, budget, flags, lane);
             } else {
                 // through the tree: the match node is the slot's active node of depth p, once the
                 // append is done (bounded wait; a job that runs out of patience is done after the
@@ -1411,22 +1136,15 @@ speculate_fused_kernel(sd_store sv, int n, const int32_t* __restrict__ d_slot, i
 
 namespace {
 
-constexpr int SMEM_PER_SM = 228 * 1024;       // shared memory of one SM; a resident block also costs 1 KB of it
 constexpr int MAX_DEVICES = 64;
 struct DeviceInfo { bool ready = false; int sm_count = 0; };
 DeviceInfo g_dev[MAX_DEVICES];
 std::mutex g_dev_mutex;
 
-// tokens of text a block of this shape can hold in shared memory beside its working set
-template <int WARPS, int MINB>
-constexpr int stage_limit_tokens() {
-    return (int)((SMEM_PER_SM / MINB - 1024 - (int)((sizeof(BlockSharedT<WARPS>) + 15) & ~(size_t)15)) / 5) & ~15;   // 4 + 1 bytes per token
-}
-
-template <bool STEP, int WARPS, int MINB, int G>
+template <bool STEP, int WARPS, int MINB>
 int raise_smem_limit() {
-    return cudaFuncSetAttribute(speculate_fused_kernel<STEP, WARPS, MINB, G>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                SMEM_PER_SM / MINB - 1024) == cudaSuccess ? SD_OK : SD_ERR_CUDA;
+    return cudaFuncSetAttribute(speculate_fused_kernel<STEP, WARPS, MINB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)sizeof(BlockSharedT<WARPS>)) == cudaSuccess ? SD_OK : SD_ERR_CUDA;
 }
 
 // once per device: raise the kernels' dynamic shared memory limit, read the SM count
@@ -1434,10 +1152,10 @@ int device_setup(int dev, int* sm_count) {
     if (dev < 0 || dev >= MAX_DEVICES) return SD_ERR_INVALID_ARG;
     std::lock_guard<std::mutex> lock(g_dev_mutex);
     if (!g_dev[dev].ready) {
-        if (raise_smem_limit<false, CTA_WARPS, 2, 8>() != SD_OK || raise_smem_limit<true, CTA_WARPS_STEP, 2, STEP_G>() != SD_OK ||
-            raise_smem_limit<false, CTA_WARPS_WIDE, 1, 8>() != SD_OK || raise_smem_limit<true, CTA_WARPS_WIDE_STEP, 1, 8>() != SD_OK ||
-            raise_smem_limit<false, CTA_WARPS_NARROW, 4, 8>() != SD_OK ||
-            raise_smem_limit<true, CTA_WARPS_NARROW_STEP, 4, STEP_G>() != SD_OK)
+        if (raise_smem_limit<false, CTA_WARPS, 2>() != SD_OK || raise_smem_limit<true, CTA_WARPS_STEP, 2>() != SD_OK ||
+            raise_smem_limit<false, CTA_WARPS_WIDE, 1>() != SD_OK || raise_smem_limit<true, CTA_WARPS_WIDE_STEP, 1>() != SD_OK ||
+            raise_smem_limit<false, CTA_WARPS_NARROW, 4>() != SD_OK ||
+            raise_smem_limit<true, CTA_WARPS_NARROW_STEP, 4>() != SD_OK)
             return SD_ERR_CUDA;
         SD_CUDA_OK(cudaDeviceGetAttribute(&g_dev[dev].sm_count, cudaDevAttrMultiProcessorCount, dev));
         g_dev[dev].ready = true;
@@ -1474,25 +1192,18 @@ static int launch_fused(sd_store* s, int32_t n, const int32_t* d_slot, const sd_
     const bool wide = n <= sms && (step || 2 * Pe > 2 * CTA_WARPS);
     // more requests than two 16-warp blocks per SM hold at once: smaller blocks, one wave
     const bool narrow = n > 2 * sms;
-    // Behind its working set a block keeps the request's text in shared memory if it fits (a
-    // longer text is not scanned: all of its per-request jobs go through the tree).
-#define SD_LAUNCH_FUSED(STEP, WARPS, MINB, G, OFF, TOK)                                                                 \
-    do {                                                                                                                 \
-        const int lim = stage_limit_tokens<WARPS, MINB>();                                                               \
-        const int stage = s->T <= lim ? ((s->T + 15) & ~15) : 0;                                                         \
-        const size_t smem = ((sizeof(BlockSharedT<WARPS>) + 15) & ~(size_t)15) + (size_t)stage * 5;                      \
-        speculate_fused_kernel<STEP, WARPS, MINB, G><<<(unsigned)n, WARPS * 32, smem, st>>>(                             \
-            *s, n, d_slot, Pe, prm->alpha, prm->max_spec, prm->flags, prm->tau, d_budget_cap, d_n_draft, d_tokens,       \
-            d_parents, d_positions, d_mask, d_chosen_tree, d_chosen_p, d_score, d_status, OFF, TOK, stage);              \
-    } while (0)
+#define SD_LAUNCH_FUSED(STEP, WARPS, MINB, OFF, TOK)                                                                     \
+    speculate_fused_kernel<STEP, WARPS, MINB><<<(unsigned)n, WARPS * 32, sizeof(BlockSharedT<WARPS>), st>>>(             \
+        *s, n, d_slot, Pe, prm->alpha, prm->max_spec, prm->flags, prm->tau, d_budget_cap, d_n_draft, d_tokens,           \
+        d_parents, d_positions, d_mask, d_chosen_tree, d_chosen_p, d_score, d_status, OFF, TOK)
     if (step) {
-        if (wide) SD_LAUNCH_FUSED(true, CTA_WARPS_WIDE_STEP, 1, 8, d_app_off, d_app_tok);
-        else if (narrow) SD_LAUNCH_FUSED(true, CTA_WARPS_NARROW_STEP, 4, STEP_G, d_app_off, d_app_tok);
-        else SD_LAUNCH_FUSED(true, CTA_WARPS_STEP, 2, STEP_G, d_app_off, d_app_tok);
+        if (wide) SD_LAUNCH_FUSED(true, CTA_WARPS_WIDE_STEP, 1, d_app_off, d_app_tok);
+        else if (narrow) SD_LAUNCH_FUSED(true, CTA_WARPS_NARROW_STEP, 4, d_app_off, d_app_tok);
+        else SD_LAUNCH_FUSED(true, CTA_WARPS_STEP, 2, d_app_off, d_app_tok);
     } else {
-        if (wide) SD_LAUNCH_FUSED(false, CTA_WARPS_WIDE, 1, 8, nullptr, nullptr);
-        else if (narrow) SD_LAUNCH_FUSED(false, CTA_WARPS_NARROW, 4, 8, nullptr, nullptr);
-        else SD_LAUNCH_FUSED(false, CTA_WARPS, 2, 8, nullptr, nullptr);
+        if (wide) SD_LAUNCH_FUSED(false, CTA_WARPS_WIDE, 1, nullptr, nullptr);
+        else if (narrow) SD_LAUNCH_FUSED(false, CTA_WARPS_NARROW, 4, nullptr, nullptr);
+        else SD_LAUNCH_FUSED(false, CTA_WARPS, 2, nullptr, nullptr);
     }
 #undef SD_LAUNCH_FUSED
     SD_CUDA_OK(cudaGetLastError());
