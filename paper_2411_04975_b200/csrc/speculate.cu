@@ -129,6 +129,32 @@ __device__ void push_children(const int4* __restrict__ ent, int cb, int n, doubl
     }
 }
 
+// ExpandSpeculationTree below the node with child run [cb, cb + n) as Algorithm 1 states it, one node
+// after the other: tokens and parents of the draft in insertion order, SCORE in `score`.  Whole warp.
+__device__ __noinline__ int expand_serial(const int4* __restrict__ ent, int cb0, int n0, int budget, unsigned flags, Frontier& F,
+                                          int32_t* out_tok, int32_t* out_par, double& score, int lane) {
+    int fh = 0, fs = 0, cnt = 0;
+    score = 0.0;
+    push_children(ent, cb0, n0, 1.0, -1, F, fh, fs, budget, lane);
+    while (cnt < budget && fs > 0) {
+        const double d = F.d[fh];
+        const int tok = F.tok[fh], par = F.par[fh], cb = F.cb[fh];
+        const int nc = (int)(F.nc[fh] & RUN_COUNT_MASK);
+        __syncwarp();
+        fh = (fh + 1) & (SD_MAX_SPEC - 1);
+        --fs;
+        if (lane == 0) { out_tok[cnt] = tok; out_par[cnt] = par; }
+        score = __dadd_rn(score, d);                            // Eq. 4, insertion order
+        const int idx = cnt++;
+        const int K = budget - cnt;
+        if (fs > K) fs = K;
+        if (flags & SD_FLAG_LINEAR) fs = 0;
+        push_children(ent, cb, nc, d, idx, F, fh, fs, K, lane);
+    }
+    __syncwarp();
+    return cnt;
+}
+
 __device__ __forceinline__ int budget_for(double alpha, int p, int cap) {
     const double b = floor(__dmul_rn(alpha, (double)p));        // Eq. 3
     if (b > (double)cap) return cap;
@@ -179,27 +205,9 @@ match_expand_kernel(sd_store sv, int n, const int32_t* __restrict__ d_slot, int 
             }
             if (node >= 0) {
                 // ---- ExpandSpeculationTree
-                Frontier& F = fr[wib];
-                int fh = 0, fs = 0;
                 const int4 e = ent[node];
-                push_children(ent, e.z, (int)((unsigned)e.w & RUN_COUNT_MASK), 1.0, -1, F, fh, fs, budget, lane);
-                int32_t* out_tok = sv.j_tok + rec * sv.M;
-                int32_t* out_par = sv.j_par + rec * sv.M;
-                while (cnt < budget && fs > 0) {
-                    const double d = F.d[fh];
-                    const int tok = F.tok[fh], par = F.par[fh], cb = F.cb[fh];
-                    const int nc = (int)(F.nc[fh] & RUN_COUNT_MASK);
-                    __syncwarp();
-                    fh = (fh + 1) & (SD_MAX_SPEC - 1);
-                    --fs;
-                    if (lane == 0) { out_tok[cnt] = tok; out_par[cnt] = par; }
-                    score = __dadd_rn(score, d);                // Eq. 4, insertion order
-                    const int idx = cnt++;
-                    const int K = budget - cnt;
-                    if (fs > K) fs = K;
-                    if (flags & SD_FLAG_LINEAR) fs = 0;
-                    push_children(ent, cb, nc, d, idx, F, fh, fs, K, lane);
-                }
+                cnt = expand_serial(ent, e.z, (int)((unsigned)e.w & RUN_COUNT_MASK), budget, flags, fr[wib], sv.j_tok + rec * sv.M,
+                                    sv.j_par + rec * sv.M, score, lane);
             }
         }
     }
@@ -282,9 +290,21 @@ constexpr int CTA_WARPS_WIDE_STEP = 16;        // registers to itself (80 per th
 constexpr int CTA_WARPS_NARROW = 8;            // batches of more than two requests per SM: four blocks per SM
 constexpr int CTA_WARPS_NARROW_STEP = 5;       // (sd_step: 96 registers)
 
-struct WarpWork {
-    Frontier F;
-    Frontier T;                               // scratch list for the children of one wide node
+// Candidates of one job: not ordered.  A candidate is put in once and looked for only when it is its turn, and most never
+// have one: the next node is usually the best child of the node just added, which one comparison with the
+// largest D in the pool tells.  (Keeping the candidates in order cost 1,800 cycles per node, two thirds of the job.)
+constexpr int POOL = 128;                     // four places per lane
+struct Pool {
+    double d[POOL];                           // 0: taken
+    int tok[POOL];
+    int cb[POOL];
+    unsigned nc[POOL];
+    unsigned char par[POOL];                  // parent index + 1
+};
+
+struct __align__(16) WarpWork {
+    Pool C;
+    Frontier T;                               // children of a wide node, by count (F of a wide match node's slices)
     int one_tok[SD_MAX_SPEC];                 // its first children of count 1, in token order
     int one_cb[SD_MAX_SPEC];
     unsigned one_nc[SD_MAX_SPEC];
@@ -300,7 +320,7 @@ struct BlockSharedT {
     int node[2][SD_MAX_DEPTH];                // match node per tree and pattern length (-1: none)
     int cb[2][SD_MAX_DEPTH];                  // its child run
     unsigned nc[2][SD_MAX_DEPTH];             // ... as the node's w field (count | flags)
-    int cost[2 * SD_MAX_DEPTH];
+    unsigned char ordp[SD_MAX_DEPTH];         // pattern lengths - 1 by the number of nodes their jobs can add at most
     int job[2 * SD_MAX_DEPTH];
     int wide[2 * SD_MAX_DEPTH];               // jobs whose match node has a wide child run
     int njobs, next, nwide, nwide_kept;
@@ -314,7 +334,8 @@ struct BlockSharedT {
     unsigned best_hi;                         // high word of the largest SCORE reached so far: a lower
                                               // bound of it (scores are non-negative doubles), which is
                                               // all the pruning needs; 32 bits keep the atomic native
-    int win_warp;
+    unsigned long long anc[SD_MAX_SPEC];      // ancestors of the chosen tree's nodes
+    signed char up[SD_MAX_SPEC];
 };
 
 __device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
@@ -400,146 +421,6 @@ __device__ __forceinline__ int4 load_window(const int4* __restrict__ ent, int ba
     return idx < limit ? ent[idx] : make_int4(-1, 0, 0, 0);
 }
 
-// A child that was not put into the frontier because it would be taken out again at once.
-struct Taken {
-    bool any;
-    double d;
-    int tok, cb;
-    unsigned w;
-};
-
-// Offer the children of a node to the frontier; `w` already holds the first 32 entries of the run.
-// With `take` (runs of at most 32 children): if the best child (largest count, then smallest
-// token: among siblings that is the order of D) beats every waiting candidate, it is the next
-// node to be added whatever else is offered, so it is handed back instead of being merged in
-// and popped again; the frontier is then bounded by K - 1.
-__device__ void push_children_w(const int4* __restrict__ ent, int cb, int n, int4 w, double d_parent, int par_index,
-                                Frontier& F, int fh, int& fs, int K, int lane, Taken* take = nullptr) {
-    if (take) take->any = false;
-    if (n <= 0 || K <= 0) return;
-    // sibling sum: the denominator of Eq. 1 (a parent's occurrences fit 31 bits)
-    unsigned part = lane < n ? (unsigned)w.y : 0u;
-    for (int base = 32; base < n; base += 128) {                // wide runs: four loads in flight
-        int y[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) { const int idx = base + u * 32 + lane; y[u] = idx < n ? ent[cb + idx].y : 0; }
-        part += (unsigned)(y[0] + y[1] + y[2] + y[3]);
-    }
-    const unsigned sum = __reduce_add_sync(FULL, part);
-    const double dsum = (double)sum;
-    int skip = -1;                                              // child handed back through `take`
-    if (take && n <= 32) {
-        const unsigned cmax = __reduce_max_sync(FULL, lane < n ? (unsigned)w.y : 0u);
-        const int b = __ffs(__ballot_sync(FULL, lane < n && (unsigned)w.y == cmax)) - 1;
-        const double db = __dmul_rn(d_parent, __ddiv_rn((double)cmax, dsum));    // Eq. 2 with Eq. 1
-        const int tb = __shfl_sync(FULL, w.x, b);
-        if (fs == 0 || better(db, tb, par_index, F.d[fh], F.tok[fh], F.par[fh])) {
-            take->any = true; take->d = db; take->tok = tb;
-            take->cb = __shfl_sync(FULL, w.z, b);
-            take->w = (unsigned)__shfl_sync(FULL, w.w, b);
-            skip = b;
-            --K;                                                // one node fewer is still to come
-            if (fs > K) fs = K;
-            if (K <= 0 || n == 1) return;
-        }
-    }
-    // With a full frontier only a child that beats its worst entry matters:
-    // D = d_parent * count / sum, so counts below `cmin` lose without any fp64 work.
-    double ld = 0.0, need = 0.0; int lt = 0, lp = 0;
-    const bool full = fs == K;
-    if (full) {
-        const int last = (fh + fs - 1) & (SD_MAX_SPEC - 1);
-        ld = F.d[last]; lt = F.tok[last]; lp = F.par[last];
-        need = ld * dsum * 0.999999;                            // count * d_parent must reach this
-    }
-    for (int base = 0; base < n; base += 32) {
-        const int idx = base + lane;
-        int4 e = w;
-        if (base != 0) { e = make_int4(0, 0, 0, 0); if (idx < n) e = ent[cb + idx]; }
-        bool pass = idx < n && idx != skip && (double)e.y * d_parent >= need;
-        if (!__any_sync(FULL, pass)) continue;
-        double dc = 0.0;
-        if (pass) {
-            dc = __dmul_rn(d_parent, __ddiv_rn((double)e.y, dsum));      // Eq. 2 with Eq. 1
-            if (full) pass = better(dc, e.x, par_index, ld, lt, lp);
-            if (pass && ((unsigned)e.w & RUN_COUNT_MASK)) prefetch_l2(ent + e.z);   // likely looked at soon
-        }
-        if (fs == 0 && n <= 32) {
-            // Nothing waits yet (the first children of a job): the candidates are siblings, and
-            // among siblings the order of D is the order of (count, then token).  Their places
-            // follow from one pass per distinct count, largest first, without any merging.
-            unsigned rem = __ballot_sync(FULL, pass);
-            const int np = __popc(rem);
-            const unsigned below = (1u << lane) - 1u;
-            int place = -1, taken = 0;
-            while (rem && taken < K) {
-                const bool in = (rem >> lane) & 1u;
-                const unsigned top = __reduce_max_sync(FULL, in ? (unsigned)e.y : 0u);
-                const unsigned grp = __ballot_sync(FULL, in && (unsigned)e.y == top);
-                if ((grp >> lane) & 1u) place = taken + __popc(grp & below);
-                taken += __popc(grp);
-                rem &= ~grp;
-            }
-            if (place >= 0 && place < K) {
-                const int q = (fh + place) & (SD_MAX_SPEC - 1);
-                F.d[q] = dc; F.tok[q] = e.x; F.par[q] = par_index; F.cb[q] = e.z; F.nc[q] = (unsigned)e.w;
-            }
-            __syncwarp();
-            fs = min(np, K);
-            return;
-        }
-        frontier_merge(F, fh, fs, K, pass, dc, e.x, par_index, e.z, (unsigned)e.w, lane);
-        if (!full && fs == K) {                                 // it filled up while merging
-            const int last = (fh + fs - 1) & (SD_MAX_SPEC - 1);
-            const double d2 = F.d[last];
-            const int t2 = F.tok[last], p2 = F.par[last];
-            // from here on compare exactly against the new worst entry (no count shortcut)
-            for (int b2 = base + 32; b2 < n; b2 += 32) {
-                const int i2 = b2 + lane;
-                int4 e2 = make_int4(0, 0, 0, 0);
-                if (i2 < n) e2 = ent[cb + i2];
-                double dc2 = 0.0;
-                bool pass2 = i2 < n;
-                if (pass2) {
-                    dc2 = __dmul_rn(d_parent, __ddiv_rn((double)e2.y, dsum));
-                    const int l3 = (fh + fs - 1) & (SD_MAX_SPEC - 1);
-                    pass2 = better(dc2, e2.x, par_index, F.d[l3], F.tok[l3], F.par[l3]);
-                }
-                frontier_merge(F, fh, fs, K, pass2, dc2, e2.x, par_index, e2.z, (unsigned)e2.w, lane);
-            }
-            (void)d2; (void)t2; (void)p2;
-            return;
-        }
-    }
-}
-
-// Children of a node whose run has a top block (see RUN_HAS_TOP): the 64 best by count are
-// listed, best first, right before the run, together with the sum of all counts.
-__device__ void push_top(const int4* __restrict__ ent, int cb, double d_parent, int par_index, Frontier& F, int fh,
-                         int& fs, int K, int lane) {
-    if (K <= 0) return;
-    const int4 hdr = ent[cb - SD_TOP_BLOCK];
-    const double dsum = (double)(((unsigned long long)(unsigned)hdr.y << 32) | (unsigned long long)(unsigned)hdr.x);
-    const int ntop = min(hdr.z, K);                             // only the K best can enter
-    for (int base = 0; base < ntop; base += 32) {
-        const int idx = base + lane;
-        bool pass = idx < ntop;
-        int4 e = make_int4(0, 0, 0, 0);
-        double dc = 0.0;
-        if (pass) {
-            e = ent[cb - SD_TOP_BLOCK + 1 + idx];
-            dc = __dmul_rn(d_parent, __ddiv_rn((double)e.y, dsum));      // Eq. 2 with Eq. 1
-            if (fs == K) {
-                const int last = (fh + fs - 1) & (SD_MAX_SPEC - 1);
-                pass = better(dc, e.x, par_index, F.d[last], F.tok[last], F.par[last]);
-            }
-            if (pass && ((unsigned)e.w & RUN_COUNT_MASK)) prefetch_l2(ent + e.z);
-        }
-        if (!__any_sync(FULL, pass)) break;                     // best first: nothing further can enter
-        frontier_merge(F, fh, fs, K, pass, dc, e.x, par_index, e.z, (unsigned)e.w, lane);
-    }
-}
-
 constexpr int WIDE_RUN = 256;                 // child runs longer than this are scanned by several warps
 
 // One pass over chunks first, first + stride, ... of a child run: adds up the counts and keeps
@@ -612,73 +493,307 @@ __device__ __forceinline__ double best_so_far(BlockShared& sh) {
     return __hiloint2double((int)__shfl_sync(FULL, *(volatile unsigned*)&sh.best_hi, 0), 0);
 }
 
-// ExpandSpeculationTree + SCORE for one (tree, p) job by one warp.  With `seeded` the frontier
-// already holds the match node's children (fs entries from ring head 0).
+// The state of a job's pool that lives in registers.
+struct PoolState {
+    int n;                                    // places used
+    unsigned top;                             // high word of the largest D in it (0: empty)
+    unsigned floor;                           // candidates whose D has a smaller high word do not matter
+};
+
+// Leaves at least the `room` best candidates and few others: the rest cannot be taken any more.
+__device__ __noinline__ PoolState pool_compact(Pool& C, PoolState P, int room, int lane) {
+    unsigned h[4];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) h[c] = c * 32 + lane < P.n ? (unsigned)__double2hiint(C.d[c * 32 + lane]) : 0u;
+    unsigned lo = 1u, hi = P.top;                               // the largest limit with at least `room` candidates at or above it
+    int at_lo = 0;
+#pragma unroll
+    for (int c = 0; c < 4; ++c) at_lo += __popc(__ballot_sync(FULL, h[c] != 0u));
+    if (at_lo > room) {
+        for (int it = 0; it < 32 && lo < hi && at_lo > room + 8; ++it) {
+            const unsigned mid = lo + (hi - lo + 1u) / 2u;
+            int k = 0;
+#pragma unroll
+            for (int c = 0; c < 4; ++c) k += __popc(__ballot_sync(FULL, h[c] >= mid));
+            if (k >= room) { lo = mid; at_lo = k; } else hi = mid - 1u;
+        }
+    }
+    // (those at the limit may be more than the places: equal D; the first by token are what counts, so they all stay
+    // unless they fill the pool, which the caller checks)
+    double d[4]; int tok[4], cb[4]; unsigned nc[4]; unsigned char par[4];
+#pragma unroll
+    for (int c = 0; c < 4; ++c)
+        if (h[c] >= lo) { const int i = c * 32 + lane; d[c] = C.d[i]; tok[c] = C.tok[i]; cb[c] = C.cb[i]; nc[c] = C.nc[i]; par[c] = C.par[i]; }
+    __syncwarp();
+    int n = 0;
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+        const unsigned m = __ballot_sync(FULL, h[c] >= lo);
+        if (h[c] >= lo) {
+            const int i = n + __popc(m & ((1u << lane) - 1u));
+            C.d[i] = d[c]; C.tok[i] = tok[c]; C.cb[i] = cb[c]; C.nc[i] = nc[c]; C.par[i] = par[c];
+        }
+        n += __popc(m);
+    }
+    __syncwarp();
+    P.n = n;
+    if (at_lo >= room) P.floor = max(P.floor, lo);
+    return P;
+}
+
+// Puts one candidate per lane with `keep` into the pool.  `room`: nodes that can still be added.  False: no
+// place (more than POOL - 32 candidates that all may matter: equal D).
+__device__ __forceinline__ bool pool_push(Pool& C, PoolState& P, int room, bool keep, double d, int tok, int par, int cb, unsigned nc,
+                                          int lane) {
+    const unsigned h = (unsigned)__double2hiint(d);
+    keep = keep && h >= P.floor;
+    const unsigned m = __ballot_sync(FULL, keep);
+    if (!m) return true;
+    if (P.n + __popc(m) > POOL) {
+        P = pool_compact(C, P, room, lane);
+        if (P.n + __popc(m) > POOL) return false;
+    }
+    if (keep) {
+        const int i = P.n + __popc(m & ((1u << lane) - 1u));
+        C.d[i] = d; C.tok[i] = tok; C.cb[i] = cb; C.nc[i] = nc; C.par[i] = (unsigned char)(par + 1);
+    }
+    P.n += __popc(m);
+    P.top = max(P.top, __reduce_max_sync(FULL, keep ? h : 0u));
+    __syncwarp();
+    return true;
+}
+
+// Place of the best candidate: larger D, then smaller token, then smaller parent index.  It leaves the pool (its
+// fields stay readable).  P.top > 0.  Where several share the largest D (`ties` of them, at most 32), none is taken:
+// their places are in `list`.
+__device__ __forceinline__ int pool_pop(Pool& C, PoolState& P, int* list, bool turns, int& ties, int lane) {
+    unsigned h[4];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+        h[c] = 0u;
+        if (c * 32 < P.n && c * 32 + lane < P.n) h[c] = (unsigned)__double2hiint(C.d[c * 32 + lane]);
+    }
+    int at = -1, eq = 0;
+    unsigned rest = 0u;                                         // the largest below the top
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+        if (c * 32 >= P.n) break;
+        const unsigned b = __ballot_sync(FULL, h[c] == P.top);
+        if (b && at < 0) at = c * 32 + __ffs(b) - 1;
+        eq += __popc(b);
+        if (h[c] != P.top) rest = max(rest, h[c]);
+    }
+    ties = 0;
+    if (eq == 1) {
+        P.top = __reduce_max_sync(FULL, rest);
+        return at;
+    }
+    // several share the high word: full comparison
+    double bd = -1.0;
+    int bt = 0x7fffffff, bp = 0x7fffffff, bi = -1;
+#pragma unroll
+    for (int c = 0; c < 4; ++c)
+        if (h[c] == P.top) {
+            const int i = c * 32 + lane;
+            const double d = C.d[i];
+            const int t = C.tok[i], p = C.par[i];
+            if (bi < 0 || better(d, t, p, bd, bt, bp)) { bd = d; bt = t; bp = p; bi = i; }
+        }
+    const unsigned mlo = __reduce_max_sync(FULL, bi >= 0 ? (unsigned)__double2loint(bd) : 0u);
+    int g = 0;
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+        const int i = c * 32 + lane;
+        const bool same = h[c] == P.top && (unsigned)__double2loint(C.d[i]) == mlo;
+        const unsigned m = __ballot_sync(FULL, same);
+        const int k = g + __popc(m & ((1u << lane) - 1u));
+        if (same && k < 32) list[k] = i;
+        g += __popc(m);
+    }
+    __syncwarp();
+    if (g > 1 && g <= 32 && turns) { ties = g; return -1; }
+    const bool in2 = bi >= 0 && (unsigned)__double2loint(bd) == mlo;
+    const unsigned mt = __reduce_min_sync(FULL, in2 ? (unsigned)bt : 0xffffffffu);
+    const bool in3 = in2 && (unsigned)bt == mt;
+    const unsigned mp = __reduce_min_sync(FULL, in3 ? (unsigned)bp : 0xffffffffu);
+    const int src = __ffs(__ballot_sync(FULL, in3 && (unsigned)bp == mp)) - 1;
+    return __shfl_sync(FULL, bi, src);                          // (others have the same high word: P.top stays)
+}
+
+// The largest high word in the pool.
+__device__ __forceinline__ unsigned pool_top(const Pool& C, int n, int lane) {
+    unsigned top = 0u;
+    for (int i = lane; i < n; i += 32) top = max(top, (unsigned)__double2hiint(C.d[i]));
+    return __reduce_max_sync(FULL, top);
+}
+
+// The best children (by count, then smallest token; at most `room`) of a node with more than 32: their entries, best
+// first, in `list`.  One class of equal counts after the other, within it in run (token) order.
+__device__ __noinline__ int list_by_count(const int4* __restrict__ ent, int cb, int n, int room, int* list, unsigned& sum_out, int lane) {
+    unsigned sum = 0, top = 0;
+    for (int base = lane; base < n; base += 128) {
+        unsigned y[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) y[u] = base + u * 32 < n ? (unsigned)ent[cb + base + u * 32].y : 0u;
+        sum += y[0] + y[1] + y[2] + y[3];                       // (a parent's occurrences fit 31 bits)
+        top = max(top, max(max(y[0], y[1]), max(y[2], y[3])));
+    }
+    sum_out = __reduce_add_sync(FULL, sum);
+    top = __reduce_max_sync(FULL, top);
+    int taken = 0;
+    while (top > 0u && taken < room) {
+        unsigned next = 0;
+        for (int base = 0; base < n; base += 128) {
+            unsigned y[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) y[u] = base + u * 32 + lane < n ? (unsigned)ent[cb + base + u * 32 + lane].y : 0u;
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const unsigned m = __ballot_sync(FULL, y[u] == top);
+                const int at = taken + __popc(m & ((1u << lane) - 1u));
+                if (y[u] == top && at < room) list[at] = cb + base + u * 32 + lane;
+                taken += __popc(m);
+                if (y[u] < top) next = max(next, y[u]);
+            }
+        }
+        top = __reduce_max_sync(FULL, next);
+    }
+    __syncwarp();
+    return min(taken, room);
+}
+
+// ExpandSpeculationTree + SCORE for one (tree, p) job by one warp.  nseed >= 0: the match node's best
+// children are in W.T (nseed of them, from ring head 0, with their D).
 template <class BlockShared>
-__device__ void expand_job(BlockShared& sh, WarpWork& W, const int4* __restrict__ ent, int limit, int tree, int p,
-                           int budget, unsigned flags, bool seeded, int fs, int lane) {
+__device__ __noinline__ void expand_job(BlockShared& sh, WarpWork& W, const int4* __restrict__ ent, int limit, int tree, int p,
+                           int budget, unsigned flags, int nseed, int lane) {
     const int order = tree * SD_MAX_DEPTH + p;                  // loop order of Algorithm 1
     const int buf = W.best_buf ^ 1;
-    int fh = 0, cnt = 0;
+    Pool& C = W.C;
+    PoolState P{0, 0u, 0u};
+    int cnt = 0;
     double score = 0.0;
-    bool dropped = false;
+    bool dropped = false, fits = true;
     // the node whose children are to be offered next: the match node first, D(N_p) = 1
     double cur_d = 1.0;
     int cur_cb = sh.cb[tree][p - 1], cur_idx = -1;
     unsigned cur_w = sh.nc[tree][p - 1];
-    int cur_n = (int)(cur_w & RUN_COUNT_MASK);
-    bool have_cur = !seeded;
-    if (!seeded) fs = 0;
+    bool have_cur = nseed < 0;
+    for (int base = 0; base < nseed && fits; base += 32) {
+        const int q = base + lane;
+        const bool keep = q < nseed;
+        fits = pool_push(C, P, budget, keep, keep ? W.T.d[q] : 0.0, keep ? W.T.tok[q] : 0, -1, keep ? W.T.cb[q] : 0, keep ? W.T.nc[q] : 0u, lane);
+    }
     int4 w = make_int4(-1, 0, 0, 0);                            // window in registers: entries wb .. wb + wvalid
     int wb = -1, wvalid = 0;
-    while (true) {
+    while (fits) {
         if (!have_cur) {
-            if (cnt >= budget || fs == 0) break;
-            cur_d = W.F.d[fh];
-            const int tok = W.F.tok[fh], par = W.F.par[fh];
-            cur_cb = W.F.cb[fh];
-            cur_w = W.F.nc[fh];
-            cur_n = (int)(cur_w & RUN_COUNT_MASK);
+            if (cnt >= budget || P.top == 0u) break;
+            int ties;
+            const int at = pool_pop(C, P, W.one_tok, !(flags & SD_FLAG_LINEAR), ties, lane);
+            if (ties > 0) {
+                // Candidates of equal D take turns: smallest token first, then smallest parent index, and an
+                // only child (C = 1: the same D again) takes its parent's place.  All of them are ahead of every
+                // other candidate, so a lane each keeps them until one has several children or all have ended.
+                // (Text that occurs a few times below the match node is just this: chains of equal D, token by token in
+                // turn.  Through the pool a node of them costs ten times as much.)
+                const bool mine = lane < ties;
+                const int place = mine ? W.one_tok[lane] : 0;
+                bool live = mine;
+                int tok = 0, par = 0, cb = 0;
+                unsigned nc = 0;
+                int4 nx = make_int4(0, 0, 0, 0);                // the only child, read ahead
+                if (mine) {
+                    tok = C.tok[place]; par = C.par[place]; cb = C.cb[place]; nc = C.nc[place];
+                    if ((nc & RUN_COUNT_MASK) == 1u) nx = ent[cb];
+                }
+                cur_d = C.d[W.one_tok[0]];
+                unsigned alive = (ties == 32 ? FULL : (1u << ties) - 1u);
+                while (cnt < budget) {
+                    if ((cnt & 3) == 0 && (score + (double)(budget - cnt) * cur_d) * 1.000000001 < best_so_far(sh)) { dropped = true; break; }
+                    const unsigned mt = __reduce_min_sync(FULL, live ? (unsigned)tok : 0xffffffffu);
+                    unsigned who = __ballot_sync(FULL, live && (unsigned)tok == mt);
+                    if (who & (who - 1u)) {
+                        const bool in = (who >> lane) & 1u;
+                        const unsigned mp = __reduce_min_sync(FULL, in ? (unsigned)par : 0xffffffffu);
+                        who = __ballot_sync(FULL, in && (unsigned)par == mp);
+                    }
+                    const int wl = __ffs(who) - 1;
+                    const int n = (int)(__shfl_sync(FULL, nc, wl) & RUN_COUNT_MASK);
+                    if (lane == wl) {
+                        W.tok[buf][cnt] = tok; W.par[buf][cnt] = (unsigned char)par;
+                        if (n == 1) {
+                            tok = nx.x; par = cnt + 1; cb = nx.z; nc = (unsigned)nx.w;
+                            if ((nc & RUN_COUNT_MASK) == 1u) nx = ent[cb];
+                        } else live = false;
+                    }
+                    score = __dadd_rn(score, cur_d);            // Eq. 4, insertion order
+                    ++cnt;
+                    if (n == 1) continue;
+                    alive &= ~(1u << wl);
+                    if (n > 1) {
+                        have_cur = true;
+                        cur_idx = cnt - 1;
+                        cur_cb = __shfl_sync(FULL, cb, wl);
+                        cur_w = __shfl_sync(FULL, nc, wl);
+                        break;
+                    }
+                    if (!alive) break;
+                }
+                if (dropped) break;
+                if (lane == 0) atomicMax(&sh.best_hi, (unsigned)__double2hiint(score));
+                if (mine) {
+                    if (live) { C.tok[place] = tok; C.par[place] = (unsigned char)par; C.cb[place] = cb; C.nc[place] = nc; }
+                    else C.d[place] = 0.0;
+                }
+                __syncwarp();
+                if (!alive) P.top = pool_top(C, P.n, lane);
+                if (!have_cur || cnt >= budget) continue;
+            } else {
+            cur_d = C.d[at];
+            const int tok = C.tok[at], par = C.par[at];
+            cur_cb = C.cb[at];
+            cur_w = C.nc[at];
             // everything still to come is at most cur_d each
             if ((score + (double)(budget - cnt) * cur_d) * 1.000000001 < best_so_far(sh)) { dropped = true; break; }
             __syncwarp();
-            fh = (fh + 1) & (SD_MAX_SPEC - 1);
-            --fs;
-            if (lane == 0) { W.tok[buf][cnt] = tok; W.par[buf][cnt] = (unsigned char)(par + 1); }
+            if (lane == 0) { C.d[at] = 0.0; W.tok[buf][cnt] = tok; W.par[buf][cnt] = (unsigned char)par; }
             score = __dadd_rn(score, cur_d);                    // Eq. 4, insertion order
             // the final SCORE of this job is at least its running value: let the others prune on it
             if (lane == 0) atomicMax(&sh.best_hi, (unsigned)__double2hiint(score));
             cur_idx = cnt++;
-            const int K = budget - cnt;
-            if (fs > K) fs = K;
-            if (flags & SD_FLAG_LINEAR) fs = 0;
+            if (flags & SD_FLAG_LINEAR) { P.n = 0; P.top = 0u; P.floor = 0u; }
+            __syncwarp();
+            }
         }
         have_cur = false;
         if (cnt >= budget) break;
+        const int cur_n = (int)(cur_w & RUN_COUNT_MASK);
         if (cur_n == 0) continue;
-        if (cur_w & RUN_HAS_TOP) {                              // long run with a ready-made list of its best children
-            push_top(ent, cur_cb, cur_d, cur_idx, W.F, fh, fs, budget - cnt, lane);
-            continue;
-        }
         if (cur_n > 32) {
-            // wide run: one pass that keeps the best children by count, then D for those only
-            const int K = budget - cnt;
-            long long sum;
-            if (fs == 0) {
-                scan_run_by_count(ent, cur_cb, cur_n, 0, 1, cur_idx, 1, W, W.F, fh, fs, K, sum, lane);
-                counts_to_d(W.F, fh, fs, cur_d, sum, lane);
-            } else if (fs == K) {
-                // full frontier: sum pass, then a pass that only looks at counts large enough
-                prefetch_run(ent, cur_cb, cur_n, lane, 64);
-                push_children_w(ent, cur_cb, cur_n, load_window(ent, cur_cb, limit, lane), cur_d, cur_idx, W.F, fh, fs, K,
-                                lane);
+            // a long run: only the best of its children, by count, can ever be added.  A ready-made list of them
+            // stands in front of the run, or is made here.
+            const int room = budget - cnt;
+            double dsum;
+            int nl;
+            if (cur_w & RUN_HAS_TOP) {
+                const int4 hdr = ent[cur_cb - SD_TOP_BLOCK];
+                dsum = (double)(((unsigned long long)(unsigned)hdr.y << 32) | (unsigned long long)(unsigned)hdr.x);
+                nl = min(hdr.z, room);
             } else {
-                // some candidates wait and there is room for more: the K best children by count go
-                // into a list of their own, which is then merged in
-                int ts;
-                scan_run_by_count(ent, cur_cb, cur_n, 0, 1, cur_idx, 1, W, W.T, 0, ts, K, sum, lane);
-                counts_to_d(W.T, 0, ts, cur_d, sum, lane);
-                frontier_merge_list(W.F, fh, fs, K, W.T, ts, cur_idx, lane);
+                unsigned sum;
+                nl = list_by_count(ent, cur_cb, cur_n, room, W.one_tok, sum, lane);
+                dsum = (double)sum;
+            }
+            for (int base = 0; base < nl && fits; base += 32) {
+                const bool keep = base + lane < nl;
+                int4 e = make_int4(0, 0, 0, 0);
+                double dc = 0.0;
+                if (keep) {
+                    e = ent[(cur_w & RUN_HAS_TOP) ? cur_cb - SD_TOP_BLOCK + 1 + base + lane : W.one_tok[base + lane]];
+                    dc = __dmul_rn(cur_d, __ddiv_rn((double)e.y, dsum));         // Eq. 2 with Eq. 1
+                }
+                fits = pool_push(C, P, room, keep, dc, e.x, cur_idx, e.z, (unsigned)e.w, lane);
             }
             continue;
         }
@@ -697,7 +812,8 @@ __device__ void expand_job(BlockShared& sh, WarpWork& W, const int4* __restrict_
                 wvalid = min(32, limit - cur_cb);
             }
         }
-        if (cur_n == 1 && (fs == 0 || W.F.d[fh] < cur_d)) {
+        const unsigned cur_hi = (unsigned)__double2hiint(cur_d);
+        if (cur_n == 1 && P.top < cur_hi) {
             // An only child has C = 1, so D stays cur_d: while the best waiting candidate is
             // strictly worse, the whole chain of only children is added in one go.
             const bool link = lane < wvalid && ((unsigned)w.w & RUN_COUNT_MASK) == 1u && w.z == cur_cb + lane + 1;
@@ -711,31 +827,50 @@ __device__ void expand_job(BlockShared& sh, WarpWork& W, const int4* __restrict_
             for (int q = 0; q < m; ++q) score = __dadd_rn(score, cur_d);
             if (lane == 0) atomicMax(&sh.best_hi, (unsigned)__double2hiint(score));
             cnt += m;
-            if (fs > budget - cnt) fs = budget - cnt;
             cur_idx = cnt - 1;
             cur_cb = __shfl_sync(FULL, w.z, m - 1);
             cur_w = (unsigned)__shfl_sync(FULL, w.w, m - 1);
-            cur_n = (int)(cur_w & RUN_COUNT_MASK);
             have_cur = true;
             if ((score + (double)(budget - cnt) * cur_d) * 1.000000001 < best_so_far(sh)) { dropped = true; break; }
             continue;
         }
-        Taken tk;
-        push_children_w(ent, cur_cb, cur_n, w, cur_d, cur_idx, W.F, fh, fs, budget - cnt, lane, &tk);
-        if (tk.any) {
-            // the same steps as taking it from the frontier at the top of the loop
-            if ((score + (double)(budget - cnt) * tk.d) * 1.000000001 < best_so_far(sh)) { dropped = true; break; }
-            if (lane == 0) { W.tok[buf][cnt] = tk.tok; W.par[buf][cnt] = (unsigned char)(cur_idx + 1); }
-            score = __dadd_rn(score, tk.d);
+        // ---- D of the children; the best of them (largest count, then smallest token: among siblings the order of D)
+        // is the next node to be added if it beats every waiting candidate
+        const bool in = lane < cur_n;
+        const unsigned y = in ? (unsigned)w.y : 0u;
+        const unsigned sum = __reduce_add_sync(FULL, y), most = __reduce_max_sync(FULL, y);      // sibling sum: the denominator of Eq. 1
+        const int b = __ffs(__ballot_sync(FULL, in && y == most)) - 1;
+        const double dc = __dmul_rn(cur_d, __ddiv_rn((double)y, (double)sum));                   // Eq. 2 with Eq. 1
+        const unsigned best_hi = (unsigned)__shfl_sync(FULL, __double2hiint(dc), b);
+        const bool take = best_hi > P.top;
+        if (cur_n > 1 || !take)
+            fits = pool_push(C, P, budget - cnt - (take ? 1 : 0), in && !(take && lane == b), dc, w.x, cur_idx, w.z, (unsigned)w.w, lane);
+        if (take) {
+            // the same steps as taking it from the pool at the top of the loop
+            cur_d = __hiloint2double((int)best_hi, __shfl_sync(FULL, __double2loint(dc), b));
+            if ((score + (double)(budget - cnt) * cur_d) * 1.000000001 < best_so_far(sh)) { dropped = true; break; }
+            const int tok = __shfl_sync(FULL, w.x, b);
+            if (lane == 0) { W.tok[buf][cnt] = tok; W.par[buf][cnt] = (unsigned char)(cur_idx + 1); }
+            score = __dadd_rn(score, cur_d);
             if (lane == 0) atomicMax(&sh.best_hi, (unsigned)__double2hiint(score));
             cur_idx = cnt++;
-            cur_d = tk.d; cur_cb = tk.cb; cur_w = tk.w;
-            cur_n = (int)(cur_w & RUN_COUNT_MASK);
-            if (flags & SD_FLAG_LINEAR) fs = 0;
+            cur_cb = __shfl_sync(FULL, w.z, b);
+            cur_w = (unsigned)__shfl_sync(FULL, w.w, b);
+            if (flags & SD_FLAG_LINEAR) { P.n = 0; P.top = 0u; P.floor = 0u; }
             have_cur = true;
         }
     }
     __syncwarp();
+    if (!fits) {
+        // more candidates of equal D than the pool holds: one node after the other, with the candidates in order
+        Frontier& F = W.T;
+        int* const otok = W.one_tok;
+        int* const opar = W.one_cb;
+        cnt = expand_serial(ent, sh.cb[tree][p - 1], (int)(sh.nc[tree][p - 1] & RUN_COUNT_MASK), budget, flags, F, otok, opar, score, lane);
+        for (int j = lane; j < cnt; j += 32) { W.tok[buf][j] = otok[j]; W.par[buf][j] = (unsigned char)(opar[j] + 1); }
+        dropped = false;
+        __syncwarp();
+    }
     if (!dropped && (score > W.best_score || (score == W.best_score && score > 0.0 && order < W.best_order))) {
         if (lane == 0) {
             W.best_score = score; W.best_order = order; W.best_n = cnt; W.best_buf = buf;
@@ -770,7 +905,7 @@ __device__ void request_tree_job(BlockShared& sh, WarpWork& W, const sd_store& s
         if (lane == 0) sh.wide[atomicAdd(&sh.nwide, 1)] = SD_MAX_DEPTH + p - 1;
         return;
     }
-    expand_job(sh, W, s_ent, (int)sv.spn, 1, p, budget, flags, false, 0, lane);
+    expand_job(sh, W, s_ent, (int)sv.spn, 1, p, budget, flags, -1, lane);
 }
 
 // One block of W warps per request.
@@ -838,8 +973,18 @@ speculate_fused_kernel(sd_store sv, int n, const int32_t* __restrict__ d_slot, i
     if (d_budget_cap && d_budget_cap[i] >= 0) cap = min(cap, d_budget_cap[i]);
     if (tid < 2 * SD_MAX_DEPTH) { (&sh.node[0][0])[tid] = -1; (&sh.nc[0][0])[tid] = 0; }
     if (tid == 0) {
-        sh.njobs = 0; sh.next = 0; sh.nwide = 0; sh.nwide_kept = 0; sh.best_hi = 0u; sh.win_warp = -1;
+        sh.njobs = 0; sh.next = 0; sh.nwide = 0; sh.nwide_kept = 0; sh.best_hi = 0u;
         sh.app_done = 0; sh.nlate = 0; sh.app.ahead = 0;
+    }
+    if (wib == WARPS - 1) {
+        const int c = lane < Pe ? min(budget_for(alpha, lane + 1, cap), 2 * (D - lane - 1)) : -1;
+        int rank = 0;
+#pragma unroll
+        for (int q = 0; q < 32; ++q) {
+            const int cq = __shfl_sync(FULL, c, q);
+            rank += (cq > c || (cq == c && q < lane)) ? 1 : 0;
+        }
+        sh.ordp[rank] = (unsigned char)lane;
     }
     WarpWork& W = sh.w[wib];
     if (lane == 0) { W.best_score = 0.0; W.best_order = 1 << 30; W.best_n = 0; W.best_buf = 0; }
@@ -909,7 +1054,10 @@ speculate_fused_kernel(sd_store sv, int n, const int32_t* __restrict__ d_slot, i
                 while (true) {
                     bool on = node >= 0 && pos < t;
                     if (!__any_sync(FULL, on)) break;
-                    const int x = on ? (pos < t_old ? text[pos] : newtok[pos - t_old]) : -1;
+                    // (of the new tokens the first ones are at hand)
+                    const int kx = pos - t_old;
+                    int x = -1;
+                    if (on) x = kx < 0 ? text[pos] : (kx < APP_AHEAD ? sh.app.tok[kx + APP_SHALLOW - 1] : newtok[kx]);
                     const int n = on ? (int)((unsigned)zw.y & RUN_COUNT_MASK) : 0;
                     const bool far = n > APP_LANES;
                     if (__any_sync(FULL, far)) {                // long runs are searched
@@ -940,39 +1088,25 @@ speculate_fused_kernel(sd_store sv, int n, const int32_t* __restrict__ d_slot, i
         group_sync();
 
         // ---------------- 2. the job queue, by the number of nodes a job can add at most
-        if (gtid < 2 * SD_MAX_DEPTH) {
-            const int tree = gtid / SD_MAX_DEPTH, p = gtid % SD_MAX_DEPTH + 1;
-            int c = 0;
-            if (tree == 0) {
-                const unsigned wf = sh.nc[0][p - 1];
-                const int nch = (int)(wf & RUN_COUNT_MASK);
-                if (p <= Pe && sh.node[0][p - 1] >= 0 && nch > 0) {
-                    // all first runs start their way to L2 now, long before a warp gets to them
-                    const int4* base = sv.g_ent + sh.cb[0][p - 1];
-                    const int lines = min(4, (nch + 7) >> 3);
-                    for (int l = 0; l < lines; ++l) prefetch_l2(base + l * 8);
-                    c = min(budget_for(alpha, p, cap), 2 * (D - p));
-                    if (c > 0 && nch > WIDE_RUN && !(wf & RUN_HAS_TOP)) { sh.wide[atomicAdd(&sh.nwide, 1)] = gtid; c = 0; }
-                    if (c > 0) c += 1000;
-                }
-            } else if (want_r && p <= Pe && p <= t) {
-                c = min(budget_for(alpha, p, cap), 2 * (D - p));
-                if (c > 0) c += 1000;
+        // (a lane per pattern length in the order of that number, the global tree's job before the request's)
+        if (gw == 0) {
+            const int p = sh.ordp[lane] + 1;
+            const int c = p <= Pe ? min(budget_for(alpha, p, cap), 2 * (D - p)) : 0;
+            const unsigned wf = c > 0 && sh.node[0][p - 1] >= 0 ? sh.nc[0][p - 1] : 0u;
+            const int nch = (int)(wf & RUN_COUNT_MASK);
+            const bool far = nch > WIDE_RUN && !(wf & RUN_HAS_TOP);
+            const bool j0 = nch > 0 && !far, j1 = c > 0 && want_r && p <= t;
+            if (j0) {
+                // all first runs start their way to L2 now, before a warp gets to them
+                const int4* base = sv.g_ent + sh.cb[0][p - 1];
+                for (int l = 0; l < min(4, (nch + 7) >> 3); ++l) prefetch_l2(base + l * 8);
             }
-            sh.cost[gtid] = c;
-        }
-        group_sync();
-        if (gtid < 2 * SD_MAX_DEPTH) {
-            const int c = sh.cost[gtid];
-            if (c > 0) {
-                int rank = 0;
-                for (int q = 0; q < 2 * SD_MAX_DEPTH; ++q) {
-                    const int cq = sh.cost[q];
-                    rank += (cq > c || (cq == c && q < gtid)) ? 1 : 0;
-                }
-                sh.job[rank] = gtid;
-                atomicAdd(&sh.njobs, 1);
-            }
+            if (far) sh.wide[atomicAdd(&sh.nwide, 1)] = p - 1;
+            const unsigned b0 = __ballot_sync(FULL, j0), b1 = __ballot_sync(FULL, j1), lt = (1u << lane) - 1u;
+            int at = __popc(b0 & lt) + __popc(b1 & lt);
+            if (j0) sh.job[at++] = p - 1;
+            if (j1) sh.job[at] = SD_MAX_DEPTH + p - 1;
+            if (lane == 0) sh.njobs = __popc(b0) + __popc(b1);
         }
         group_sync();
         if (STEP) asm volatile("bar.arrive %0, %1;" ::"r"(BAR_JOIN), "r"(NT) : "memory");   // warp 0 may come in
@@ -993,7 +1127,7 @@ speculate_fused_kernel(sd_store sv, int n, const int32_t* __restrict__ d_slot, i
             // the parent's D among its children)
             if ((double)min(budget, D - p) * 1.000000001 < best_so_far(sh)) continue;
             if (tree == 0) {
-                expand_job(sh, W, sv.g_ent, (int)sv.g_cap, 0, p, budget, flags, false, 0, lane);
+                expand_job(sh, W, sv.g_ent, (int)sv.g_cap, 0, p, budget, flags, -1, lane);
             } else {
                 // through the tree: the match node is the slot's active node of depth p, once the
                 // append is done (bounded wait; a job that runs out of patience is done after the
@@ -1027,107 +1161,120 @@ speculate_fused_kernel(sd_store sv, int n, const int32_t* __restrict__ d_slot, i
             if (tid == 0) ss->g_gen = ss->gen - 1;
         }
     }
-    for (int q = wib; q < sh.nlate && usable; q += CTA_WARPS) {
-        const int p = sh.late[q];
-        const int budget = budget_for(alpha, p, cap);
-        if ((double)min(budget, D - p) * 1.000000001 < best_so_far(sh)) continue;
-        request_tree_job(sh, W, sv, ss, s_ent, t, p, budget, flags, lane);
-    }
-    __syncthreads();
-    // Jobs that start at a wide node (short patterns, hence small budgets): most cannot reach
-    // the best score any more and are dropped here.  For the rest the warps of the block share
-    // the scan of the run, then one warp merges the partial lists and finishes the job.
-    if (tid == 0) {
-        const double best = __hiloint2double((int)sh.best_hi, 0);
-        int kept = 0;
-        for (int q = 0; q < sh.nwide && usable; ++q) {
-            const int p = sh.wide[q] % SD_MAX_DEPTH + 1;
-            if (!((double)min(budget_for(alpha, p, cap), D - p) * 1.000000001 < best)) sh.wide[kept++] = sh.wide[q];
-        }
-        sh.nwide_kept = kept;
-    }
-    __syncthreads();
-    const int nwide = sh.nwide_kept;
-    for (int base = 0; base < nwide; base += CTA_WARPS) {
-        const int nj = min(CTA_WARPS, nwide - base);
-        const int G = CTA_WARPS / nj;                           // warps per job
-        const int my_job = wib / G, my_slice = wib % G;
-        const bool active = my_job < nj;
-        int tree = 0, p = 1, budget = 0, fs = 0;
-        const int4* ent = sv.g_ent;
-        if (active) {
-            const int code = sh.wide[base + my_job];
-            tree = code / SD_MAX_DEPTH; p = code % SD_MAX_DEPTH + 1;
-            budget = budget_for(alpha, p, cap);
-            ent = tree == 0 ? sv.g_ent : s_ent;
-            long long sum;
-            scan_run_by_count(ent, sh.cb[tree][p - 1], (int)(sh.nc[tree][p - 1] & RUN_COUNT_MASK), my_slice, G, -1, 1, W,
-                              W.F, 0, fs, budget, sum, lane);
-            if (lane == 0) { sh.slice_sum[wib] = sum; sh.slice_fs[wib] = fs; }
+    if (sh.nlate > 0 || sh.nwide > 0) {                         // (either only grows before the barrier above)
+        for (int q = wib; q < sh.nlate && usable; q += CTA_WARPS) {
+            const int p = sh.late[q];
+            const int budget = budget_for(alpha, p, cap);
+            if ((double)min(budget, D - p) * 1.000000001 < best_so_far(sh)) continue;
+            request_tree_job(sh, W, sv, ss, s_ent, t, p, budget, flags, lane);
         }
         __syncthreads();
-        if (active && my_slice == 0) {
-            long long sum = sh.slice_sum[wib];
-            for (int g = 1; g < G; ++g) {
-                const Frontier& O = sh.w[wib + g].F;
-                const int ofs = sh.slice_fs[wib + g];
-                sum += sh.slice_sum[wib + g];
-                frontier_merge_list(W.F, 0, fs, budget, O, ofs, -1, lane);
+        // Jobs that start at a wide node (short patterns, hence small budgets): most cannot reach
+        // the best score any more and are dropped here.  For the rest the warps of the block share
+        // the scan of the run, then one warp merges the partial lists and finishes the job.
+        if (tid == 0) {
+            const double best = __hiloint2double((int)sh.best_hi, 0);
+            int kept = 0;
+            for (int q = 0; q < sh.nwide && usable; ++q) {
+                const int p = sh.wide[q] % SD_MAX_DEPTH + 1;
+                if (!((double)min(budget_for(alpha, p, cap), D - p) * 1.000000001 < best)) sh.wide[kept++] = sh.wide[q];
             }
-            counts_to_d(W.F, 0, fs, 1.0, sum, lane);
-            expand_job(sh, W, ent, tree == 0 ? (int)sv.g_cap : (int)sv.spn, tree, p, budget, flags, true, fs, lane);
+            sh.nwide_kept = kept;
         }
         __syncthreads();
+        const int nwide = sh.nwide_kept;
+        for (int base = 0; base < nwide; base += CTA_WARPS) {
+            const int nj = min(CTA_WARPS, nwide - base);
+            const int G = CTA_WARPS / nj;                           // warps per job
+            const int my_job = wib / G, my_slice = wib % G;
+            const bool active = my_job < nj;
+            int tree = 0, p = 1, budget = 0, fs = 0;
+            const int4* ent = sv.g_ent;
+            if (active) {
+                const int code = sh.wide[base + my_job];
+                tree = code / SD_MAX_DEPTH; p = code % SD_MAX_DEPTH + 1;
+                budget = budget_for(alpha, p, cap);
+                ent = tree == 0 ? sv.g_ent : s_ent;
+                long long sum;
+                scan_run_by_count(ent, sh.cb[tree][p - 1], (int)(sh.nc[tree][p - 1] & RUN_COUNT_MASK), my_slice, G, -1, 1, W,
+                                  W.T, 0, fs, budget, sum, lane);
+                if (lane == 0) { sh.slice_sum[wib] = sum; sh.slice_fs[wib] = fs; }
+            }
+            __syncthreads();
+            if (active && my_slice == 0) {
+                long long sum = sh.slice_sum[wib];
+                for (int g = 1; g < G; ++g) {
+                    const Frontier& O = sh.w[wib + g].T;
+                    const int ofs = sh.slice_fs[wib + g];
+                    sum += sh.slice_sum[wib + g];
+                    frontier_merge_list(W.T, 0, fs, budget, O, ofs, -1, lane);
+                }
+                counts_to_d(W.T, 0, fs, 1.0, sum, lane);
+                expand_job(sh, W, ent, tree == 0 ? (int)sv.g_cap : (int)sv.spn, tree, p, budget, flags, fs, lane);
+            }
+            __syncthreads();
+        }
     }
+    if (wib != 0) return;
 
-    // ---------------- 4. select (first in loop order among the largest scores) and emit
-    if (wib == 0) {
-        double sc = lane < CTA_WARPS ? sh.w[lane].best_score : 0.0;
-        int od = lane < CTA_WARPS ? sh.w[lane].best_order : 1 << 30;
-        int ww = lane;
+    // ---------------- 4. select (first in loop order among the largest scores) and emit: one warp
+    double best = lane < CTA_WARPS ? sh.w[lane].best_score : 0.0;
+    int od = lane < CTA_WARPS ? sh.w[lane].best_order : 1 << 30;
+    int win = lane;
 #pragma unroll
-        for (int off = 16; off > 0; off >>= 1) {
-            const double osc = __shfl_xor_sync(FULL, sc, off);
-            const int ood = __shfl_xor_sync(FULL, od, off);
-            const int oww = __shfl_xor_sync(FULL, ww, off);
-            if (osc > sc || (osc == sc && ood < od)) { sc = osc; od = ood; ww = oww; }
-        }
-        // Section 3.2: the tree is used only if its score exceeds the threshold (tau = 0: any score above 0)
-        if (lane == 0) sh.win_warp = (usable && sc > 0.0 && sc > tau) ? ww : -1;
+    for (int off = 16; off > 0; off >>= 1) {
+        const double osc = __shfl_xor_sync(FULL, best, off);
+        const int ood = __shfl_xor_sync(FULL, od, off);
+        const int oww = __shfl_xor_sync(FULL, win, off);
+        if (osc > best || (osc == best && ood < od)) { best = osc; od = ood; win = oww; }
     }
-    __syncthreads();
-    const int win = sh.win_warp;
-    int nd = 0, ctree = -1, cp = 0;
-    double best = 0.0;
-    const int* wtok = nullptr;
-    const unsigned char* wpar = nullptr;
-    if (win >= 0) {
-        const WarpWork& B = sh.w[win];
-        nd = B.best_n; best = B.best_score;
-        ctree = B.best_order / SD_MAX_DEPTH; cp = B.best_order % SD_MAX_DEPTH;
-        if (cp == 0) { cp = SD_MAX_DEPTH; ctree -= 1; }          // order = tree * 32 + p with p in 1..32
-        wtok = B.tok[B.best_buf]; wpar = B.par[B.best_buf];
+    // Section 3.2: the tree is used only if its score exceeds the threshold (tau = 0: any score above 0)
+    const bool used = usable && best > 0.0 && best > tau;
+    const WarpWork& B = sh.w[win];
+    const int nd = used ? B.best_n : 0;
+    int tok[2], par[2], up[2];
+    unsigned long long bits[2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const int j = lane + 32 * h;
+        tok[h] = -1; par[h] = -1; bits[h] = 0ull;
+        if (j < nd) { tok[h] = B.tok[B.best_buf][j]; par[h] = (int)B.par[B.best_buf][j] - 1; bits[h] = 1ull << j; }
+        up[h] = par[h];
+        sh.anc[j] = bits[h]; sh.up[j] = (signed char)up[h];
     }
-    for (int j = tid; j < M; j += NT) {
-        int tok = -1, par = -1, pos = -1;
-        unsigned long long bits = 0;
-        if (j < nd) {
-            tok = wtok[j];
-            par = (int)wpar[j] - 1;
-            int depth = 0;
-            for (int a = j, hops = 0; a >= 0 && hops < SD_MAX_SPEC; a = (int)wpar[a] - 1, ++hops) {
-                bits |= 1ull << a;
-                ++depth;
-            }
-            pos = t + depth - 1;
+    __syncwarp();
+    // ancestors by pointer doubling: bits gathered so far, and the next ancestor to ask
+    while (__any_sync(FULL, up[0] >= 0 || up[1] >= 0)) {
+        unsigned long long add[2];
+        int nu[2];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            add[h] = up[h] >= 0 ? sh.anc[up[h]] : 0ull;
+            nu[h] = up[h] >= 0 ? (int)sh.up[up[h]] : -1;
         }
+        __syncwarp();
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            bits[h] |= add[h];
+            up[h] = nu[h];
+            sh.anc[lane + 32 * h] = bits[h]; sh.up[lane + 32 * h] = (signed char)up[h];
+        }
+        __syncwarp();
+    }
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const int j = lane + 32 * h;
+        if (j >= M) continue;
         const long long o = (long long)i * M + j;
-        d_tokens[o] = tok; d_parents[o] = par; d_positions[o] = pos;
-        d_mask[o * words] = (uint32_t)bits;
-        if (words > 1) d_mask[o * words + 1] = (uint32_t)(bits >> 32);
+        d_tokens[o] = tok[h]; d_parents[o] = par[h]; d_positions[o] = j < nd ? t + __popcll(bits[h]) - 1 : -1;
+        d_mask[o * words] = (uint32_t)bits[h];
+        if (words > 1) d_mask[o * words + 1] = (uint32_t)(bits[h] >> 32);
     }
-    if (tid == 0) {
-        d_n_draft[i] = nd; d_chosen_tree[i] = ctree; d_chosen_p[i] = cp; d_score[i] = best;
+    if (lane == 0) {
+        d_n_draft[i] = nd;
+        d_chosen_tree[i] = used ? (od - 1) / SD_MAX_DEPTH : -1;  // order = tree * 32 + p with p in 1 .. 32
+        d_chosen_p[i] = used ? (od - 1) % SD_MAX_DEPTH + 1 : 0;
+        d_score[i] = used ? best : 0.0;
         if (d_status) d_status[i] = status;
     }
 }
