@@ -1,7 +1,7 @@
 // Offline build of the global suffix tree (Section 3, "Suffix Tree Construction")
 // on the GPU: depth-capped suffix sort by prefix doubling, adjacent-suffix LCPs,
-// then all depths at once: ballot scans over (lcp, len) give every node's rank, range
-// and parent, and one kernel lays the nodes down as sorted child runs in pre-order.
+// then all depths at once, a lane per depth: sweeps over (lcp, len) give every node's count, children
+// and place, and one kernel lays the nodes down as sorted child runs in pre-order.
 // Hand-written LSD radix sort and scans (no CUB / Thrust).
 // Also: sd_build_requests (the trees of a batch of new requests by the same pipeline).
 #include <algorithm>
@@ -10,7 +10,7 @@
 #include <stdio.h>
 #include <string.h>
 
-#include "common.cuh"
+#include "append_core.cuh"
 
 namespace {
 
@@ -346,295 +346,429 @@ block_suffix_sort_kernel(const int32_t* tok, const int64_t* seq_off, int D, uint
     for (int i = tid; i < n; i += BS_THREADS) sa[b + i] = (uint32_t)(b + idx[i]);
 }
 
-// lcp[j] = common prefix (capped) of sorted suffixes j-1 and j; len[j] = capped length of suffix j
-__global__ void lcp_kernel(const int32_t* tok, const uint32_t* sa, const int* end_pos, i64 n, int D, uint8_t* lcp,
-                           uint8_t* len) {
-    i64 j = (i64)blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= n) return;
-    i64 b = sa[j];
-    int lb = min((i64)D, (i64)end_pos[b] - b);
-    len[j] = (uint8_t)lb;
-    int l = 0;
-    if (j > 0) {
-        i64 a = sa[j - 1];
-        int la = min((i64)D, (i64)end_pos[a] - a);
-        int m = min(la, lb);
-        while (l < m && tok[a + l] == tok[b + l]) ++l;
-    }
-    lcp[j] = (uint8_t)l;
-}
-
-struct NewNodes {             // nodes opened by suffix j: one at every depth in (lcp[j], len[j]]
-    const uint8_t* lcp;
-    const uint8_t* len;
-    __device__ int operator()(i64 j) const { return (int)len[j] - (int)lcp[j]; }
-};
-
 // ------------------------------------------------------------------ all depths at once
-// Everything the tree needs beyond the suffix order follows from lcp[] and len[], for all
-// depths d = 1 .. D together.  "Channel" c stands for depth d = c + 1:
-//   opens_c(i)  = lcp[i] <= c < len[i]    suffix i opens a node at depth d
-//   bound_c(i)  = lcp[i] <= c             suffix i starts a new range of equal d-token prefixes
-//   E_c[j]      = #{ i < j : opens_c(i) }                  rank of a depth-d node among all of them
-//   end(j, d)   = min{ i > j : bound_c(i) } (else N)        one past the node's range: count = end - j
-//   before(j)   = max{ i < j : lcp[i] < lcp[j] }            first suffix of the parent's range when
-//                                                           the parent was opened by another suffix
-// One warp scans a tile of 32 x CHUNKS suffixes, 32 at a time: a ballot per channel turns the 32
-// suffixes' flags into one word, lane c keeps the running state of channel c.  Three launches:
-// tile totals, carries across tiles (one small block), then the tile again with its carries.
-// Nodes are numbered in depth-first pre-order: the root is 0 and the node that suffix j opens
-// at depth d is 1 + nbase[j] + (d - lcp[j] - 1).  Pre-order is what makes paths contiguous:
-// child runs are laid down in node order, so the run of a node's first child directly follows
-// the node's own run, and a chain of only children is one run of consecutive entries.
-constexpr int MS_CHUNKS = 32;                     // chunks of 32 suffixes per tile
-constexpr int MS_CHUNKS_SMALL = 4;                // ... when there are few suffixes (more, shorter tiles: more warps at work)
-constexpr i64 MS_SMALL_N = 1 << 17;
-constexpr int MS_WARPS = 4;                       // tiles (warps) per block
+// Everything the tree needs beyond the suffix order follows from lcp[] (common prefix of a suffix with the one
+// before it) and len[], both capped at D.  Suffix j opens a node at every depth d in (lcp[j], len[j]].  A
+// warp goes through a tile of suffixes with a lane per depth:
+//   end_d(j)   = min{ i > j : lcp[i] < d }, else N      one past the node's range: count = end - j
+//   F_d(j)     = #{ i in (j, end_d(j)) : lcp[i] == d < len[i] }  children that later suffixes open below it
+//   children   = F_d(j) + 1 if d < len[j]
+//   G_d(j)     = sum of F_a(j) over 1 <= a < d
+// The nodes are numbered in depth-first pre-order and child runs are laid down in node order, so the run of a
+// node's first child directly follows the node's own run and a chain of only children is a run of consecutive
+// entries.  What lies in front of a node's run are the nodes (below depth 1) that earlier suffixes opened, those
+// that j itself opened down to depth d, and the children that later suffixes will open below the node's ancestors:
+//   run(j, d)  = S(j) + (d - max(lcp[j], 1)) + G_d(j),  S(j) = nodes below depth 1 opened by suffixes before j
+// so a node's run needs no table of all nodes, only running state per depth:
+//   from behind  (F, end): at suffix i, F_d + 1 if lcp[i] == d < len[i], both reset if lcp[i] < d.  In terms of G: G_d
+//                becomes G_{lcp+1} (+ 1 if the suffix opens a node) for all d > lcp (0 if lcp is 0): one shuffle; F_d = G_{d+1} - G_d
+//   from the front  R_d: the end of the run of the last node opened at depth d.  The first node that suffix j opens has
+//                F_lcp(j) siblings behind it: its entry is R_lcp - 1 - F_lcp(j); every further one is its parent's
+//                first child.
+// Three sweeps over the suffixes: (1) lcp and what a tile does to the state from behind, (2) the R a tile leaves behind,
+// (3) the entries; between them the state is carried over the tiles, a block per depth.  Per suffix that reads a row of D
+// tokens twice and writes 16 B per node.  (A table of ranks per depth and suffix, and per node its range, children and
+// run, written and read back by six kernels, took 2.5 ms for 4.2 M suffixes of 48.6 M nodes.)
+constexpr int TS_SUB = 16;                        // suffixes whose state from behind is kept in registers
+constexpr int TS_WARPS = 4;                       // tiles (warps) per block
+constexpr int TS_TILES = 8192;                    // tiles are made longer to have no more of them than that, as far as
+constexpr int TS_MAX_LEN = 1024;                  // the shared memory for their state goes
+constexpr int TS_CARRY = 256;                     // threads per block of the carry kernels
+constexpr unsigned TS_FULL = 0xffffffffu;
 
-struct LevelTables {
-    int* E;               // [D][N + 1]
-    int* node_end;        // [n_nodes + 1], by node id
-    int* before;          // [N]
-    int* agg;             // [3][32][tiles]: opens counts, last bound index, first bound index, per channel
-    i64 N;
-    int D, tiles;
+struct TreeScan {
+    const int32_t* tok;
+    const uint32_t* sa;
+    const int* end_pos;
+    uint8_t *lcp, *len;
+    int N, D;
+    int tile_len, tiles;                          // a multiple of 32
+    int* f;                                       // [32][tiles] (1): children counted, bit 31: state reset; carried: F from behind
+    int* e;                                       // [32][tiles] (1): first reset in the tile; carried: end from behind
+    int* r;                                       // [32][tiles] (2): R left behind (-1: none); carried: R from the front
+    int* s;                                       // [tiles + 1] nodes below depth 1, carried: S
+    int* n1;                                      // [tiles + 1] nodes of depth 1, carried: before the tile
+    int* wide;                                    // [4]: long runs, entries they take with their top blocks, cursors of both
 };
 
-template <int CHUNKS>
-__global__ void __launch_bounds__(MS_WARPS * 32)
-ms_tile_kernel(const uint8_t* __restrict__ lcp, const uint8_t* __restrict__ len, LevelTables T) {
-    const int lane = threadIdx.x & 31;
-    const int tile = blockIdx.x * MS_WARPS + (threadIdx.x >> 5);
-    if (tile >= T.tiles) return;
-    const i64 t0 = (i64)tile * (32 * CHUNKS);
-    int cnt = 0, last = -1, first = 0x7fffffff;                 // of channel `lane`
-    for (int ch = 0; ch < CHUNKS; ++ch) {
-        const i64 base = t0 + (i64)ch * 32, i = base + lane;
-        const int l = i < T.N ? lcp[i] : 255, n = i < T.N ? len[i] : 0;
+__device__ __forceinline__ int ts_scan(int v, int lane) {       // inclusive
 #pragma unroll
-        for (int c = 0; c < 32; ++c) {
-            const unsigned ob = __ballot_sync(0xffffffffu, l <= c && c < n);
-            const unsigned bb = __ballot_sync(0xffffffffu, l <= c);
-            if (lane == c) {
-                cnt += __popc(ob);
-                if (bb) {
-                    last = (int)base + 31 - __clz(bb);
-                    if (first == 0x7fffffff) first = (int)base + __ffs(bb) - 1;
-                }
-            }
-        }
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(TS_FULL, v, o);
+        if (lane >= o) v += y;
     }
-    T.agg[(i64)lane * T.tiles + tile] = cnt;
-    T.agg[(i64)(32 + lane) * T.tiles + tile] = last;
-    T.agg[(i64)(64 + lane) * T.tiles + tile] = first;
+    return v;
 }
 
-// In place: counts -> sum over the tiles before; last -> nearest bound index before the tile
-// (-1: none); first -> nearest bound index behind the tile (N: none).  Also E_c[N].
-// One block per column (kind, channel) of agg[96][tiles]; every thread takes a contiguous
-// stretch of tiles, the stretches' totals are combined in shared memory.
-constexpr int MC_THREADS = 256;
-__global__ void __launch_bounds__(MC_THREADS) ms_carry_kernel(LevelTables T) {
-    __shared__ int part[MC_THREADS];
-    const int kind = blockIdx.x >> 5, c = blockIdx.x & 31;
-    int* col = T.agg + (i64)blockIdx.x * T.tiles;
-    const int per = (T.tiles + MC_THREADS - 1) / MC_THREADS;
-    // kind 2 runs over the tiles from the last to the first
-    const int ident = kind == 0 ? 0 : (kind == 1 ? -1 : (int)T.N);
-    auto at = [&](int k) { return kind == 2 ? T.tiles - 1 - k : k; };
-    auto op = [&](int x, int y) { return kind == 0 ? x + y : (kind == 1 ? max(x, y) : min(x, y)); };
+// (1)
+__global__ void __launch_bounds__(TS_WARPS * 32)
+ts_tiles_kernel(TreeScan T) {
+    const int lane = threadIdx.x & 31, tile = blockIdx.x * TS_WARPS + (threadIdx.x >> 5), d = lane + 1;
+    if (tile >= T.tiles) return;
+    const int t0 = tile * T.tile_len, t1 = min(T.N, t0 + T.tile_len);
+    int px = -1, pl = 0;                                        // the row before: its tokens, its length
+    if (t0 > 0) {
+        const int q = (int)T.sa[t0 - 1];
+        pl = min(T.D, T.end_pos[q] - q);
+        if (lane < pl) px = T.tok[q + lane];
+    }
+    bool seen = false;
+    int cnt = 0, first = T.N, below = 0, top = 0;
+    for (int jb = t0; jb < t1; jb += 32) {
+        const int m = min(32, t1 - jb);
+        int q = 0, ln = 0, own = 0;
+        if (lane < m) { q = (int)T.sa[jb + lane]; ln = min(T.D, T.end_pos[q] - q); }
+        for (int i0 = 0; i0 < m; i0 += 8) {
+            int x[8], L[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {                       // eight rows in flight
+                const int at = __shfl_sync(TS_FULL, q, i0 + u);
+                L[u] = __shfl_sync(TS_FULL, ln, i0 + u);
+                x[u] = lane < L[u] ? T.tok[at + lane] : -1;
+            }
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                if (i0 + u >= m) break;
+                const unsigned ne = __ballot_sync(TS_FULL, x[u] != px || lane >= L[u] || lane >= pl);
+                const int l = ne ? __ffs(ne) - 1 : 32;
+                if (lane == i0 + u) own = l;
+                if (!seen) {
+                    cnt += l == d && L[u] > l ? 1 : 0;
+                    if (l < d) { seen = true; first = jb + i0 + u; }
+                }
+                px = x[u]; pl = L[u];
+            }
+        }
+        if (lane < m) {
+            T.lcp[jb + lane] = (uint8_t)own; T.len[jb + lane] = (uint8_t)ln;
+            below += ln - max(own, 1);
+            top += own == 0 ? 1 : 0;
+        }
+    }
+    T.f[(i64)lane * T.tiles + tile] = cnt | (seen ? (int)0x80000000 : 0);
+    T.e[(i64)lane * T.tiles + tile] = first;
+    below = (int)__reduce_add_sync(TS_FULL, (unsigned)below);
+    top = (int)__reduce_add_sync(TS_FULL, (unsigned)top);
+    if (lane == 0) { T.s[tile] = below; T.n1[tile] = top; }
+}
+
+// What lies behind (f, e: the tiles to the right; blocks 0 .. 31) or in front of a tile (s, n1: block 32).
+__global__ void __launch_bounds__(TS_CARRY) ts_carry_kernel(TreeScan T) {
+    __shared__ int p0[TS_CARRY / 32], p1[TS_CARRY / 32];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int per = (T.tiles + TS_CARRY - 1) / TS_CARRY;
     const int k0 = threadIdx.x * per, k1 = min(T.tiles, k0 + per);
-    int acc = ident;
-    for (int k = k0; k < k1; ++k) acc = op(acc, col[at(k)]);
-    part[threadIdx.x] = acc;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        int run = ident;
-        for (int t = 0; t < MC_THREADS; ++t) { const int v = part[t]; part[t] = run; run = op(run, v); }
-        if (kind == 0 && c < T.D) T.E[(i64)c * (T.N + 1) + T.N] = run;
+    if (blockIdx.x == 32) {
+        int a = 0, b = 0;
+        for (int k = k0; k < k1; ++k) { a += T.s[k]; b += T.n1[k]; }
+        const int ia = ts_scan(a, lane), ib = ts_scan(b, lane);
+        if (lane == 31) { p0[w] = ia; p1[w] = ib; }
+        __syncthreads();
+        int ra = ia - a, rb = ib - b, ta = 0, tb = 0;
+        for (int q = 0; q < TS_CARRY / 32; ++q) { if (q < w) { ra += p0[q]; rb += p1[q]; } ta += p0[q]; tb += p1[q]; }
+        for (int k = k0; k < k1; ++k) { a = T.s[k]; b = T.n1[k]; T.s[k] = ra; T.n1[k] = rb; ra += a; rb += b; }
+        if (threadIdx.x == 0) { T.s[T.tiles] = ta; T.n1[T.tiles] = tb; }
+        return;
     }
-    __syncthreads();
-    int run = part[threadIdx.x];
-    for (int k = k0; k < k1; ++k) { const int v = col[at(k)]; col[at(k)] = run; run = op(run, v); }
-}
-
-template <int CHUNKS>
-__global__ void __launch_bounds__(MS_WARPS * 32)
-ms_apply_kernel(const uint8_t* __restrict__ lcp, const uint8_t* __restrict__ len, const int* __restrict__ nbase,
-                LevelTables T) {
-    __shared__ unsigned bmask[MS_WARPS][CHUNKS][32];            // bound words of the tile, by chunk and channel
-    __shared__ int sfirst[MS_WARPS][32];
-    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-    const int tile = blockIdx.x * MS_WARPS + wib;
-    if (tile >= T.tiles) return;
-    const i64 t0 = (i64)tile * (32 * CHUNKS);
-    const unsigned lt = (1u << lane) - 1u;
-    int run_cnt = T.agg[(i64)lane * T.tiles + tile], run_last = T.agg[(i64)(32 + lane) * T.tiles + tile],
-        run_first = T.agg[(i64)(64 + lane) * T.tiles + tile];
-    // forward: E and `before`
-    for (int ch = 0; ch < CHUNKS; ++ch) {
-        const i64 base = t0 + (i64)ch * 32, i = base + lane;
-        const int l = i < T.N ? lcp[i] : 255, n = i < T.N ? len[i] : 0;
-        const int prev_last = run_last;
+    int* const f = T.f + (i64)blockIdx.x * T.tiles;
+    int* const e = T.e + (i64)blockIdx.x * T.tiles;
+    // (tile T.tiles - 1 - k: from the last to the first.)  v: children since the last reset, bit 31: there was one
+    auto join = [](int& v, int& x, int nv, int nx) { if (nv < 0) { v = nv; x = nx; } else v += nv; };        // further to the left
+    int v = 0, x = T.N;
+    for (int k = k0; k < k1; ++k) join(v, x, f[T.tiles - 1 - k], e[T.tiles - 1 - k]);
+    int iv = v, ix = x;
 #pragma unroll
-        for (int c = 0; c < 32; ++c) {
-            const unsigned ob = __ballot_sync(0xffffffffu, l <= c && c < n);
-            const unsigned bb = __ballot_sync(0xffffffffu, l <= c);
-            const int carry = __shfl_sync(0xffffffffu, run_cnt, c);
-            if (c < T.D && i < T.N) T.E[(i64)c * (T.N + 1) + i] = carry + __popc(ob & lt);
-            if (lane == c) {
-                run_cnt += __popc(ob);
-                if (bb) run_last = (int)base + 31 - __clz(bb);
-                bmask[wib][ch][c] = bb;
-            }
-        }
-        __syncwarp();
-        // nearest earlier suffix with a smaller lcp: bound channel lcp - 1
-        const int src = (l >= 1 && l <= 32) ? l - 1 : 0;
-        const int far = __shfl_sync(0xffffffffu, prev_last, src);
-        if (i < T.N) {
-            int b = -1;
-            if (l >= 1) {
-                const unsigned m = bmask[wib][ch][src] & lt;
-                b = m ? (int)base + 31 - __clz(m) : far;
-            }
-            T.before[i] = b;
-        }
+    for (int o = 1; o < 32; o <<= 1) {
+        int yv = __shfl_up_sync(TS_FULL, iv, o), yx = __shfl_up_sync(TS_FULL, ix, o);
+        if (lane >= o) { join(yv, yx, iv, ix); iv = yv; ix = yx; }
     }
-    // backward: the end of every node's range
-    for (int ch = CHUNKS - 1; ch >= 0; --ch) {
-        const i64 base = t0 + (i64)ch * 32, i = base + lane;
-        sfirst[wib][lane] = run_first;
-        __syncwarp();
-        if (i < T.N) {
-            const int l = lcp[i], n = len[i];
-            const unsigned gt = ~lt & ~(1u << lane);
-            int nid = 1 + nbase[i];
-            for (int d = l + 1; d <= n; ++d, ++nid) {
-                const unsigned m = bmask[wib][ch][d - 1] & gt;
-                T.node_end[nid] = m ? (int)base + __ffs(m) - 1 : sfirst[wib][d - 1];
-            }
-        }
-        __syncwarp();
-        const unsigned bb = bmask[wib][ch][lane];
-        if (bb) run_first = (int)base + __ffs(bb) - 1;
+    if (lane == 31) { p0[w] = iv; p1[w] = ix; }
+    int bv = __shfl_up_sync(TS_FULL, iv, 1), bx = __shfl_up_sync(TS_FULL, ix, 1);      // of the lanes before
+    __syncthreads();
+    int rv = 0, rx = T.N;
+    for (int q = 0; q < w; ++q) join(rv, rx, p0[q], p1[q]);
+    if (lane > 0) join(rv, rx, bv, bx);
+    for (int k = k0; k < k1; ++k) {
+        const int t = T.tiles - 1 - k;
+        const int fv = f[t], fx = e[t];
+        f[t] = rv & 0x7fffffff; e[t] = rx;
+        join(rv, rx, fv, fx);
     }
 }
 
-// children per node: the depth d + 1 nodes opened inside the node's range
-__global__ void count_children_kernel(const uint8_t* __restrict__ lcp, const uint8_t* __restrict__ len,
-                                      const int* __restrict__ nbase, LevelTables T, int* nchild) {
-    const i64 i = (i64)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i == 0) nchild[0] = T.E[T.N];                            // the root's children: all depth-1 nodes
-    if (i >= T.N) return;
-    const int l = lcp[i], n = len[i];
-    int nid = 1 + nbase[i];
-    for (int d = l + 1; d <= n; ++d, ++nid) {
-        int nc = 0;
-        if (d < T.D) {
-            const int* row = T.E + (i64)d * (T.N + 1);          // channel of depth d + 1
-            nc = row[T.node_end[nid]] - row[i];
+// R from the front: the last one left behind by a tile to the left.
+__global__ void __launch_bounds__(TS_CARRY) ts_carry_front_kernel(TreeScan T) {
+    __shared__ int part[TS_CARRY / 32];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int per = (T.tiles + TS_CARRY - 1) / TS_CARRY;
+    const int k0 = threadIdx.x * per, k1 = min(T.tiles, k0 + per);
+    int* const r = T.r + (i64)blockIdx.x * T.tiles;
+    int v = -1;
+    for (int k = k0; k < k1; ++k) { const int n = r[k]; if (n >= 0) v = n; }
+    int iv = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(TS_FULL, iv, o);
+        if (lane >= o && iv < 0) iv = y;
+    }
+    if (lane == 31) part[w] = iv;
+    const int b = __shfl_up_sync(TS_FULL, iv, 1);
+    __syncthreads();
+    int run = -1;
+    for (int q = 0; q < w; ++q) if (part[q] >= 0) run = part[q];
+    if (lane > 0 && b >= 0) run = b;
+    for (int k = k0; k < k1; ++k) { const int n = r[k]; r[k] = run; if (n >= 0) run = n; }
+}
+
+// The state from behind at a tile's right end: G of this lane's depth.
+__device__ __forceinline__ int ts_g_in(const TreeScan& T, int tile, int lane) {
+    const int f = T.f[(i64)lane * T.tiles + tile];
+    return ts_scan(f, lane) - f;
+}
+
+// G in front of a suffix with lcp l and length n (uniform)
+__device__ __forceinline__ int ts_g_step(int g, int l, int n, int d) {
+    const int v = __shfl_sync(TS_FULL, g, min(l, 31)) + (n > l ? 1 : 0);
+    return d > l ? (l == 0 ? 0 : v) : g;
+}
+
+__device__ __forceinline__ int ts_f_of(int g, int lane) {       // F from G (no node of depth 32 has children)
+    const int up = __shfl_down_sync(TS_FULL, g, 1);
+    return lane == 31 ? 0 : up - g;
+}
+
+// (2) TOP: also counts the long runs.
+template <bool TOP>
+__global__ void __launch_bounds__(TS_WARPS * 32)
+ts_runs_kernel(TreeScan T) {
+    const int lane = threadIdx.x & 31, tile = blockIdx.x * TS_WARPS + (threadIdx.x >> 5), d = lane + 1;
+    if (tile >= T.tiles) return;
+    const int t0 = tile * T.tile_len, t1 = min(T.N, t0 + T.tile_len);
+    int g = ts_g_in(T, tile, lane);
+    int s_end = T.s[tile + 1], R = -1, n_wide = 0, room = 0;
+    for (int jb = t0 + ((t1 - t0 - 1) & ~31); jb >= t0; jb -= 32) {
+        const int m = min(32, t1 - jb);
+        int l_own = 0, n_own = 0, c = 0;
+        if (lane < m) { l_own = T.lcp[jb + lane]; n_own = T.len[jb + lane]; c = n_own - max(l_own, 1); }
+        const int inc = ts_scan(c, lane);
+        const int all = __shfl_sync(TS_FULL, inc, 31);
+        const int s_own = s_end - all + inc - c;
+        s_end -= all;
+        for (int i = m - 1; i >= 0; --i) {
+            const int l = __shfl_sync(TS_FULL, l_own, i), n = __shfl_sync(TS_FULL, n_own, i);
+            const bool opens = d > l && d <= n;
+            if (TOP || __any_sync(TS_FULL, opens && R < 0)) {
+                const int kids = ts_f_of(g, lane) + (d < n ? 1 : 0);
+                const int s = __shfl_sync(TS_FULL, s_own, i);
+                if (opens && R < 0) R = s + d - max(l, 1) + g + kids;
+                if (TOP && opens && kids > SD_TOP_MIN) { ++n_wide; room += kids + SD_TOP_BLOCK; }
+            }
+            g = ts_g_step(g, l, n, d);
         }
-        nchild[nid] = nc;
+    }
+    T.r[(i64)lane * T.tiles + tile] = R;
+    if (TOP) {
+        n_wide = (int)__reduce_add_sync(TS_FULL, (unsigned)n_wide);
+        room = (int)__reduce_add_sync(TS_FULL, (unsigned)room);
+        if (lane == 0 && n_wide) { atomicAdd(&T.wide[0], n_wide); atomicAdd(&T.wide[1], room); }
     }
 }
 
-__device__ __forceinline__ int top_block_of(int nid, int nc) { return (nid > 0 && nc > SD_TOP_MIN) ? SD_TOP_BLOCK : 0; }
-
-struct RunAlloc {             // entries a node's child run takes, top block included
-    const int* nchild;
-    int top_blocks;
-    __device__ int operator()(i64 nid) const {
-        return nchild[nid] + (top_blocks ? top_block_of((int)nid, nchild[nid]) : 0);
-    }
+// Where the trees go: one tree (the global one), or one per request, whose suffixes are consecutive in the order.
+struct TreeOut {
+    int4* ent;                                    // global tree
+    int32_t* root;
+    int4* wide;                                   // its long runs: entry of the node, run, children, -
+    sd_store sv;                                  // requests
+    int n_req;
+    const int32_t* slot;
+    const int64_t* off;                           // [n_req + 1]
+    const int *s_req, *n1_req;                    // [n_req + 1] S and depth-1 nodes before the request's first suffix
 };
 
-__global__ void collect_wide_kernel(const int* nchild, i64 n_nodes_plus1, int* list, int* counter) {
-    i64 nid = (i64)blockIdx.x * blockDim.x + threadIdx.x;
-    if (nid >= n_nodes_plus1) return;
-    if (top_block_of((int)nid, nchild[nid])) list[atomicAdd(counter, 1)] = (int)nid;
-}
-
-// One block per long run: header (sum of counts) and the 64 best children by (count desc,
-// token asc), found by 64 rounds of "largest key below the previous one".
-__global__ void fill_top_kernel(const int* list, const int* nchild, const int* runstart, int4* ent) {
-    __shared__ u64 skey[256];
-    __shared__ int sidx[256];
-    __shared__ u64 ssum[256];
-    const int nid = list[blockIdx.x];
-    const int n = nchild[nid];
-    const int top = runstart[nid];                 // header; the run itself starts SD_TOP_BLOCK later
-    const int4* run = ent + top + SD_TOP_BLOCK;
-    u64 sum = 0;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) sum += (u64)(unsigned)run[i].y;
-    ssum[threadIdx.x] = sum;
-    __syncthreads();
-    for (int o = 128; o > 0; o >>= 1) {
-        if (threadIdx.x < o) ssum[threadIdx.x] += ssum[threadIdx.x + o];
-        __syncthreads();
-    }
-    const int ntop = n < 64 ? n : 64;
-    if (threadIdx.x == 0) ent[top] = make_int4((int)(unsigned)(ssum[0] & 0xffffffffu), (int)(unsigned)(ssum[0] >> 32), ntop, 0);
-    u64 prev = ~0ull;
-    for (int r = 0; r < ntop; ++r) {
-        u64 best = 0;
-        int bi = -1;
-        for (int i = threadIdx.x; i < n; i += blockDim.x) {
-            const int4 e = run[i];
-            const u64 key = ((u64)(unsigned)e.y << 32) | (u64)(0xffffffffu - (unsigned)e.x);
-            if (key < prev && (bi < 0 || key > best)) { best = key; bi = i; }
-        }
-        skey[threadIdx.x] = bi >= 0 ? best : 0;
-        sidx[threadIdx.x] = bi;
-        __syncthreads();
-        for (int o = 128; o > 0; o >>= 1) {
-            if (threadIdx.x < o) {
-                const int oi = sidx[threadIdx.x + o];
-                if (oi >= 0 && (sidx[threadIdx.x] < 0 || skey[threadIdx.x + o] > skey[threadIdx.x])) {
-                    skey[threadIdx.x] = skey[threadIdx.x + o];
-                    sidx[threadIdx.x] = oi;
-                }
+// (3)
+template <bool REQ>
+__global__ void __launch_bounds__(TS_WARPS * 32)
+ts_emit_kernel(TreeScan T, TreeOut O) {
+    extern __shared__ int2 ts_state[];                          // [TS_WARPS][tile_len / TS_SUB][32]: G and end behind each sub-tile
+    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5, tile = blockIdx.x * TS_WARPS + wib, d = lane + 1;
+    if (tile >= T.tiles) return;
+    const int t0 = tile * T.tile_len, t1 = min(T.N, t0 + T.tile_len);
+    const int subs = (t1 - t0 + TS_SUB - 1) / TS_SUB;
+    int2* const st = ts_state + (i64)wib * (T.tile_len / TS_SUB) * 32;
+    {
+        int g = ts_g_in(T, tile, lane), e = T.e[(i64)lane * T.tiles + tile];
+        for (int c = subs - 1; c >= 0; --c) {
+            st[c * 32 + lane] = make_int2(g, e);
+            if (c == 0) break;
+            const int jb = t0 + c * TS_SUB, m = min(TS_SUB, t1 - jb);
+            const int l_own = lane < m ? T.lcp[jb + lane] : 0, n_own = lane < m ? T.len[jb + lane] : 0;
+            for (int i = m - 1; i >= 0; --i) {
+                const int l = __shfl_sync(TS_FULL, l_own, i);
+                g = ts_g_step(g, l, __shfl_sync(TS_FULL, n_own, i), d);
+                if (d > l) e = jb + i;
             }
-            __syncthreads();
         }
-        prev = skey[0];
-        if (threadIdx.x == 0) ent[top + 1 + r] = run[sidx[0]];
-        __syncthreads();
+        __syncwarp();
+    }
+    int R = T.r[(i64)lane * T.tiles + tile];
+    int s_at = T.s[tile], n1_at = T.n1[tile];
+    // the tree this suffix belongs to: entries, root table, what turns S into a place, first token, depth-1 nodes before it
+    int4* ent = O.ent;
+    int32_t* root = O.root;
+    int shift = 0, first_tok = 0, n1_0 = 0, q = 0, next_req = 0x7fffffff;
+    bool fits = true;
+    auto enter = [&]() {                                        // request q
+        const int n1 = O.n1_req[q + 1] - O.n1_req[q], used = n1 + O.s_req[q + 1] - O.s_req[q], slot = O.slot[q];
+        fits = used <= O.sv.spn && O.off[q + 1] - O.off[q] <= O.sv.T && slot >= 0 && slot < O.sv.R;
+        ent = O.sv.s_ent + (i64)(fits ? slot : 0) * O.sv.spn;
+        root = O.sv.s_root + (i64)(fits ? slot : 0) * O.sv.V;
+        shift = n1 - O.s_req[q]; n1_0 = O.n1_req[q]; first_tok = q * O.sv.V;
+        next_req = (int)O.off[q + 1];
+    };
+    if (REQ) {
+        int lo = 0, hi = O.n_req;                               // the last request that starts at or before t0
+        while (hi - lo > 1) { const int mid = (lo + hi) >> 1; if (O.off[mid] <= t0) lo = mid; else hi = mid; }
+        q = lo;
+        enter();
+    } else {
+        shift = T.n1[T.tiles];
+    }
+    for (int c = 0; c < subs; ++c) {
+        const int jb = t0 + c * TS_SUB, m = min(TS_SUB, t1 - jb);
+        int l_own = 255, n_own = 0, sa_own = 0, below = 0, top = 0;
+        if (lane < m) {
+            l_own = T.lcp[jb + lane]; n_own = T.len[jb + lane]; sa_own = (int)T.sa[jb + lane];
+            below = n_own - max(l_own, 1); top = l_own == 0 ? 1 : 0;
+        }
+        const int ib = ts_scan(below, lane), it = ts_scan(top, lane);
+        const int s_own = s_at + ib - below, n1_own = n1_at + it - top;
+        s_at += __shfl_sync(TS_FULL, ib, 31);
+        n1_at += __shfl_sync(TS_FULL, it, 31);
+        int x[TS_SUB], gs[TS_SUB], es[TS_SUB];
+        const int2 in = st[c * 32 + lane];
+        int g = in.x, e = in.y;
+#pragma unroll
+        for (int i = TS_SUB - 1; i >= 0; --i) {
+            const int n = __shfl_sync(TS_FULL, n_own, i), at = __shfl_sync(TS_FULL, sa_own, i);
+            x[i] = lane < n ? T.tok[at + lane] : 0;
+            gs[i] = g; es[i] = e;
+            const int l = __shfl_sync(TS_FULL, l_own, i);
+            if (i < m) {
+                g = ts_g_step(g, l, n, d);
+                if (d > l) e = jb + i;
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < TS_SUB; ++i) {
+            if (i >= m) break;
+            const int j = jb + i;
+            if (REQ && j >= next_req) { while (j >= (int)O.off[q + 1]) ++q; enter(); }
+            const int l = __shfl_sync(TS_FULL, l_own, i), n = __shfl_sync(TS_FULL, n_own, i);
+            const int run = __shfl_sync(TS_FULL, s_own, i) + d - max(l, 1) + gs[i], depth1 = __shfl_sync(TS_FULL, n1_own, i) - n1_0;
+            const int later = ts_f_of(gs[i], lane);
+            const int kids = later + (d < n ? 1 : 0);
+            const bool opens = d > l && d <= n;
+            // the entry of the next depth's node: this node's first child, or the next of its other children
+            const int place = __shfl_up_sync(TS_FULL, opens ? run : R - 1 - later, 1);
+            if (opens) R = run + kids;
+            if (opens && fits) {
+                const int pos = lane == 0 ? depth1 : place + shift;
+                ent[pos] = make_int4(x[i] - first_tok, es[i] - j, kids > 0 ? run + shift : 0, kids > 0 ? (int)((unsigned)kids | RUN_STATIC) : 0);
+                if (lane == 0) root[x[i] - first_tok] = pos;
+                if (!REQ && kids > SD_TOP_MIN) O.wide[atomicAdd(&T.wide[2], 1)] = make_int4(pos, run + shift, kids, 0);
+            }
+        }
     }
 }
 
-// Write the nodes that suffix j opens.  A node's entry sits in its parent's child run at its
-// rank among the siblings (suffix order = token order).  The first node a suffix opens hangs
-// below a node of an earlier suffix (or the root); every further one is the only-so-far child
-// of the one before it.
-__global__ void emit_nodes_kernel(const int32_t* tok, const uint32_t* sa, const uint8_t* lcp, const uint8_t* len, i64 n,
-                                  LevelTables T, const int* nbase, const int* nchild, const int* runstart, int4* ent,
-                                  int32_t* root) {
-    const i64 j = (i64)blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= n) return;
-    const int l = lcp[j], m = len[j];
-    if (m <= l) return;
-    int nid = 1 + nbase[j];
-    int pnid = 0, rank = T.E[j];                                  // depth 1: below the root
-    if (l >= 1) {
-        const int jx = T.before[j];                               // its first suffix opened the parent
-        pnid = 1 + nbase[jx] + (l - (int)lcp[jx] - 1);
-        const int* row = T.E + (i64)l * (T.N + 1);                // channel of depth l + 1
-        rank = row[j] - row[jx];
+// Long runs of the global tree move behind the others, with room for a top block in front: first every node of one
+// gets its new run (its entry may itself lie in a run that moves), then the runs are copied.
+__global__ void ts_wide_place_kernel(TreeScan T, int4* wide, int4* ent, int first) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= T.wide[0]) return;
+    int4 w = wide[i];
+    w.w = first + atomicAdd(&T.wide[3], w.z + SD_TOP_BLOCK);
+    wide[i] = w;
+    ent[w.x].z = w.w + SD_TOP_BLOCK;
+    ent[w.x].w = (int)((unsigned)w.z | RUN_STATIC | RUN_HAS_TOP);
+}
+
+// One block per long run: the run, and in front of it the sum of its counts and the 64 best children by (count desc, token asc).
+// The smallest count among them is found by halving; children that occur more often are fewer than 64 and placed by comparing
+// them with one another, those with that very count follow in run (token) order.
+constexpr int TOP_THREADS = 256;
+__global__ void __launch_bounds__(TOP_THREADS)
+ts_wide_fill_kernel(const int4* wide, int4* ent) {
+    __shared__ int part[TOP_THREADS / 32];
+    __shared__ u64 psum[TOP_THREADS / 32];
+    __shared__ int cand[64];
+    __shared__ u64 ckey[64];
+    __shared__ int n_cand, limit;
+    const int4 w = wide[blockIdx.x];
+    const int n = w.z, tid = threadIdx.x, lane = tid & 31, wib = tid >> 5;
+    const int4* const from = ent + w.y;
+    int4* const to = ent + w.w + SD_TOP_BLOCK;
+    int4* const topb = ent + w.w;
+    u64 sum = 0;
+    unsigned most = 0;
+    for (int i = tid; i < n; i += TOP_THREADS) {
+        const int4 e = from[i];
+        to[i] = e;
+        sum += (unsigned)e.y;
+        most = max(most, (unsigned)e.y);
     }
-    const i64 text = (i64)sa[j];
-    for (int d = l + 1; d <= m; ++d, ++nid) {
-        const int nc = nchild[nid];
-        int4 e;
-        e.x = tok[text + d - 1];
-        e.y = T.node_end[nid] - (int)j;                           // every suffix in the range is an occurrence
-        const int tb = top_block_of(nid, nc);
-        e.z = nc > 0 ? runstart[nid] + tb : 0;
-        e.w = nc > 0 ? (int)((unsigned)nc | RUN_STATIC | (tb ? RUN_HAS_TOP : 0u)) : 0;
-        const int pos = runstart[pnid] + top_block_of(pnid, nchild[pnid]) + rank;
-        ent[pos] = e;
-        if (d == 1) root[e.x] = pos;
-        pnid = nid; rank = 0;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(TS_FULL, sum, o);
+    most = __reduce_max_sync(TS_FULL, most);
+    if (lane == 0) { psum[wib] = sum; part[wib] = (int)most; }
+    if (tid == 0) n_cand = 0;
+    __syncthreads();
+    const int want = min(n, 64);
+    if (tid == 0) {
+        for (int k = 1; k < TOP_THREADS / 32; ++k) { sum += psum[k]; most = max(most, (unsigned)part[k]); }
+        limit = (int)most;
+        topb[0] = make_int4((int)(unsigned)(sum & 0xffffffffu), (int)(unsigned)(sum >> 32), want, 0);
+    }
+    __syncthreads();
+    // the largest count c with at least `want` children at or above it
+    int lo = 1, hi = limit;
+    while (lo < hi) {
+        const int mid = lo + (hi - lo + 1) / 2;
+        int k = 0;
+        for (int i = tid; i < n; i += TOP_THREADS) k += from[i].y >= mid ? 1 : 0;
+        k = (int)__reduce_add_sync(TS_FULL, (unsigned)k);
+        __syncthreads();
+        if (lane == 0) part[wib] = k;
+        __syncthreads();
+        k = 0;
+        for (int q = 0; q < TOP_THREADS / 32; ++q) k += part[q];
+        if (k >= want) lo = mid; else hi = mid - 1;
+    }
+    for (int i = tid; i < n; i += TOP_THREADS) {
+        const int4 e = from[i];
+        if (e.y > lo) {
+            const int k = atomicAdd(&n_cand, 1);
+            cand[k] = i; ckey[k] = ((u64)(unsigned)e.y << 32) | (0xffffffffu - (unsigned)e.x);
+        }
+    }
+    __syncthreads();
+    const int nc = n_cand;
+    if (tid < nc) {
+        int rank = 0;
+        for (int q = 0; q < nc; ++q) rank += ckey[q] > ckey[tid] ? 1 : 0;
+        topb[1 + rank] = from[cand[tid]];
+    }
+    if (wib == 0) {
+        int k = nc;
+        for (int base = 0; base < n && k < want; base += 32) {
+            int4 e = make_int4(0, 0, 0, 0);
+            if (base + lane < n) e = from[base + lane];
+            const unsigned m = __ballot_sync(TS_FULL, e.y == lo);
+            const int at = k + __popc(m & ((1u << lane) - 1u));
+            if (e.y == lo && at < want) topb[1 + at] = e;
+            k += __popc(m);
+        }
     }
 }
 
@@ -835,61 +969,54 @@ static void store_release(sd_store* s, cudaStream_t st) {
     delete s;
 }
 
-// Everything up to the placement of the child runs, for one array of sequences: suffix
-// order, LCPs, children per node (pre-order node ids) and the start of every child run.
+// Everything up to the writing of the entries, for one array of sequences: suffix order and the sweeps over it.
 struct Pipeline {
     DeviceArena tmp;
     explicit Pipeline(cudaStream_t st) : tmp(st) {}
     SortBuffers sb;
     int *end_pos = nullptr, *rank[8] = {nullptr}, *comb[2] = {nullptr, nullptr}, *ex = nullptr;
-    uint8_t *lcp = nullptr, *len = nullptr;
-    int* wide_counter = nullptr;
-    const uint32_t* sa = nullptr;
-    LevelTables lv;
-    int *nbase = nullptr, *nchild = nullptr, *runstart = nullptr, *big_tmp = nullptr, *wide_list = nullptr;
-    i64 N = 0, n_nodes = 0, used_entries = 0;
-    int n_wide = 0;
+    TreeScan ts;
+    i64 N = 0;
 };
 
-// max_token: largest token value + 1 (sets the number of radix passes).  top_blocks: reserve
-// room for top blocks in front of long runs.  per_seq_max_len > 0: the sequences are independent
+// max_token: largest token value + 1 (sets the number of radix passes).  top_blocks: count the
+// long runs.  per_seq_max_len > 0: the sequences are independent
 // (tokens of different sequences never compare equal, sequence k's tokens below sequence k + 1's)
 // and none is longer than that, so each is sorted by a block of its own.
-// no_readback: nothing is read back to the host on the way (no stream synchronisation): the
-// node arrays are sized for the most nodes N tokens can have (N * D) instead of the number
-// counted, and n_nodes / used_entries / n_wide are not filled in.  For small builds without
-// top blocks (a few prompts in the middle of a decode loop), where a round trip to the host
-// costs as much as the kernels between two of them.
+// Nothing is read back to the host.
 // Returns SD_OK, SD_ERR_NOMEM or SD_ERR_CUDA.
 static int pipeline_run(Pipeline& P, const int32_t* d_tok, const int64_t* d_seq_offsets, int n_seqs, i64 N,
-                        i64 max_token, int D, bool top_blocks, cudaStream_t st, i64 per_seq_max_len = 0,
-                        bool no_readback = false) {
+                        i64 max_token, int D, bool top_blocks, cudaStream_t st, i64 per_seq_max_len = 0) {
     const int T256 = 256;
     P.N = N;
     DeviceArena& tmp = P.tmp;
     SortBuffers& sb = P.sb;
-    cudaError_t ce = cudaSuccess;
     const int nblk = (int)((N + RS_TILE - 1) / RS_TILE);
+    const bool block_sort = per_seq_max_len > 0 && per_seq_max_len <= BS_MAX_LEN;
+    TreeScan& ts = P.ts;
+    ts.N = (int)N; ts.D = D; ts.tok = d_tok;
+    ts.tile_len = 32;
+    while ((N + ts.tile_len - 1) / ts.tile_len > TS_TILES && ts.tile_len < TS_MAX_LEN) ts.tile_len *= 2;
+    ts.tiles = (int)((N + ts.tile_len - 1) / ts.tile_len);
     int m = 0;
     while ((2 << m) <= D) ++m;                    // 2^m <= D < 2^(m+1)
     {
         const i64 scan_ints = scan_tmp_ints(std::max<i64>((i64)256 * nblk, N + 1));
         tmp.reserve((long long)N * (16 + 8 + 4 + 4 + 2 + 4 * (m + 1) + 8 + 4) + 4ll * ((i64)256 * nblk + 1 + scan_ints) +
-                    64 * 256);
+                    4ll * 100 * ts.tiles + 64 * 256);
     }
-    bool ok = tmp.get(&sb.keys[0], N) && tmp.get(&sb.keys[1], N) && tmp.get(&sb.vals[0], N) &&
+    bool ok = tmp.get(&ts.lcp, N) && tmp.get(&ts.len, N) && tmp.get(&ts.f, 32 * (i64)ts.tiles) && tmp.get(&ts.e, 32 * (i64)ts.tiles) &&
+              tmp.get(&ts.r, 32 * (i64)ts.tiles) && tmp.get(&ts.s, ts.tiles + 1) && tmp.get(&ts.n1, ts.tiles + 1) && tmp.get(&ts.wide, 4);
+    ok = ok && tmp.get(&sb.keys[0], N) && tmp.get(&sb.keys[1], N) && tmp.get(&sb.vals[0], N) &&
               tmp.get(&sb.vals[1], N) && tmp.get(&sb.hist, (i64)256 * nblk + 1) &&
               tmp.get(&sb.scan_tmp, scan_tmp_ints(std::max<i64>((i64)256 * nblk, N + 1))) &&
-              tmp.get(&P.end_pos, N) && tmp.get(&P.ex, N + 1) && tmp.get(&P.lcp, N) && tmp.get(&P.len, N) &&
-              tmp.get(&P.wide_counter, 1);
+              tmp.get(&P.end_pos, N) && tmp.get(&P.ex, N + 1);
     for (int k = 0; ok && k <= m; ++k) ok = tmp.get(&P.rank[k], N);
     ok = ok && tmp.get(&P.comb[0], N) && tmp.get(&P.comb[1], N);
     if (!ok) return SD_ERR_NOMEM;
     int *end_pos = P.end_pos, **rank = P.rank, **comb = P.comb, *ex = P.ex;
-    uint8_t *lcp = P.lcp, *len = P.len;
 
     seq_end_kernel<<<grid_for(N, T256), T256, 0, st>>>(d_seq_offsets, n_seqs, N, end_pos);
-    const bool block_sort = per_seq_max_len > 0 && per_seq_max_len <= BS_MAX_LEN;
     if (block_sort) {
         i64 np = 1;
         while (np < per_seq_max_len) np <<= 1;
@@ -936,55 +1063,25 @@ static int pipeline_run(Pipeline& P, const int32_t* d_tok, const int64_t* d_seq_
             }
         }
     }
-    P.sa = sb.vals[sorted];
-    lcp_kernel<<<grid_for(N, T256), T256, 0, st>>>(d_tok, P.sa, end_pos, N, D, lcp, len);
-    ok = tmp.get(&P.nbase, N + 1);
-    if (!ok) return SD_ERR_NOMEM;
-    exclusive_scan(NewNodes{lcp, len}, N, P.nbase, sb.scan_tmp, st);
-    int h_nodes = 0;
-    if (!no_readback) {
-        ce = cudaMemcpyAsync(&h_nodes, P.nbase + N, sizeof(int), cudaMemcpyDeviceToHost, st);
-        if (ce == cudaSuccess) ce = cudaStreamSynchronize(st);
-        if (ce != cudaSuccess) return SD_ERR_CUDA;
-    }
-    const i64 n_nodes = no_readback ? N * D : (i64)h_nodes;      // (an upper bound: every suffix opens at most D nodes)
-    P.n_nodes = no_readback ? 0 : n_nodes;
+    ts.sa = sb.vals[sorted];
+    ts.end_pos = end_pos;
+    const unsigned grid = (unsigned)((ts.tiles + TS_WARPS - 1) / TS_WARPS);
+    if (top_blocks && cudaMemsetAsync(ts.wide, 0, 4 * sizeof(int), st) != cudaSuccess) return SD_ERR_CUDA;
+    ts_tiles_kernel<<<grid, TS_WARPS * 32, 0, st>>>(ts);
+    ts_carry_kernel<<<33, TS_CARRY, 0, st>>>(ts);
+    if (top_blocks) ts_runs_kernel<true><<<grid, TS_WARPS * 32, 0, st>>>(ts);
+    else ts_runs_kernel<false><<<grid, TS_WARPS * 32, 0, st>>>(ts);
+    ts_carry_front_kernel<<<32, TS_CARRY, 0, st>>>(ts);
+    return SD_OK;
+}
 
-    LevelTables& lv = P.lv;
-    lv.N = N; lv.D = D;
-    const bool small_tiles = N <= MS_SMALL_N;
-    const int tile_len = 32 * (small_tiles ? MS_CHUNKS_SMALL : MS_CHUNKS);
-    lv.tiles = (int)((N + tile_len - 1) / tile_len);
-    tmp.reserve(4ll * ((i64)D * (N + 1) + 3 * (n_nodes + 2) + N + (i64)lv.tiles * 96 + scan_tmp_ints(n_nodes + 1) +
-                       n_nodes / SD_TOP_MIN + 2) + 64 * 256);
-    ok = tmp.get(&lv.E, (i64)D * (N + 1)) && tmp.get(&lv.node_end, n_nodes + 1) && tmp.get(&lv.before, N) &&
-         tmp.get(&lv.agg, (i64)lv.tiles * 96) && tmp.get(&P.nchild, n_nodes + 1) &&
-         tmp.get(&P.runstart, n_nodes + 2) && tmp.get(&P.big_tmp, scan_tmp_ints(n_nodes + 1)) &&
-         tmp.get(&P.wide_list, n_nodes / SD_TOP_MIN + 2);
-    if (!ok) return SD_ERR_NOMEM;
-    const unsigned ms_grid = (unsigned)((lv.tiles + MS_WARPS - 1) / MS_WARPS);
-    if (small_tiles) ms_tile_kernel<MS_CHUNKS_SMALL><<<ms_grid, MS_WARPS * 32, 0, st>>>(lcp, len, lv);
-    else ms_tile_kernel<MS_CHUNKS><<<ms_grid, MS_WARPS * 32, 0, st>>>(lcp, len, lv);
-    ms_carry_kernel<<<96, MC_THREADS, 0, st>>>(lv);
-    if (small_tiles) ms_apply_kernel<MS_CHUNKS_SMALL><<<ms_grid, MS_WARPS * 32, 0, st>>>(lcp, len, P.nbase, lv);
-    else ms_apply_kernel<MS_CHUNKS><<<ms_grid, MS_WARPS * 32, 0, st>>>(lcp, len, P.nbase, lv);
-    // (with the bound, the node ids behind the last real node have no children)
-    if (no_readback) ce = cudaMemsetAsync(P.nchild, 0, sizeof(int) * (size_t)(n_nodes + 1), st);
-    if (ce != cudaSuccess) return SD_ERR_CUDA;
-    count_children_kernel<<<grid_for(N, T256), T256, 0, st>>>(lcp, len, P.nbase, lv, P.nchild);
-    // child runs (with their top blocks) in node (pre-)order
-    exclusive_scan(RunAlloc{P.nchild, top_blocks ? 1 : 0}, n_nodes + 1, P.runstart, P.big_tmp, st);
-    int* wide_counter = P.wide_counter;
-    ce = cudaMemsetAsync(wide_counter, 0, sizeof(int), st);
-    if (top_blocks)
-        collect_wide_kernel<<<grid_for(n_nodes + 1, T256), T256, 0, st>>>(P.nchild, n_nodes + 1, P.wide_list, wide_counter);
-    if (no_readback) return ce == cudaSuccess ? SD_OK : SD_ERR_CUDA;
-    int h_total = 0;
-    if (ce == cudaSuccess) ce = cudaMemcpyAsync(&h_total, P.runstart + n_nodes + 1, sizeof(int), cudaMemcpyDeviceToHost, st);
-    if (ce == cudaSuccess) ce = cudaMemcpyAsync(&P.n_wide, wide_counter, sizeof(int), cudaMemcpyDeviceToHost, st);
-    if (ce == cudaSuccess) ce = cudaStreamSynchronize(st);
-    if (ce != cudaSuccess) return SD_ERR_CUDA;
-    P.used_entries = h_total;
+template <bool REQ>
+static int emit_entries(const TreeScan& ts, const TreeOut& out, cudaStream_t st) {
+    const unsigned grid = (unsigned)((ts.tiles + TS_WARPS - 1) / TS_WARPS);
+    const size_t smem = sizeof(int2) * 32 * (size_t)TS_WARPS * (ts.tile_len / TS_SUB);
+    if (smem > 48 * 1024)
+        SD_CUDA_OK(cudaFuncSetAttribute(ts_emit_kernel<REQ>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    ts_emit_kernel<REQ><<<grid, TS_WARPS * 32, smem, st>>>(ts, out);
     return SD_OK;
 }
 
@@ -1029,6 +1126,8 @@ extern "C" int sd_build(const sd_build_params* p, const int32_t* d_corpus, const
     Pipeline P(st);
     const int T256 = 256;
     i64 n_nodes = 0, used_entries = 0;
+    int h_wide[2] = {0, 0};
+    int4* wide_list = nullptr;
     if (N > 0) {
         {
             int* bad = nullptr;
@@ -1044,8 +1143,15 @@ extern "C" int sd_build(const sd_build_params* p, const int32_t* d_corpus, const
         }
         const int rc = pipeline_run(P, d_corpus, d_seq_offsets, n_seqs, N, s->V, D, true, st);
         if (rc != SD_OK) { store_release(s, st); return rc; }
-        n_nodes = P.n_nodes;
-        used_entries = P.used_entries;
+        int h_s = 0, h_n1 = 0;
+        ce = cudaMemcpyAsync(&h_s, P.ts.s + P.ts.tiles, sizeof(int), cudaMemcpyDeviceToHost, st);
+        if (ce == cudaSuccess) ce = cudaMemcpyAsync(&h_n1, P.ts.n1 + P.ts.tiles, sizeof(int), cudaMemcpyDeviceToHost, st);
+        if (ce == cudaSuccess) ce = cudaMemcpyAsync(h_wide, P.ts.wide, 2 * sizeof(int), cudaMemcpyDeviceToHost, st);
+        if (ce == cudaSuccess) ce = cudaStreamSynchronize(st);
+        if (ce != cudaSuccess) { store_release(s, st); return SD_ERR_CUDA; }
+        n_nodes = (i64)h_s + h_n1;
+        used_entries = n_nodes + h_wide[1];                     // (a long run leaves its first place empty)
+        if (h_wide[0] > 0 && !P.tmp.get(&wide_list, h_wide[0])) { store_release(s, st); return SD_ERR_NOMEM; }
     }
 
     i64 extra = p->global_extra_nodes >= 0 ? p->global_extra_nodes : std::max<i64>(1ll << 22, n_nodes);
@@ -1054,10 +1160,15 @@ extern "C" int sd_build(const sd_build_params* p, const int32_t* d_corpus, const
     if (!store_alloc(s, &s->g_ent, s->g_cap, st)) { store_release(s, st); return SD_ERR_NOMEM; }
 
     if (N > 0) {
-        // write the entries
-        emit_nodes_kernel<<<grid_for(N, T256), T256, 0, st>>>(d_corpus, P.sa, P.lcp, P.len, N, P.lv, P.nbase, P.nchild,
-                                                             P.runstart, s->g_ent, s->g_root);
-        if (P.n_wide > 0) fill_top_kernel<<<P.n_wide, 256, 0, st>>>(P.wide_list, P.nchild, P.runstart, s->g_ent);
+        TreeOut out;
+        memset(&out, 0, sizeof(out));
+        out.ent = s->g_ent; out.root = s->g_root; out.wide = wide_list;
+        const int erc = emit_entries<false>(P.ts, out, st);
+        if (erc != SD_OK) { store_release(s, st); return erc; }
+        if (h_wide[0] > 0) {
+            ts_wide_place_kernel<<<grid_for(h_wide[0], T256), T256, 0, st>>>(P.ts, wide_list, s->g_ent, (int)n_nodes);
+            ts_wide_fill_kernel<<<(unsigned)h_wide[0], TOP_THREADS, 0, st>>>(wide_list, s->g_ent);
+        }
     }
     init_global_state_kernel<<<1, 1, 0, st>>>(s->g_state, (int)used_entries, (int)n_nodes, N);
     ce = cudaStreamSynchronize(st);
@@ -1110,8 +1221,9 @@ __global__ void map_tokens_kernel(const int32_t* tok, const int64_t* off, int n,
 }
 
 // one block per request: forget the slot's old tree and store the new text
-__global__ void requests_prepare_kernel(sd_store sv, int n, const int32_t* slot_ids, const int64_t* off,
-                                        const int32_t* tok) {
+constexpr int PREP_THREADS = 1024;
+__global__ void __launch_bounds__(PREP_THREADS)
+requests_prepare_kernel(sd_store sv, int n, const int32_t* slot_ids, const int64_t* off, const int32_t* tok) {
     const int q = blockIdx.x;
     if (q >= n) return;
     const int slot = slot_ids[q];
@@ -1127,99 +1239,59 @@ __global__ void requests_prepare_kernel(sd_store sv, int n, const int32_t* slot_
         for (i64 k = threadIdx.x; k < hi - lo; k += blockDim.x) text[k] = tok[lo + k];
 }
 
-struct RequestLayout {       // where request q's nodes go (device arrays of n entries)
-    int* run_base;           // global position of its first child run
-    int* n1;                 // its depth-1 nodes
-    int* r1lo;               // depth-1 nodes of earlier requests
-    int* used;               // entries it takes
-    int* live;               // nodes
-    int* ok;                 // fits its pool and text buffer
-};
-
-__global__ void requests_layout_kernel(sd_store sv, int n, const int64_t* off, const int* nbase, const int* runstart,
-                                       const int* r1, RequestLayout L) {
-    const int q = blockIdx.x * blockDim.x + threadIdx.x;
-    if (q >= n) return;
-    const i64 lo = off[q], hi = off[q + 1];
-    const int first = 1 + nbase[lo], next = 1 + nbase[hi];
-    const int rb = runstart[first], re = runstart[next];
-    const int n1 = r1[hi] - r1[lo];
-    L.run_base[q] = rb; L.n1[q] = n1; L.r1lo[q] = r1[lo];
-    L.used[q] = n1 + (re - rb); L.live[q] = next - first;
-    L.ok[q] = ((i64)n1 + (re - rb) <= sv.spn && hi - lo <= sv.T) ? 1 : 0;
-}
-
-__global__ void emit_nodes_slots_kernel(sd_store sv, int n_req, const int32_t* slot_ids, const int64_t* off,
-                                        const int32_t* mtok, const uint32_t* sa, const uint8_t* lcp, const uint8_t* len,
-                                        i64 n, LevelTables T, const int* nbase, const int* nchild, const int* runstart,
-                                        RequestLayout L) {
-    const i64 j = (i64)blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= n) return;
-    const int l = lcp[j], m = len[j];
-    if (m <= l) return;
-    const i64 text = (i64)sa[j];
-    const int q = seq_rank_of(off, n_req, text);
-    const int slot = slot_ids[q];
-    if (!L.ok[q] || slot < 0 || slot >= sv.R) return;
-    int4* ent = sv.s_ent + (i64)slot * sv.spn;
-    const int shift = L.n1[q] - L.run_base[q];                  // global run position -> index in the slot pool
-    int nid = 1 + nbase[j];
-    int pos = T.E[j] - L.r1lo[q];                               // depth 1: the request's own root table
-    if (l >= 1) {
-        const int jx = T.before[j];
-        const int pnid = 1 + nbase[jx] + (l - (int)lcp[jx] - 1);
-        const int* row = T.E + (i64)l * (T.N + 1);
-        pos = runstart[pnid] + (row[j] - row[jx]) + shift;
-    }
-    for (int d = l + 1; d <= m; ++d, ++nid) {
-        const int nc = nchild[nid];
-        int4 e;
-        e.x = mtok[text + d - 1] - q * sv.V;
-        e.y = T.node_end[nid] - (int)j;
-        e.z = nc > 0 ? runstart[nid] + shift : 0;
-        e.w = nc > 0 ? (int)((unsigned)nc | RUN_STATIC) : 0;
-        ent[pos] = e;
-        if (d == 1) (sv.s_root + (i64)slot * sv.V)[e.x] = pos;
-        pos = runstart[nid] + shift;                             // the next one is this node's first child
+// S and the depth-1 nodes in front of every request's first suffix (the requests' suffixes are consecutive in the
+// order): a block per request, [n] = all
+__global__ void requests_bounds_kernel(TreeScan T, int n, const int64_t* off, int* s_req, int* n1_req) {
+    __shared__ int part[2][4];
+    const int q = blockIdx.x;
+    const int j = (int)off[q], tile = j / T.tile_len;
+    int a = 0, b = 0;
+    for (int i = tile * T.tile_len + threadIdx.x; i < j; i += 128) { const int l = T.lcp[i]; a += T.len[i] - max(l, 1); b += l == 0 ? 1 : 0; }
+    a = (int)__reduce_add_sync(TS_FULL, (unsigned)a);
+    b = (int)__reduce_add_sync(TS_FULL, (unsigned)b);
+    if ((threadIdx.x & 31) == 0) { part[0][threadIdx.x >> 5] = a; part[1][threadIdx.x >> 5] = b; }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int k = 1; k < 4; ++k) { a += part[0][k]; b += part[1][k]; }
+        s_req[q] = T.s[tile] + a; n1_req[q] = T.n1[tile] + b;
     }
 }
 
-// one warp per request: bookkeeping and the active nodes (lane d-1: node of the last d tokens)
-__global__ void requests_finalize_kernel(sd_store sv, int n, const int32_t* slot_ids, const int64_t* off,
-                                         RequestLayout L) {
-    const int q = (int)((blockIdx.x * (i64)blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
+// one block per request: bookkeeping and the active nodes (eight lanes per depth: node of the last d tokens)
+__global__ void __launch_bounds__(256)
+requests_finalize_kernel(sd_store sv, int n, const int32_t* slot_ids, const int64_t* off, const int* s_req, const int* n1_req) {
+    const int q = blockIdx.x, lane = threadIdx.x & 31, d = threadIdx.x / APP_LANES + 1;
     if (q >= n) return;
     const int slot = slot_ids[q];
     if (slot < 0 || slot >= sv.R) return;
     SlotState* ss = sv.s_state + slot;
-    const bool ok = L.ok[q] != 0;
+    const int n1 = n1_req ? n1_req[q + 1] - n1_req[q] : 0, used = n1_req ? n1 + s_req[q + 1] - s_req[q] : 0;
+    const bool ok = used <= sv.spn && off[q + 1] - off[q] <= sv.T;
     const int len = ok ? (int)(off[q + 1] - off[q]) : 0;
     const int4* ent = sv.s_ent + (i64)slot * sv.spn;
     const int32_t* root = sv.s_root + (i64)slot * sv.V;
     const int32_t* text = sv.s_text + (i64)slot * sv.T;
-    int node = -1, rcb = 0;
-    unsigned rw = 0;
-    const int d = lane + 1;
+    int node = -1;
+    int2 zw = make_int2(0, 0);
     if (d <= len && d <= sv.D) {
         node = root[text[len - d]];
-        int4 e = make_int4(0, 0, 0, 0);
-        if (node >= 0) e = ent[node];
-        for (int k = 1; k < d && node >= 0; ++k) {
-            const int x = text[len - d + k];
-            const int cb = e.z, nn = (int)((unsigned)e.w & RUN_COUNT_MASK);
-            int lo = 0, hi = nn;
-            while (lo < hi) {                                    // at most 24 rounds
-                const int mid = (lo + hi) >> 1;
-                if (ent[cb + mid].x < x) lo = mid + 1; else hi = mid;
-            }
-            node = -1;
-            if (lo < nn) { e = ent[cb + lo]; if (e.x == x) node = cb + lo; }
-        }
-        if (node >= 0) { rcb = e.z; rw = (unsigned)e.w; }
+        if (node >= 0) zw = *reinterpret_cast<const int2*>(&ent[node].z);
     }
-    ss->active[lane] = node; ss->room[lane] = 0; ss->run_cb[lane] = rcb; ss->run_w[lane] = rw;
-    if (lane == 0) {
-        ss->len = len; ss->used = ok ? L.used[q] : 0; ss->live = ok ? L.live[q] : 0;
+    for (int k = 1; k < SD_MAX_DEPTH; ++k) {
+        const bool on = node >= 0 && k < d;
+        if (!__any_sync(TS_FULL, on)) break;
+        const int x = on ? text[len - d + k] : -1;
+        int place;
+        int2 next;
+        const int at = group_lookup(RunSearch{ent + zw.x, 0, on ? (int)((unsigned)zw.y & RUN_COUNT_MASK) : 0}, x, lane, place, next);
+        if (on) { node = at >= 0 ? zw.x + at : -1; zw = next; }
+    }
+    if ((lane & (APP_LANES - 1)) == 0) {
+        ss->active[d - 1] = node; ss->room[d - 1] = 0;
+        ss->run_cb[d - 1] = node >= 0 ? zw.x : 0; ss->run_w[d - 1] = node >= 0 ? (unsigned)zw.y : 0u;
+    }
+    if (threadIdx.x == 0) {
+        ss->len = len; ss->used = ok ? used : 0; ss->live = ok ? used : 0;
         ss->status = ok ? 0 : SD_STATUS_POOL_FULL;
         ss->gen += 1;
     }
@@ -1254,10 +1326,9 @@ extern "C" int sd_build_requests(sd_store* s, int32_t n, const int32_t* h_slot, 
     int32_t *d_slot = nullptr, *mtok = nullptr;
     int64_t* d_off = nullptr;
     int* bad = nullptr;
-    RequestLayout L;
+    int *s_req = nullptr, *n1_req = nullptr;
     bool ok = P.tmp.get(&d_slot, n) && P.tmp.get(&d_off, n + 1) && P.tmp.get(&mtok, N) && P.tmp.get(&bad, 1) &&
-              P.tmp.get(&L.run_base, n) && P.tmp.get(&L.n1, n) && P.tmp.get(&L.r1lo, n) &&
-              P.tmp.get(&L.used, n) && P.tmp.get(&L.live, n) && P.tmp.get(&L.ok, n);
+              P.tmp.get(&s_req, n + 1) && P.tmp.get(&n1_req, n + 1);
     if (!ok) return SD_ERR_NOMEM;
     SD_CUDA_OK(cudaMemcpyAsync(d_slot, h_slot, sizeof(int32_t) * n, cudaMemcpyHostToDevice, st));
     SD_CUDA_OK(cudaMemcpyAsync(d_off, h_offsets, sizeof(int64_t) * (n + 1), cudaMemcpyHostToDevice, st));
@@ -1269,23 +1340,20 @@ extern "C" int sd_build_requests(sd_store* s, int32_t n, const int32_t* h_slot, 
         SD_CUDA_OK(cudaStreamSynchronize(st));
         if (h_bad) return SD_ERR_INVALID_ARG;                    // nothing was changed yet
     }
-    requests_prepare_kernel<<<(unsigned)n, T256, 0, st>>>(*s, n, d_slot, d_off, d_tokens);
+    requests_prepare_kernel<<<(unsigned)n, PREP_THREADS, 0, st>>>(*s, n, d_slot, d_off, d_tokens);
     if (N > 0) {
         i64 max_len = 0;
         for (int q = 0; q < n; ++q) max_len = std::max<i64>(max_len, h_offsets[q + 1] - h_offsets[q]);
-        // a handful of prompts: no round trips to the host on the way
-        const bool small = N <= 65536;
-        const int rc = pipeline_run(P, mtok, d_off, n, N, (i64)n * s->V, D, false, st, max_len, small);
+        int rc = pipeline_run(P, mtok, d_off, n, N, (i64)n * s->V, D, false, st, max_len);
         if (rc != SD_OK) return rc;
-        requests_layout_kernel<<<grid_for(n, T256), T256, 0, st>>>(*s, n, d_off, P.nbase, P.runstart, P.lv.E, L);
-        emit_nodes_slots_kernel<<<grid_for(N, T256), T256, 0, st>>>(*s, n, d_slot, d_off, mtok, P.sa, P.lcp, P.len, N, P.lv,
-                                                                   P.nbase, P.nchild, P.runstart, L);
-    } else {
-        SD_CUDA_OK(cudaMemsetAsync(L.ok, 0xFF, sizeof(int) * n, st));
-        SD_CUDA_OK(cudaMemsetAsync(L.used, 0, sizeof(int) * n, st));
-        SD_CUDA_OK(cudaMemsetAsync(L.live, 0, sizeof(int) * n, st));
+        requests_bounds_kernel<<<(unsigned)n + 1, 128, 0, st>>>(P.ts, n, d_off, s_req, n1_req);
+        TreeOut out;
+        memset(&out, 0, sizeof(out));
+        out.sv = *s; out.n_req = n; out.slot = d_slot; out.off = d_off; out.s_req = s_req; out.n1_req = n1_req;
+        rc = emit_entries<true>(P.ts, out, st);
+        if (rc != SD_OK) return rc;
     }
-    requests_finalize_kernel<<<grid_for((i64)n * 32, T256), T256, 0, st>>>(*s, n, d_slot, d_off, L);
+    requests_finalize_kernel<<<(unsigned)n, 256, 0, st>>>(*s, n, d_slot, d_off, N > 0 ? s_req : nullptr, N > 0 ? n1_req : nullptr);
     // (no synchronisation: the temporaries stay in the store's workspace, and a later call on
     // another stream must be ordered behind this one by the caller like any other use of the store)
     SD_CUDA_OK(cudaGetLastError());
