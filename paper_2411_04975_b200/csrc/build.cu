@@ -5,10 +5,14 @@
 // Hand-written LSD radix sort and scans (no CUB / Thrust).
 // Also: sd_build_requests (the trees of a batch of new requests by the same pipeline).
 #include <algorithm>
+#include <chrono>
 #include <mutex>
 #include <new>
 #include <stdio.h>
 #include <string.h>
+
+#include <unordered_map>
+#include <vector>
 
 #include "append_core.cuh"
 
@@ -894,62 +898,64 @@ __global__ void init_global_state_kernel(GlobalState* g, int used, int live, lon
 
 }  // namespace
 
-// Device memory comes from one stream-ordered pool per device, which keeps up to 1/32 of the
-// device's memory (5.7 GB of a B200's) from store to store and gives everything above that back
-// at the next synchronisation.  Mapping fresh memory is what a build or a short-lived store
-// would otherwise spend its time on: 20 cudaMalloc / cudaFree calls took 2.7 ms of the 3.7 ms of a
-// 32,768-token build and up to 70 ms of a 4 M-token one.  An allocation that fails empties the
-// pool and is tried once more, so the memory kept never stands in the way of a store.
+// Device memory: blocks that stores and builds have given back are kept for the next ones, up to 1/32 of the
+// device's memory (5.7 GB of a B200's); the oldest go first when there are more, all of them when an allocation
+// fails (which is then tried once more), and those that nobody has wanted for half a minute.  Getting
+// and returning memory is what a build or a short-lived store would otherwise spend its time on: 20
+// cudaMalloc / cudaFree calls took 2.7 ms of the 3.7 ms of a 32,768-token build and up to 70 ms of a
+// 4 M-token one.  (CUDA's own stream-ordered pools cost 6.2 ms per GB whenever they grow or shrink, cudaMalloc
+// 0.3 - 0.8 ms at any of these sizes.)  A block is given back when the work on it has ended, so the next owner may be
+// on any stream or thread.
 //
 // Test hook: the k-th device allocation from now on fails (k = 1: the next one); 0 switches it off.
-// Only the allocation-failure tests use it.  While it is on, memory comes from a second pool that
-// keeps nothing.
+// Only the allocation-failure tests use it.  While it is on nothing is kept.
 namespace {
 
-constexpr int POOL_DEVICES = 64;
-constexpr int POOL_KEEP_FRACTION = 32;
+constexpr int CACHE_DEVICES = 64;
+constexpr int CACHE_FRACTION = 32;
+constexpr double CACHE_SECONDS = 30.0;
 constexpr int KEPT_STREAMS = 8;
 
+typedef std::chrono::steady_clock Clock;
 struct StreamSet { cudaStream_t aux; cudaEvent_t ev_fork, ev_join; };
-struct DevicePool {
-    cudaMemPool_t pool[2] = {nullptr, nullptr};       // [0] keeps memory, [1] keeps none
-    StreamSet idle[KEPT_STREAMS];                     // stream and events of freed stores, for the next ones
-    int n_idle = 0;
+struct FreeBlock { void* p; size_t bytes; Clock::time_point since; };
+struct DeviceCache {
+    std::vector<FreeBlock> idle;                      // oldest first
+    size_t bytes = 0, most = 0;
+    StreamSet streams[KEPT_STREAMS];                  // stream and events of freed stores, for the next ones
+    int n_streams = 0;
 };
-DevicePool g_pool[POOL_DEVICES];
-std::mutex g_pool_mutex;
+struct OwnedBlock { size_t bytes; int dev; };
+DeviceCache g_cache[CACHE_DEVICES];
+std::unordered_map<void*, OwnedBlock> g_owned;        // blocks in use
+std::mutex g_cache_mutex;
 long long g_fail_alloc_in = 0;
 bool g_fail_alloc_on = false;
 
-cudaError_t pool_of(int dev, int which, cudaMemPool_t* out) {
-    if (dev < 0 || dev >= POOL_DEVICES) return cudaErrorInvalidDevice;
-    std::lock_guard<std::mutex> lock(g_pool_mutex);
-    cudaMemPool_t& p = g_pool[dev].pool[which];
-    if (!p) {
-        size_t free_bytes = 0, total = 0;
-        cudaError_t e = cudaMemGetInfo(&free_bytes, &total);
-        if (e != cudaSuccess) return e;
-        cudaMemPoolProps props;
-        memset(&props, 0, sizeof(props));
-        props.allocType = cudaMemAllocationTypePinned;
-        props.location.type = cudaMemLocationTypeDevice;
-        props.location.id = dev;
-        e = cudaMemPoolCreate(&p, &props);
-        if (e != cudaSuccess) { p = nullptr; return e; }
-        uint64_t keep = which == 0 ? (uint64_t)total / POOL_KEEP_FRACTION : 0;
-        e = cudaMemPoolSetAttribute(p, cudaMemPoolAttrReleaseThreshold, &keep);
-        if (e != cudaSuccess) return e;
+// gives back the oldest blocks until at most `bytes` are kept (the mutex is held)
+void cache_trim(DeviceCache& c, size_t bytes) {
+    size_t n = 0;
+    while (n < c.idle.size() && c.bytes > bytes) { cudaFree(c.idle[n].p); c.bytes -= c.idle[n].bytes; ++n; }
+    c.idle.erase(c.idle.begin(), c.idle.begin() + n);
+}
+
+void cache_expire(DeviceCache& c) {
+    const Clock::time_point now = Clock::now();
+    size_t n = 0;
+    while (n < c.idle.size() && std::chrono::duration<double>(now - c.idle[n].since).count() > CACHE_SECONDS) {
+        cudaFree(c.idle[n].p);
+        c.bytes -= c.idle[n].bytes;
+        ++n;
     }
-    *out = p;
-    return cudaSuccess;
+    c.idle.erase(c.idle.begin(), c.idle.begin() + n);
 }
 
 // a stream and two events for a store on the current device
 bool take_streams(int dev, StreamSet* out) {
-    if (dev >= 0 && dev < POOL_DEVICES) {
-        std::lock_guard<std::mutex> lock(g_pool_mutex);
-        DevicePool& d = g_pool[dev];
-        if (d.n_idle > 0) { *out = d.idle[--d.n_idle]; return true; }
+    if (dev >= 0 && dev < CACHE_DEVICES) {
+        std::lock_guard<std::mutex> lock(g_cache_mutex);
+        DeviceCache& d = g_cache[dev];
+        if (d.n_streams > 0) { *out = d.streams[--d.n_streams]; return true; }
     }
     out->aux = nullptr; out->ev_fork = nullptr; out->ev_join = nullptr;
     if (cudaStreamCreateWithFlags(&out->aux, cudaStreamNonBlocking) == cudaSuccess &&
@@ -964,9 +970,9 @@ bool take_streams(int dev, StreamSet* out) {
 
 void give_streams(int dev, const StreamSet& s) {
     {
-        std::lock_guard<std::mutex> lock(g_pool_mutex);
-        if (dev >= 0 && dev < POOL_DEVICES && g_pool[dev].n_idle < KEPT_STREAMS) {
-            g_pool[dev].idle[g_pool[dev].n_idle++] = s;
+        std::lock_guard<std::mutex> lock(g_cache_mutex);
+        if (dev >= 0 && dev < CACHE_DEVICES && g_cache[dev].n_streams < KEPT_STREAMS) {
+            g_cache[dev].streams[g_cache[dev].n_streams++] = s;
             return;
         }
     }
@@ -977,27 +983,63 @@ void give_streams(int dev, const StreamSet& s) {
 
 }  // namespace
 
-cudaError_t sd_device_malloc(void** p, size_t bytes, cudaStream_t st) {
+cudaError_t sd_device_malloc(void** p, size_t bytes) {
     *p = nullptr;
     if (g_fail_alloc_in > 0 && --g_fail_alloc_in == 0) return cudaErrorMemoryAllocation;
     int dev = -1;
-    cudaMemPool_t pool;
     cudaError_t e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = pool_of(dev, g_fail_alloc_on ? 1 : 0, &pool);
     if (e != cudaSuccess) return e;
-    e = cudaMallocFromPoolAsync(p, bytes, pool, st);
-    if (e != cudaSuccess) {
-        cudaGetLastError();
-        cudaStreamSynchronize(st);
-        cudaMemPoolTrimTo(pool, 0);
-        e = cudaMallocFromPoolAsync(p, bytes, pool, st);
-        if (e != cudaSuccess) *p = nullptr;
+    if (dev < 0 || dev >= CACHE_DEVICES) return cudaErrorInvalidDevice;
+    // (up to a multiple of an eighth of the next lower power of two, 32 MB at most, so that sizes that differ a little share blocks)
+    size_t unit = 512;
+    while (unit * 16 <= bytes && unit < (32u << 20)) unit *= 2;
+    bytes = (bytes + unit - 1) / unit * unit;
+    std::lock_guard<std::mutex> lock(g_cache_mutex);
+    DeviceCache& c = g_cache[dev];
+    if (!g_fail_alloc_on) {
+        cache_expire(c);
+        // the smallest kept block that is not much too large
+        size_t best = c.idle.size();
+        for (size_t k = 0; k < c.idle.size(); ++k)
+            if (c.idle[k].bytes >= bytes && c.idle[k].bytes <= bytes + bytes / 4 && (best == c.idle.size() || c.idle[k].bytes < c.idle[best].bytes))
+                best = k;
+        if (best < c.idle.size()) {
+            *p = c.idle[best].p;
+            g_owned[*p] = OwnedBlock{c.idle[best].bytes, dev};
+            c.bytes -= c.idle[best].bytes;
+            c.idle.erase(c.idle.begin() + best);
+            return cudaSuccess;
+        }
     }
-    return e;
+    e = cudaMalloc(p, bytes);
+    if (e != cudaSuccess && !c.idle.empty()) {
+        cudaGetLastError();
+        cache_trim(c, 0);
+        e = cudaMalloc(p, bytes);
+    }
+    if (e != cudaSuccess) { *p = nullptr; return e; }
+    g_owned[*p] = OwnedBlock{bytes, dev};
+    return cudaSuccess;
 }
 
-// behind everything `st` holds at the call
-void sd_device_free(void* p, cudaStream_t st) { if (p) cudaFreeAsync(p, st); }
+void sd_device_free(void* p) {
+    if (!p) return;
+    std::lock_guard<std::mutex> lock(g_cache_mutex);
+    auto it = g_owned.find(p);
+    if (it == g_owned.end()) return;
+    const OwnedBlock b = it->second;
+    g_owned.erase(it);
+    DeviceCache& c = g_cache[b.dev];
+    if (c.most == 0) {
+        size_t free_bytes = 0, total = 0;
+        if (cudaMemGetInfo(&free_bytes, &total) == cudaSuccess) c.most = total / CACHE_FRACTION;
+    }
+    if (g_fail_alloc_on || b.bytes > c.most) { cudaFree(p); return; }
+    cache_expire(c);
+    cache_trim(c, c.most - b.bytes);
+    c.idle.push_back(FreeBlock{p, b.bytes, Clock::now()});
+    c.bytes += b.bytes;
+}
 
 extern "C" void sd_debug_fail_alloc(int64_t k) { g_fail_alloc_in = k; g_fail_alloc_on = k > 0; }
 
@@ -1011,13 +1053,17 @@ struct DeviceArena {          // temporaries of one build: freed together, or ke
     long long chunk_left = 0;
     cudaStream_t st;                                  // the buffers belong to the work on this stream
     explicit DeviceArena(cudaStream_t stream) : st(stream) {}
-    ~DeviceArena() { if (!keep) for (int i = 0; i < n; ++i) sd_device_free(ptr[i], st); }
+    ~DeviceArena() {
+        if (keep || n == 0) return;
+        cudaStreamSynchronize(st);
+        for (int i = 0; i < n; ++i) sd_device_free(ptr[i]);
+    }
     // One allocation for the buffers to come (an allocation of its own costs far more than the
     // kernels that use a buffer).  If it fails the buffers are simply allocated one by one.
     void reserve(long long bytes) {
         if (keep || n >= 48 || bytes <= 0) return;
         void* p = nullptr;
-        if (sd_device_malloc(&p, (size_t)bytes, st) != cudaSuccess) { cudaGetLastError(); return; }
+        if (sd_device_malloc(&p, (size_t)bytes) != cudaSuccess) { cudaGetLastError(); return; }
         ptr[n++] = p;
         chunk = (char*)p; chunk_left = bytes;
     }
@@ -1034,17 +1080,17 @@ struct DeviceArena {          // temporaries of one build: freed together, or ke
         if (keep) {
             const int k = n++;
             if (keep->bytes[k] < need) {
-                sd_device_free(keep->ptr[k], st);
+                if (keep->ptr[k]) { cudaStreamSynchronize(st); sd_device_free(keep->ptr[k]); }
                 keep->ptr[k] = nullptr; keep->bytes[k] = 0;
                 const long long want = need + need / 4 + 256;
-                if (sd_device_malloc(&keep->ptr[k], (size_t)want, st) != cudaSuccess) { cudaGetLastError(); return false; }
+                if (sd_device_malloc(&keep->ptr[k], (size_t)want) != cudaSuccess) { cudaGetLastError(); return false; }
                 keep->bytes[k] = want;
             }
             *out = (T*)keep->ptr[k];
             return true;
         }
         void* p = nullptr;
-        if (sd_device_malloc(&p, (size_t)need, st) != cudaSuccess) { cudaGetLastError(); return false; }
+        if (sd_device_malloc(&p, (size_t)need) != cudaSuccess) { cudaGetLastError(); return false; }
         ptr[n++] = p;
         *out = (T*)p;
         return true;
@@ -1062,25 +1108,25 @@ int bits_for(i64 maxval) {
 }  // namespace
 
 template <class T>
-static bool store_alloc(sd_store* s, T** out, long long count, cudaStream_t st) {
+static bool store_alloc(sd_store* s, T** out, long long count) {
     void* p = nullptr;
     if (count < 1) count = 1;
-    if (sd_device_malloc(&p, (size_t)count * sizeof(T), st) != cudaSuccess) { cudaGetLastError(); return false; }
+    if (sd_device_malloc(&p, (size_t)count * sizeof(T)) != cudaSuccess) { cudaGetLastError(); return false; }
     s->device_bytes += count * (long long)sizeof(T);
     *out = (T*)p;
     return true;
 }
 
-// Releases what a store holds, on `st`: the caller has waited for every other stream that used the store.
+// Releases what a store holds, behind the work on `st`: the caller has waited for every other stream that used the store.
 static void store_release(sd_store* s, cudaStream_t st) {
     if (!s) return;
+    cudaStreamSynchronize(st);
     void* const own[] = {s->g_ent, s->g_root, s->g_state, s->s_ent, s->s_root, s->s_text, s->s_state};
-    for (void* p : own) sd_device_free(p, st);
+    for (void* p : own) sd_device_free(p);
     if (s->ws) {
-        for (int k = 0; k < 48; ++k) sd_device_free(s->ws->ptr[k], st);
+        for (int k = 0; k < 48; ++k) sd_device_free(s->ws->ptr[k]);
         delete s->ws;
     }
-    cudaStreamSynchronize(st);                        // the memory is free for any stream from here on
     if (s->aux) give_streams(s->device, StreamSet{s->aux, s->ev_fork, s->ev_join});
     delete s;
 }
@@ -1229,9 +1275,9 @@ extern "C" int sd_build(const sd_build_params* p, const int32_t* d_corpus, const
     s->spn = p->slot_pool_nodes > 0 ? p->slot_pool_nodes : 2ll * s->T * D;
     if (s->spn >= (1ll << 31) - 2) { delete s; return SD_ERR_INVALID_ARG; }
 
-    bool ok = store_alloc(s, &s->g_root, s->V, st) && store_alloc(s, &s->g_state, 1, st) &&
-              store_alloc(s, &s->s_ent, (i64)s->R * s->spn, st) && store_alloc(s, &s->s_root, (i64)s->R * s->V, st) &&
-              store_alloc(s, &s->s_text, (i64)s->R * s->T, st) && store_alloc(s, &s->s_state, s->R, st);
+    bool ok = store_alloc(s, &s->g_root, s->V) && store_alloc(s, &s->g_state, 1) &&
+              store_alloc(s, &s->s_ent, (i64)s->R * s->spn) && store_alloc(s, &s->s_root, (i64)s->R * s->V) &&
+              store_alloc(s, &s->s_text, (i64)s->R * s->T) && store_alloc(s, &s->s_state, s->R);
     if (!ok) { store_release(s, st); return SD_ERR_NOMEM; }
     StreamSet streams;
     if (!take_streams(s->device, &streams)) { store_release(s, st); return SD_ERR_CUDA; }
@@ -1275,7 +1321,7 @@ extern "C" int sd_build(const sd_build_params* p, const int32_t* d_corpus, const
     i64 extra = p->global_extra_nodes >= 0 ? p->global_extra_nodes : std::max<i64>(1ll << 22, n_nodes);
     s->g_cap = used_entries + extra;
     if (s->g_cap >= (1ll << 31) - 2) { store_release(s, st); return SD_ERR_INVALID_ARG; }
-    if (!store_alloc(s, &s->g_ent, s->g_cap, st)) { store_release(s, st); return SD_ERR_NOMEM; }
+    if (!store_alloc(s, &s->g_ent, s->g_cap)) { store_release(s, st); return SD_ERR_NOMEM; }
 
     if (N > 0) {
         TreeOut out;

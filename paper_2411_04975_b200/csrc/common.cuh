@@ -116,9 +116,9 @@ __host__ __device__ inline uint32_t sd_run_capacity(uint32_t w) {
         if (_e != cudaSuccess) return SD_ERR_CUDA;         \
     } while (0)
 
-// Device memory of the library (build.cu): from a pool, ordered on `st`.
-cudaError_t sd_device_malloc(void** p, size_t bytes, cudaStream_t st);
-void sd_device_free(void* p, cudaStream_t st);
+// Device memory of the library (build.cu), and back when the work on it has ended.
+cudaError_t sd_device_malloc(void** p, size_t bytes);
+void sd_device_free(void* p);
 
 // Every entry point refuses a store that lives on another device than the current one.
 #define SD_CHECK_DEVICE(s)                                                   \

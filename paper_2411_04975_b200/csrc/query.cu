@@ -267,10 +267,10 @@ extern "C" int sd_entropy(sd_store* s, int32_t tree, double* h_entropy, void* st
     struct Small { unsigned long long total, wsum; double acc; int count[SD_MAX_DEPTH + 1]; } h_small;
     int2* queue = nullptr;
     Small* d_small = nullptr;
-    if (sd_device_malloc((void**)&queue, sizeof(int2) * 2 * (size_t)room, st) != cudaSuccess ||
-        sd_device_malloc((void**)&d_small, sizeof(Small), st) != cudaSuccess) {
+    if (sd_device_malloc((void**)&queue, sizeof(int2) * 2 * (size_t)room) != cudaSuccess ||
+        sd_device_malloc((void**)&d_small, sizeof(Small)) != cudaSuccess) {
         cudaGetLastError();
-        sd_device_free(queue, st); sd_device_free(d_small, st);
+        sd_device_free(queue); sd_device_free(d_small);
         return SD_ERR_NOMEM;
     }
     cudaError_t ce = cudaMemsetAsync(d_small, 0, sizeof(Small), st);
@@ -283,9 +283,10 @@ extern "C" int sd_entropy(sd_store* s, int32_t tree, double* h_entropy, void* st
         entropy_runs_kernel<<<grid, ENT_THREADS, 0, st>>>(ent, queue + (g & 1) * room, &d_small->count[g], queue + ((g & 1) ^ 1) * room,
                                                           &d_small->count[g + 1], &d_small->acc, &d_small->wsum);
     if (ce == cudaSuccess) ce = cudaMemcpyAsync(&h_small, d_small, sizeof(Small), cudaMemcpyDeviceToHost, st);
-    sd_device_free(queue, st);
-    sd_device_free(d_small, st);
-    if (ce == cudaSuccess) ce = cudaStreamSynchronize(st);
+    const cudaError_t done = cudaStreamSynchronize(st);
+    if (ce == cudaSuccess) ce = done;
+    sd_device_free(queue);
+    sd_device_free(d_small);
     if (ce == cudaSuccess) ce = cudaGetLastError();
     if (ce != cudaSuccess) return SD_ERR_CUDA;
     *h_entropy = h_small.wsum ? h_small.acc / (double)h_small.wsum : 0.0;
@@ -346,13 +347,14 @@ extern "C" int sd_enumerate(sd_store* s, int32_t tree, int64_t max_nodes, int32_
     const long long room = max_nodes > 0 ? max_nodes : 1;        // nodes with children among the records written
     int *fe[2] = {nullptr, nullptr}, *fr[2] = {nullptr, nullptr};
     unsigned char* small = nullptr;                              // n_out, frontier sizes
-    bool okm = sd_device_malloc((void**)&small, 64, st) == cudaSuccess;
+    bool okm = sd_device_malloc((void**)&small, 64) == cudaSuccess;
     for (int b = 0; b < 2 && okm; ++b)
-        okm = sd_device_malloc((void**)&fe[b], sizeof(int) * (size_t)room, st) == cudaSuccess &&
-              sd_device_malloc((void**)&fr[b], sizeof(int) * (size_t)room, st) == cudaSuccess;
+        okm = sd_device_malloc((void**)&fe[b], sizeof(int) * (size_t)room) == cudaSuccess &&
+              sd_device_malloc((void**)&fr[b], sizeof(int) * (size_t)room) == cudaSuccess;
     auto release = [&]() {
-        sd_device_free(small, st);
-        for (int b = 0; b < 2; ++b) { sd_device_free(fe[b], st); sd_device_free(fr[b], st); }
+        cudaStreamSynchronize(st);
+        sd_device_free(small);
+        for (int b = 0; b < 2; ++b) { sd_device_free(fe[b]); sd_device_free(fr[b]); }
     };
     if (!okm) { cudaGetLastError(); release(); return SD_ERR_NOMEM; }
     unsigned long long* n_out = (unsigned long long*)small;
