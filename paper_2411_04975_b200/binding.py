@@ -8,6 +8,7 @@ wraps them with output allocation.
 from __future__ import annotations
 
 import ctypes as C
+import functools
 import os
 from typing import Dict, Optional
 
@@ -93,6 +94,9 @@ def library() -> C.CDLL:
 def _ptr(t: Optional[torch.Tensor], dtype: torch.dtype, name: str) -> Optional[int]:
     if t is None:
         return None
+    # (the usual case first: a small batch's draft takes the GPU no longer than such checks take the host)
+    if t.dtype is dtype and t.is_cuda and t.is_contiguous():
+        return t.data_ptr()
     # pinned host memory has a device address of its own (unified addressing): the kernels then
     # read or write it across the bus, with no copy before or after the call
     if not (t.is_cuda or t.is_pinned()) or t.dtype != dtype or not t.is_contiguous():
@@ -101,8 +105,30 @@ def _ptr(t: Optional[torch.Tensor], dtype: torch.dtype, name: str) -> Optional[i
     return t.data_ptr()
 
 
+_current_device = torch._C._cuda_getDevice if hasattr(torch._C, "_cuda_getDevice") else torch.cuda.current_device
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
 def _stream() -> int:
+    if _raw_stream is not None and torch.cuda.is_initialized():
+        return _raw_stream(_current_device())
     return torch.cuda.current_stream().cuda_stream
+
+
+_OUT_FIELDS = (("n_draft", torch.int32), ("tokens", torch.int32), ("parents", torch.int32), ("positions", torch.int32),
+               ("mask", torch.int32), ("chosen_tree", torch.int32), ("chosen_p", torch.int32), ("score", torch.float64),
+               ("status", torch.int32))
+
+
+def _out_ptrs(out: Dict[str, torch.Tensor]) -> list:
+    return [_ptr(out[name], dtype, name) for name, dtype in _OUT_FIELDS]
+
+
+@functools.lru_cache(maxsize=64)
+def _spec_params(P: int, alpha: float, max_spec: int, flags: int, tau: float):
+    """The converted parameters of a draft (read by the library only) and a pointer to them."""
+    prm = _SpecParams(P, alpha, max_spec, flags, tau)
+    return prm, C.pointer(prm)
 
 
 # ---- the C entry points, one to one ------------------------------------------------------
@@ -132,14 +158,9 @@ def sd_append(store: int, slots: torch.Tensor, offsets: torch.Tensor, tokens: to
 
 def sd_speculate(store: int, slots: torch.Tensor, P: int, alpha: float, max_spec: int, flags: int,
                  budget_cap: Optional[torch.Tensor], out: Dict[str, torch.Tensor], tau: float = 0.0) -> None:
-    prm = _SpecParams(P, alpha, max_spec, flags, tau)
     rc = library().sd_speculate(
-        store, int(slots.numel()), _ptr(slots, torch.int32, "slots"), C.byref(prm),
-        _ptr(budget_cap, torch.int32, "budget_cap"), _ptr(out["n_draft"], torch.int32, "n_draft"),
-        _ptr(out["tokens"], torch.int32, "tokens"), _ptr(out["parents"], torch.int32, "parents"),
-        _ptr(out["positions"], torch.int32, "positions"), _ptr(out["mask"], torch.int32, "mask"),
-        _ptr(out["chosen_tree"], torch.int32, "chosen_tree"), _ptr(out["chosen_p"], torch.int32, "chosen_p"),
-        _ptr(out["score"], torch.float64, "score"), _ptr(out["status"], torch.int32, "status"), _stream())
+        store, slots.numel(), _ptr(slots, torch.int32, "slots"), _spec_params(P, alpha, max_spec, flags, tau)[1],
+        _ptr(budget_cap, torch.int32, "budget_cap"), *_out_ptrs(out), _stream())
     if rc != 0:
         raise SuffixSpecError(rc, "sd_speculate")
 
@@ -150,14 +171,9 @@ def sd_speculate_noalloc(store: int, slots: torch.Tensor, P: int, alpha: float, 
     records live in a fixed array inside the library, so the batch is limited
     (n * 2 * depth_cap <= 4096 jobs) and calls on one device must not overlap.
     `out` must be preallocated by the caller; nothing is allocated here."""
-    prm = _SpecParams(P, alpha, max_spec, flags, tau)
     rc = library().sd_speculate_noalloc(
-        store, int(slots.numel()), _ptr(slots, torch.int32, "slots"), C.byref(prm),
-        _ptr(budget_cap, torch.int32, "budget_cap"), _ptr(out["n_draft"], torch.int32, "n_draft"),
-        _ptr(out["tokens"], torch.int32, "tokens"), _ptr(out["parents"], torch.int32, "parents"),
-        _ptr(out["positions"], torch.int32, "positions"), _ptr(out["mask"], torch.int32, "mask"),
-        _ptr(out["chosen_tree"], torch.int32, "chosen_tree"), _ptr(out["chosen_p"], torch.int32, "chosen_p"),
-        _ptr(out["score"], torch.float64, "score"), _ptr(out["status"], torch.int32, "status"), _stream())
+        store, slots.numel(), _ptr(slots, torch.int32, "slots"), _spec_params(P, alpha, max_spec, flags, tau)[1],
+        _ptr(budget_cap, torch.int32, "budget_cap"), *_out_ptrs(out), _stream())
     if rc != 0:
         raise SuffixSpecError(rc, "sd_speculate_noalloc")
 
@@ -179,11 +195,7 @@ class BoundStep:
         self._args = (
             store._h, int(slots.numel()), _ptr(slots, torch.int32, "slots"), _ptr(offsets, torch.int64, "offsets"),
             _ptr(new_tokens, torch.int32, "new_tokens"), C.byref(self._prm), _ptr(budget_cap, torch.int32, "budget_cap"),
-            _ptr(out["n_draft"], torch.int32, "n_draft"), _ptr(out["tokens"], torch.int32, "tokens"),
-            _ptr(out["parents"], torch.int32, "parents"), _ptr(out["positions"], torch.int32, "positions"),
-            _ptr(out["mask"], torch.int32, "mask"), _ptr(out["chosen_tree"], torch.int32, "chosen_tree"),
-            _ptr(out["chosen_p"], torch.int32, "chosen_p"), _ptr(out["score"], torch.float64, "score"),
-            _ptr(out["status"], torch.int32, "status"), stream)
+            *_out_ptrs(out), stream)
 
     def __call__(self) -> Dict[str, torch.Tensor]:
         rc = self._fn(*self._args)
@@ -284,15 +296,10 @@ class SuffixStore:
         then speculate.  Same result as append() followed by speculate()."""
         if out is None:
             out = self.alloc_outputs(int(slots.numel()))
-        prm = _SpecParams(P, alpha, max_spec, flags, tau)
         rc = library().sd_step(
-            self._h, int(slots.numel()), _ptr(slots, torch.int32, "slots"), _ptr(offsets, torch.int64, "offsets"),
-            _ptr(new_tokens, torch.int32, "new_tokens"), C.byref(prm), _ptr(budget_cap, torch.int32, "budget_cap"),
-            _ptr(out["n_draft"], torch.int32, "n_draft"), _ptr(out["tokens"], torch.int32, "tokens"),
-            _ptr(out["parents"], torch.int32, "parents"), _ptr(out["positions"], torch.int32, "positions"),
-            _ptr(out["mask"], torch.int32, "mask"), _ptr(out["chosen_tree"], torch.int32, "chosen_tree"),
-            _ptr(out["chosen_p"], torch.int32, "chosen_p"), _ptr(out["score"], torch.float64, "score"),
-            _ptr(out["status"], torch.int32, "status"), _stream())
+            self._h, slots.numel(), _ptr(slots, torch.int32, "slots"), _ptr(offsets, torch.int64, "offsets"),
+            _ptr(new_tokens, torch.int32, "new_tokens"), _spec_params(P, alpha, max_spec, flags, tau)[1],
+            _ptr(budget_cap, torch.int32, "budget_cap"), *_out_ptrs(out), _stream())
         if rc != 0:
             raise SuffixSpecError(rc, "sd_step")
         return out
