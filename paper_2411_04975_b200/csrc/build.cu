@@ -49,30 +49,31 @@ __global__ void validate_kernel(const int32_t* tok, i64 n, int V, const int64_t*
 // Suffix order of a whole corpus by prefix doubling, in one cooperative launch.  After a round every suffix has
 // the rank of its first k tokens, and the order by the tokens behind those is the current order moved k places back, so
 // a round only has to sort by rank, stably, with LSD radix passes of 8 bits.  A last round that adds fewer than k
-// tokens looks at an overlapping window.  A rank also tells whether the sequence ends right behind the k tokens, so
-// that suffixes of equal rank either all go on or are equal altogether, and the ones that have nothing k places on
-// may take any place.  Order: by the first D tokens, a suffix that ends earlier before its extensions.
+// tokens looks at an overlapping window.  A rank also tells whether the sequence ends right behind the k tokens (its
+// lowest bit: the sequence goes on), so that suffixes of equal rank either all go on or are equal altogether, the ones
+// that have nothing k places on may take any place, and no look-up of a sequence's end is needed.  Order: by the first D tokens, a suffix that ends earlier before its extensions.
 //
 // A block owns a chunk of consecutive places throughout.  A pass: digit counts per block; a warp per digit adds them up
 // over the blocks; the blocks go through their chunks, SG_THREADS x ITEMS places at a time, ordering each lot in shared
 // memory so that what is written is consecutive.  Three grid barriers of about 1.5 us, and for 4.2 M suffixes, which stay
-// in L2, what the lots cost in barriers and ranking ballots.  (Separate histogram, scan and scatter launches over 64-bit
+// in L2, one random read per suffix for the keys, one for the new ranks, and what the lots cost in barriers and ballots.  (Separate histogram, scan and scatter launches over 64-bit
 // keys, six passes a round: 2.2 ms for 4.2 M suffixes, 0.45 ms for 32,768, of 100 launches.)
 constexpr int SG_THREADS = 512;
 constexpr int SG_WARPS = SG_THREADS / 32;
 constexpr int SG_BINS = 256;
+constexpr int SG_BATCH = 8;                       // random reads in flight per thread
 
 struct CorpusSort {
     const int32_t* tok;
     const int64_t* seq_off;
     int n_seqs;
     const int* end_pos;
-    int N, chunk;                                 // chunk: a multiple of SG_THREADS * ITEMS
+    int N, chunk;                                 // chunk: a multiple of 32
     unsigned key_bits;                            // of a token and one more
     int D;
     uint32_t *key[2], *val[2];
-    int* rank;                                    // [N]
-    unsigned* flags;                              // [N / 32 + 1] places where a new rank starts
+    int* rank;                                    // [N] rank from 0, times two, + 1: the sequence goes on behind its k tokens
+    unsigned *flags, *go;                         // [N / 32 + 1] by place: a new rank starts, the sequence goes on
     int* table;                                   // [SG_BINS][blocks]
     int* total;                                   // [SG_BINS]
     int* count;                                   // [blocks]
@@ -119,30 +120,47 @@ corpus_sort_kernel(CorpusSort A) {
     const unsigned lt = (1u << lane) - 1u;
     int cur = 0;                                                // the order so far: val[cur], with its keys in key[cur]
 
-    // digit counts of this block's chunk; `item` gives the key of a place
-    auto count_digits = [&](int shift, auto item) {
+    // digit counts of this block's chunk; `items` gives the keys of SG_BATCH places, SG_THREADS apart
+    auto count_digits = [&](int shift, auto items) {
         for (int d = tid; d < SG_BINS; d += SG_THREADS) sh.tot[d] = 0;
         __syncthreads();
-        for (int p = p_begin + tid; p < p_end; p += SG_THREADS) atomicAdd(&sh.tot[(item(p) >> shift) & (SG_BINS - 1)], 1);
+        for (int p = p_begin + tid; p < p_end; p += SG_THREADS * SG_BATCH) {
+            uint32_t k[SG_BATCH];
+            items(p, k);
+#pragma unroll
+            for (int u = 0; u < SG_BATCH; ++u)
+                if (p + u * SG_THREADS < p_end) atomicAdd(&sh.tot[(k[u] >> shift) & (SG_BINS - 1)], 1);
+        }
         __syncthreads();
         for (int d = tid; d < SG_BINS; d += SG_THREADS) A.table[(i64)d * G + blk] = sh.tot[d];
+    };
+    auto stored_keys = [&](int p, uint32_t (&k)[SG_BATCH]) {
+#pragma unroll
+        for (int u = 0; u < SG_BATCH; ++u) k[u] = p + u * SG_THREADS < p_end ? A.key[cur][p + u * SG_THREADS] : 0u;
     };
     // the counted pass: key / val [cur] to [cur ^ 1]
     auto scatter = [&](int shift) {
         grid.sync();
-        for (int d = blk * SG_WARPS + wib; d < SG_BINS; d += G * SG_WARPS) {
+        for (int d = wib * G + blk; d < SG_BINS; d += G * SG_WARPS) {
             int* const row = A.table + (i64)d * G;
             int run = 0;
-            for (int k0 = 0; k0 < G; k0 += 32) {
-                const int k = k0 + lane, v = k < G ? row[k] : 0;
-                int inc = v;
+            for (int k0 = 0; k0 < G; k0 += 32 * 10) {
+                int v[10];
 #pragma unroll
-                for (int o = 1; o < 32; o <<= 1) {
-                    const int y = __shfl_up_sync(0xffffffffu, inc, o);
-                    if (lane >= o) inc += y;
+                for (int u = 0; u < 10; ++u) { const int k = k0 + u * 32 + lane; v[u] = k < G ? row[k] : 0; }
+#pragma unroll
+                for (int u = 0; u < 10; ++u) {
+                    const int k = k0 + u * 32 + lane;
+                    int inc = v[u];
+#pragma unroll
+                    for (int o = 1; o < 32; o <<= 1) {
+                        const int y = __shfl_up_sync(0xffffffffu, inc, o);
+                        if (lane >= o) inc += y;
+                    }
+                    if (k < G) row[k] = run + inc - v[u];
+                    run += __shfl_sync(0xffffffffu, inc, 31);
+                    if (k0 + (u + 1) * 32 >= G) break;
                 }
-                if (k < G) row[k] = run + inc - v;
-                run += __shfl_sync(0xffffffffu, inc, 31);
             }
             if (lane == 0) A.total[d] = run;
         }
@@ -157,22 +175,25 @@ corpus_sort_kernel(CorpusSort A) {
         const uint32_t* const vi = A.val[cur];
         uint32_t* const ko = A.key[cur ^ 1];
         uint32_t* const vo = A.val[cur ^ 1];
-        for (int lot = p_begin; lot < p_end; lot += LOT) {
-            const int m = min(LOT, p_end - lot);
+        // lots of about the same size, every warp the same share of a lot: `per` items per thread, consecutive for the warp
+        const int lots = (p_end - p_begin + LOT - 1) / LOT;
+        const int per = lots > 0 ? ((p_end - p_begin + lots - 1) / lots + SG_THREADS - 1) / SG_THREADS : 1;
+        for (int lot = p_begin; lot < p_end; lot += per * SG_THREADS) {
+            const int m = min(per * SG_THREADS, p_end - lot);
             uint32_t key[ITEMS], val[ITEMS];
-            const int q0 = wib * 32 * ITEMS + lane;             // a warp's places are consecutive
+            const int q0 = wib * 32 * per + lane, q1 = min(m, (wib + 1) * 32 * per);
 #pragma unroll
             for (int u = 0; u < ITEMS; ++u) {
                 const int q = q0 + u * 32;
-                key[u] = q < m ? ki[lot + q] : 0u;
-                val[u] = q < m ? vi[lot + q] : 0u;
+                key[u] = q < q1 ? ki[lot + q] : 0u;
+                val[u] = q < q1 ? vi[lot + q] : 0u;
             }
             for (int d = lane; d < SG_BINS; d += 32) sh.cnt[wib][d] = 0;
             __syncwarp();
             int at[ITEMS];
 #pragma unroll
             for (int u = 0; u < ITEMS; ++u) {
-                const bool in = q0 + u * 32 < m;
+                const bool in = q0 + u * 32 < q1;
                 unsigned peers = __ballot_sync(0xffffffffu, in);
                 at[u] = 0;
                 if (!peers) continue;
@@ -202,7 +223,7 @@ corpus_sort_kernel(CorpusSort A) {
             __syncthreads();
 #pragma unroll
             for (int u = 0; u < ITEMS; ++u)
-                if (q0 + u * 32 < m) {
+                if (q0 + u * 32 < q1) {
                     const int digit = (int)((key[u] >> shift) & (SG_BINS - 1));
                     const int q = sh.start[digit] + sh.cnt[wib][digit] + at[u];
                     sh.key[q] = key[u]; sh.val[q] = val[u];
@@ -221,21 +242,36 @@ corpus_sort_kernel(CorpusSort A) {
         cur ^= 1;
         grid.sync();
     };
-    // ranks (from 0) of the order, a new one where the key or `second` differs from the place before; returns their number
+    // ranks (from 0) of the order, a new one where the key or what `second` makes of the value differs from the place before;
+    // returns their number
     auto rerank = [&](auto second) -> int {
         const uint32_t* const k = A.key[cur];
         const uint32_t* const v = A.val[cur];
         int mine = 0;
-        for (int w = p_begin / 32 + wib; w * 32 < p_end; w += SG_WARPS) {          // (chunks are multiples of 32)
-            const int p = w * 32 + lane;
-            uint32_t kk = 0, pk = 0;
-            int s = 0, ps = 0;
-            if (p < p_end) { kk = k[p]; s = second((int)v[p]); }
-            pk = __shfl_up_sync(0xffffffffu, kk, 1);
-            ps = __shfl_up_sync(0xffffffffu, s, 1);
-            if (lane == 0 && p > 0) { pk = k[p - 1]; ps = second((int)v[p - 1]); }
-            const unsigned f = __ballot_sync(0xffffffffu, p < p_end && (p == 0 || kk != pk || s != ps));
-            if (lane == 0) { A.flags[w] = f; mine += __popc(f); }
+        for (int w0 = p_begin / 32 + wib * SG_BATCH; w0 * 32 < p_end; w0 += SG_WARPS * SG_BATCH) {   // (chunks are multiples of 32)
+            uint32_t kk[SG_BATCH], pk;
+            int sv[SG_BATCH], ps;
+#pragma unroll
+            for (int u = 0; u < SG_BATCH; ++u) {
+                const int p = (w0 + u) * 32 + lane;
+                kk[u] = p < p_end ? k[p] : 0u;
+                sv[u] = p < p_end ? (int)v[p] : 0;
+            }
+            pk = w0 > 0 ? k[w0 * 32 - 1] : 0u;
+            ps = w0 > 0 ? (int)v[w0 * 32 - 1] : 0;
+            second(kk, sv, pk, ps);
+#pragma unroll
+            for (int u = 0; u < SG_BATCH; ++u) {
+                const int p = (w0 + u) * 32 + lane;
+                uint32_t bk = __shfl_up_sync(0xffffffffu, kk[u], 1);
+                int bs = __shfl_up_sync(0xffffffffu, sv[u], 1);
+                if (lane == 0) { bk = pk; bs = ps; }
+                pk = __shfl_sync(0xffffffffu, kk[u], 31); ps = __shfl_sync(0xffffffffu, sv[u], 31);
+                const unsigned f = __ballot_sync(0xffffffffu, p < p_end && (p == 0 || kk[u] != bk || sv[u] != bs));
+                // (goes on behind the first half and behind the second; the first round has no second half)
+                const unsigned go = __ballot_sync(0xffffffffu, (kk[u] & 1u) != 0u && sv[u] != -1 && (sv[u] & 1) != 0);
+                if (lane == 0 && (w0 + u) * 32 < p_end) { A.flags[w0 + u] = f; A.go[w0 + u] = go; mine += __popc(f); }
+            }
         }
         int all;
         sg_block_scan(mine, sh.wsum, tid, all);
@@ -256,13 +292,23 @@ corpus_sort_kernel(CorpusSort A) {
             const int c = w * 32 < p_end ? __popc(A.flags[w]) : 0;
             int n_lot;
             const int off = before + sg_block_scan(c, sh.wsum, tid, n_lot);
-            for (int q = 0; q < 32; ++q) {
-                const int ww = w0 + wib * 32 + q;
-                if (ww * 32 >= p_end) break;
-                const int p = ww * 32 + lane;
-                const int o = __shfl_sync(0xffffffffu, off, q);
-                const unsigned f = A.flags[ww];
-                if (p < p_end) A.rank[v[p]] = o + __popc(f & (lt | (1u << lane))) - 1;
+            for (int q0 = 0; q0 < 32; q0 += SG_BATCH) {
+                if ((w0 + wib * 32 + q0) * 32 >= p_end) break;
+                uint32_t x[SG_BATCH];
+                unsigned f[SG_BATCH], go[SG_BATCH];
+#pragma unroll
+                for (int u = 0; u < SG_BATCH; ++u) {
+                    const int ww = w0 + wib * 32 + q0 + u, p = ww * 32 + lane;
+                    x[u] = p < p_end ? v[p] : 0u;
+                    f[u] = ww * 32 < p_end ? A.flags[ww] : 0u;
+                    go[u] = ww * 32 < p_end ? A.go[ww] : 0u;
+                }
+#pragma unroll
+                for (int u = 0; u < SG_BATCH; ++u) {
+                    const int p = (w0 + wib * 32 + q0 + u) * 32 + lane;
+                    const int o = __shfl_sync(0xffffffffu, off, q0 + u);
+                    if (p < p_end) A.rank[x[u]] = (o + __popc(f[u] & (lt | (1u << lane))) - 1) * 2 + (int)((go[u] >> lane) & 1u);
+                }
             }
             before += n_lot;
         }
@@ -277,40 +323,64 @@ corpus_sort_kernel(CorpusSort A) {
     }
     __syncthreads();
     for (unsigned shift = 0; shift < A.key_bits; shift += 8) {
-        count_digits((int)shift, [&](int p) { return A.key[cur][p]; });
+        count_digits((int)shift, stored_keys);
         scatter((int)shift);
     }
     for (int k = 1, off; k < A.D; k += off) {
         off = min(k, A.D - k);
         const int o = k >> 1;                                   // (every round but the last doubles)
-        const int ranks = k == 1 ? rerank([&](int) { return 0; })
-                                 : rerank([&](int i) { return i + o < A.end_pos[i] ? A.rank[i + o] : -1; });
+        const int ranks = k == 1 ? rerank([&](const uint32_t (&)[SG_BATCH], int (&x)[SG_BATCH], uint32_t, int& y) {
+#pragma unroll
+            for (int u = 0; u < SG_BATCH; ++u) x[u] = 1;
+            y = 1;
+        }) : rerank([&](const uint32_t (&kk)[SG_BATCH], int (&x)[SG_BATCH], uint32_t pk, int& y) {
+#pragma unroll
+            for (int u = 0; u < SG_BATCH; ++u) x[u] = (kk[u] & 1u) ? A.rank[x[u] + o] : -1;
+            y = (pk & 1u) ? A.rank[y + o] : -1;
+        });
         if (ranks == N) break;                                  // no two alike: the order is final
         // the order by what follows `off` places on, then by rank
         {
             const uint32_t* const from = A.val[cur];
             uint32_t* const ko = A.key[cur ^ 1];
             uint32_t* const vo = A.val[cur ^ 1];
-            count_digits(0, [&](int p) {
-                const int t = (int)from[p], e = A.end_pos[t];
-                int i = t - off;
-                if (i < 0 || A.end_pos[i] != e) {
-                    // one of its sequence's first `off`: it stands for one of the last, which have nothing `off` places on
-                    int lo = 0, hi = A.n_seqs;                  // largest q with seq_off[q] <= t
-                    while (hi - lo > 1) { const int mid = (lo + hi) >> 1; if (A.seq_off[mid] <= t) lo = mid; else hi = mid; }
-                    const int b = (int)A.seq_off[lo];
-                    i = e - min(off, e - b) + (t - b);
+            count_digits(1, [&](int p, uint32_t (&k)[SG_BATCH]) {
+                int t[SG_BATCH];
+                bool in[SG_BATCH], edge = false;
+#pragma unroll
+                for (int u = 0; u < SG_BATCH; ++u) {
+                    in[u] = p + u * SG_THREADS < p_end;
+                    t[u] = in[u] ? (int)from[p + u * SG_THREADS] : off;
                 }
-                const uint32_t key = (uint32_t)A.rank[i];
-                ko[p] = key; vo[p] = (uint32_t)i;
-                return key;
+#pragma unroll
+                for (int u = 0; u < SG_BATCH; ++u) k[u] = t[u] >= off ? (uint32_t)A.rank[t[u] - off] : 0u;
+#pragma unroll
+                for (int u = 0; u < SG_BATCH; ++u) edge |= in[u] && (k[u] & 1u) == 0u;
+                if (edge) {
+#pragma unroll 1
+                    for (int u = 0; u < SG_BATCH; ++u) {
+                        if (!in[u] || (k[u] & 1u)) continue;
+                        // the sequence of the suffix `off` places back ends within its k tokens, if it is the same sequence at all
+                        const int e = A.end_pos[t[u]];
+                        if (t[u] >= off && A.end_pos[t[u] - off] == e) continue;
+                        // one of its sequence's first `off`: it stands for one of the last, which have nothing `off` places on
+                        int lo = 0, hi = A.n_seqs;              // largest q with seq_off[q] <= t
+                        while (hi - lo > 1) { const int mid = (lo + hi) >> 1; if (A.seq_off[mid] <= t[u]) lo = mid; else hi = mid; }
+                        const int b = (int)A.seq_off[lo];
+                        t[u] = e - min(off, e - b) + (t[u] - b) + off;
+                        k[u] = (uint32_t)A.rank[t[u] - off];
+                    }
+                }
+#pragma unroll
+                for (int u = 0; u < SG_BATCH; ++u)
+                    if (in[u]) { ko[p + u * SG_THREADS] = k[u]; vo[p + u * SG_THREADS] = (uint32_t)(t[u] - off); }
             });
             cur ^= 1;
         }
-        scatter(0);
+        scatter(1);                                             // (the lowest bit is the same for equal ranks)
         for (int shift = 8; shift < 32 && ((unsigned)(ranks - 1) >> shift) != 0u; shift += 8) {
-            count_digits(shift, [&](int p) { return A.key[cur][p]; });
-            scatter(shift);
+            count_digits(shift + 1, stored_keys);
+            scatter(shift + 1);
         }
     }
     for (int p = p_begin + tid; p < p_end; p += SG_THREADS) A.sa[p] = A.val[cur][p];
@@ -1206,9 +1276,10 @@ static int pipeline_run(Pipeline& P, const int32_t* d_tok, const int64_t* d_seq_
         const i64 lot = (i64)SG_THREADS * (small ? 2 : 8);
         const i64 lots = (N + lot - 1) / lot;
         const i64 per_block = (lots + most_blocks - 1) / most_blocks;
-        A.chunk = (int)(lot * per_block);
+        // (as many blocks as fit, the last lot of each part full: a multiple of 32)
+        A.chunk = (int)(per_block == 1 ? lot : ((N + most_blocks - 1) / most_blocks + 31) / 32 * 32);
         ok = tmp.get(&A.key[0], N) && tmp.get(&A.key[1], N) && tmp.get(&A.val[0], N) && tmp.get(&A.val[1], N) && tmp.get(&A.rank, N) &&
-             tmp.get(&A.flags, N / 32 + 1) && tmp.get(&A.table, (i64)SG_BINS * most_blocks) && tmp.get(&A.total, SG_BINS) &&
+             tmp.get(&A.flags, N / 32 + 1) && tmp.get(&A.go, N / 32 + 1) && tmp.get(&A.table, (i64)SG_BINS * most_blocks) && tmp.get(&A.total, SG_BINS) &&
              tmp.get(&A.count, most_blocks);
         if (!ok) return SD_ERR_NOMEM;
         rc = small ? corpus_sort<2>(A, st) : corpus_sort<8>(A, st);
