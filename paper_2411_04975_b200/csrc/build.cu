@@ -707,10 +707,33 @@ __global__ void __launch_bounds__(TS_CARRY) ts_carry_kernel(TreeScan T) {
     }
 }
 
-// R from the front: the last one left behind by a tile to the left.
-__global__ void __launch_bounds__(TS_CARRY) ts_carry_front_kernel(TreeScan T) {
-    __shared__ int part[TS_CARRY / 32];
+// S and the depth-1 nodes in front of every request's first suffix (the requests' suffixes are consecutive in the
+// order); entry n: all of them.
+struct RequestBounds {
+    int n;                                        // -1: no requests
+    const int64_t* off;                           // [n + 1]
+    int *s, *n1;                                  // [n + 1]
+};
+
+// R from the front: the last one left behind by a tile to the left (blocks 0 .. 31); the others: a request each.
+__global__ void __launch_bounds__(TS_CARRY) ts_carry_front_kernel(TreeScan T, RequestBounds Q) {
+    __shared__ int part[TS_CARRY / 32], part1[TS_CARRY / 32];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    if (blockIdx.x >= 32) {
+        const int q = blockIdx.x - 32;
+        const int j = (int)Q.off[q], tile = j / T.tile_len;
+        int a = 0, b = 0;
+        for (int i = tile * T.tile_len + threadIdx.x; i < j; i += TS_CARRY) { const int l = T.lcp[i]; a += T.len[i] - max(l, 1); b += l == 0 ? 1 : 0; }
+        a = (int)__reduce_add_sync(TS_FULL, (unsigned)a);
+        b = (int)__reduce_add_sync(TS_FULL, (unsigned)b);
+        if (lane == 0) { part[w] = a; part1[w] = b; }
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            for (int k = 1; k < TS_CARRY / 32; ++k) { a += part[k]; b += part1[k]; }
+            Q.s[q] = T.s[tile] + a; Q.n1[q] = T.n1[tile] + b;
+        }
+        return;
+    }
     const int per = (T.tiles + TS_CARRY - 1) / TS_CARRY;
     const int k0 = threadIdx.x * per, k1 = min(T.tiles, k0 + per);
     int* const r = T.r + (i64)blockIdx.x * T.tiles;
@@ -795,6 +818,7 @@ struct TreeOut {
     const int32_t* slot;
     const int64_t* off;                           // [n_req + 1]
     const int *s_req, *n1_req;                    // [n_req + 1] S and depth-1 nodes before the request's first suffix
+    const int* bad;                               // not 0: a token is outside the vocabulary, nothing may change
 };
 
 // (3)
@@ -803,7 +827,7 @@ __global__ void __launch_bounds__(TS_WARPS * 32)
 ts_emit_kernel(TreeScan T, TreeOut O) {
     extern __shared__ int2 ts_state[];                          // [TS_WARPS][tile_len / TS_SUB][32]: G and end behind each sub-tile
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5, tile = blockIdx.x * TS_WARPS + wib, d = lane + 1;
-    if (tile >= T.tiles) return;
+    if (tile >= T.tiles || (REQ && *O.bad)) return;
     const int t0 = tile * T.tile_len, t1 = min(T.N, t0 + T.tile_len);
     const int subs = (t1 - t0 + TS_SUB - 1) / TS_SUB;
     int2* const st = ts_state + (i64)wib * (T.tile_len / TS_SUB) * 32;
@@ -1008,12 +1032,13 @@ constexpr double CACHE_SECONDS = 30.0;
 constexpr int KEPT_STREAMS = 8;
 
 typedef std::chrono::steady_clock Clock;
-struct StreamSet { cudaStream_t aux; cudaEvent_t ev_fork, ev_join; };
+// What a store holds besides device memory: a stream and events, and pinned memory for the arguments of sd_build_requests.
+struct StreamSet { cudaStream_t aux; cudaEvent_t ev_fork, ev_join, ev_check; void* stage; size_t stage_bytes; };
 struct FreeBlock { void* p; size_t bytes; Clock::time_point since; };
 struct DeviceCache {
     std::vector<FreeBlock> idle;                      // oldest first
     size_t bytes = 0, most = 0;
-    StreamSet streams[KEPT_STREAMS];                  // stream and events of freed stores, for the next ones
+    StreamSet streams[KEPT_STREAMS];                  // of freed stores, for the next ones
     int n_streams = 0;
 };
 struct OwnedBlock { size_t bytes; int dev; };
@@ -1041,21 +1066,34 @@ void cache_expire(DeviceCache& c) {
     c.idle.erase(c.idle.begin(), c.idle.begin() + n);
 }
 
-// a stream and two events for a store on the current device
-bool take_streams(int dev, StreamSet* out) {
+void drop_streams(const StreamSet& s) {
+    for (cudaEvent_t e : {s.ev_fork, s.ev_join, s.ev_check}) if (e) cudaEventDestroy(e);
+    if (s.aux) cudaStreamDestroy(s.aux);
+    if (s.stage) cudaFreeHost(s.stage);
+}
+
+// for a store on the current device, with at least `stage_bytes` of pinned memory
+bool take_streams(int dev, size_t stage_bytes, StreamSet* out) {
     if (dev >= 0 && dev < CACHE_DEVICES) {
         std::lock_guard<std::mutex> lock(g_cache_mutex);
         DeviceCache& d = g_cache[dev];
-        if (d.n_streams > 0) { *out = d.streams[--d.n_streams]; return true; }
+        for (int k = d.n_streams - 1; k >= 0; --k)
+            if (d.streams[k].stage_bytes >= stage_bytes) {
+                *out = d.streams[k];
+                d.streams[k] = d.streams[--d.n_streams];
+                return true;
+            }
     }
-    out->aux = nullptr; out->ev_fork = nullptr; out->ev_join = nullptr;
+    memset(out, 0, sizeof(*out));
+    out->stage_bytes = std::max<size_t>(stage_bytes, 16384);
     if (cudaStreamCreateWithFlags(&out->aux, cudaStreamNonBlocking) == cudaSuccess &&
         cudaEventCreateWithFlags(&out->ev_fork, cudaEventDisableTiming) == cudaSuccess &&
-        cudaEventCreateWithFlags(&out->ev_join, cudaEventDisableTiming) == cudaSuccess)
+        cudaEventCreateWithFlags(&out->ev_join, cudaEventDisableTiming) == cudaSuccess &&
+        cudaEventCreateWithFlags(&out->ev_check, cudaEventDisableTiming) == cudaSuccess &&
+        cudaHostAlloc(&out->stage, out->stage_bytes, cudaHostAllocPortable | cudaHostAllocMapped) == cudaSuccess)
         return true;
     cudaGetLastError();
-    if (out->ev_fork) cudaEventDestroy(out->ev_fork);
-    if (out->aux) cudaStreamDestroy(out->aux);
+    drop_streams(*out);
     return false;
 }
 
@@ -1067,9 +1105,7 @@ void give_streams(int dev, const StreamSet& s) {
             return;
         }
     }
-    cudaEventDestroy(s.ev_fork);
-    cudaEventDestroy(s.ev_join);
-    cudaStreamDestroy(s.aux);
+    drop_streams(s);
 }
 
 }  // namespace
@@ -1198,6 +1234,9 @@ int bits_for(i64 maxval) {
 
 }  // namespace
 
+// Arguments of sd_build_requests for n requests: offsets, slots, a zero; and the host's flag.
+static size_t stage_bytes_for(i64 n) { return (size_t)(8 * (n + 1) + 4 * n + 4 + 16) / 16 * 16 + 16; }
+
 template <class T>
 static bool store_alloc(sd_store* s, T** out, long long count) {
     void* p = nullptr;
@@ -1218,7 +1257,7 @@ static void store_release(sd_store* s, cudaStream_t st) {
         for (int k = 0; k < 48; ++k) sd_device_free(s->ws->ptr[k]);
         delete s->ws;
     }
-    if (s->aux) give_streams(s->device, StreamSet{s->aux, s->ev_fork, s->ev_join});
+    if (s->aux) give_streams(s->device, StreamSet{s->aux, s->ev_fork, s->ev_join, s->ev_check, s->stage, s->stage_bytes});
     delete s;
 }
 
@@ -1233,10 +1272,12 @@ struct Pipeline {
 // long runs.  per_seq_max_len > 0: the sequences are independent
 // (tokens of different sequences never compare equal, sequence k's tokens below sequence k + 1's)
 // and none is longer than that, so each is sorted by a block of its own.
+// end_pos: one past the last token of every token's sequence, if that is known already.
 // Nothing is read back to the host.
 // Returns SD_OK, SD_ERR_NOMEM or SD_ERR_CUDA.
 static int pipeline_run(Pipeline& P, const int32_t* d_tok, const int64_t* d_seq_offsets, int n_seqs, i64 N,
-                        i64 max_token, int D, bool top_blocks, cudaStream_t st, i64 per_seq_max_len = 0) {
+                        i64 max_token, int D, bool top_blocks, cudaStream_t st, i64 per_seq_max_len = 0,
+                        int* end_pos = nullptr, RequestBounds bounds = RequestBounds{-1, nullptr, nullptr, nullptr}) {
     const int T256 = 256;
     DeviceArena& tmp = P.tmp;
     const bool block_sort = per_seq_max_len > 0 && per_seq_max_len <= BS_MAX_LEN;
@@ -1251,13 +1292,13 @@ static int pipeline_run(Pipeline& P, const int32_t* d_tok, const int64_t* d_seq_
     const int most_blocks = 2 * sms;
     if (!block_sort)
         tmp.reserve((long long)N * (16 + 4 + 4 + 4 + 2 + 1) + 4ll * (100 * (i64)ts.tiles + (SG_BINS + 1) * (i64)most_blocks + SG_BINS) + 64 * 256);
-    int* end_pos = nullptr;
+    const bool have_ends = end_pos != nullptr;
     uint32_t* sa = nullptr;
     bool ok = tmp.get(&ts.lcp, N) && tmp.get(&ts.len, N) && tmp.get(&ts.f, 32 * (i64)ts.tiles) && tmp.get(&ts.e, 32 * (i64)ts.tiles) &&
               tmp.get(&ts.r, 32 * (i64)ts.tiles) && tmp.get(&ts.s, ts.tiles + 1) && tmp.get(&ts.n1, ts.tiles + 1) && tmp.get(&ts.wide, 4) &&
-              tmp.get(&end_pos, N) && tmp.get(&sa, N);
+              (have_ends || tmp.get(&end_pos, N)) && tmp.get(&sa, N);
     if (!ok) return SD_ERR_NOMEM;
-    seq_end_kernel<<<grid_for(N, T256), T256, 0, st>>>(d_seq_offsets, n_seqs, N, end_pos);
+    if (!have_ends) seq_end_kernel<<<grid_for(N, T256), T256, 0, st>>>(d_seq_offsets, n_seqs, N, end_pos);
     int rc;
     if (block_sort) {
         const int V = (int)(max_token / n_seqs);                // (a sequence's tokens lie in a range of V of their own)
@@ -1293,7 +1334,7 @@ static int pipeline_run(Pipeline& P, const int32_t* d_tok, const int64_t* d_seq_
     ts_carry_kernel<<<33, TS_CARRY, 0, st>>>(ts);
     if (top_blocks) ts_runs_kernel<true><<<grid, TS_WARPS * 32, 0, st>>>(ts);
     else ts_runs_kernel<false><<<grid, TS_WARPS * 32, 0, st>>>(ts);
-    ts_carry_front_kernel<<<32, TS_CARRY, 0, st>>>(ts);
+    ts_carry_front_kernel<<<(unsigned)(32 + bounds.n + 1), TS_CARRY, 0, st>>>(ts, bounds);
     return SD_OK;
 }
 
@@ -1338,8 +1379,9 @@ extern "C" int sd_build(const sd_build_params* p, const int32_t* d_corpus, const
               store_alloc(s, &s->s_text, (i64)s->R * s->T) && store_alloc(s, &s->s_state, s->R);
     if (!ok) { store_release(s, st); return SD_ERR_NOMEM; }
     StreamSet streams;
-    if (!take_streams(s->device, &streams)) { store_release(s, st); return SD_ERR_CUDA; }
-    s->aux = streams.aux; s->ev_fork = streams.ev_fork; s->ev_join = streams.ev_join;
+    if (!take_streams(s->device, stage_bytes_for(s->R), &streams)) { store_release(s, st); return SD_ERR_CUDA; }
+    s->aux = streams.aux; s->ev_fork = streams.ev_fork; s->ev_join = streams.ev_join; s->ev_check = streams.ev_check;
+    s->stage = streams.stage; s->stage_bytes = streams.stage_bytes;
     cudaError_t ce = cudaMemsetAsync(s->g_root, 0xFF, sizeof(int32_t) * (size_t)s->V, st);
     if (ce == cudaSuccess) ce = cudaMemsetAsync(s->s_root, 0xFF, sizeof(int32_t) * (size_t)s->R * s->V, st);
     if (ce == cudaSuccess) ce = cudaMemsetAsync(s->s_state, 0, sizeof(SlotState) * (size_t)s->R, st);
@@ -1434,20 +1476,25 @@ __device__ __forceinline__ int seq_rank_of(const int64_t* off, int n, i64 pos) {
     return lo;
 }
 
-__global__ void map_tokens_kernel(const int32_t* tok, const int64_t* off, int n, i64 N, int V, int32_t* out, int* bad) {
-    i64 i = (i64)blockIdx.x * blockDim.x + threadIdx.x;
+// The tokens in ranges of their own, request by request, and where their request ends.  A token outside the vocabulary
+// sets both flags (the host's one lies in its memory).
+__global__ void map_tokens_kernel(const int32_t* tok, const int64_t* off, int n, i64 N, int V, int32_t* out, int* end_pos, int* bad,
+                                  int* host_bad) {
+    const i64 i = (i64)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= N) return;
-    const int t = tok[i];
-    if (t < 0 || t >= V) { atomicOr(bad, 1); out[i] = 0; return; }
-    out[i] = seq_rank_of(off, n, i) * V + t;
+    int t = tok[i];
+    if (t < 0 || t >= V) { *bad = 1; *host_bad = 1; t = 0; }
+    const int q = seq_rank_of(off, n, i);
+    out[i] = q * V + t;
+    end_pos[i] = (int)off[q + 1];
 }
 
 // one block per request: forget the slot's old tree and store the new text
 constexpr int PREP_THREADS = 1024;
 __global__ void __launch_bounds__(PREP_THREADS)
-requests_prepare_kernel(sd_store sv, int n, const int32_t* slot_ids, const int64_t* off, const int32_t* tok) {
+requests_prepare_kernel(sd_store sv, int n, const int32_t* slot_ids, const int64_t* off, const int32_t* tok, const int* bad) {
     const int q = blockIdx.x;
-    if (q >= n) return;
+    if (q >= n || *bad) return;
     const int slot = slot_ids[q];
     if (slot < 0 || slot >= sv.R) return;
     SlotState* ss = sv.s_state + slot;
@@ -1461,29 +1508,12 @@ requests_prepare_kernel(sd_store sv, int n, const int32_t* slot_ids, const int64
         for (i64 k = threadIdx.x; k < hi - lo; k += blockDim.x) text[k] = tok[lo + k];
 }
 
-// S and the depth-1 nodes in front of every request's first suffix (the requests' suffixes are consecutive in the
-// order): a block per request, [n] = all
-__global__ void requests_bounds_kernel(TreeScan T, int n, const int64_t* off, int* s_req, int* n1_req) {
-    __shared__ int part[2][4];
-    const int q = blockIdx.x;
-    const int j = (int)off[q], tile = j / T.tile_len;
-    int a = 0, b = 0;
-    for (int i = tile * T.tile_len + threadIdx.x; i < j; i += 128) { const int l = T.lcp[i]; a += T.len[i] - max(l, 1); b += l == 0 ? 1 : 0; }
-    a = (int)__reduce_add_sync(TS_FULL, (unsigned)a);
-    b = (int)__reduce_add_sync(TS_FULL, (unsigned)b);
-    if ((threadIdx.x & 31) == 0) { part[0][threadIdx.x >> 5] = a; part[1][threadIdx.x >> 5] = b; }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        for (int k = 1; k < 4; ++k) { a += part[0][k]; b += part[1][k]; }
-        s_req[q] = T.s[tile] + a; n1_req[q] = T.n1[tile] + b;
-    }
-}
-
 // one block per request: bookkeeping and the active nodes (eight lanes per depth: node of the last d tokens)
 __global__ void __launch_bounds__(256)
-requests_finalize_kernel(sd_store sv, int n, const int32_t* slot_ids, const int64_t* off, const int* s_req, const int* n1_req) {
+requests_finalize_kernel(sd_store sv, int n, const int32_t* slot_ids, const int64_t* off, const int* s_req, const int* n1_req,
+                         const int* bad) {
     const int q = blockIdx.x, lane = threadIdx.x & 31, d = threadIdx.x / APP_LANES + 1;
-    if (q >= n) return;
+    if (q >= n || *bad) return;
     const int slot = slot_ids[q];
     if (slot < 0 || slot >= sv.R) return;
     SlotState* ss = sv.s_state + slot;
@@ -1528,9 +1558,14 @@ extern "C" int sd_build_requests(sd_store* s, int32_t n, const int32_t* h_slot, 
     if (n == 0) return SD_OK;
     if (!h_slot || !h_offsets || n > s->R) return SD_ERR_INVALID_ARG;
     if (h_offsets[0] != 0) return SD_ERR_INVALID_ARG;
-    for (int q = 0; q < n; ++q) {
-        if (h_offsets[q + 1] < h_offsets[q] || h_slot[q] < 0 || h_slot[q] >= s->R) return SD_ERR_INVALID_ARG;
-        for (int r = 0; r < q; ++r) if (h_slot[r] == h_slot[q]) return SD_ERR_INVALID_ARG;   // a slot once per call
+    try {
+        std::vector<bool> seen((size_t)s->R);
+        for (int q = 0; q < n; ++q) {
+            if (h_offsets[q + 1] < h_offsets[q] || h_slot[q] < 0 || h_slot[q] >= s->R || seen[h_slot[q]]) return SD_ERR_INVALID_ARG;
+            seen[h_slot[q]] = true;                              // a slot once per call
+        }
+    } catch (const std::bad_alloc&) {
+        return SD_ERR_NOMEM;
     }
     const i64 N = h_offsets[n];
     if (N > 0 && !d_tokens) return SD_ERR_INVALID_ARG;
@@ -1545,38 +1580,48 @@ extern "C" int sd_build_requests(sd_store* s, int32_t n, const int32_t* h_slot, 
         memset(s->ws, 0, sizeof(*s->ws));
     }
     P.tmp.keep = s->ws;                                          // temporaries are kept for the next call
-    int32_t *d_slot = nullptr, *mtok = nullptr;
-    int64_t* d_off = nullptr;
-    int* bad = nullptr;
-    int *s_req = nullptr, *n1_req = nullptr;
-    bool ok = P.tmp.get(&d_slot, n) && P.tmp.get(&d_off, n + 1) && P.tmp.get(&mtok, N) && P.tmp.get(&bad, 1) &&
-              P.tmp.get(&s_req, n + 1) && P.tmp.get(&n1_req, n + 1);
+    // Arguments go over in one copy from pinned memory, which ends with a zero: the flag that a bad token sets.  Everything is
+    // queued behind the check of the tokens and changes nothing if it fails; the host waits for the check alone, so
+    // the GPU does not run dry meanwhile (it did, for some 50 us of a 185 us refill).
+    const size_t arg_bytes = 8 * ((size_t)n + 1) + 4 * (size_t)n + 4;
+    unsigned char* d_args = nullptr;
+    int32_t* mtok = nullptr;
+    int *end_pos = nullptr, *s_req = nullptr, *n1_req = nullptr;
+    bool ok = P.tmp.get(&d_args, (i64)arg_bytes) && P.tmp.get(&mtok, N) && P.tmp.get(&end_pos, N) && P.tmp.get(&s_req, n + 1) &&
+              P.tmp.get(&n1_req, n + 1);
     if (!ok) return SD_ERR_NOMEM;
-    SD_CUDA_OK(cudaMemcpyAsync(d_slot, h_slot, sizeof(int32_t) * n, cudaMemcpyHostToDevice, st));
-    SD_CUDA_OK(cudaMemcpyAsync(d_off, h_offsets, sizeof(int64_t) * (n + 1), cudaMemcpyHostToDevice, st));
-    SD_CUDA_OK(cudaMemsetAsync(bad, 0, sizeof(int), st));
-    if (N > 0) {
-        map_tokens_kernel<<<grid_for(N, T256), T256, 0, st>>>(d_tokens, d_off, n, N, s->V, mtok, bad);
-        int h_bad = 0;
-        SD_CUDA_OK(cudaMemcpyAsync(&h_bad, bad, sizeof(int), cudaMemcpyDeviceToHost, st));
-        SD_CUDA_OK(cudaStreamSynchronize(st));
-        if (h_bad) return SD_ERR_INVALID_ARG;                    // nothing was changed yet
-    }
-    requests_prepare_kernel<<<(unsigned)n, PREP_THREADS, 0, st>>>(*s, n, d_slot, d_off, d_tokens);
+    int64_t* const d_off = reinterpret_cast<int64_t*>(d_args);
+    int32_t* const d_slot = reinterpret_cast<int32_t*>(d_off + n + 1);
+    int* const bad = d_slot + n;
+    unsigned char* const h_args = (unsigned char*)s->stage + 16;
+    volatile int* const h_bad = (volatile int*)s->stage;
+    *h_bad = 0;
+    memcpy(h_args, h_offsets, 8 * ((size_t)n + 1));
+    memcpy(h_args + 8 * ((size_t)n + 1), h_slot, 4 * (size_t)n);
+    memset(h_args + arg_bytes - 4, 0, 4);
+    SD_CUDA_OK(cudaMemcpyAsync(d_args, h_args, arg_bytes, cudaMemcpyHostToDevice, st));
+    if (N > 0) map_tokens_kernel<<<grid_for(N, T256), T256, 0, st>>>(d_tokens, d_off, n, N, s->V, mtok, end_pos, bad, (int*)s->stage);
+    SD_CUDA_OK(cudaEventRecord(s->ev_check, st));
+    int rc = SD_OK;
     if (N > 0) {
         i64 max_len = 0;
         for (int q = 0; q < n; ++q) max_len = std::max<i64>(max_len, h_offsets[q + 1] - h_offsets[q]);
-        int rc = pipeline_run(P, mtok, d_off, n, N, (i64)n * s->V, D, false, st, max_len);
-        if (rc != SD_OK) return rc;
-        requests_bounds_kernel<<<(unsigned)n + 1, 128, 0, st>>>(P.ts, n, d_off, s_req, n1_req);
+        rc = pipeline_run(P, mtok, d_off, n, N, (i64)n * s->V, D, false, st, max_len, end_pos, RequestBounds{n, d_off, s_req, n1_req});
+    }
+    if (rc == SD_OK) requests_prepare_kernel<<<(unsigned)n, PREP_THREADS, 0, st>>>(*s, n, d_slot, d_off, d_tokens, bad);
+    if (rc == SD_OK && N > 0) {
         TreeOut out;
         memset(&out, 0, sizeof(out));
-        out.sv = *s; out.n_req = n; out.slot = d_slot; out.off = d_off; out.s_req = s_req; out.n1_req = n1_req;
+        out.sv = *s; out.n_req = n; out.slot = d_slot; out.off = d_off; out.s_req = s_req; out.n1_req = n1_req; out.bad = bad;
         rc = emit_entries<true>(P.ts, out, st);
-        if (rc != SD_OK) return rc;
     }
-    requests_finalize_kernel<<<(unsigned)n, 256, 0, st>>>(*s, n, d_slot, d_off, N > 0 ? s_req : nullptr, N > 0 ? n1_req : nullptr);
-    // (no synchronisation: the temporaries stay in the store's workspace, and a later call on
+    if (rc == SD_OK)
+        requests_finalize_kernel<<<(unsigned)n, 256, 0, st>>>(*s, n, d_slot, d_off, N > 0 ? s_req : nullptr, N > 0 ? n1_req : nullptr, bad);
+    const cudaError_t checked = cudaEventSynchronize(s->ev_check);               // (the pinned memory is free again, too)
+    if (rc != SD_OK) return rc;
+    if (checked != cudaSuccess) return SD_ERR_CUDA;
+    if (*h_bad) return SD_ERR_INVALID_ARG;
+    // (the temporaries stay in the store's workspace, and a later call on
     // another stream must be ordered behind this one by the caller like any other use of the store)
     SD_CUDA_OK(cudaGetLastError());
     return SD_OK;

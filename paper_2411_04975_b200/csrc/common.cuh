@@ -91,6 +91,10 @@ struct sd_store {
     // (they share nothing), on this stream, forked from and joined to the caller's stream
     cudaStream_t aux;
     cudaEvent_t ev_fork, ev_join;
+    // HOST: sd_build_requests stages its arguments in pinned memory and waits for the check of the tokens
+    cudaEvent_t ev_check;
+    void* stage;
+    size_t stage_bytes;
 };
 
 __host__ __device__ inline uint32_t sd_pow2ceil(uint32_t n) {
