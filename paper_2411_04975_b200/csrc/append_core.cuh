@@ -207,6 +207,40 @@ __device__ __forceinline__ int group_lookup(RunSearch a, int x, int lane, int& p
     return eq ? a.lo + k : -1;
 }
 
+// All lanes of the warp call; the eight lanes of a group go `steps` tokens (token(0), ...) down from `node` with child run zw; on
+// return node is the node reached or -1.  The eight entries at hand hold the next levels, too, where they are only
+// children (most of them are): a token then costs no load.  Long runs are searched.
+template <class F>
+__device__ __forceinline__ void group_walk(const int4* ent, int limit, int& node, int2& zw, int steps, int lane, F token) {
+    const unsigned FULL = 0xffffffffu;
+    const int l = lane & (APP_LANES - 1), gb = lane & ~(APP_LANES - 1);
+    int wb = -64, k = 0;
+    int4 e = make_int4(-1, 0, 0, 0);
+    while (true) {
+        bool on = node >= 0 && k < steps;
+        if (!__any_sync(FULL, on)) break;
+        const int x = on ? token(k) : -1;
+        const int n = on ? (int)((unsigned)zw.y & RUN_COUNT_MASK) : 0;
+        const bool far = n > APP_LANES;
+        if (__any_sync(FULL, far)) {
+            int place;
+            int2 next;
+            const int at = group_lookup(RunSearch{ent + zw.x, 0, far ? n : 0}, x, lane, place, next);
+            if (far) { node = at >= 0 ? zw.x + at : -1; zw = next; ++k; on = false; }
+        }
+        if (!__any_sync(FULL, on)) continue;
+        if (on && (zw.x < wb || zw.x + n > wb + APP_LANES)) {
+            wb = zw.x;
+            if (wb + l < limit) e = ent[wb + l];
+        }
+        const int off = zw.x - wb;
+        const unsigned eq = (__ballot_sync(FULL, on && l >= off && l < off + n && e.x == x) >> gb) & 0xffu;
+        const int q = eq ? __ffs(eq) - 1 : 0;
+        const int nz = __shfl_sync(FULL, e.z, q, APP_LANES), nw = __shfl_sync(FULL, e.w, q, APP_LANES);
+        if (on) { node = eq ? wb + q : -1; zw = make_int2(nz, nw); ++k; }
+    }
+}
+
 // The tokens sh.tok holds: token 0 of the append is sh.tok[APP_SHALLOW - 1].
 __device__ __forceinline__ void append_stage_tokens(AppendShared& sh, const int32_t* text, int t_old, const int32_t* newtok, int n_new,
                                                     int tid, int nthreads) {

@@ -411,6 +411,7 @@ constexpr int BS_WARPS = BS_THREADS / 32;
 constexpr int BS_MAX_LEN = 16384;              // longest sequence (two passes of 7 bits per round; 112 KB)
 constexpr int BS_BITS = 7;
 constexpr int BS_BINS = 1 << BS_BITS;
+constexpr int BS_ROW = BS_BINS + 1;            // (rows of 128 counters put the eight threads that add up a digit on one bank: a sort of 4 x 4,096 tokens took 60 us, 49 now)
 
 // ITEMS per thread: sequences of up to 1,024 x ITEMS tokens
 template <int ITEMS>
@@ -418,8 +419,8 @@ __global__ void __launch_bounds__(BS_THREADS, ITEMS <= 4 ? 2 : 1)
 block_suffix_sort_kernel(const int32_t* tok, const int64_t* seq_off, int V, int tok_bits, int D, uint32_t* sa_out) {
     extern __shared__ __align__(16) unsigned char bs_smem[];
     __shared__ int wsum[BS_WARPS];
-    int (*hist)[BS_BINS] = reinterpret_cast<int (*)[BS_BINS]>(bs_smem);              // [BS_WARPS][BS_BINS]
-    unsigned short* const rank = reinterpret_cast<unsigned short*>(bs_smem + sizeof(int) * BS_WARPS * BS_BINS);
+    int (*hist)[BS_ROW] = reinterpret_cast<int (*)[BS_ROW]>(bs_smem);                // [BS_WARPS][BS_ROW]
+    unsigned short* const rank = reinterpret_cast<unsigned short*>(bs_smem + sizeof(int) * BS_WARPS * BS_ROW);
     unsigned short* cur = rank + BS_THREADS * ITEMS;                                // the order so far
     unsigned short* nxt = cur + BS_THREADS * ITEMS;
     const i64 b = seq_off[blockIdx.x];
@@ -550,7 +551,7 @@ block_suffix_sort_kernel(const int32_t* tok, const int64_t* seq_off, int V, int 
 
 template <int ITEMS>
 int block_suffix_sort(const int32_t* tok, const int64_t* seq_off, int n_seqs, int V, int tok_bits, int D, uint32_t* sa, cudaStream_t st) {
-    const int smem = (int)(sizeof(int) * BS_WARPS * BS_BINS + 3 * sizeof(unsigned short) * BS_THREADS * ITEMS);
+    const int smem = (int)(sizeof(int) * BS_WARPS * BS_ROW + 3 * sizeof(unsigned short) * BS_THREADS * ITEMS);
     if (smem > 48 * 1024)
         SD_CUDA_OK(cudaFuncSetAttribute(block_suffix_sort_kernel<ITEMS>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
     block_suffix_sort_kernel<ITEMS><<<(unsigned)n_seqs, BS_THREADS, smem, st>>>(tok, seq_off, V, tok_bits, D, sa);
@@ -1523,21 +1524,16 @@ requests_finalize_kernel(sd_store sv, int n, const int32_t* slot_ids, const int6
     const int4* ent = sv.s_ent + (i64)slot * sv.spn;
     const int32_t* root = sv.s_root + (i64)slot * sv.V;
     const int32_t* text = sv.s_text + (i64)slot * sv.T;
+    __shared__ int tail[SD_MAX_DEPTH];                           // the last tokens
+    if (threadIdx.x < SD_MAX_DEPTH && (int)threadIdx.x < len) tail[threadIdx.x] = text[len - 1 - threadIdx.x];
+    __syncthreads();
     int node = -1;
     int2 zw = make_int2(0, 0);
     if (d <= len && d <= sv.D) {
-        node = root[text[len - d]];
+        node = root[tail[d - 1]];
         if (node >= 0) zw = *reinterpret_cast<const int2*>(&ent[node].z);
     }
-    for (int k = 1; k < SD_MAX_DEPTH; ++k) {
-        const bool on = node >= 0 && k < d;
-        if (!__any_sync(TS_FULL, on)) break;
-        const int x = on ? text[len - d + k] : -1;
-        int place;
-        int2 next;
-        const int at = group_lookup(RunSearch{ent + zw.x, 0, on ? (int)((unsigned)zw.y & RUN_COUNT_MASK) : 0}, x, lane, place, next);
-        if (on) { node = at >= 0 ? zw.x + at : -1; zw = next; }
-    }
+    group_walk(ent, (int)sv.spn, node, zw, d - 1, lane, [&](int k) { return tail[d - 2 - k]; });
     if ((lane & (APP_LANES - 1)) == 0) {
         ss->active[d - 1] = node; ss->room[d - 1] = 0;
         ss->run_cb[d - 1] = node >= 0 ? zw.x : 0; ss->run_w[d - 1] = node >= 0 ? (unsigned)zw.y : 0u;

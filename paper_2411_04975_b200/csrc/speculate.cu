@@ -1043,40 +1043,13 @@ speculate_fused_kernel(sd_store sv, int n, const int32_t* __restrict__ d_slot, i
             for (int p0 = 0; p0 < Pe; p0 += GT / APP_LANES) {
                 const int d = p0 + gtid / APP_LANES + 1;
                 int node = d <= Pe ? sh.src_node[d - 1] : -1;
-                int pos = d <= Pe ? sh.src_from[d - 1] : t;
+                const int pos = d <= Pe ? sh.src_from[d - 1] : t;
                 int2 zw = make_int2(0, 0);
                 if (node >= 0) zw = *reinterpret_cast<const int2*>(&sv.g_ent[node].z);
-                // The eight entries at hand hold the next levels, too, where they are only children (most of them
-                // are): a token then costs no load.
-                int wb = -64;
-                int4 e = make_int4(-1, 0, 0, 0);
-                const int l = lane & (APP_LANES - 1), gb = lane & ~(APP_LANES - 1);
-                while (true) {
-                    bool on = node >= 0 && pos < t;
-                    if (!__any_sync(FULL, on)) break;
-                    // (of the new tokens the first ones are at hand)
-                    const int kx = pos - t_old;
-                    int x = -1;
-                    if (on) x = kx < 0 ? text[pos] : (kx < APP_AHEAD ? sh.app.tok[kx + APP_SHALLOW - 1] : newtok[kx]);
-                    const int n = on ? (int)((unsigned)zw.y & RUN_COUNT_MASK) : 0;
-                    const bool far = n > APP_LANES;
-                    if (__any_sync(FULL, far)) {                // long runs are searched
-                        int place;
-                        int2 next;
-                        const int at = group_lookup(RunSearch{sv.g_ent + zw.x, 0, far ? n : 0}, x, lane, place, next);
-                        if (far) { node = at >= 0 ? zw.x + at : -1; zw = next; ++pos; on = false; }
-                    }
-                    if (!__any_sync(FULL, on)) continue;
-                    if (on && (zw.x < wb || zw.x + n > wb + APP_LANES)) {
-                        wb = zw.x;
-                        if (wb + l < (int)sv.g_cap) e = sv.g_ent[wb + l];
-                    }
-                    const int off = zw.x - wb;
-                    const unsigned eq = (__ballot_sync(FULL, on && l >= off && l < off + n && e.x == x) >> gb) & 0xffu;
-                    const int k = eq ? __ffs(eq) - 1 : 0;
-                    const int nz = __shfl_sync(FULL, e.z, k, APP_LANES), nw = __shfl_sync(FULL, e.w, k, APP_LANES);
-                    if (on) { node = eq ? wb + k : -1; zw = make_int2(nz, nw); ++pos; }
-                }
+                group_walk(sv.g_ent, (int)sv.g_cap, node, zw, t - pos, lane, [&](int k) {
+                    const int kx = pos + k - t_old;            // (of the new tokens the first ones are at hand)
+                    return kx < 0 ? text[pos + k] : (kx < APP_AHEAD ? sh.app.tok[kx + APP_SHALLOW - 1] : newtok[kx]);
+                });
                 if ((lane & (APP_LANES - 1)) == 0 && d <= Pe) {
                     ss->g_node[d - 1] = node;
                     sh.node[0][d - 1] = node;
