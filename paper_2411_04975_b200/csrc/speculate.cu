@@ -280,11 +280,11 @@ __global__ void select_emit_kernel(sd_store sv, int n, const int32_t* __restrict
 
 // ---------------------------------------------------------------------------------------------
 // Fused path: one block of W warps per request (the kernel itself is described where it is
-// defined).  Two blocks per SM is the usual shape: W = 10 with 96 registers per thread.  A batch
+// defined).  Two blocks per SM is the usual shape.  A batch
 // of at most one request per SM gets bigger blocks (W = 24 / 16), a batch of more than two
 // requests per SM smaller ones (W = 8 / 5, four per SM) to stay in one wave.
-constexpr int CTA_WARPS = 10;                  // the usual block (96 registers; 16 warps x 64 registers spill: 87 us against 83.5)
-constexpr int CTA_WARPS_STEP = 10;             // the usual block of sd_step
+constexpr int CTA_WARPS = 14;                  // the usual block; 256 requests: 44.2 us (10 warps 51.5, 12 52.1, 13 45.6, 15 48.9, 16 49.3)
+constexpr int CTA_WARPS_STEP = 14;             // of sd_step: 58.6 us per step (8 warps 63.1, 10 60.1, 12 59.2, 16 58.6)
 constexpr int CTA_WARPS_WIDE = 24;             // small batches (one block per SM at most): the block has the SM's
 constexpr int CTA_WARPS_WIDE_STEP = 16;        // registers to itself (80 per thread; sd_step: 128)
 constexpr int CTA_WARPS_NARROW = 8;            // batches of more than two requests per SM: four blocks per SM
