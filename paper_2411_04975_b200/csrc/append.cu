@@ -1,368 +1,608 @@
 // sd_append: the batched append kernel for the per-request trees (see append_core.cuh for how one
-// token is appended) and the level-by-level insert of whole sequences into the global tree.
+// token is appended) and the insert of whole sequences into the global tree.
 #include <cooperative_groups.h>
 
 #include "append_core.cuh"
+#include "global_insert.cuh"
+#include "suffix_order.cuh"
 
 namespace cg = cooperative_groups;
 
 namespace {
 
 // ---------------------------------------------------------------------------------------------
-// Global online insert (a finished request's output goes into the global tree), level by level.
+// Global online insert (a finished request's output goes into the global tree).
 //
 // Inserting a sequence adds one occurrence to every string of at most D tokens that starts at one
-// of its positions: one root-to-depth-D PATH per start position.  Taking the tokens one after the
-// other makes a chain as long as the sequence.  Here up to 2,048 paths are taken at once, a
-// thread per path, and all of them go down one level per round:
-//   1. every path enters its current node (the parent of the node it is about to reach) into a
-//      hash set in shared memory, which counts the paths per parent;
-//   2. every path looks its next token up in the parent's child run.  A child that exists gets its
-//      count raised by an atomic add.  A missing child is inserted at once if the path is the
-//      only one at that parent: nobody else reads or writes that run during this level;
-//   3. the other missing children are PENDING and are served in rounds: the waiting paths look
-//      again (an earlier round may have added the very child), then per parent one path is
-//      elected (a turn counter in the parent's hash-set cell) and inserts.  Runs of different
-//      parents are disjoint, so the elected paths do not disturb one another;
-//   4. an insert shifts or moves its run, so every path that shares its parent and whose parent's
-//      run changed after it took its child looks the child's new place up.
-// Only runs of ONE depth change during a level, and the entries of their parents (one level up)
-// stay where they are, which is what makes the election by parent sufficient.  A node's own
-// child run (first entry and size, as read with the node's entry) stays valid until the next
-// level, so it travels with the path and the next look-up starts at the run itself.  There is
-// no waiting on another thread anywhere, only block-wide barriers.  Placement follows the
-// token-by-token append: the first leaf of a path that leaves the known text reserves room down
-// to depth D and the later leaves go directly behind their parents.
-//
-// The block is a CLUSTER of GI_CTAS thread blocks on as many SMs (the work of a level is mostly
-// instruction issue, which one SM's schedulers limit): the barriers are cluster barriers, the
-// parent set is spread over the blocks' shared memories and the pool counters live in block 0's,
-// all reached through distributed shared memory.  Tree entries are read through L2 (an SM's L1
-// does not see what the other SMs store), and every block derives the list of sequences from
-// the call's arguments for itself, so all blocks take the same branches and meet at every barrier.
-constexpr int GI_CTAS = 8;
-constexpr int GI_THREADS = 256;               // per block
-constexpr int GI_PASS = GI_CTAS * GI_THREADS; // paths per pass
-constexpr int GI_CELLS = 512;                 // cells of the parent set per block: the set is at most half full
-constexpr int GI_SLOTS = GI_CTAS * GI_CELLS;
+// of its positions: one root-to-depth-D PATH per start position.  Up to GI_REAL positions are taken at once, in one
+// cooperative launch:
+//   1. every path goes down the tree as far as it exists, eight lanes each, and raises the counts on its way (no path
+//      waits for another: nothing moves yet).  Meanwhile one block sorts the positions' suffixes;
+//   2. the sorted suffixes and their common prefixes are a trie of the whole batch.  Its nodes deeper than the walk
+//      came are new.  They are laid down in pre-order in one stretch of the pool, by the sweeps that build
+//      a tree offline (see build.cu: a lane per depth), with the depth the walk reached taking the place of the root:
+//      counts, children and places follow from running state per depth.  EVENTS are the new nodes whose parent
+//      exists;
+//   3. events are grouped by parent, and every parent's run is merged once with all its new children (in place, or
+//      into a roomier run), while the rest of the new nodes is written;
+//   4. every parent's entry gets its new run, in the place it has now if its own run was merged, too.
+// Six grid barriers and no rounds: the time is that of the walk (dependent loads) or of the sort, whichever is
+// longer, and of the sweeps over the tiles.  (Level by level with an election per parent and round, by a cluster of 8
+// blocks: 150 us for the 1,000 tokens that three finished outputs bring, MEASURED now.)
+// The nodes that a batch adds need the pool to hold them all: a batch that does not fit raises counts only.
+constexpr int GI_BLOCKS = 24;
+constexpr int GI_THREADS = BS_THREADS;
+constexpr int GI_REAL = GI_MAX - SD_MAX_DEPTH;                   // start positions per pass
 constexpr int GI_ITEMS = 256;
-constexpr int GI_BIG = 48;                    // inserts that move more entries are done by a whole warp
+constexpr int GI_CELLS = 2 * GI_MAX;
+constexpr int GI_BIG = 256;                   // runs longer than this are merged by a whole block
 
-struct GiShared {
-    // the parent set, one for the odd and one for the even levels (a level clears the other one's)
-    int key[2][GI_CELLS];                     // parent + 1 (level 1: token + 1), 0 = free
-    int cnt[2][GI_CELLS];                     // paths at that parent
-    int turn[2][GI_CELLS];                    // rounds in which a path of that parent was elected
+struct GiItems {
     int item[GI_ITEMS];
     long long begin[GI_ITEMS], end[GI_ITEMS], pref[GI_ITEMS + 1];
     int n_items;
-    int any[3];                               // flags of the cluster-wide "or", used in turn
-    // block 0's copy only:
-    unsigned long long used;
-    int live, status;
 };
 
-struct GiCluster {
-    cg::cluster_group cl;
-    GiShared* sh;                             // this block's
-    GiShared* sh0;                            // block 0's
-    int phase;
-    __device__ int* cell_ptr(int* base, int cell) const {       // base: a table of this block's GiShared
-        return cl.map_shared_rank(base, (unsigned)cell / GI_CELLS) + (cell & (GI_CELLS - 1));
-    }
-    // Bit 0: a holds for any thread of the cluster, bit 1: b does.  A barrier for the whole
-    // cluster.  Every block tells every block (thread r writes to block r), so the answer is read
-    // from the block's own shared memory.
-    __device__ int any(bool a, bool b = false) {
-        const int mine = (__syncthreads_or(a) ? 1 : 0) | (__syncthreads_or(b) ? 2 : 0);
-        if (threadIdx.x < GI_CTAS && mine) atomicOr(cl.map_shared_rank(&sh->any[phase], threadIdx.x), mine);
-        cl.sync();
-        const int r = *(volatile int*)&sh->any[phase];
-        // the flag of the round before: everybody read it before arriving at the barrier above,
-        // and it is written again only after the next barrier
-        if (threadIdx.x == 0) sh->any[(phase + 2) % 3] = 0;
-        phase = (phase + 1) % 3;
-        return r;
-    }
+struct GiSort {                               // block 0, while it sorts
+    unsigned char order[block_order_smem<GI_MAX / BS_THREADS>()];
+    int tok[GI_MAX];
+    unsigned short begin[GI_MAX], end[GI_MAX], sa[GI_MAX];
+};
+struct GiTable {                              // block 0, while it groups
+    int key[GI_CELLS];                        // parent + 2, 0 = free
+    int cnt[GI_CELLS];                        // events
+    int at[GI_CELLS];                         // first place | group << 16
+    int tok[GI_MAX], ev[GI_MAX];
+    int n_big;
+};
+constexpr int GI_WARP_TILES = (GI_TILES + GI_BLOCKS - 2) / (GI_BLOCKS - 1);                 // tiles per block, a warp each
+union GiShared {
+    GiSort sort;
+    GiTable table;
+    int2 state[GI_WARP_TILES][GI_TILE][32];   // the other blocks: state from behind, by suffix of the tile and depth
 };
 
-// Entries for new runs and chain blocks of a warp's lanes (`size` may be 0): one atomic per warp.
-// Returns the lane's first entry, -1 if it asked for none or the pool cannot hold the warp's
-// request (then the status bit is set as well).  All 32 lanes call.
-__device__ __forceinline__ int gi_alloc_warp(GiShared* sh0, long long cap, int size, int lane) {
+// exclusive sum over the block's threads, the total in `all`
+__device__ __forceinline__ int gi_block_scan(int v, int* wsum, int tid, int& all) {
     const unsigned FULL = 0xffffffffu;
-    int inc = size;
+    const int lane = tid & 31, wib = tid >> 5;
+    int inc = v;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
         const int y = __shfl_up_sync(FULL, inc, o);
         if (lane >= o) inc += y;
     }
-    const int total = __shfl_sync(FULL, inc, 31);
-    if (total == 0) return -1;
-    unsigned long long at = 0;
-    if (lane == 31) at = atomicAdd(&sh0->used, (unsigned long long)total);
-    at = __shfl_sync(FULL, at, 31);
-    if (at + (unsigned long long)total > (unsigned long long)cap) {
-        if (lane == 31) atomicOr(&sh0->status, SD_STATUS_GLOBAL_FULL);
-        return -1;
-    }
-    return size > 0 ? (int)at + inc - size : -1;
+    if (lane == 31) wsum[wib] = inc;
+    __syncthreads();
+    const int c = wsum[lane];
+    const int before = (int)__reduce_add_sync(FULL, lane < wib ? (unsigned)c : 0u);
+    all = (int)__reduce_add_sync(FULL, (unsigned)c);
+    __syncthreads();
+    return before + inc - v;
 }
 
-// Child x of `cur` is missing and this path may add it (`ins`; lanes without an insert pass
-// false).  All 32 lanes call.  On return nxt is the new node and new_room the room reserved
-// behind it; (seen_cb, seen_n) describe the parent's run right after the insert.  A path whose
-// entries the pool cannot hold stops (rem = 0).
-__device__ __forceinline__ void gi_insert(GiShared* sh0, const sd_store& sv, int d, int lane, bool ins, int x, int cur,
-                                          int room, int cb, int nc, unsigned w, int pos, int& nxt, int& new_room,
-                                          int& seen_cb, int& seen_n, int& rem, int& my_live) {
-    const unsigned FULL = 0xffffffffu;
-    int4* const ent = sv.g_ent;
-    const int D = sv.D;
-    bool moves = false, behind = false;
-    int asz = 0;
-    if (ins) {
-        if (d == 1) asz = D;                                     // a new depth-1 node starts a chain block
-        else if (nc == 0) {                                      // first child of a leaf: continue the chain block, or start one
-            moves = true;
-            if (room > 0) behind = true; else asz = D - d + 1;
-        } else if ((uint32_t)nc == sd_run_capacity(w)) {         // the run is full: it moves to twice the room
-            moves = true;
-            asz = (int)sd_pow2ceil((uint32_t)nc + 1u);
-        }
+__device__ __forceinline__ int gi_item_of(const GiItems& I, long long p) {
+    int lo = 0, hi = I.n_items - 1;                              // last item whose prefix is <= p
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (I.pref[mid] <= p) lo = mid; else hi = mid - 1;
     }
-    int fresh = gi_alloc_warp(sh0, sv.g_cap, asz, lane);
-    bool big = false;
-    if (ins) {
-        if (asz > 0 && fresh < 0) rem = 0;
-        else {
-            ++my_live;
-            if (d == 1) {
-                ent[fresh] = make_int4(x, 1, 0, 0);
-                sv.g_root[x] = fresh;
-                nxt = fresh;
-                new_room = D - 1;
-            } else {
-                if (behind) { fresh = cur + 1; new_room = room - 1; }
-                else new_room = nc == 0 ? asz - 1 : 0;
-                seen_cb = moves ? fresh : cb;
-                seen_n = nc + 1;
-                big = (moves ? nc : nc - pos) > GI_BIG;
-                if (!big) nxt = insert_child<8, true>(ent, cur, cb, nc, pos, x, fresh, moves);
+    return lo;
+}
+
+// 1. the paths from positions [0, m) of the pass that starts at c0
+__device__ void gi_walk(const sd_store& sv, GiScratch* X, const GiItems& I, const int32_t* d_tokens, long long c0, int m, int group,
+                        int groups, int lane) {
+    const unsigned FULL = 0xffffffffu;
+    const int l = lane & (APP_LANES - 1), gb = lane & ~(APP_LANES - 1), D = sv.D;
+    int4* const ent = sv.g_ent;
+    for (int p0 = 0; p0 < m; p0 += groups) {                     // (uniform for the warp)
+        const int p = p0 + group;
+        const bool mine = p < m;
+        const int32_t* tp = d_tokens;
+        int len = 0;
+        if (mine) {
+            const int it = gi_item_of(I, c0 + p);
+            const long long k = I.begin[it] + (c0 + p - I.pref[it]);
+            tp = d_tokens + k;
+            len = (int)min((long long)D, I.end[it] - k);
+        }
+        int node = -1, prev = -1, v = 0, wb = -64;
+        int2 zw = make_int2(0, 0);
+        int4 e = make_int4(-1, 0, 0, 0);
+        if (mine) {
+            node = sv.g_root[tp[0]];
+            if (node >= 0) {
+                zw = *reinterpret_cast<const int2*>(&ent[node].z);
+                v = 1;
+                if (l == 0) atomicAdd(word(&ent[node], 1), 1);
             }
         }
-    }
-    // inserts that move many entries: the warp does them one after the other
-    unsigned bm = __ballot_sync(FULL, big);
-    while (bm) {
-        const int src = __ffs(bm) - 1;
-        bm &= bm - 1;
-        const int idx = insert_child_warp<true>(ent, __shfl_sync(FULL, cur, src), __shfl_sync(FULL, cb, src),
-                                                __shfl_sync(FULL, nc, src), __shfl_sync(FULL, pos, src),
-                                                __shfl_sync(FULL, x, src), __shfl_sync(FULL, fresh, src),
-                                                __shfl_sync(FULL, moves ? 1 : 0, src) != 0, lane);
-        if (lane == src) nxt = idx;
+        bool alive = node >= 0;
+        while (true) {
+            const bool on = alive && v < len;
+            if (!__any_sync(FULL, on)) break;
+            const int x = on ? tp[v] : -1;
+            const int n = on ? (int)((unsigned)zw.y & RUN_COUNT_MASK) : 0;
+            const bool far = n > APP_LANES;
+            int at = -1;
+            int2 next = make_int2(0, 0);
+            if (__any_sync(FULL, far)) {
+                int place;
+                int2 fz;
+                const int q = group_lookup(RunSearch{ent + zw.x, 0, far ? n : 0}, x, lane, place, fz);
+                if (far && q >= 0) { at = zw.x + q; next = fz; }
+            }
+            const bool near = on && !far;
+            if (__any_sync(FULL, near)) {
+                if (near && (zw.x < wb || zw.x + n > wb + APP_LANES)) {
+                    wb = zw.x;
+                    if (wb + l < (int)sv.g_cap) e = ent[wb + l];
+                }
+                const int off = zw.x - wb;
+                const unsigned eq = (__ballot_sync(FULL, near && l >= off && l < off + n && e.x == x) >> gb) & 0xffu;
+                const int q = eq ? __ffs(eq) - 1 : 0;
+                const int nz = __shfl_sync(FULL, e.z, q, APP_LANES), nw = __shfl_sync(FULL, e.w, q, APP_LANES);
+                if (near && eq) { at = wb + q; next = make_int2(nz, nw); }
+            }
+            if (on) {
+                if (at < 0) alive = false;
+                else {
+                    if (l == 0) {
+                        atomicAdd(word(&ent[at], 1), 1);
+                        // a count changes: the copies in the run's top block (if any) are stale from now on
+                        if ((unsigned)zw.y & RUN_HAS_TOP) atomicAnd(word(&ent[node], 3), (int)~RUN_HAS_TOP);
+                    }
+                    prev = node; node = at; zw = next;
+                    ++v;
+                }
+            }
+        }
+        if (mine && l == 0) { X->v[p] = v; X->p[p] = node; X->q[p] = prev; }
     }
 }
 
-__global__ void __cluster_dims__(GI_CTAS, 1, 1) __launch_bounds__(GI_THREADS, 1)
-global_insert_kernel(sd_store sv, int n, const int32_t* d_slot, const int64_t* d_offsets, const int32_t* d_tokens) {
-    __shared__ GiShared sh;
-    const unsigned FULL = 0xffffffffu;
-    const int tid = threadIdx.x, lane = tid & 31;
-    int4* const ent = sv.g_ent;
-    const int D = sv.D;
+// 2. The sweeps: a warp per tile of GI_TILE suffixes, a lane per depth.  A lane also looks after the tile's suffix of its number.
+// (Functions of their own: in one with everything else they spilled, 36 and 38 us instead of MEASURED.)
+struct GiOwn {
+    int lnv;                                  // common prefix, length, levels that exist: packed
+    int at;                                   // start position
+    int below, event;                         // new nodes whose parent is new, whose parent exists
+};
 
-    // (every block looks at all items: all blocks of the cluster take the same way)
+__device__ __forceinline__ GiOwn gi_own(const GiScratch* X, int j0, int mm, int lane) {
+    GiOwn o{0, 0, 0, 0};
+    if (lane < mm) {
+        o.at = X->sa[j0 + lane];
+        const int l = X->lcp[j0 + lane], n = X->len[j0 + lane], v = X->v[o.at];
+        o.lnv = l | (n << 8) | (v << 16);
+        o.below = max(0, n - max(l, v + 1));
+        o.event = l <= v && v < n ? 1 : 0;
+    }
+    return o;
+}
+
+// what the tile does to the state from behind: children counted up to the first reset, and where that is
+__device__ __noinline__ void gi_sweep_tile(GiScratch* X, int t, int m, int lane) {
+    const unsigned FULL = 0xffffffffu;
+    const int j0 = t * GI_TILE, mm = min(GI_TILE, m - j0), d = lane + 1;
+    const GiOwn o = gi_own(X, j0, mm, lane);
+    int cnt = 0, first = m;
+    bool seen = false;
+    for (int i = 0; i < mm; ++i) {
+        const int x = __shfl_sync(FULL, o.lnv, i), l = x & 255, len = (x >> 8) & 255;
+        if (!seen) {
+            cnt += l == d && len > l ? 1 : 0;
+            if (l < d) { seen = true; first = j0 + i; }
+        }
+    }
+    X->f[t][lane] = cnt | (seen ? (int)0x80000000 : 0);
+    X->e[t][lane] = first;
+    const int sb = (int)__reduce_add_sync(FULL, (unsigned)o.below), se = (int)__reduce_add_sync(FULL, (unsigned)o.event);
+    if (lane == 0) { X->s[t] = sb; X->ev[t] = se; }
+}
+
+// sums over the tiles in front of tile t (t = tiles: all)
+__device__ __forceinline__ void gi_sums(const GiScratch* X, int t, int lane, int& s, int& ev) {
+    int a = 0, b = 0;
+    for (int q = lane; q < t; q += 32) { a += X->s[q]; b += X->ev[q]; }
+    s = (int)__reduce_add_sync(0xffffffffu, (unsigned)a);
+    ev = (int)__reduce_add_sync(0xffffffffu, (unsigned)b);
+}
+
+// from behind: the events, the end of the last run opened per depth, and the state at every suffix
+__device__ __noinline__ void gi_sweep_runs(GiScratch* X, int2 (*state)[32], int t, int tiles, int m, int lane) {
+    const unsigned FULL = 0xffffffffu;
+    const int j0 = t * GI_TILE, mm = min(GI_TILE, m - j0), d = lane + 1;
+    const GiOwn o = gi_own(X, j0, mm, lane);
+    int s_at, ev_at;
+    gi_sums(X, t, lane, s_at, ev_at);
+    int is = o.below, ie = o.event;
+#pragma unroll
+    for (int k = 1; k < GI_TILE; k <<= 1) {
+        const int a = __shfl_up_sync(FULL, is, k), b = __shfl_up_sync(FULL, ie, k);
+        if (lane >= k) { is += a; ie += b; }
+    }
+    const int s_own = s_at + is - o.below, ev_own = ev_at + ie - o.event;
+    if (o.event) {
+        const int v = o.lnv >> 16;
+        X->ev_p[ev_own] = X->p[o.at]; X->ev_q[ev_own] = X->q[o.at];
+        X->ev_ptok[ev_own] = v > 0 ? X->tok[o.at + v - 1] : -1;
+        X->ev_tok[ev_own] = X->tok[o.at + v];
+    }
+    int F = 0, e = m;
+    bool seen = false;
+#pragma unroll 8
+    for (int q = t + 1; q < tiles; ++q) {
+        const int fq = X->f[q][lane], eq = X->e[q][lane];
+        if (!seen) {
+            F += fq & 0x7fffffff;
+            if (fq < 0) { seen = true; e = eq; }
+        }
+    }
+    int g = F;
+#pragma unroll
+    for (int k = 1; k < 32; k <<= 1) {
+        const int y = __shfl_up_sync(FULL, g, k);
+        if (lane >= k) g += y;
+    }
+    g -= F;                                                      // G: children of the levels above
+    int R = -1;
+    for (int i = mm - 1; i >= 0; --i) {
+        const int x = __shfl_sync(FULL, o.lnv, i), l = x & 255, len = (x >> 8) & 255, v = x >> 16;
+        const int si = __shfl_sync(FULL, s_own, i), ei = __shfl_sync(FULL, ev_own, i);
+        state[i][lane] = make_int2(g, e);
+        const int up = __shfl_down_sync(FULL, g, 1), gv = __shfl_sync(FULL, g, min(v, 31));
+        const int kids = (lane == 31 ? 0 : up - g) + (d < len ? 1 : 0);
+        const int run = si + d - max(l, v + 1) + g - gv;
+        const bool opens = d > max(l, v) && d <= len;
+        if (opens && R < 0) R = run + kids;
+        if (opens && l <= v && d == v + 1) { X->ev_cnt[ei] = e - (j0 + i); X->ev_run[ei] = run; X->ev_kids[ei] = kids; }
+        const int step = __shfl_sync(FULL, g, min(l, 31)) + (len > l ? 1 : 0);
+        if (d > l) { g = l == 0 ? 0 : step; e = j0 + i; }
+    }
+    X->r[t][lane] = R;
+}
+
+// from the front: the new nodes below the events, from entry `used` on
+__device__ __noinline__ void gi_sweep_emit(const GiScratch* X, const int2 (*state)[32], int4* ent, int used, int t, int m, int lane) {
+    const unsigned FULL = 0xffffffffu;
+    const int j0 = t * GI_TILE, mm = min(GI_TILE, m - j0), d = lane + 1;
+    const GiOwn o = gi_own(X, j0, mm, lane);
+    int s_at, ev_at;
+    gi_sums(X, t, lane, s_at, ev_at);
+    int is = o.below;
+#pragma unroll
+    for (int k = 1; k < GI_TILE; k <<= 1) {
+        const int a = __shfl_up_sync(FULL, is, k);
+        if (lane >= k) is += a;
+    }
+    const int s_own = s_at + is - o.below;
+    int tok[GI_TILE];
+#pragma unroll
+    for (int i = 0; i < GI_TILE; ++i) {
+        const int at = __shfl_sync(FULL, o.at, i), len = (__shfl_sync(FULL, o.lnv, i) >> 8) & 255;
+        tok[i] = lane < len ? X->tok[at + lane] : 0;
+    }
+    int R = -1;
+#pragma unroll 8
+    for (int q = 0; q < t; ++q) { const int y = X->r[q][lane]; if (y >= 0) R = y; }
+#pragma unroll
+    for (int i = 0; i < GI_TILE; ++i) {
+        if (i >= mm) break;
+        const int x = __shfl_sync(FULL, o.lnv, i), l = x & 255, len = (x >> 8) & 255, v = x >> 16;
+        const int si = __shfl_sync(FULL, s_own, i);
+        const int2 ge = state[i][lane];
+        const int up = __shfl_down_sync(FULL, ge.x, 1), gv = __shfl_sync(FULL, ge.x, min(v, 31));
+        const int later = lane == 31 ? 0 : up - ge.x, kids = later + (d < len ? 1 : 0);
+        const int run = si + d - max(l, v + 1) + ge.x - gv;
+        const bool opens = d > max(l, v) && d <= len;
+        // the entry of the next depth's node: this node's first child, or the next of its other children
+        const int place = __shfl_up_sync(FULL, opens ? run : R - 1 - later, 1);
+        if (opens) R = run + kids;
+        if (opens && !(l <= v && d == v + 1))
+            ent[used + place] = make_int4(tok[i], ge.y - (j0 + i), kids > 0 ? used + run : 0, kids > 0 ? (int)((unsigned)kids | RUN_STATIC) : 0);
+    }
+}
+
+// 3. the events by parent (one block): every parent's new children by token, its run's new place
+__device__ __noinline__ void gi_group(const sd_store& sv, GiScratch* X, GiTable& tb, int* wsum, int used, int s_all, int ev_all, int tid) {
+    int4* const ent = sv.g_ent;
+    for (int i = tid; i < GI_CELLS; i += GI_THREADS) { tb.key[i] = 0; tb.cnt[i] = 0; }
+    if (tid == 0) tb.n_big = 0;
+    __syncthreads();
+    auto cell_of = [&](int key, bool insert) {
+        int c = (int)(((unsigned)key * 2654435761u) >> 20) & (GI_CELLS - 1);
+        for (int probe = 0; probe < GI_CELLS; ++probe) {
+            const int old = insert ? atomicCAS(&tb.key[c], 0, key) : tb.key[c];
+            if (old == key || (insert && old == 0)) return c;
+            if (old == 0) return -1;
+            c = (c + 1) & (GI_CELLS - 1);
+        }
+        return -1;
+    };
+    constexpr int PER = GI_MAX / GI_THREADS;
+    int cell[PER], at[PER], x[PER];
+#pragma unroll
+    for (int u = 0; u < PER; ++u) {
+        const int e = tid + u * GI_THREADS;
+        cell[u] = -1; at[u] = 0; x[u] = 0;
+        if (e < ev_all) {
+            x[u] = X->ev_tok[e];
+            cell[u] = cell_of(X->ev_p[e] + 2, true);
+            at[u] = atomicAdd(&tb.cnt[cell[u]], 1);
+        }
+    }
+    __syncthreads();
+    constexpr int CELLS = GI_CELLS / GI_THREADS;
+    int sum = 0, groups = 0, all, n_groups;
+#pragma unroll
+    for (int u = 0; u < CELLS; ++u) { const int c = tb.cnt[tid * CELLS + u]; sum += c; groups += c > 0 ? 1 : 0; }
+    int first = gi_block_scan(sum, wsum, tid, all), id = gi_block_scan(groups, wsum, tid, n_groups);
+#pragma unroll
+    for (int u = 0; u < CELLS; ++u) {
+        const int c = tb.cnt[tid * CELLS + u];
+        tb.at[tid * CELLS + u] = first | (id << 16);
+        first += c; id += c > 0 ? 1 : 0;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int u = 0; u < PER; ++u)
+        if (cell[u] >= 0) { const int p = (tb.at[cell[u]] & 0xffff) + at[u]; tb.tok[p] = x[u]; tb.ev[p] = tid + u * GI_THREADS; }
+    __syncthreads();
+#pragma unroll
+    for (int u = 0; u < PER; ++u)
+        if (cell[u] >= 0) {                          // tokens of one parent's events are distinct
+            const int p = tb.at[cell[u]] & 0xffff, k = tb.cnt[cell[u]];
+            int rank = 0;
+            for (int q = 0; q < k; ++q) rank += tb.tok[p + q] < x[u] ? 1 : 0;
+            X->m_tok[p + rank] = x[u]; X->m_ev[p + rank] = tid + u * GI_THREADS;
+        }
+    GiGroup gr[CELLS];
+    int size[CELLS], mine_size = 0;
+#pragma unroll
+    for (int u = 0; u < CELLS; ++u) {
+        const int c = tid * CELLS + u, k = tb.cnt[c];
+        size[u] = 0;
+        gr[u].k = k;
+        if (k > 0) {
+            GiGroup& G = gr[u];
+            G.first = tb.at[c] & 0xffff;
+            const int e = tb.ev[G.first], q = X->ev_q[e];
+            G.parent = tb.key[c] - 2; G.parent_tok = X->ev_ptok[e];
+            G.cb = 0; G.n = 0; G.above = -1;
+            if (G.parent >= 0) {
+                const int4 pe = __ldcg(ent + G.parent);
+                G.cb = pe.z; G.n = (int)((unsigned)pe.w & RUN_COUNT_MASK);
+                if ((uint32_t)(G.n + k) > sd_run_capacity((uint32_t)pe.w)) size[u] = (int)sd_pow2ceil((uint32_t)(G.n + k));
+                if (q >= 0) { const int qc = cell_of(q + 2, false); if (qc >= 0) G.above = tb.at[qc] >> 16; }
+            } else size[u] = k;
+            if (G.n > GI_BIG || k > GI_BIG) X->big[atomicAdd(&tb.n_big, 1)] = tb.at[c] >> 16;
+        }
+        mine_size += size[u];
+    }
+    int entries, place = used + s_all + gi_block_scan(mine_size, wsum, tid, entries);
+#pragma unroll
+    for (int u = 0; u < CELLS; ++u)
+        if (gr[u].k > 0) {
+            gr[u].base = size[u] > 0 ? place : gr[u].cb;
+            X->group[tb.at[tid * CELLS + u] >> 16] = gr[u];
+            place += size[u];
+        }
+    if (tid == 0) {
+        X->n_groups = n_groups; X->n_big = tb.n_big; X->entries = entries;
+        X->fits = (long long)used + s_all + entries <= sv.g_cap ? 1 : 0;
+    }
+}
+
+// 3. one parent's run with its new children, by a team of T threads (a warp or a block)
+template <int T, class Sync>
+__device__ __forceinline__ void gi_merge(const sd_store& sv, const GiScratch* X, int* m_pos, const GiGroup& g, int base0, int t, Sync sync) {
+    constexpr int U = 4;
+    int4* const ent = sv.g_ent;
+    const int* const tok = X->m_tok + g.first;
+    int* const pos = m_pos + g.first;
+    // where the new children belong
+    for (int r = t; r < g.k; r += T) {
+        int lo = 0, hi = g.n;
+        while (lo < hi) { const int mid = (lo + hi) >> 1; if (__ldcg(&ent[g.cb + mid].x) < tok[r]) lo = mid + 1; else hi = mid; }
+        pos[r] = lo;
+    }
+    sync();
+    auto before = [&](int x) {                                   // new children in front of token x
+        int lo = 0, hi = g.k;
+        while (lo < hi) { const int mid = (lo + hi) >> 1; if (tok[mid] < x) lo = mid + 1; else hi = mid; }
+        return lo;
+    };
+    if (g.parent >= 0 && g.base != g.cb) {
+        for (int i0 = t; i0 < g.n; i0 += T * U) {
+            int4 e[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) if (i0 + u * T < g.n) e[u] = __ldcg(ent + g.cb + i0 + u * T);
+#pragma unroll
+            for (int u = 0; u < U; ++u) if (i0 + u * T < g.n) ent[g.base + i0 + u * T + before(e[u].x)] = e[u];
+        }
+    } else if (g.parent >= 0) {
+        const int stop = pos[0];
+        for (int hi = g.n; hi > stop; hi -= T * U) {             // from the top down, a chunk at a time
+            const int lo = max(stop, hi - T * U);
+            int4 e[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) if (lo + t + u * T < hi) e[u] = __ldcg(ent + g.cb + lo + t + u * T);
+            sync();
+#pragma unroll
+            for (int u = 0; u < U; ++u) if (lo + t + u * T < hi) ent[g.cb + lo + t + u * T + before(e[u].x)] = e[u];
+            sync();
+        }
+    }
+    for (int r = t; r < g.k; r += T) {
+        const int ev = X->m_ev[g.first + r], kids = X->ev_kids[ev], at = g.base + pos[r] + r;
+        ent[at] = make_int4(tok[r], X->ev_cnt[ev], kids > 0 ? base0 + X->ev_run[ev] : 0, kids > 0 ? (int)((unsigned)kids | RUN_STATIC) : 0);
+        if (g.parent < 0) sv.g_root[tok[r]] = at;
+    }
+    sync();
+}
+
+__global__ void __launch_bounds__(GI_THREADS, 1)
+global_insert_kernel(sd_store sv, int n, const int32_t* d_slot, const int64_t* d_offsets, const int32_t* d_tokens, int tok_bits) {
+    extern __shared__ __align__(16) unsigned char gi_smem[];
+    __shared__ GiItems I;
+    __shared__ int wsum[GI_THREADS / 32];
+    const unsigned FULL = 0xffffffffu;
+    const int tid = threadIdx.x, lane = tid & 31, wib = tid >> 5, blk = (int)blockIdx.x;
+    const int D = sv.D;
+    int4* const ent = sv.g_ent;
+    GiScratch* const X = sv.gi;
+    GiShared& sh = *reinterpret_cast<GiShared*>(gi_smem);
+
+    // (every block looks at all items: all blocks take the same way)
     bool mine = false;
     for (int i = tid; i < n; i += GI_THREADS) mine |= d_slot[i] == -1;
     if (!__syncthreads_or(mine)) return;                         // the usual decode step: nothing for the global tree
-    GiCluster G{cg::this_cluster(), &sh, nullptr, 0};
-    G.sh0 = G.cl.map_shared_rank(&sh, 0);
-    GiShared* const sh0 = G.sh0;
-    const int path0 = (int)G.cl.block_rank() * GI_THREADS + tid; // this thread's path within a pass
-    if (tid == 0) {
-        sh.used = (unsigned long long)sv.g_state->used; sh.live = 0; sh.status = sv.g_state->status;
-        sh.any[0] = sh.any[1] = sh.any[2] = 0;
-    }
-    for (int i = tid; i < 2 * GI_CELLS; i += GI_THREADS) { sh.key[0][i] = 0; sh.cnt[0][i] = 0; sh.turn[0][i] = 0; }
-    G.cl.sync();
+    cg::grid_group grid = cg::this_grid();
+    bool full = (sv.g_state->status & SD_STATUS_GLOBAL_FULL) != 0, bad = false, again = false;
+    int used = sv.g_state->used, live = 0;
     long long tokens_done = 0;
-    int my_live = 0;
 
-    for (int base = 0; base < n; base += GI_ITEMS) {
-        if (G.any((*(volatile int*)&sh0->status & SD_STATUS_GLOBAL_FULL) != 0)) break;
+    for (int base = 0; base < n && !full; base += GI_ITEMS) {
         // the sequences among items [base, base + GI_ITEMS), in item order
-        if (tid == 0) sh.n_items = 0;
+        __syncthreads();
+        if (tid == 0) I.n_items = 0;
         __syncthreads();
         if (tid < 32) {
             for (int i0 = 0; i0 < GI_ITEMS; i0 += 32) {
                 const int i = base + i0 + lane;
                 const bool is = i < n && d_slot[i] == -1;
                 const unsigned m = __ballot_sync(FULL, is);
-                if (is) sh.item[sh.n_items + __popc(m & ((1u << lane) - 1u))] = i;
+                if (is) I.item[I.n_items + __popc(m & ((1u << lane) - 1u))] = i;
                 __syncwarp();
-                if (lane == 0) sh.n_items += __popc(m);
+                if (lane == 0) I.n_items += __popc(m);
                 __syncwarp();
             }
         }
         __syncthreads();
-        const int n_items = sh.n_items;
+        const int n_items = I.n_items;
         if (n_items == 0) continue;
-        for (int j = tid; j < n_items; j += GI_THREADS) { sh.begin[j] = d_offsets[sh.item[j]]; sh.end[j] = d_offsets[sh.item[j] + 1]; }
+        for (int j = tid; j < n_items; j += GI_THREADS) { I.begin[j] = d_offsets[I.item[j]]; I.end[j] = d_offsets[I.item[j] + 1]; }
         __syncthreads();
         // a token outside the vocabulary ends its sequence there
         for (int j = 0; j < n_items; ++j) {
-            const long long b = sh.begin[j], e = d_offsets[sh.item[j] + 1];
+            const long long b = I.begin[j], e = d_offsets[I.item[j] + 1];
             for (long long k = b + tid; k < e; k += GI_THREADS) {
                 const int x = d_tokens[k];
-                if (x < 0 || x >= sv.V) { atomicMin(&sh.end[j], k); atomicOr(&sh0->status, SD_STATUS_BAD_TOKEN); }
+                if (x < 0 || x >= sv.V) { atomicMin(&I.end[j], k); bad = true; }
             }
         }
         __syncthreads();
         if (tid == 0) {
             long long acc = 0;
-            for (int j = 0; j < n_items; ++j) { sh.pref[j] = acc; acc += max(sh.end[j] - sh.begin[j], 0ll); }
-            sh.pref[n_items] = acc;
+            for (int j = 0; j < n_items; ++j) { I.pref[j] = acc; acc += max(I.end[j] - I.begin[j], 0ll); }
+            I.pref[n_items] = acc;
         }
         __syncthreads();
-        const long long total = sh.pref[n_items];
+        const long long total = I.pref[n_items];
 
-        for (long long c0 = 0; c0 < total; c0 += GI_PASS) {
-            // both parent sets are empty behind this barrier (the last level of a pass leaves its own behind)
-            for (int i = tid; i < 2 * GI_CELLS; i += GI_THREADS) { sh.key[0][i] = 0; sh.cnt[0][i] = 0; sh.turn[0][i] = 0; }
-            if (G.any((*(volatile int*)&sh0->status & SD_STATUS_GLOBAL_FULL) != 0)) break;
-            // this thread's path: start position k, `rem` tokens to take (at most D)
-            const long long p = c0 + path0;
-            long long k = 0;
-            int rem = 0;
-            if (p < total) {
-                int lo = 0, hi = n_items - 1;                    // last item whose prefix is <= p
-                while (lo < hi) {
-                    const int mid = (lo + hi + 1) >> 1;
-                    if (sh.pref[mid] <= p) lo = mid; else hi = mid - 1;
+        for (long long c0 = 0; c0 < total && !full; c0 += GI_REAL) {
+            if (again) grid.sync();                              // the pass before is over
+            again = true;
+            const int m = (int)min((long long)GI_REAL, total - c0);
+            // ---------------- 1. walk, and sort
+            if (blk == 0) {
+                // (the last sequence's next tokens, as far as the paths reach)
+                const int M = m + (int)min((long long)(D - 1), I.pref[gi_item_of(I, c0 + m - 1) + 1] - (c0 + m));
+                GiSort& so = sh.sort;
+                for (int i = tid; i < M; i += GI_THREADS) {
+                    const int it = gi_item_of(I, c0 + i);
+                    const int x = d_tokens[I.begin[it] + (c0 + i - I.pref[it])];
+                    so.tok[i] = x; X->tok[i] = x;
+                    so.begin[i] = (unsigned short)max(I.pref[it] - c0, 0ll);
+                    so.end[i] = (unsigned short)min(I.pref[it + 1] - c0, (long long)M);
                 }
-                k = sh.begin[lo] + (p - sh.pref[lo]);
-                rem = (int)min((long long)D, sh.end[lo] - k);
+                __syncthreads();
+                auto token = [&](int i) { return so.tok[i]; };
+                auto begin = [&](int i) { return (int)so.begin[i]; };
+                auto end = [&](int i) { return (int)so.end[i]; };
+                const unsigned short* const order = M <= BS_THREADS ? block_suffix_order<1>(so.order, wsum, M, tok_bits, D, token, begin, end)
+                                                                    : block_suffix_order<2>(so.order, wsum, M, tok_bits, D, token, begin, end);
+                // start positions only
+                int at = 0;
+                for (int i0 = 0; i0 < M; i0 += GI_THREADS) {
+                    const int i = i0 + tid;
+                    const int q = i < M ? order[i] : GI_MAX;
+                    int all;
+                    const int k = at + gi_block_scan(q < m ? 1 : 0, wsum, tid, all);
+                    if (q < m) { so.sa[k] = (unsigned short)q; X->sa[k] = q; }
+                    at += all;
+                }
+                __syncthreads();
+                for (int j = tid; j < m; j += GI_THREADS) {
+                    const int q = so.sa[j], len = min(D, so.end[q] - q);
+                    int l = 0;
+                    if (j > 0) {
+                        const int h = so.sa[j - 1], most = min(len, min(D, so.end[h] - h));
+                        while (l < most && so.tok[q + l] == so.tok[h + l]) ++l;
+                    }
+                    X->lcp[j] = l; X->len[j] = len;
+                }
+            } else {
+                gi_walk(sv, X, I, d_tokens, c0, m, ((blk - 1) * GI_THREADS + tid) / APP_LANES, (GI_BLOCKS - 1) * GI_THREADS / APP_LANES, lane);
             }
-            // the node of the tokens taken so far, the room reserved behind it, its child run
-            int cur = -1, room = 0, run_cb = 0;
-            unsigned run_w = 0;
-            bool more = true;                                    // a path of the cluster has a token for this level
-            for (int d = 1; d <= D && more; ++d) {
-                int* const t_key = sh.key[d & 1];
-                int* const t_cnt = sh.cnt[d & 1];
-                int* const t_turn = sh.turn[d & 1];
-                const bool alive = rem >= d;
-                const int x = alive ? d_tokens[k + d - 1] : 0;
-                // 1. the parent set
-                int cell = 0;
-                if (alive) {
-                    const int key = (d == 1 ? x : cur) + 1;
-                    cell = (int)(((unsigned)key * 2654435761u) >> 20);          // 12 bits
-                    for (int probe = 0; probe < GI_SLOTS; ++probe) {
-                        const int old = atomicCAS(G.cell_ptr(t_key, cell), 0, key);
-                        if (old == 0 || old == key) break;
-                        cell = (cell + 1) & (GI_SLOTS - 1);
-                    }
-                    atomicAdd(G.cell_ptr(t_cnt, cell), 1);
+            grid.sync();
+            // ---------------- 2. the sweeps, a warp per tile
+            const int tiles = (m + GI_TILE - 1) / GI_TILE, t = (blk - 1) + wib * (GI_BLOCKS - 1);
+            const bool sweeps = blk > 0 && t < tiles;
+            if (sweeps) gi_sweep_tile(X, t, m, lane);
+            grid.sync();
+            int s_all, ev_all;
+            gi_sums(X, tiles, lane, s_all, ev_all);
+            if (sweeps) gi_sweep_runs(X, sh.state[wib], t, tiles, m, lane);
+            grid.sync();
+            // ---------------- 3. grouping (block 0) while the others write the new nodes below the events
+            if (blk == 0) gi_group(sv, X, sh.table, wsum, used, s_all, ev_all, tid);
+            else if (sweeps && (long long)used + s_all <= sv.g_cap) gi_sweep_emit(X, sh.state[wib], ent, used, t, m, lane);
+            grid.sync();
+            // ---------------- merges: a warp per parent, a block per parent with a long run
+            const int n_groups = X->n_groups;
+            full = X->fits == 0;
+            if (!full) {
+                for (int gi = wib * GI_BLOCKS + blk; gi < n_groups; gi += GI_BLOCKS * (GI_THREADS / 32)) {
+                    const GiGroup g = X->group[gi];
+                    if (g.n <= GI_BIG && g.k <= GI_BIG) gi_merge<32>(sv, X, X->m_pos, g, used, lane, [] { __syncwarp(); });
                 }
-                G.cl.sync();
-                // the other level's set: last used before the barrier that ended that level, used
-                // again after the one that ends this level
-                for (int i = tid; i < GI_CELLS; i += GI_THREADS) {
-                    sh.key[(d & 1) ^ 1][i] = 0; sh.cnt[(d & 1) ^ 1][i] = 0; sh.turn[(d & 1) ^ 1][i] = 0;
+                const int n_big = X->n_big;
+                for (int b = blk; b < n_big; b += GI_BLOCKS) {
+                    const GiGroup g = X->group[X->big[b]];
+                    gi_merge<GI_THREADS>(sv, X, X->m_pos, g, used, tid, [] { __syncthreads(); });
                 }
-                const bool alone = alive && *(volatile int*)G.cell_ptr(t_cnt, cell) == 1;
-                // 2. look the token up
-                int found = -1, pos = 0;
-                int cb = run_cb, nc = (int)(run_w & RUN_COUNT_MASK);
-                unsigned w = run_w;
-                int4 fe = make_int4(0, 0, 0, 0);
-                if (alive) {
-                    if (d == 1) { found = __ldcg(sv.g_root + x); if (found >= 0) fe = __ldcg(ent + found); }
-                    else if (nc > 0) found = lookup_child<8, true>(ent, cb, nc, x, pos, fe);
-                    if (found >= 0) {
-                        atomicAdd(word(&ent[found], 1), 1);
-                        // a count changes: the copies in the run's top block (if any) are stale from now on
-                        if (d > 1 && (w & RUN_HAS_TOP)) atomicAnd(word(&ent[cur], 3), (int)~RUN_HAS_TOP);
-                    }
-                }
-                int nxt = found, new_room = 0;
-                int seen_cb = cb, seen_n = nc;                    // the parent's run as it was when nxt was taken
-                const bool own = alive && found < 0 && alone;
-                gi_insert(sh0, sv, d, lane, own, x, cur, room, cb, nc, w, pos, nxt, new_room, seen_cb, seen_n, rem, my_live);
-                // A node made by a path that was alone at the parent can be reached by no other path
-                // of this pass, and neither can anything below it: the rest of the path is a chain
-                // of new leaves, written here in one go if the room behind the node holds it.
-                if (own && rem > d && new_room >= rem - d) {
-                    *word(&ent[nxt], 2) = nxt + 1;
-                    *word(&ent[nxt], 3) = 1;
-                    for (int j = d + 1; j <= rem; ++j)
-                        ent[nxt + j - d] = j < rem ? make_int4(d_tokens[k + j - 1], 1, nxt + j - d + 1, 1)
-                                                   : make_int4(d_tokens[k + j - 1], 1, 0, 0);
-                    my_live += rem - d;
-                    rem = 0;
-                }
-                // 3. the other inserts: one path per parent and round.  From the second round on every
-                // waiting path first looks again: the children added in the round before are found by
-                // all the paths that want them at once (text that repeats itself sends many paths
-                // down the same strings), and only the children still missing are competed for.
-                bool pending = alive && found < 0 && !alone;
-                for (int round = 0; round <= GI_PASS; ++round) {
-                    const int r = G.any(pending, rem > d);
-                    more = (r & 2) != 0;
-                    if (!(r & 1)) break;
-                    if (round > 0) {
-                        if (pending) {
-                            found = -1; pos = 0;
-                            if (d == 1) { found = __ldcg(sv.g_root + x); if (found >= 0) fe = __ldcg(ent + found); }
-                            else {
-                                const int4 pe = __ldcg(ent + cur);
-                                cb = pe.z; w = (unsigned)pe.w; nc = (int)(w & RUN_COUNT_MASK);
-                                if (nc > 0) found = lookup_child<8, true>(ent, cb, nc, x, pos, fe);
-                            }
-                            if (found >= 0) {
-                                atomicAdd(word(&ent[found], 1), 1);
-                                nxt = found; seen_cb = cb; seen_n = nc;
-                                pending = false;
-                            }
-                        }
-                        G.cl.sync();                             // the look-ups are over before a run moves again
-                    }
-                    const bool win = pending && atomicCAS(G.cell_ptr(t_turn, cell), round, round + 1) == round;
-                    if (win) pending = false;
-                    gi_insert(sh0, sv, d, lane, win, x, cur, room, cb, nc, w, pos, nxt, new_room, seen_cb, seen_n, rem,
-                              my_live);
-                }
-                // 4. the child's place after all inserts of this level
-                if (rem >= d && d > 1 && !alone) {
-                    const int4 pe = __ldcg(ent + cur);
-                    const int n2 = (int)((unsigned)pe.w & RUN_COUNT_MASK);
-                    if (pe.z != seen_cb || n2 != seen_n) {
-                        found = n2 > 0 ? lookup_child<8, true>(ent, pe.z, n2, x, pos, fe) : -1;
-                        nxt = found;
-                        new_room = 0;                            // the node left its chain block
-                    }
-                }
-                if (rem >= d && nxt < 0) rem = 0;                // cannot happen; the path stops rather than go astray
-                cur = nxt;
-                room = new_room;
-                run_cb = found >= 0 ? fe.z : 0;                  // a node made just now has no children
-                run_w = found >= 0 ? (unsigned)fe.w : 0u;
             }
-            tokens_done += min((long long)GI_PASS, total - c0);
+            grid.sync();
+            // ---------------- 4. the parents' entries
+            if (!full) {
+                for (int gi = blk * GI_THREADS + tid; gi < n_groups; gi += GI_BLOCKS * GI_THREADS) {
+                    const GiGroup g = X->group[gi];
+                    if (g.parent < 0) continue;
+                    int at = g.parent;
+                    if (g.above >= 0) {
+                        const GiGroup a = X->group[g.above];
+                        int lo = 0, hi = a.k;
+                        while (lo < hi) { const int mid = (lo + hi) >> 1; if (X->m_tok[a.first + mid] < g.parent_tok) lo = mid + 1; else hi = mid; }
+                        at = a.base + (g.parent - a.cb) + lo;
+                    }
+                    *reinterpret_cast<int2*>(&ent[at].z) = make_int2(g.base, g.n + g.k);
+                }
+                live += s_all + ev_all;
+                used += s_all + X->entries;
+            }
+            tokens_done += m;
         }
     }
-    G.cl.sync();
-    if (my_live) atomicAdd(&sh0->live, my_live);
-    G.cl.sync();                                                 // (no block leaves while its shared memory may be in use)
-    if (tid == 0 && G.cl.block_rank() == 0) {
+    bad = __syncthreads_or(bad) != 0;
+    if (tid == 0 && blk == 0) {
         GlobalState* gs = sv.g_state;
         gs->epoch += 1;                              // cached match nodes of every slot are stale now
-        gs->used = (int)min(sh.used, (unsigned long long)sv.g_cap);
-        gs->live += sh.live;
-        gs->status = sh.status;
+        gs->used = used;
+        gs->live += live;
+        gs->status |= (full ? SD_STATUS_GLOBAL_FULL : 0) | (bad ? SD_STATUS_BAD_TOKEN : 0);
         gs->tokens += tokens_done;
     }
 }
@@ -429,8 +669,11 @@ extern "C" int sd_append(sd_store* s, int32_t n, const int32_t* d_slot, const in
     cudaStream_t st = (cudaStream_t)stream;
     SD_CUDA_OK(cudaEventRecord(s->ev_fork, st));
     SD_CUDA_OK(cudaStreamWaitEvent(s->aux, s->ev_fork, 0));
-    global_insert_kernel<<<GI_CTAS, GI_THREADS, 0, s->aux>>>(*s, n, d_slot, d_offsets, d_tokens);
-    SD_CUDA_OK(cudaGetLastError());
+    int tok_bits = 1;
+    while (tok_bits < 31 && (1 << tok_bits) < s->V) ++tok_bits;
+    void* args[] = {(void*)s, (void*)&n, (void*)&d_slot, (void*)&d_offsets, (void*)&d_tokens, (void*)&tok_bits};
+    SD_CUDA_OK(cudaFuncSetAttribute(global_insert_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(GiShared)));
+    SD_CUDA_OK(cudaLaunchCooperativeKernel((void*)global_insert_kernel, dim3(GI_BLOCKS), dim3(GI_THREADS), args, sizeof(GiShared), s->aux));
     SD_CUDA_OK(cudaEventRecord(s->ev_join, s->aux));
     append_kernel<<<(unsigned)n, APPEND_THREADS, 0, st>>>(*s, d_slot, d_offsets, d_tokens, d_reset);
     SD_CUDA_OK(cudaGetLastError());

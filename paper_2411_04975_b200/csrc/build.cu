@@ -17,6 +17,8 @@
 #include <cooperative_groups.h>
 
 #include "append_core.cuh"
+#include "global_insert.cuh"
+#include "suffix_order.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -397,161 +399,24 @@ int corpus_sort(CorpusSort& A, cudaStream_t st) {
 }
 
 // Suffix order of sequences that are sorted one by one (the trees of different requests share
-// nothing, so no suffix of one request is ever compared with a suffix of another): one block per
-// sequence, everything in shared memory, by prefix doubling.  After a round every suffix has the rank of its
-// first k tokens, and the order by the tokens behind those is the current order moved k places back, so a
-// round only has to sort by rank, stably: one or two radix passes of 7 bits.  A last round that adds fewer
-// than k tokens looks at an overlapping window.  A rank also tells whether the sequence ends right
-// behind the k tokens, so that suffixes of equal rank either all go on or are equal altogether, and the ones that
-// have nothing k places on may take any place.  Order: by the first D tokens, a suffix that ends earlier before its
-// extensions.  Bound by the latency of a pass (one block: barriers, and 32 items per warp and step ranked by
-// ballots).  (A bitonic sort that compared tokens took 78 - 91 stages: 83 us for 4 x 4,096 tokens, 390 for 64 x 8,192.)
-constexpr int BS_THREADS = 1024;
-constexpr int BS_WARPS = BS_THREADS / 32;
-constexpr int BS_MAX_LEN = 16384;              // longest sequence (two passes of 7 bits per round; 112 KB)
-constexpr int BS_BITS = 7;
-constexpr int BS_BINS = 1 << BS_BITS;
-constexpr int BS_ROW = BS_BINS + 1;            // (rows of 128 counters put the eight threads that add up a digit on one bank: a sort of 4 x 4,096 tokens took 60 us, 49 now)
-
-// ITEMS per thread: sequences of up to 1,024 x ITEMS tokens
+// nothing, so no suffix of one request is ever compared with a suffix of another): one block per sequence.
 template <int ITEMS>
 __global__ void __launch_bounds__(BS_THREADS, ITEMS <= 4 ? 2 : 1)
 block_suffix_sort_kernel(const int32_t* tok, const int64_t* seq_off, int V, int tok_bits, int D, uint32_t* sa_out) {
     extern __shared__ __align__(16) unsigned char bs_smem[];
     __shared__ int wsum[BS_WARPS];
-    int (*hist)[BS_ROW] = reinterpret_cast<int (*)[BS_ROW]>(bs_smem);                // [BS_WARPS][BS_ROW]
-    unsigned short* const rank = reinterpret_cast<unsigned short*>(bs_smem + sizeof(int) * BS_WARPS * BS_ROW);
-    unsigned short* cur = rank + BS_THREADS * ITEMS;                                // the order so far
-    unsigned short* nxt = cur + BS_THREADS * ITEMS;
     const i64 b = seq_off[blockIdx.x];
     const int n = (int)(seq_off[blockIdx.x + 1] - b), first_tok = (int)blockIdx.x * V;
-    const int tid = threadIdx.x, lane = tid & 31, wib = tid >> 5;
     if (n <= 0) return;
     const int32_t* const t = tok + b;
-    const unsigned lt = (1u << lane) - 1u;
-    const int p0 = wib * 32 * ITEMS + lane;                     // a warp's places are consecutive, 32 per step
-
-    // one stable pass: `val` of every place goes by bits [shift, shift + 7) of its key
-    unsigned short val[ITEMS];
-    auto pass = [&](int shift, auto key_of) {
-        for (int k = lane; k < BS_BINS; k += 32) hist[wib][k] = 0;
-        __syncwarp();
-        int at[ITEMS];                                          // digit, and place among the warp's items of that digit
-#pragma unroll
-        for (int u = 0; u < ITEMS; ++u) {
-            const bool in = p0 + u * 32 < n;
-            const unsigned active = __ballot_sync(0xffffffffu, in);
-            at[u] = 0;
-            if (!active) continue;
-            const int digit = in ? (int)((key_of(val[u]) >> shift) & (BS_BINS - 1)) : 0;
-            unsigned peers = active;
-#pragma unroll
-            for (int k = 0; k < BS_BITS; ++k) {
-                const unsigned m = __ballot_sync(0xffffffffu, (digit >> k) & 1);
-                peers &= ((digit >> k) & 1) ? m : ~m;
-            }
-            int base = 0;
-            if (in) base = hist[wib][digit];
-            __syncwarp();
-            if (in && (peers & lt) == 0u) hist[wib][digit] = base + __popc(peers);
-            __syncwarp();
-            at[u] = digit | ((base + __popc(peers & lt)) << BS_BITS);
-        }
-        __syncthreads();
-        {
-            // counts to first places, in the order (digit, warp): a thread takes four warps of one digit
-            const int digit = tid >> 3, w0 = (tid & 7) * 4;
-            int c[4], sum = 0;
-#pragma unroll
-            for (int q = 0; q < 4; ++q) { c[q] = hist[w0 + q][digit]; sum += c[q]; }
-            int inc = sum;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const int y = __shfl_up_sync(0xffffffffu, inc, o);
-                if (lane >= o) inc += y;
-            }
-            if (lane == 31) wsum[wib] = inc;
-            __syncthreads();
-            int before = lane < wib ? wsum[lane] : 0;
-            before = (int)__reduce_add_sync(0xffffffffu, (unsigned)before) + inc - sum;
-#pragma unroll
-            for (int q = 0; q < 4; ++q) { hist[w0 + q][digit] = before; before += c[q]; }
-        }
-        __syncthreads();
-#pragma unroll
-        for (int u = 0; u < ITEMS; ++u)
-            if (p0 + u * 32 < n) nxt[hist[wib][at[u] & (BS_BINS - 1)] + (at[u] >> BS_BITS)] = val[u];
-        __syncthreads();
-        unsigned short* const x = cur; cur = nxt; nxt = x;
-    };
-    auto load = [&]() {
-#pragma unroll
-        for (int u = 0; u < ITEMS; ++u) val[u] = p0 + u * 32 < n ? cur[p0 + u * 32] : 0;
-    };
-    // ranks (from 0) of the order `cur`, a new one where `differs` from the suffix before; returns their number
-    auto rerank = [&](auto differs) -> int {
-        load();
-        unsigned flags[ITEMS];
-        int mine = 0;
-#pragma unroll
-        for (int u = 0; u < ITEMS; ++u) {
-            const int p = p0 + u * 32;
-            flags[u] = __ballot_sync(0xffffffffu, p < n && (p == 0 || differs((int)val[u], (int)cur[p - 1])));
-            mine += __popc(flags[u]);
-        }
-        if (lane == 0) wsum[wib] = mine;
-        __syncthreads();                                        // all old ranks have been read
-        const int c = wsum[lane];
-        int r = (int)__reduce_add_sync(0xffffffffu, lane < wib ? (unsigned)c : 0u) - 1;
-        const int all = (int)__reduce_add_sync(0xffffffffu, (unsigned)c);
-#pragma unroll
-        for (int u = 0; u < ITEMS; ++u) {
-            if (p0 + u * 32 < n) rank[val[u]] = (unsigned short)(r + __popc(flags[u] & (lt | (1u << lane))));
-            r += __popc(flags[u]);
-        }
-        __syncthreads();
-        return all;
-    };
-
-    // ---- by the first token, and whether it is the last one
-    auto token_key = [&](int i) -> unsigned { return ((unsigned)(t[i] - first_tok) << 1) | (i + 1 < n ? 1u : 0u); };
-#pragma unroll
-    for (int u = 0; u < ITEMS; ++u) val[u] = (unsigned short)(p0 + u * 32);
-    for (int shift = 0; shift < tok_bits + 1; shift += BS_BITS) {
-        if (shift > 0) load();
-        pass(shift, [&](int i) { return token_key(i); });
-    }
-    for (int k = 1, off; k < D; k += off) {
-        off = min(k, D - k);
-        // ranks of the first k tokens
-        int ranks;
-        if (k == 1) ranks = rerank([&](int i, int h) { return token_key(i) != token_key(h); });
-        else {
-            const int o = k >> 1;                               // (every round but the last doubles)
-            ranks = rerank([&](int i, int h) {
-                return rank[i] != rank[h] || (i + o < n ? (int)rank[i + o] : -1) != (h + o < n ? (int)rank[h + o] : -1);
-            });
-        }
-        if (ranks == n) break;                                  // no two alike: the order is final
-        // the order by what follows `off` places on, then by rank
-        load();
-#pragma unroll
-        for (int u = 0; u < ITEMS; ++u) {
-            const int q = val[u];
-            val[u] = (unsigned short)(q >= off ? q - off : n - min(off, n) + q);
-        }
-        __syncthreads();
-        pass(0, [&](int i) { return (unsigned)rank[i]; });
-        if (ranks > BS_BINS) { load(); __syncthreads(); pass(BS_BITS, [&](int i) { return (unsigned)rank[i]; }); }
-    }
-    load();
-#pragma unroll
-    for (int u = 0; u < ITEMS; ++u) if (p0 + u * 32 < n) sa_out[b + p0 + u * 32] = (uint32_t)(b + val[u]);
+    const unsigned short* const order = block_suffix_order<ITEMS>(
+        bs_smem, wsum, n, tok_bits, D, [&](int i) { return t[i] - first_tok; }, [](int) { return 0; }, [&](int) { return n; });
+    for (int p = threadIdx.x; p < n; p += BS_THREADS) sa_out[b + p] = (uint32_t)(b + order[p]);
 }
 
 template <int ITEMS>
 int block_suffix_sort(const int32_t* tok, const int64_t* seq_off, int n_seqs, int V, int tok_bits, int D, uint32_t* sa, cudaStream_t st) {
-    const int smem = (int)(sizeof(int) * BS_WARPS * BS_ROW + 3 * sizeof(unsigned short) * BS_THREADS * ITEMS);
+    constexpr int smem = block_order_smem<ITEMS>();
     if (smem > 48 * 1024)
         SD_CUDA_OK(cudaFuncSetAttribute(block_suffix_sort_kernel<ITEMS>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
     block_suffix_sort_kernel<ITEMS><<<(unsigned)n_seqs, BS_THREADS, smem, st>>>(tok, seq_off, V, tok_bits, D, sa);
@@ -1252,7 +1117,7 @@ static bool store_alloc(sd_store* s, T** out, long long count) {
 static void store_release(sd_store* s, cudaStream_t st) {
     if (!s) return;
     cudaStreamSynchronize(st);
-    void* const own[] = {s->g_ent, s->g_root, s->g_state, s->s_ent, s->s_root, s->s_text, s->s_state};
+    void* const own[] = {s->g_ent, s->g_root, s->g_state, s->gi, s->s_ent, s->s_root, s->s_text, s->s_state};
     for (void* p : own) sd_device_free(p);
     if (s->ws) {
         for (int k = 0; k < 48; ++k) sd_device_free(s->ws->ptr[k]);
@@ -1375,7 +1240,7 @@ extern "C" int sd_build(const sd_build_params* p, const int32_t* d_corpus, const
     s->spn = p->slot_pool_nodes > 0 ? p->slot_pool_nodes : 2ll * s->T * D;
     if (s->spn >= (1ll << 31) - 2) { delete s; return SD_ERR_INVALID_ARG; }
 
-    bool ok = store_alloc(s, &s->g_root, s->V) && store_alloc(s, &s->g_state, 1) &&
+    bool ok = store_alloc(s, &s->g_root, s->V) && store_alloc(s, &s->g_state, 1) && store_alloc(s, &s->gi, 1) &&
               store_alloc(s, &s->s_ent, (i64)s->R * s->spn) && store_alloc(s, &s->s_root, (i64)s->R * s->V) &&
               store_alloc(s, &s->s_text, (i64)s->R * s->T) && store_alloc(s, &s->s_state, s->R);
     if (!ok) { store_release(s, st); return SD_ERR_NOMEM; }

@@ -73,6 +73,7 @@ struct sd_store {
     long long g_cap;
     int32_t* g_root;          // [V]
     GlobalState* g_state;
+    struct GiScratch* gi;     // of the online insert into the global tree
     // per-request trees
     int4* s_ent;              // [R][spn]
     long long spn;
