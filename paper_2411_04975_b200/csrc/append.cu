@@ -28,10 +28,10 @@ namespace {
 //   4. every parent's entry gets its new run, in the place it has now if its own run was merged, too.
 // Six grid barriers and no rounds: the time is that of the walk (dependent loads) or of the sort, whichever is
 // longer, and of the sweeps over the tiles.  (Level by level with an election per parent and round, by a cluster of 8
-// blocks: 150 us for the 1,000 tokens that three finished outputs bring, MEASURED now.)
+// blocks: 150 us for 352 paths, 58 for 91; now 56 and 42, of which the walk 16 and 12, grouping 8 and 6.)
 // The nodes that a batch adds need the pool to hold them all: a batch that does not fit raises counts only.
 constexpr int GI_BLOCKS = 24;
-constexpr int GI_THREADS = BS_THREADS;
+constexpr int GI_THREADS = 512;               // (1,024 leave 64 registers: the sweeps spill)
 constexpr int GI_REAL = GI_MAX - SD_MAX_DEPTH;                   // start positions per pass
 constexpr int GI_ITEMS = 256;
 constexpr int GI_CELLS = 2 * GI_MAX;
@@ -44,7 +44,7 @@ struct GiItems {
 };
 
 struct GiSort {                               // block 0, while it sorts
-    unsigned char order[block_order_smem<GI_MAX / BS_THREADS>()];
+    unsigned char order[block_order_smem<GI_THREADS, GI_MAX / GI_THREADS>()];
     int tok[GI_MAX];
     unsigned short begin[GI_MAX], end[GI_MAX], sa[GI_MAX];
 };
@@ -56,10 +56,15 @@ struct GiTable {                              // block 0, while it groups
     int n_big;
 };
 constexpr int GI_WARP_TILES = (GI_TILES + GI_BLOCKS - 2) / (GI_BLOCKS - 1);                 // tiles per block, a warp each
+struct GiSweep {                              // the other blocks
+    int2 state[GI_WARP_TILES][GI_TILE][32];   // state from behind, by suffix of a tile and depth
+    int f[GI_TILES][32], e[GI_TILES][32];     // of all tiles; f then r
+    int s[GI_TILES], ev[GI_TILES];
+};
 union GiShared {
     GiSort sort;
     GiTable table;
-    int2 state[GI_WARP_TILES][GI_TILE][32];   // the other blocks: state from behind, by suffix of the tile and depth
+    GiSweep sweep;
 };
 
 // exclusive sum over the block's threads, the total in `all`
@@ -74,7 +79,7 @@ __device__ __forceinline__ int gi_block_scan(int v, int* wsum, int tid, int& all
     }
     if (lane == 31) wsum[wib] = inc;
     __syncthreads();
-    const int c = wsum[lane];
+    const int c = lane < GI_THREADS / 32 ? wsum[lane] : 0;
     const int before = (int)__reduce_add_sync(FULL, lane < wib ? (unsigned)c : 0u);
     all = (int)__reduce_add_sync(FULL, (unsigned)c);
     __syncthreads();
@@ -163,32 +168,44 @@ __device__ void gi_walk(const sd_store& sv, GiScratch* X, const GiItems& I, cons
 }
 
 // 2. The sweeps: a warp per tile of GI_TILE suffixes, a lane per depth.  A lane also looks after the tile's suffix of its number.
-// (Functions of their own: in one with everything else they spilled, 36 and 38 us instead of MEASURED.)
+// What a sweep waits for are reads of what other blocks have just written (about 1,500 cycles behind a grid barrier), so
+// everything about a tile's suffixes is read once and kept in registers, and what the tiles leave for one another comes
+// into shared memory in one go.
 struct GiOwn {
     int lnv;                                  // common prefix, length, levels that exist: packed
     int at;                                   // start position
     int below, event;                         // new nodes whose parent is new, whose parent exists
+    int p, q, ptok, xtok;                     // of the event: the parent, the node above it, the parent's token and its own
+    int tok[GI_TILE];                         // token of this lane's depth, by suffix of the tile
 };
 
-__device__ __forceinline__ GiOwn gi_own(const GiScratch* X, int j0, int mm, int lane) {
-    GiOwn o{0, 0, 0, 0};
+__device__ __forceinline__ void gi_own(GiOwn& o, const GiScratch* X, int j0, int mm, int lane) {
+    const unsigned FULL = 0xffffffffu;
+    o.lnv = 0; o.at = 0; o.below = 0; o.event = 0; o.p = -1; o.q = -1; o.ptok = -1; o.xtok = 0;
     if (lane < mm) {
         o.at = X->sa[j0 + lane];
         const int l = X->lcp[j0 + lane], n = X->len[j0 + lane], v = X->v[o.at];
+        o.p = X->p[o.at]; o.q = X->q[o.at];
         o.lnv = l | (n << 8) | (v << 16);
         o.below = max(0, n - max(l, v + 1));
         o.event = l <= v && v < n ? 1 : 0;
     }
-    return o;
+#pragma unroll
+    for (int i = 0; i < GI_TILE; ++i) {
+        const int at = __shfl_sync(FULL, o.at, i), x = __shfl_sync(FULL, o.lnv, i);
+        o.tok[i] = lane < ((x >> 8) & 255) ? X->tok[at + lane] : 0;
+        const int v = x >> 16, t1 = __shfl_sync(FULL, o.tok[i], min(v, 31)), t0 = __shfl_sync(FULL, o.tok[i], max(v - 1, 0));
+        if (lane == i) { o.xtok = t1; o.ptok = v > 0 ? t0 : -1; }
+    }
 }
 
 // what the tile does to the state from behind: children counted up to the first reset, and where that is
-__device__ __noinline__ void gi_sweep_tile(GiScratch* X, int t, int m, int lane) {
+__device__ __forceinline__ void gi_sweep_tile(GiScratch* X, const GiOwn& o, int t, int m, int lane) {
     const unsigned FULL = 0xffffffffu;
     const int j0 = t * GI_TILE, mm = min(GI_TILE, m - j0), d = lane + 1;
-    const GiOwn o = gi_own(X, j0, mm, lane);
     int cnt = 0, first = m;
     bool seen = false;
+#pragma unroll 1
     for (int i = 0; i < mm; ++i) {
         const int x = __shfl_sync(FULL, o.lnv, i), l = x & 255, len = (x >> 8) & 255;
         if (!seen) {
@@ -202,44 +219,38 @@ __device__ __noinline__ void gi_sweep_tile(GiScratch* X, int t, int m, int lane)
     if (lane == 0) { X->s[t] = sb; X->ev[t] = se; }
 }
 
-// sums over the tiles in front of tile t (t = tiles: all)
-__device__ __forceinline__ void gi_sums(const GiScratch* X, int t, int lane, int& s, int& ev) {
-    int a = 0, b = 0;
-    for (int q = lane; q < t; q += 32) { a += X->s[q]; b += X->ev[q]; }
-    s = (int)__reduce_add_sync(0xffffffffu, (unsigned)a);
-    ev = (int)__reduce_add_sync(0xffffffffu, (unsigned)b);
+// sums over the first t tiles
+__device__ __forceinline__ void gi_sums(const int* s, const int* ev, int t, int lane, int& a, int& b) {
+    a = 0; b = 0;
+    for (int q = lane; q < t; q += 32) { a += s[q]; b += ev[q]; }
+    a = (int)__reduce_add_sync(0xffffffffu, (unsigned)a);
+    b = (int)__reduce_add_sync(0xffffffffu, (unsigned)b);
 }
 
-// from behind: the events, the end of the last run opened per depth, and the state at every suffix
-__device__ __noinline__ void gi_sweep_runs(GiScratch* X, int2 (*state)[32], int t, int tiles, int m, int lane) {
+// from behind: the events, the end of the last run opened per depth, and the state at every suffix.  s_own: new nodes with a
+// new parent in front of the lane's suffix.
+__device__ __forceinline__ void gi_sweep_runs(GiScratch* X, GiSweep& sw, const GiOwn& o, int wib, int t, int tiles, int m, int lane,
+                                              int& s_own) {
     const unsigned FULL = 0xffffffffu;
     const int j0 = t * GI_TILE, mm = min(GI_TILE, m - j0), d = lane + 1;
-    const GiOwn o = gi_own(X, j0, mm, lane);
     int s_at, ev_at;
-    gi_sums(X, t, lane, s_at, ev_at);
+    gi_sums(sw.s, sw.ev, t, lane, s_at, ev_at);
     int is = o.below, ie = o.event;
 #pragma unroll
     for (int k = 1; k < GI_TILE; k <<= 1) {
         const int a = __shfl_up_sync(FULL, is, k), b = __shfl_up_sync(FULL, ie, k);
         if (lane >= k) { is += a; ie += b; }
     }
-    const int s_own = s_at + is - o.below, ev_own = ev_at + ie - o.event;
-    if (o.event) {
-        const int v = o.lnv >> 16;
-        X->ev_p[ev_own] = X->p[o.at]; X->ev_q[ev_own] = X->q[o.at];
-        X->ev_ptok[ev_own] = v > 0 ? X->tok[o.at + v - 1] : -1;
-        X->ev_tok[ev_own] = X->tok[o.at + v];
-    }
+    s_own = s_at + is - o.below;
+    const int ev_own = ev_at + ie - o.event;
+    if (o.event) { X->ev_p[ev_own] = o.p; X->ev_q[ev_own] = o.q; X->ev_ptok[ev_own] = o.ptok; X->ev_tok[ev_own] = o.xtok; }
     int F = 0, e = m;
-    bool seen = false;
-#pragma unroll 8
     for (int q = t + 1; q < tiles; ++q) {
-        const int fq = X->f[q][lane], eq = X->e[q][lane];
-        if (!seen) {
-            F += fq & 0x7fffffff;
-            if (fq < 0) { seen = true; e = eq; }
-        }
+        const int fq = sw.f[q][lane];
+        F += fq & 0x7fffffff;
+        if (fq < 0) { e = sw.e[q][lane]; break; }
     }
+    __syncwarp();
     int g = F;
 #pragma unroll
     for (int k = 1; k < 32; k <<= 1) {
@@ -248,10 +259,11 @@ __device__ __noinline__ void gi_sweep_runs(GiScratch* X, int2 (*state)[32], int 
     }
     g -= F;                                                      // G: children of the levels above
     int R = -1;
+#pragma unroll 1
     for (int i = mm - 1; i >= 0; --i) {
         const int x = __shfl_sync(FULL, o.lnv, i), l = x & 255, len = (x >> 8) & 255, v = x >> 16;
         const int si = __shfl_sync(FULL, s_own, i), ei = __shfl_sync(FULL, ev_own, i);
-        state[i][lane] = make_int2(g, e);
+        sw.state[wib][i][lane] = make_int2(g, e);
         const int up = __shfl_down_sync(FULL, g, 1), gv = __shfl_sync(FULL, g, min(v, 31));
         const int kids = (lane == 31 ? 0 : up - g) + (d < len ? 1 : 0);
         const int run = si + d - max(l, v + 1) + g - gv;
@@ -264,35 +276,20 @@ __device__ __noinline__ void gi_sweep_runs(GiScratch* X, int2 (*state)[32], int 
     X->r[t][lane] = R;
 }
 
-// from the front: the new nodes below the events, from entry `used` on
-__device__ __noinline__ void gi_sweep_emit(const GiScratch* X, const int2 (*state)[32], int4* ent, int used, int t, int m, int lane) {
+// from the front: the new nodes below the events, from entry `used` on (sw.f holds what the tiles left in r)
+__device__ __forceinline__ void gi_sweep_emit(const GiSweep& sw, const GiOwn& o, int4* ent, int used, int wib, int t, int m, int lane,
+                                              int s_own) {
     const unsigned FULL = 0xffffffffu;
     const int j0 = t * GI_TILE, mm = min(GI_TILE, m - j0), d = lane + 1;
-    const GiOwn o = gi_own(X, j0, mm, lane);
-    int s_at, ev_at;
-    gi_sums(X, t, lane, s_at, ev_at);
-    int is = o.below;
-#pragma unroll
-    for (int k = 1; k < GI_TILE; k <<= 1) {
-        const int a = __shfl_up_sync(FULL, is, k);
-        if (lane >= k) is += a;
-    }
-    const int s_own = s_at + is - o.below;
-    int tok[GI_TILE];
-#pragma unroll
-    for (int i = 0; i < GI_TILE; ++i) {
-        const int at = __shfl_sync(FULL, o.at, i), len = (__shfl_sync(FULL, o.lnv, i) >> 8) & 255;
-        tok[i] = lane < len ? X->tok[at + lane] : 0;
-    }
     int R = -1;
-#pragma unroll 8
-    for (int q = 0; q < t; ++q) { const int y = X->r[q][lane]; if (y >= 0) R = y; }
+    for (int q = t - 1; q >= 0 && R < 0; --q) R = sw.f[q][lane];
+    __syncwarp();
 #pragma unroll
     for (int i = 0; i < GI_TILE; ++i) {
         if (i >= mm) break;
         const int x = __shfl_sync(FULL, o.lnv, i), l = x & 255, len = (x >> 8) & 255, v = x >> 16;
         const int si = __shfl_sync(FULL, s_own, i);
-        const int2 ge = state[i][lane];
+        const int2 ge = sw.state[wib][i][lane];
         const int up = __shfl_down_sync(FULL, ge.x, 1), gv = __shfl_sync(FULL, ge.x, min(v, 31));
         const int later = lane == 31 ? 0 : up - ge.x, kids = later + (d < len ? 1 : 0);
         const int run = si + d - max(l, v + 1) + ge.x - gv;
@@ -301,12 +298,12 @@ __device__ __noinline__ void gi_sweep_emit(const GiScratch* X, const int2 (*stat
         const int place = __shfl_up_sync(FULL, opens ? run : R - 1 - later, 1);
         if (opens) R = run + kids;
         if (opens && !(l <= v && d == v + 1))
-            ent[used + place] = make_int4(tok[i], ge.y - (j0 + i), kids > 0 ? used + run : 0, kids > 0 ? (int)((unsigned)kids | RUN_STATIC) : 0);
+            ent[used + place] = make_int4(o.tok[i], ge.y - (j0 + i), kids > 0 ? used + run : 0, kids > 0 ? (int)((unsigned)kids | RUN_STATIC) : 0);
     }
 }
 
 // 3. the events by parent (one block): every parent's new children by token, its run's new place
-__device__ __noinline__ void gi_group(const sd_store& sv, GiScratch* X, GiTable& tb, int* wsum, int used, int s_all, int ev_all, int tid) {
+__device__ __forceinline__ void gi_group(const sd_store& sv, GiScratch* X, GiTable& tb, int* wsum, int used, int s_all, int ev_all, int tid) {
     int4* const ent = sv.g_ent;
     for (int i = tid; i < GI_CELLS; i += GI_THREADS) { tb.key[i] = 0; tb.cnt[i] = 0; }
     if (tid == 0) tb.n_big = 0;
@@ -358,37 +355,39 @@ __device__ __noinline__ void gi_group(const sd_store& sv, GiScratch* X, GiTable&
             for (int q = 0; q < k; ++q) rank += tb.tok[p + q] < x[u] ? 1 : 0;
             X->m_tok[p + rank] = x[u]; X->m_ev[p + rank] = tid + u * GI_THREADS;
         }
-    GiGroup gr[CELLS];
-    int size[CELLS], mine_size = 0;
-#pragma unroll
+    __syncthreads();                                             // (the counts have been read: they become sizes)
+    int mine_size = 0;
+#pragma unroll 1
     for (int u = 0; u < CELLS; ++u) {
         const int c = tid * CELLS + u, k = tb.cnt[c];
-        size[u] = 0;
-        gr[u].k = k;
-        if (k > 0) {
-            GiGroup& G = gr[u];
-            G.first = tb.at[c] & 0xffff;
-            const int e = tb.ev[G.first], q = X->ev_q[e];
-            G.parent = tb.key[c] - 2; G.parent_tok = X->ev_ptok[e];
-            G.cb = 0; G.n = 0; G.above = -1;
-            if (G.parent >= 0) {
-                const int4 pe = __ldcg(ent + G.parent);
-                G.cb = pe.z; G.n = (int)((unsigned)pe.w & RUN_COUNT_MASK);
-                if ((uint32_t)(G.n + k) > sd_run_capacity((uint32_t)pe.w)) size[u] = (int)sd_pow2ceil((uint32_t)(G.n + k));
-                if (q >= 0) { const int qc = cell_of(q + 2, false); if (qc >= 0) G.above = tb.at[qc] >> 16; }
-            } else size[u] = k;
-            if (G.n > GI_BIG || k > GI_BIG) X->big[atomicAdd(&tb.n_big, 1)] = tb.at[c] >> 16;
-        }
-        mine_size += size[u];
+        if (k == 0) continue;
+        GiGroup G;
+        const int id = tb.at[c] >> 16;
+        G.first = tb.at[c] & 0xffff; G.k = k;
+        const int e = tb.ev[G.first], q = X->ev_q[e];
+        G.parent = tb.key[c] - 2; G.parent_tok = X->ev_ptok[e];
+        G.cb = 0; G.n = 0; G.above = -1; G.base = 0;
+        int size = 0;
+        if (G.parent >= 0) {
+            const int4 pe = __ldcg(ent + G.parent);
+            G.cb = pe.z; G.n = (int)((unsigned)pe.w & RUN_COUNT_MASK);
+            if ((uint32_t)(G.n + k) > sd_run_capacity((uint32_t)pe.w)) size = (int)sd_pow2ceil((uint32_t)(G.n + k));
+            if (q >= 0) { const int qc = cell_of(q + 2, false); if (qc >= 0) G.above = tb.at[qc] >> 16; }
+        } else size = k;
+        if (G.n > GI_BIG || k > GI_BIG) X->big[atomicAdd(&tb.n_big, 1)] = id;
+        X->group[id] = G;
+        tb.cnt[c] = size;                                        // (only this thread looks at this cell's count)
+        mine_size += size;
     }
     int entries, place = used + s_all + gi_block_scan(mine_size, wsum, tid, entries);
-#pragma unroll
-    for (int u = 0; u < CELLS; ++u)
-        if (gr[u].k > 0) {
-            gr[u].base = size[u] > 0 ? place : gr[u].cb;
-            X->group[tb.at[tid * CELLS + u] >> 16] = gr[u];
-            place += size[u];
-        }
+#pragma unroll 1
+    for (int u = 0; u < CELLS; ++u) {
+        const int c = tid * CELLS + u, size = tb.cnt[c];
+        if (tb.key[c] == 0) continue;
+        GiGroup* const G = &X->group[tb.at[c] >> 16];
+        G->base = size > 0 ? place : G->cb;
+        place += size;
+    }
     if (tid == 0) {
         X->n_groups = n_groups; X->n_big = tb.n_big; X->entries = entries;
         X->fits = (long long)used + s_all + entries <= sv.g_cap ? 1 : 0;
@@ -522,8 +521,9 @@ global_insert_kernel(sd_store sv, int n, const int32_t* d_slot, const int64_t* d
                 auto token = [&](int i) { return so.tok[i]; };
                 auto begin = [&](int i) { return (int)so.begin[i]; };
                 auto end = [&](int i) { return (int)so.end[i]; };
-                const unsigned short* const order = M <= BS_THREADS ? block_suffix_order<1>(so.order, wsum, M, tok_bits, D, token, begin, end)
-                                                                    : block_suffix_order<2>(so.order, wsum, M, tok_bits, D, token, begin, end);
+                const unsigned short* order;
+                if (M <= GI_THREADS) order = block_suffix_order<GI_THREADS, 1>(so.order, wsum, M, tok_bits, D, token, begin, end);
+                else order = block_suffix_order<GI_THREADS, GI_MAX / GI_THREADS>(so.order, wsum, M, tok_bits, D, token, begin, end);
                 // start positions only
                 int at = 0;
                 for (int i0 = 0; i0 < M; i0 += GI_THREADS) {
@@ -545,21 +545,42 @@ global_insert_kernel(sd_store sv, int n, const int32_t* d_slot, const int64_t* d
                     X->lcp[j] = l; X->len[j] = len;
                 }
             } else {
-                gi_walk(sv, X, I, d_tokens, c0, m, ((blk - 1) * GI_THREADS + tid) / APP_LANES, (GI_BLOCKS - 1) * GI_THREADS / APP_LANES, lane);
+                gi_walk(sv, X, I, d_tokens, c0, m, tid / APP_LANES * (GI_BLOCKS - 1) + blk - 1,
+                        (GI_BLOCKS - 1) * GI_THREADS / APP_LANES, lane);
             }
             grid.sync();
             // ---------------- 2. the sweeps, a warp per tile
             const int tiles = (m + GI_TILE - 1) / GI_TILE, t = (blk - 1) + wib * (GI_BLOCKS - 1);
             const bool sweeps = blk > 0 && t < tiles;
-            if (sweeps) gi_sweep_tile(X, t, m, lane);
+            GiOwn own;
+            int s_own = 0;
+            if (sweeps) {
+                gi_own(own, X, t * GI_TILE, min(GI_TILE, m - t * GI_TILE), lane);
+                gi_sweep_tile(X, own, t, m, lane);
+            }
             grid.sync();
             int s_all, ev_all;
-            gi_sums(X, tiles, lane, s_all, ev_all);
-            if (sweeps) gi_sweep_runs(X, sh.state[wib], t, tiles, m, lane);
+            if (blk == 0) gi_sums(X->s, X->ev, tiles, lane, s_all, ev_all);
+            else {
+                GiSweep& sw = sh.sweep;
+                for (int i = tid; i < tiles * 8; i += GI_THREADS) {                 // (four depths at a time)
+                    reinterpret_cast<int4*>(sw.f)[i] = reinterpret_cast<const int4*>(X->f)[i];
+                    reinterpret_cast<int4*>(sw.e)[i] = reinterpret_cast<const int4*>(X->e)[i];
+                }
+                for (int i = tid; i < tiles; i += GI_THREADS) { sw.s[i] = X->s[i]; sw.ev[i] = X->ev[i]; }
+                __syncthreads();
+                gi_sums(sw.s, sw.ev, tiles, lane, s_all, ev_all);
+                if (sweeps) gi_sweep_runs(X, sw, own, wib, t, tiles, m, lane, s_own);
+            }
             grid.sync();
             // ---------------- 3. grouping (block 0) while the others write the new nodes below the events
             if (blk == 0) gi_group(sv, X, sh.table, wsum, used, s_all, ev_all, tid);
-            else if (sweeps && (long long)used + s_all <= sv.g_cap) gi_sweep_emit(X, sh.state[wib], ent, used, t, m, lane);
+            else {
+                GiSweep& sw = sh.sweep;
+                for (int i = tid; i < tiles * 8; i += GI_THREADS) reinterpret_cast<int4*>(sw.f)[i] = reinterpret_cast<const int4*>(X->r)[i];
+                __syncthreads();
+                if (sweeps && (long long)used + s_all <= sv.g_cap) gi_sweep_emit(sw, own, ent, used, wib, t, m, lane, s_own);
+            }
             grid.sync();
             // ---------------- merges: a warp per parent, a block per parent with a long run
             const int n_groups = X->n_groups;

@@ -404,19 +404,19 @@ template <int ITEMS>
 __global__ void __launch_bounds__(BS_THREADS, ITEMS <= 4 ? 2 : 1)
 block_suffix_sort_kernel(const int32_t* tok, const int64_t* seq_off, int V, int tok_bits, int D, uint32_t* sa_out) {
     extern __shared__ __align__(16) unsigned char bs_smem[];
-    __shared__ int wsum[BS_WARPS];
+    __shared__ int wsum[BS_THREADS / 32];
     const i64 b = seq_off[blockIdx.x];
     const int n = (int)(seq_off[blockIdx.x + 1] - b), first_tok = (int)blockIdx.x * V;
     if (n <= 0) return;
     const int32_t* const t = tok + b;
-    const unsigned short* const order = block_suffix_order<ITEMS>(
+    const unsigned short* const order = block_suffix_order<BS_THREADS, ITEMS>(
         bs_smem, wsum, n, tok_bits, D, [&](int i) { return t[i] - first_tok; }, [](int) { return 0; }, [&](int) { return n; });
     for (int p = threadIdx.x; p < n; p += BS_THREADS) sa_out[b + p] = (uint32_t)(b + order[p]);
 }
 
 template <int ITEMS>
 int block_suffix_sort(const int32_t* tok, const int64_t* seq_off, int n_seqs, int V, int tok_bits, int D, uint32_t* sa, cudaStream_t st) {
-    constexpr int smem = block_order_smem<ITEMS>();
+    constexpr int smem = block_order_smem<BS_THREADS, ITEMS>();
     if (smem > 48 * 1024)
         SD_CUDA_OK(cudaFuncSetAttribute(block_suffix_sort_kernel<ITEMS>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
     block_suffix_sort_kernel<ITEMS><<<(unsigned)n_seqs, BS_THREADS, smem, st>>>(tok, seq_off, V, tok_bits, D, sa);

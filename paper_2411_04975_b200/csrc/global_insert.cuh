@@ -16,7 +16,7 @@ struct GiGroup {
     int base;                                 // where the run goes (cb: it stays)
 };
 
-struct GiScratch {
+struct __align__(16) GiScratch {
     int tok[GI_MAX];                          // by position
     int v[GI_MAX], p[GI_MAX], q[GI_MAX];      // by start position: levels that exist, the node there, the node above that
     int sa[GI_MAX], lcp[GI_MAX], len[GI_MAX]; // by place in the suffix order

@@ -15,25 +15,26 @@ namespace {
 // extensions.  Bound by the latency of a pass (one block: barriers, and 32 items per warp and step ranked by
 // ballots).  (A bitonic sort that compared tokens took 78 - 91 stages: 83 us for 4 x 4,096 tokens, 390 for 64 x 8,192;
 // now 49 and 105.)
-constexpr int BS_THREADS = 1024;
-constexpr int BS_WARPS = BS_THREADS / 32;
+constexpr int BS_THREADS = 1024;               // of the kernel that sorts prompts
 constexpr int BS_MAX_LEN = 16384;              // most tokens (two passes of 7 bits per round; 112 KB)
 constexpr int BS_BITS = 7;
 constexpr int BS_BINS = 1 << BS_BITS;
 constexpr int BS_ROW = BS_BINS + 1;            // (rows of 128 counters put the eight threads that add up a digit on one bank: a sort of 4 x 4,096 tokens took 60 us, 49 now)
 
-template <int ITEMS>
-constexpr int block_order_smem() { return (int)(sizeof(int) * BS_WARPS * BS_ROW + 3 * sizeof(unsigned short) * BS_THREADS * ITEMS); }
+template <int THREADS, int ITEMS>
+constexpr int block_order_smem() { return (int)(sizeof(int) * (THREADS / 32) * BS_ROW + 3 * sizeof(unsigned short) * THREADS * ITEMS); }
 
-// All BS_THREADS threads call; ITEMS per thread: n <= BS_THREADS * ITEMS tokens.  token(i) < 2^tok_bits; position i belongs to the
+// All THREADS (512 or 1,024) threads call; ITEMS per thread: n <= THREADS * ITEMS tokens.  token(i) < 2^tok_bits; position i belongs to the
 // sequence [begin(i), end(i)).  Returns the order (positions, in shared memory).
-template <int ITEMS, class Tok, class Begin, class End>
+template <int THREADS, int ITEMS, class Tok, class Begin, class End>
 __device__ __forceinline__ unsigned short* block_suffix_order(unsigned char* smem, int* wsum, int n, int tok_bits, int D, Tok token,
                                                               Begin begin, End end) {
-    int (*hist)[BS_ROW] = reinterpret_cast<int (*)[BS_ROW]>(smem);                  // [BS_WARPS][BS_ROW]
-    unsigned short* const rank = reinterpret_cast<unsigned short*>(smem + sizeof(int) * BS_WARPS * BS_ROW);
-    unsigned short* cur = rank + BS_THREADS * ITEMS;                                // the order so far
-    unsigned short* nxt = cur + BS_THREADS * ITEMS;
+    constexpr int WARPS = THREADS / 32, SHARE = WARPS / 4;      // threads that add up one digit, four warps' counts each
+    static_assert(BS_BINS * SHARE == THREADS, "a thread per digit and four warps");
+    int (*hist)[BS_ROW] = reinterpret_cast<int (*)[BS_ROW]>(smem);                  // [WARPS][BS_ROW]
+    unsigned short* const rank = reinterpret_cast<unsigned short*>(smem + sizeof(int) * WARPS * BS_ROW);
+    unsigned short* cur = rank + THREADS * ITEMS;                                // the order so far
+    unsigned short* nxt = cur + THREADS * ITEMS;
     const int tid = threadIdx.x, lane = tid & 31, wib = tid >> 5;
     const unsigned lt = (1u << lane) - 1u;
     const int p0 = wib * 32 * ITEMS + lane;                     // a warp's places are consecutive, 32 per step
@@ -67,7 +68,7 @@ __device__ __forceinline__ unsigned short* block_suffix_order(unsigned char* sme
         __syncthreads();
         {
             // counts to first places, in the order (digit, warp): a thread takes four warps of one digit
-            const int digit = tid >> 3, w0 = (tid & 7) * 4;
+            const int digit = tid / SHARE, w0 = tid % SHARE * 4;
             int c[4], sum = 0;
 #pragma unroll
             for (int q = 0; q < 4; ++q) { c[q] = hist[w0 + q][digit]; sum += c[q]; }
@@ -108,7 +109,7 @@ __device__ __forceinline__ unsigned short* block_suffix_order(unsigned char* sme
         }
         if (lane == 0) wsum[wib] = mine;
         __syncthreads();                                        // all old ranks have been read
-        const int c = wsum[lane];
+        const int c = lane < WARPS ? wsum[lane] : 0;
         int r = (int)__reduce_add_sync(0xffffffffu, lane < wib ? (unsigned)c : 0u) - 1;
         const int all = (int)__reduce_add_sync(0xffffffffu, (unsigned)c);
 #pragma unroll
