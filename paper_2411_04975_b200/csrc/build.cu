@@ -459,7 +459,7 @@ struct TreeScan {
     const int* end_pos;
     uint8_t *lcp, *len;
     int N, D;
-    int tile_len, tiles;                          // a multiple of 32
+    int tile_len, tiles;                          // TS_SUB times a power of two
     int* f;                                       // [32][tiles] (1): children counted, bit 31: state reset; carried: F from behind
     int* e;                                       // [32][tiles] (1): first reset in the tile; carried: end from behind
     int* r;                                       // [32][tiles] (2): R left behind (-1: none); carried: R from the front
@@ -1149,7 +1149,7 @@ static int pipeline_run(Pipeline& P, const int32_t* d_tok, const int64_t* d_seq_
     const bool block_sort = per_seq_max_len > 0 && per_seq_max_len <= BS_MAX_LEN;
     TreeScan& ts = P.ts;
     ts.N = (int)N; ts.D = D; ts.tok = d_tok;
-    ts.tile_len = 32;
+    ts.tile_len = TS_SUB;
     while ((N + ts.tile_len - 1) / ts.tile_len > TS_TILES && ts.tile_len < TS_MAX_LEN) ts.tile_len *= 2;
     ts.tiles = (int)((N + ts.tile_len - 1) / ts.tile_len);
     int sms = 0, dev = 0;
