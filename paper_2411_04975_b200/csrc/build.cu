@@ -30,6 +30,7 @@ typedef long long i64;
 // ------------------------------------------------------------------ suffix order
 // end_pos[i]: one past the last token of the sequence that holds position i.
 __global__ void seq_end_kernel(const int64_t* seq_offsets, int n_seqs, i64 n, int* end_pos) {
+    sd_chain_begin();
     i64 i = (i64)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     int lo = 0, hi = n_seqs;                          // largest s with seq_offsets[s] <= i
@@ -403,6 +404,7 @@ int corpus_sort(CorpusSort& A, cudaStream_t st) {
 template <int ITEMS>
 __global__ void __launch_bounds__(BS_THREADS, ITEMS <= 4 ? 2 : 1)
 block_suffix_sort_kernel(const int32_t* tok, const int64_t* seq_off, int V, int tok_bits, int D, uint32_t* sa_out) {
+    sd_chain_begin();
     extern __shared__ __align__(16) unsigned char bs_smem[];
     __shared__ int wsum[BS_THREADS / 32];
     const i64 b = seq_off[blockIdx.x];
@@ -419,7 +421,7 @@ int block_suffix_sort(const int32_t* tok, const int64_t* seq_off, int n_seqs, in
     constexpr int smem = block_order_smem<BS_THREADS, ITEMS>();
     if (smem > 48 * 1024)
         SD_CUDA_OK(cudaFuncSetAttribute(block_suffix_sort_kernel<ITEMS>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    block_suffix_sort_kernel<ITEMS><<<(unsigned)n_seqs, BS_THREADS, smem, st>>>(tok, seq_off, V, tok_bits, D, sa);
+    SD_CUDA_OK(sd_launch(block_suffix_sort_kernel<ITEMS>, (unsigned)n_seqs, BS_THREADS, smem, st, tok, seq_off, V, tok_bits, D, sa));
     return SD_OK;
 }
 
@@ -480,6 +482,7 @@ __device__ __forceinline__ int ts_scan(int v, int lane) {       // inclusive
 // (1)
 __global__ void __launch_bounds__(TS_WARPS * 32)
 ts_tiles_kernel(TreeScan T) {
+    sd_chain_begin();
     const int lane = threadIdx.x & 31, tile = blockIdx.x * TS_WARPS + (threadIdx.x >> 5), d = lane + 1;
     if (tile >= T.tiles) return;
     const int t0 = tile * T.tile_len, t1 = min(T.N, t0 + T.tile_len);
@@ -531,6 +534,7 @@ ts_tiles_kernel(TreeScan T) {
 
 // What lies behind (f, e: the tiles to the right; blocks 0 .. 31) or in front of a tile (s, n1: block 32).
 __global__ void __launch_bounds__(TS_CARRY) ts_carry_kernel(TreeScan T) {
+    sd_chain_begin();
     __shared__ int p0[TS_CARRY / 32], p1[TS_CARRY / 32];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int per = (T.tiles + TS_CARRY - 1) / TS_CARRY;
@@ -583,6 +587,7 @@ struct RequestBounds {
 
 // R from the front: the last one left behind by a tile to the left (blocks 0 .. 31); the others: a request each.
 __global__ void __launch_bounds__(TS_CARRY) ts_carry_front_kernel(TreeScan T, RequestBounds Q) {
+    sd_chain_begin();
     __shared__ int part[TS_CARRY / 32], part1[TS_CARRY / 32];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     if (blockIdx.x >= 32) {
@@ -641,6 +646,7 @@ __device__ __forceinline__ int ts_f_of(int g, int lane) {       // F from G (no 
 template <bool TOP>
 __global__ void __launch_bounds__(TS_WARPS * 32)
 ts_runs_kernel(TreeScan T) {
+    sd_chain_begin();
     const int lane = threadIdx.x & 31, tile = blockIdx.x * TS_WARPS + (threadIdx.x >> 5), d = lane + 1;
     if (tile >= T.tiles) return;
     const int t0 = tile * T.tile_len, t1 = min(T.N, t0 + T.tile_len);
@@ -691,6 +697,7 @@ struct TreeOut {
 template <bool REQ>
 __global__ void __launch_bounds__(TS_WARPS * 32)
 ts_emit_kernel(TreeScan T, TreeOut O) {
+    sd_chain_begin();
     extern __shared__ int2 ts_state[];                          // [TS_WARPS][tile_len / TS_SUB][32]: G and end behind each sub-tile
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5, tile = blockIdx.x * TS_WARPS + wib, d = lane + 1;
     if (tile >= T.tiles || (REQ && *O.bad)) return;
@@ -786,6 +793,7 @@ ts_emit_kernel(TreeScan T, TreeOut O) {
 // Long runs of the global tree move behind the others, with room for a top block in front: first every node of one
 // gets its new run (its entry may itself lie in a run that moves), then the runs are copied.
 __global__ void ts_wide_place_kernel(TreeScan T, int4* wide, int4* ent, int first) {
+    sd_chain_begin();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= T.wide[0]) return;
     int4 w = wide[i];
@@ -801,6 +809,7 @@ __global__ void ts_wide_place_kernel(TreeScan T, int4* wide, int4* ent, int firs
 constexpr int TOP_THREADS = 256;
 __global__ void __launch_bounds__(TOP_THREADS)
 ts_wide_fill_kernel(const int4* wide, int4* ent) {
+    sd_chain_begin();
     __shared__ int part[TOP_THREADS / 32];
     __shared__ u64 psum[TOP_THREADS / 32];
     __shared__ int cand[64];
@@ -1164,7 +1173,7 @@ static int pipeline_run(Pipeline& P, const int32_t* d_tok, const int64_t* d_seq_
               tmp.get(&ts.r, 32 * (i64)ts.tiles) && tmp.get(&ts.s, ts.tiles + 1) && tmp.get(&ts.n1, ts.tiles + 1) && tmp.get(&ts.wide, 4) &&
               (have_ends || tmp.get(&end_pos, N)) && tmp.get(&sa, N);
     if (!ok) return SD_ERR_NOMEM;
-    if (!have_ends) seq_end_kernel<<<grid_for(N, T256), T256, 0, st>>>(d_seq_offsets, n_seqs, N, end_pos);
+    if (!have_ends) SD_CUDA_OK(sd_launch(seq_end_kernel, grid_for(N, T256), T256, 0, st, d_seq_offsets, n_seqs, N, end_pos));
     int rc;
     if (block_sort) {
         const int V = (int)(max_token / n_seqs);                // (a sequence's tokens lie in a range of V of their own)
@@ -1196,11 +1205,11 @@ static int pipeline_run(Pipeline& P, const int32_t* d_tok, const int64_t* d_seq_
     ts.end_pos = end_pos;
     const unsigned grid = (unsigned)((ts.tiles + TS_WARPS - 1) / TS_WARPS);
     if (top_blocks && cudaMemsetAsync(ts.wide, 0, 4 * sizeof(int), st) != cudaSuccess) return SD_ERR_CUDA;
-    ts_tiles_kernel<<<grid, TS_WARPS * 32, 0, st>>>(ts);
-    ts_carry_kernel<<<33, TS_CARRY, 0, st>>>(ts);
-    if (top_blocks) ts_runs_kernel<true><<<grid, TS_WARPS * 32, 0, st>>>(ts);
-    else ts_runs_kernel<false><<<grid, TS_WARPS * 32, 0, st>>>(ts);
-    ts_carry_front_kernel<<<(unsigned)(32 + bounds.n + 1), TS_CARRY, 0, st>>>(ts, bounds);
+    SD_CUDA_OK(sd_launch(ts_tiles_kernel, grid, TS_WARPS * 32, 0, st, ts));
+    SD_CUDA_OK(sd_launch(ts_carry_kernel, 33, TS_CARRY, 0, st, ts));
+    if (top_blocks) SD_CUDA_OK(sd_launch(ts_runs_kernel<true>, grid, TS_WARPS * 32, 0, st, ts));
+    else SD_CUDA_OK(sd_launch(ts_runs_kernel<false>, grid, TS_WARPS * 32, 0, st, ts));
+    SD_CUDA_OK(sd_launch(ts_carry_front_kernel, (unsigned)(32 + bounds.n + 1), TS_CARRY, 0, st, ts, bounds));
     return SD_OK;
 }
 
@@ -1210,7 +1219,7 @@ static int emit_entries(const TreeScan& ts, const TreeOut& out, cudaStream_t st)
     const size_t smem = sizeof(int2) * 32 * (size_t)TS_WARPS * (ts.tile_len / TS_SUB);
     if (smem > 48 * 1024)
         SD_CUDA_OK(cudaFuncSetAttribute(ts_emit_kernel<REQ>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    ts_emit_kernel<REQ><<<grid, TS_WARPS * 32, smem, st>>>(ts, out);
+    SD_CUDA_OK(sd_launch(ts_emit_kernel<REQ>, grid, TS_WARPS * 32, smem, st, ts, out));
     return SD_OK;
 }
 
@@ -1346,6 +1355,7 @@ __device__ __forceinline__ int seq_rank_of(const int64_t* off, int n, i64 pos) {
 // sets both flags (the host's one lies in its memory).
 __global__ void map_tokens_kernel(const int32_t* tok, const int64_t* off, int n, i64 N, int V, int32_t* out, int* end_pos, int* bad,
                                   int* host_bad) {
+    sd_chain_begin();
     const i64 i = (i64)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= N) return;
     int t = tok[i];
@@ -1359,6 +1369,7 @@ __global__ void map_tokens_kernel(const int32_t* tok, const int64_t* off, int n,
 constexpr int PREP_THREADS = 1024;
 __global__ void __launch_bounds__(PREP_THREADS)
 requests_prepare_kernel(sd_store sv, int n, const int32_t* slot_ids, const int64_t* off, const int32_t* tok, const int* bad) {
+    sd_chain_begin();
     const int q = blockIdx.x;
     if (q >= n || *bad) return;
     const int slot = slot_ids[q];
@@ -1378,6 +1389,7 @@ requests_prepare_kernel(sd_store sv, int n, const int32_t* slot_ids, const int64
 __global__ void __launch_bounds__(256)
 requests_finalize_kernel(sd_store sv, int n, const int32_t* slot_ids, const int64_t* off, const int* s_req, const int* n1_req,
                          const int* bad) {
+    sd_chain_begin();
     const int q = blockIdx.x, lane = threadIdx.x & 31, d = threadIdx.x / APP_LANES + 1;
     if (q >= n || *bad) return;
     const int slot = slot_ids[q];
@@ -1461,7 +1473,7 @@ extern "C" int sd_build_requests(sd_store* s, int32_t n, const int32_t* h_slot, 
     memcpy(h_args + 8 * ((size_t)n + 1), h_slot, 4 * (size_t)n);
     memset(h_args + arg_bytes - 4, 0, 4);
     SD_CUDA_OK(cudaMemcpyAsync(d_args, h_args, arg_bytes, cudaMemcpyHostToDevice, st));
-    if (N > 0) map_tokens_kernel<<<grid_for(N, T256), T256, 0, st>>>(d_tokens, d_off, n, N, s->V, mtok, end_pos, bad, (int*)s->stage);
+    if (N > 0) SD_CUDA_OK(sd_launch(map_tokens_kernel, grid_for(N, T256), T256, 0, st, d_tokens, d_off, n, N, s->V, mtok, end_pos, bad, (int*)s->stage));
     SD_CUDA_OK(cudaEventRecord(s->ev_check, st));
     int rc = SD_OK;
     if (N > 0) {
@@ -1469,7 +1481,7 @@ extern "C" int sd_build_requests(sd_store* s, int32_t n, const int32_t* h_slot, 
         for (int q = 0; q < n; ++q) max_len = std::max<i64>(max_len, h_offsets[q + 1] - h_offsets[q]);
         rc = pipeline_run(P, mtok, d_off, n, N, (i64)n * s->V, D, false, st, max_len, end_pos, RequestBounds{n, d_off, s_req, n1_req});
     }
-    if (rc == SD_OK) requests_prepare_kernel<<<(unsigned)n, PREP_THREADS, 0, st>>>(*s, n, d_slot, d_off, d_tokens, bad);
+    if (rc == SD_OK) SD_CUDA_OK(sd_launch(requests_prepare_kernel, (unsigned)n, PREP_THREADS, 0, st, *s, n, d_slot, d_off, d_tokens, bad));
     if (rc == SD_OK && N > 0) {
         TreeOut out;
         memset(&out, 0, sizeof(out));
@@ -1477,7 +1489,7 @@ extern "C" int sd_build_requests(sd_store* s, int32_t n, const int32_t* h_slot, 
         rc = emit_entries<true>(P.ts, out, st);
     }
     if (rc == SD_OK)
-        requests_finalize_kernel<<<(unsigned)n, 256, 0, st>>>(*s, n, d_slot, d_off, N > 0 ? s_req : nullptr, N > 0 ? n1_req : nullptr, bad);
+        SD_CUDA_OK(sd_launch(requests_finalize_kernel, (unsigned)n, 256, 0, st, *s, n, d_slot, d_off, N > 0 ? s_req : nullptr, N > 0 ? n1_req : nullptr, bad));
     const cudaError_t checked = cudaEventSynchronize(s->ev_check);               // (the pinned memory is free again, too)
     if (rc != SD_OK) return rc;
     if (checked != cudaSuccess) return SD_ERR_CUDA;

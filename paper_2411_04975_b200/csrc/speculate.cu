@@ -932,6 +932,7 @@ speculate_fused_kernel(sd_store sv, int n, const int32_t* __restrict__ d_slot, i
                        int32_t* d_tokens, int32_t* d_parents, int32_t* d_positions, uint32_t* d_mask, int32_t* d_chosen_tree,
                        int32_t* d_chosen_p, double* d_score, int32_t* d_status, const int64_t* __restrict__ d_app_off,
                        const int32_t* __restrict__ d_app_tok) {
+    sd_chain_begin();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     using BlockShared = BlockSharedT<WARPS>;
     constexpr int CTA_WARPS = WARPS;
@@ -1313,9 +1314,9 @@ static int launch_fused(sd_store* s, int32_t n, const int32_t* d_slot, const sd_
     // more requests than two 16-warp blocks per SM hold at once: smaller blocks, one wave
     const bool narrow = n > 2 * sms;
 #define SD_LAUNCH_FUSED(STEP, WARPS, MINB, OFF, TOK)                                                                     \
-    speculate_fused_kernel<STEP, WARPS, MINB><<<(unsigned)n, WARPS * 32, sizeof(BlockSharedT<WARPS>), st>>>(             \
-        *s, n, d_slot, Pe, prm->alpha, prm->max_spec, prm->flags, prm->tau, d_budget_cap, d_n_draft, d_tokens,           \
-        d_parents, d_positions, d_mask, d_chosen_tree, d_chosen_p, d_score, d_status, OFF, TOK)
+    SD_CUDA_OK(sd_launch(speculate_fused_kernel<STEP, WARPS, MINB>, (unsigned)n, WARPS * 32, sizeof(BlockSharedT<WARPS>), st, \
+                         *s, n, d_slot, Pe, prm->alpha, prm->max_spec, prm->flags, prm->tau, d_budget_cap, d_n_draft, d_tokens, \
+                         d_parents, d_positions, d_mask, d_chosen_tree, d_chosen_p, d_score, d_status, OFF, TOK))
     if (step) {
         if (wide) SD_LAUNCH_FUSED(true, CTA_WARPS_WIDE_STEP, 1, d_app_off, d_app_tok);
         else if (narrow) SD_LAUNCH_FUSED(true, CTA_WARPS_NARROW_STEP, 4, d_app_off, d_app_tok);
