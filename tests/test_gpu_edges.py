@@ -1,0 +1,140 @@
+"""Sizes at which the kernels change over or could slip: remainders and edges of tiles, lots and passes, the smallest and
+largest of a range, runs that are merged by a warp or a block, candidates of equal D.  Everything against the CPU oracle."""
+import numpy as np
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def U():
+    import gpu_util
+    return gpu_util
+
+
+def _text(rng, n, vocab, period=60):
+    """Repeats itself with a few fresh tokens in between: many equal suffixes, few nodes."""
+    base = rng.integers(0, vocab, size=period)
+    t = np.tile(base, n // period + 1)[:n].astype(np.int32)
+    hit = rng.random(n) < 20.0 / max(n, 40)
+    t[hit] = rng.integers(0, vocab, size=int(hit.sum()))
+    return t
+
+
+@pytest.mark.parametrize("longest,D,vocab", [(1, 1, 2), (33, 32, 3), (1024, 17, 130), (1025, 32, 50), (2049, 2, 7), (4096, 24, 128256),
+                                             (4097, 32, 300), (8193, 31, 65), (16384, 32, 40), (16385, 32, 40)])
+def test_prompts_at_the_edges_of_the_block_sort(U, longest, D, vocab):
+    rng = np.random.default_rng(longest)
+    lens = sorted({1, 2, 15, 16, 17, max(1, longest - 1), longest} & set(range(1, longest + 1)))
+    prompts = [_text(rng, n, vocab) for n in lens] + [np.zeros(0, np.int32)]
+    pr = U.Pair([], vocab=vocab, D=D, n_slots=len(prompts), max_req_tokens=longest + 8, M=32)
+    off, flat = U.ragged(prompts)
+    for _ in range(2):                                          # the second time over trees that are there
+        pr.g.build_requests(np.arange(len(prompts)), off, U.dev_i32(flat))
+    pr.o.slot_append_batch(list(range(len(prompts))), prompts)
+    for s in range(len(prompts)):
+        pr.check_tree(s)
+    pr.append(list(range(len(prompts))), [_text(rng, 5, vocab) for _ in prompts])       # the active nodes are right
+    for s in range(len(prompts)):
+        pr.check_tree(s)
+    pr.check_speculate(list(range(len(prompts))), 8, 2.0, 32)
+    pr.close()
+
+
+@pytest.mark.parametrize("n,D,vocab", [(1, 32, 5), (1023, 32, 9), (1025, 17, 4000), (9000, 24, 60), (303104, 3, 12), (303137, 6, 90)])
+def test_corpora_at_the_edges_of_the_sort(U, n, D, vocab):
+    rng = np.random.default_rng(n)
+    text = _text(rng, n, vocab, period=200)
+    cuts = np.unique(np.concatenate([[0, n, n], rng.integers(0, n + 1, size=6), [min(n, 1), min(n, 34)]]))
+    seqs = [text[a:b] for a, b in zip(cuts[:-1], cuts[1:])]
+    seqs.insert(1, np.zeros(0, np.int32))
+    pr = U.Pair(seqs, vocab=vocab, D=D, n_slots=1, max_req_tokens=64)
+    pr.check_tree(-1)
+    want = pr.o.entropy(-1)
+    assert abs(pr.g.entropy(-1) - want) <= 1e-9 * max(1.0, want)            # the tree as built
+    pr.append([-1], [text[:1]])
+    want = pr.o.entropy(-1)
+    assert abs(pr.g.entropy(-1) - want) <= 1e-9 * max(1.0, want)            # ... and inserted into: by traversal
+    pr.close()
+
+
+@pytest.mark.parametrize("sizes,D,vocab,fresh", [([1], 32, 4, False), ([7, 8, 9], 32, 6, False), ([511, 1, 0, 2], 17, 30, False),
+                                                 ([513], 32, 2, False), ([2015], 32, 5, False), ([2016], 8, 700, True),
+                                                 ([2017, 3], 32, 40, False), ([1000, 1000, 1000, 1100], 24, 900, True)])
+def test_global_insert_at_the_edges_of_a_pass(U, sizes, D, vocab, fresh):
+    rng = np.random.default_rng(sum(sizes) + D)
+    base = [_text(rng, 400, vocab), rng.integers(0, vocab, size=300).astype(np.int32)]
+    pr = U.Pair(base, vocab=vocab, D=D, n_slots=2, max_req_tokens=64)
+    for _ in range(2):
+        seqs = [rng.integers(0, vocab, size=n).astype(np.int32) if fresh else _text(rng, n, vocab, 45) for n in sizes]
+        pr.append([-1] * len(seqs) + [1], seqs + [base[0][:3]])
+        pr.check_tree(-1)
+    pr.append([0], [base[0][:20]])
+    pr.check_speculate([0, 1], 12, 2.0, 32)
+    pr.close()
+
+
+def test_global_insert_merges_long_runs(U):
+    """One token with hundreds of children: runs that move and runs with room, merged by a block, children of which get children."""
+    rng = np.random.default_rng(5)
+    vocab = 4000
+    def fan(tokens):
+        return np.stack([np.zeros(len(tokens), np.int64), tokens], 1).reshape(-1).astype(np.int32)
+    perm = 1 + rng.permutation(vocab - 1)
+    pr = U.Pair([fan(perm[:600])], vocab=vocab, D=4, n_slots=1, max_req_tokens=64)
+    for lo, hi in ((550, 950), (950, 960), (0, 300), (960, 1500), (1500, 1501)):
+        pr.append([-1, -1], [fan(perm[lo:hi]), fan(perm[hi - 1:lo:-7])])
+        pr.check_tree(-1)
+    pr.append([0], [np.array([3, 0], np.int32)])
+    pr.check_speculate([0], 4, 4.0, 64)
+    pr.close()
+
+
+@pytest.mark.parametrize("fan,deep,budget", [(2, 20, 64), (31, 3, 64), (32, 2, 64), (33, 2, 64), (30, 1, 64), (40, 6, 48)])
+def test_candidates_of_equal_d(U, fan, deep, budget):
+    """A node with `fan` children that all occur equally often, each the start of a chain, and of further fans: equal D in
+    numbers up to and above a warp and the pool."""
+    rng = np.random.default_rng(fan * 100 + deep)
+    seqs = []
+    for c in range(fan):
+        chain = (rng.permutation(500)[:deep] + 100 * (c % 3)).tolist()
+        for e in range(3 if deep < 4 else 1):
+            seqs.append(np.array([7, 8, 10 + c] + chain + [900 + (e * 37 + c) % 60, 960 + e], np.int32))
+    wide = [np.array([7, 9, 10 + c, 700 + e], np.int32) for c in range(min(fan, 30)) for e in range(30)]
+    pr = U.Pair(seqs + wide, vocab=1024, D=32, n_slots=3, max_req_tokens=64)
+    pr.append([0, 1, 2], [np.array([7, 8], np.int32), np.array([7, 9], np.int32), np.array([5, 7], np.int32)])
+    for flags in (0, 4):
+        pr.check_speculate([0, 1, 2], 3, 32.0, budget, flags=flags)
+    pr.close()
+
+
+def test_a_bad_token_leaves_the_slots_as_they_are(U):
+    import paper_2411_04975_b200 as sfx
+    rng = np.random.default_rng(9)
+    pr = U.Pair([], vocab=20, D=8, n_slots=3, max_req_tokens=200)
+    pr.append([0, 1, 2], [_text(rng, 50, 20) for _ in range(3)])
+    prompts = [_text(rng, 120, 20), _text(rng, 90, 20)]
+    off, flat = U.ragged(prompts)
+    flat[130] = 20
+    for _ in range(2):
+        with pytest.raises(sfx.SuffixSpecError) as e:
+            pr.g.build_requests([2, 0], off, U.dev_i32(flat))
+        assert e.value.code == -1
+        for s in range(3):
+            pr.check_tree(s)
+        pr.check_speculate([0, 1, 2], 8, 2.0, 32)
+    pr.close()
+
+
+def test_memory_kept_between_stores_is_bounded():
+    import paper_2411_04975_b200 as sfx
+    torch.cuda.synchronize()
+    free0, total = torch.cuda.mem_get_info()
+    for k in range(6):
+        stores = [sfx.SuffixStore(None, None, vocab=1000, depth_cap=32, max_requests=64, max_req_tokens=2000 + 997 * j + 311 * k, max_spec_cap=64)
+                  for j in range(3)]
+        for s in stores:
+            s.free()
+    torch.cuda.synchronize()
+    assert free0 - torch.cuda.mem_get_info()[0] <= total // 32 + (64 << 20)
