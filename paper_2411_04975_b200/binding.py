@@ -1,4 +1,5 @@
-"""ctypes binding of libsuffixspec.so: argument marshalling only.
+"""Binding of libsuffixspec.so: argument marshalling only (ctypes; the calls that a serving loop
+makes every step go through the native module _call, see csrc/call.cpp).
 
 Tensors are torch CUDA tensors used as plain device buffers; the stream is
 torch's current stream.  The module-level functions sd_build / sd_append /
@@ -8,7 +9,6 @@ wraps them with output allocation.
 from __future__ import annotations
 
 import ctypes as C
-import functools
 import os
 from typing import Dict, Optional
 
@@ -47,15 +47,16 @@ class _Stats(C.Structure):
 
 
 _lib = None
+_call = None               # the module of the per-step calls; loaded with the library
 
 
 def library() -> C.CDLL:
     """Load libsuffixspec.so (building it with nvcc if the sources are newer).
     Raises if it cannot be had: there is no fallback path."""
-    global _lib
+    global _lib, _call
     if _lib is None:
         path = _build.LIB
-        if not os.path.exists(path) or os.environ.get("SUFFIXSPEC_REBUILD"):
+        if not (os.path.exists(path) and os.path.exists(_build.CALL)) or os.environ.get("SUFFIXSPEC_REBUILD"):
             path = _build.build()
         lib = C.CDLL(path)
         vp = C.c_void_p
@@ -87,16 +88,15 @@ def library() -> C.CDLL:
         lib.sd_debug_fail_alloc.argtypes = [C.c_int64]
         lib.sd_strerror.restype = C.c_char_p
         lib.sd_strerror.argtypes = [C.c_int]
-        _lib = lib
+        from . import _call as call
+        call.setup(*(C.cast(f, vp).value for f in (lib.sd_speculate, lib.sd_step, lib.sd_append)), _ptr)
+        _lib, _call = lib, call
     return _lib
 
 
 def _ptr(t: Optional[torch.Tensor], dtype: torch.dtype, name: str) -> Optional[int]:
     if t is None:
         return None
-    # (the usual case first: a small batch's draft takes the GPU no longer than such checks take the host)
-    if t.dtype is dtype and t.is_cuda and t.is_contiguous():
-        return t.data_ptr()
     # pinned host memory has a device address of its own (unified addressing): the kernels then
     # read or write it across the bus, with no copy before or after the call
     if not (t.is_cuda or t.is_pinned()) or t.dtype != dtype or not t.is_contiguous():
@@ -124,11 +124,10 @@ def _out_ptrs(out: Dict[str, torch.Tensor]) -> list:
     return [_ptr(out[name], dtype, name) for name, dtype in _OUT_FIELDS]
 
 
-@functools.lru_cache(maxsize=64)
-def _spec_params(P: int, alpha: float, max_spec: int, flags: int, tau: float):
-    """The converted parameters of a draft (read by the library only) and a pointer to them."""
-    prm = _SpecParams(P, alpha, max_spec, flags, tau)
-    return prm, C.pointer(prm)
+def _loaded():
+    """The module of the per-step calls."""
+    library()
+    return _call
 
 
 # ---- the C entry points, one to one ------------------------------------------------------
@@ -149,18 +148,14 @@ def sd_build(corpus: Optional[torch.Tensor], seq_offsets: Optional[torch.Tensor]
 
 def sd_append(store: int, slots: torch.Tensor, offsets: torch.Tensor, tokens: torch.Tensor,
               reset: Optional[torch.Tensor] = None) -> None:
-    rc = library().sd_append(store, int(slots.numel()), _ptr(slots, torch.int32, "slots"),
-                             _ptr(offsets, torch.int64, "offsets"), _ptr(tokens, torch.int32, "tokens"),
-                             _ptr(reset, torch.uint8, "reset"), _stream())
+    rc = (_call or _loaded()).append(store, slots, offsets, tokens, reset)
     if rc != 0:
         raise SuffixSpecError(rc, "sd_append")
 
 
 def sd_speculate(store: int, slots: torch.Tensor, P: int, alpha: float, max_spec: int, flags: int,
                  budget_cap: Optional[torch.Tensor], out: Dict[str, torch.Tensor], tau: float = 0.0) -> None:
-    rc = library().sd_speculate(
-        store, slots.numel(), _ptr(slots, torch.int32, "slots"), _spec_params(P, alpha, max_spec, flags, tau)[1],
-        _ptr(budget_cap, torch.int32, "budget_cap"), *_out_ptrs(out), _stream())
+    rc = (_call or _loaded()).speculate(store, slots, P, alpha, max_spec, flags, tau, budget_cap, out)
     if rc != 0:
         raise SuffixSpecError(rc, "sd_speculate")
 
@@ -172,8 +167,8 @@ def sd_speculate_noalloc(store: int, slots: torch.Tensor, P: int, alpha: float, 
     (n * 2 * depth_cap <= 4096 jobs) and calls on one device must not overlap.
     `out` must be preallocated by the caller; nothing is allocated here."""
     rc = library().sd_speculate_noalloc(
-        store, slots.numel(), _ptr(slots, torch.int32, "slots"), _spec_params(P, alpha, max_spec, flags, tau)[1],
-        _ptr(budget_cap, torch.int32, "budget_cap"), *_out_ptrs(out), _stream())
+        store, slots.numel(), _ptr(slots, torch.int32, "slots"),
+        C.byref(_SpecParams(P, alpha, max_spec, flags, tau)), _ptr(budget_cap, torch.int32, "budget_cap"), *_out_ptrs(out), _stream())
     if rc != 0:
         raise SuffixSpecError(rc, "sd_speculate_noalloc")
 
@@ -296,10 +291,8 @@ class SuffixStore:
         then speculate.  Same result as append() followed by speculate()."""
         if out is None:
             out = self.alloc_outputs(int(slots.numel()))
-        rc = library().sd_step(
-            self._h, slots.numel(), _ptr(slots, torch.int32, "slots"), _ptr(offsets, torch.int64, "offsets"),
-            _ptr(new_tokens, torch.int32, "new_tokens"), _spec_params(P, alpha, max_spec, flags, tau)[1],
-            _ptr(budget_cap, torch.int32, "budget_cap"), *_out_ptrs(out), _stream())
+        rc = (_call or _loaded()).step(self._h, slots, offsets, new_tokens, P, alpha, max_spec, flags, tau, budget_cap,
+                                       out)
         if rc != 0:
             raise SuffixSpecError(rc, "sd_step")
         return out

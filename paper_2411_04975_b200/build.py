@@ -1,13 +1,15 @@
-"""Build the CUDA library in-tree with nvcc for sm_100a."""
+"""Build the CUDA library in-tree with nvcc for sm_100a, and the calls' host path beside it."""
 from __future__ import annotations
 
 import os
 import subprocess
+import sysconfig
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 _ROOT = os.path.dirname(_HERE)
 CSRC = os.path.join(_HERE, "csrc")
 LIB = os.path.join(_HERE, "libsuffixspec.so")
+CALL = os.path.join(_HERE, "_call.so")
 SOURCES = ["build.cu", "append.cu", "speculate.cu", "query.cu"]
 
 
@@ -17,18 +19,39 @@ def _newest_source() -> float:
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
-    """Compile csrc/*.cu into libsuffixspec.so (cross-compiles without a GPU)."""
-    if not force and os.path.exists(LIB) and os.path.getmtime(LIB) >= _newest_source():
-        return LIB
-    nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
-    cmd = [nvcc, "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
-           "-shared", "-Xcompiler", "-fPIC", "-I", os.path.join(_ROOT, "include"), "-I", CSRC,
-           "-cudart", "shared", "-o", LIB]
-    if verbose:
-        cmd += ["-Xptxas", "-v"]
-    cmd += [os.path.join(CSRC, f) for f in SOURCES]
-    subprocess.check_call(cmd)
+    """Compile csrc/*.cu into libsuffixspec.so (cross-compiles without a GPU) and csrc/call.cpp into the
+    module _call.  Returns the library's path."""
+    newest = _newest_source()
+
+    def fresh(path):
+        return not force and os.path.exists(path) and os.path.getmtime(path) >= newest
+
+    if not fresh(LIB):
+        nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
+        cmd = [nvcc, "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
+               "-shared", "-Xcompiler", "-fPIC", "-I", os.path.join(_ROOT, "include"), "-I", CSRC,
+               "-cudart", "shared", "-o", LIB]
+        if verbose:
+            cmd += ["-Xptxas", "-v"]
+        cmd += [os.path.join(CSRC, f) for f in SOURCES]
+        subprocess.check_call(cmd)
+    if not fresh(CALL):
+        _build_call()
     return LIB
+
+
+def _build_call() -> None:
+    import torch
+    from torch.utils.cpp_extension import include_paths
+    cuda = os.path.dirname(os.path.dirname(os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")))
+    includes = [os.path.join(_ROOT, "include"), sysconfig.get_paths()["include"], os.path.join(cuda, "include"),
+                *include_paths()]
+    lib = os.path.join(os.path.dirname(torch.__file__), "lib")
+    cmd = ["g++", "-O2", "-std=c++17", "-shared", "-fPIC", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}"]
+    for path in includes:
+        cmd += ["-isystem", path]
+    cmd += [os.path.join(CSRC, "call.cpp"), "-L", lib, "-ltorch_python", "-ltorch_cpu", "-lc10", "-lc10_cuda", "-o", CALL]
+    subprocess.check_call(cmd)
 
 
 if __name__ == "__main__":

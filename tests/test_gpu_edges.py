@@ -138,3 +138,27 @@ def test_memory_kept_between_stores_is_bounded():
             s.free()
     torch.cuda.synchronize()
     assert free0 - torch.cuda.mem_get_info()[0] <= total // 32 + (64 << 20)
+
+
+@pytest.mark.parametrize("name,bad,error", [
+    ("slots", lambda t: t.long(), TypeError), ("slots", lambda t: t.cpu(), TypeError), ("slots", lambda t: None, Exception),
+    ("offsets", lambda t: t.int(), TypeError), ("new_tokens", lambda t: t.repeat(2)[::2], TypeError),
+    ("new_tokens", lambda t: t.tolist(), Exception), ("P", lambda t: "4", TypeError), ("alpha", lambda t: None, TypeError),
+    ("budget_cap", lambda t: torch.ones(3, dtype=torch.float32, device="cuda"), TypeError), ("out", lambda t: {}, KeyError)])
+def test_arguments_of_the_calls_of_every_step(U, name, bad, error):
+    pr = U.Pair([], vocab=20, D=8, n_slots=3, max_req_tokens=200)
+    pr.append([0, 1, 2], [np.arange(9, dtype=np.int32) % 4 for _ in range(3)])
+    args = dict(slots=U.dev_i32(np.arange(3)), offsets=torch.zeros(4, dtype=torch.int64, device="cuda"), new_tokens=U.dev_i32(np.zeros(2)),
+                P=4, alpha=2.0, max_spec=8, flags=0, budget_cap=None, out=None, tau=0.0)
+    bad_args = dict(args, **{name: bad(args[name])})
+    with pytest.raises(error):
+        pr.g.step(**bad_args)
+    if name in ("slots", "P", "alpha", "budget_cap", "out"):
+        with pytest.raises(error):
+            pr.g.speculate(**{k: v for k, v in bad_args.items() if k not in ("offsets", "new_tokens")})
+    host = {k: v.pin_memory() if isinstance(v, torch.Tensor) else v for k, v in
+            dict(args, slots=args["slots"].cpu(), offsets=args["offsets"].cpu(), new_tokens=args["new_tokens"].cpu()).items()}
+    a, b = pr.g.step(**args), pr.g.step(**host)                 # the store is as it was; pinned host tensors are taken
+    for k in ("n_draft", "chosen_tree", "chosen_p", "score", "status"):
+        assert torch.equal(a[k], b[k])
+    pr.close()
