@@ -693,6 +693,16 @@ struct TreeOut {
     const int* bad;                               // not 0: a token is outside the vocabulary, nothing may change
 };
 
+// What the lanes need of a suffix in one word, so that one shuffle hands it out: lcp and length (at most 32), S and the
+// depth-1 nodes relative to the first of up to 32 suffixes (at most 31 * 31, 31).  ts_emit_kernel mostly shuffles: 13 -> 8
+// of them per suffix, and the next sub-tile read ahead, 767 -> 569 us for 4.2 M suffixes.  (ts_runs_kernel is bound by
+// its arithmetic: taking words apart made it 226 -> 251 us.)
+__device__ __forceinline__ int ts_pack(int l, int n, int s, int n1) { return l | n << 6 | s << 12 | n1 << 22; }
+__device__ __forceinline__ int ts_l(int w) { return w & 63; }
+__device__ __forceinline__ int ts_n(int w) { return (w >> 6) & 63; }
+__device__ __forceinline__ int ts_s(int w) { return (w >> 12) & 1023; }
+__device__ __forceinline__ int ts_n1(int w) { return w >> 22; }
+
 // (3)
 template <bool REQ>
 __global__ void __launch_bounds__(TS_WARPS * 32)
@@ -710,10 +720,10 @@ ts_emit_kernel(TreeScan T, TreeOut O) {
             st[c * 32 + lane] = make_int2(g, e);
             if (c == 0) break;
             const int jb = t0 + c * TS_SUB, m = min(TS_SUB, t1 - jb);
-            const int l_own = lane < m ? T.lcp[jb + lane] : 0, n_own = lane < m ? T.len[jb + lane] : 0;
+            const int own = lane < m ? ts_pack(T.lcp[jb + lane], T.len[jb + lane], 0, 0) : 0;
             for (int i = m - 1; i >= 0; --i) {
-                const int l = __shfl_sync(TS_FULL, l_own, i);
-                g = ts_g_step(g, l, __shfl_sync(TS_FULL, n_own, i), d);
+                const int w = __shfl_sync(TS_FULL, own, i), l = ts_l(w);
+                g = ts_g_step(g, l, ts_n(w), d);
                 if (d > l) e = jb + i;
             }
         }
@@ -742,38 +752,42 @@ ts_emit_kernel(TreeScan T, TreeOut O) {
     } else {
         shift = T.n1[T.tiles];
     }
+    int l_own = 0, n_own = 0, sa_own = 0;                       // of the sub-tile's suffixes, read one sub-tile ahead
+    auto fetch = [&](int j) {
+        const bool in = lane < TS_SUB && j + lane < t1;
+        l_own = in ? T.lcp[j + lane] : 0; n_own = in ? T.len[j + lane] : 0; sa_own = in ? (int)T.sa[j + lane] : 0;
+    };
+    fetch(t0);
     for (int c = 0; c < subs; ++c) {
         const int jb = t0 + c * TS_SUB, m = min(TS_SUB, t1 - jb);
-        int l_own = 255, n_own = 0, sa_own = 0, below = 0, top = 0;
-        if (lane < m) {
-            l_own = T.lcp[jb + lane]; n_own = T.len[jb + lane]; sa_own = (int)T.sa[jb + lane];
-            below = n_own - max(l_own, 1); top = l_own == 0 ? 1 : 0;
-        }
-        const int ib = ts_scan(below, lane), it = ts_scan(top, lane);
-        const int s_own = s_at + ib - below, n1_own = n1_at + it - top;
+        const int below = lane < m ? n_own - max(l_own, 1) : 0;
+        const unsigned tops = __ballot_sync(TS_FULL, lane < m && l_own == 0);
+        const int ib = ts_scan(below, lane);
+        const int own = ts_pack(l_own, n_own, ib - below, __popc(tops & ((1u << lane) - 1u))), at_own = sa_own;
+        const int s0 = s_at, n1_at0 = n1_at;
         s_at += __shfl_sync(TS_FULL, ib, 31);
-        n1_at += __shfl_sync(TS_FULL, it, 31);
+        n1_at += __popc(tops);
         int x[TS_SUB], gs[TS_SUB], es[TS_SUB];
         const int2 in = st[c * 32 + lane];
         int g = in.x, e = in.y;
 #pragma unroll
         for (int i = TS_SUB - 1; i >= 0; --i) {
-            const int n = __shfl_sync(TS_FULL, n_own, i), at = __shfl_sync(TS_FULL, sa_own, i);
+            const int w = __shfl_sync(TS_FULL, own, i), at = __shfl_sync(TS_FULL, at_own, i), l = ts_l(w), n = ts_n(w);
             x[i] = lane < n ? T.tok[at + lane] : 0;
             gs[i] = g; es[i] = e;
-            const int l = __shfl_sync(TS_FULL, l_own, i);
             if (i < m) {
                 g = ts_g_step(g, l, n, d);
                 if (d > l) e = jb + i;
             }
         }
+        fetch(jb + TS_SUB);
 #pragma unroll
         for (int i = 0; i < TS_SUB; ++i) {
             if (i >= m) break;
             const int j = jb + i;
             if (REQ && j >= next_req) { while (j >= (int)O.off[q + 1]) ++q; enter(); }
-            const int l = __shfl_sync(TS_FULL, l_own, i), n = __shfl_sync(TS_FULL, n_own, i);
-            const int run = __shfl_sync(TS_FULL, s_own, i) + d - max(l, 1) + gs[i], depth1 = __shfl_sync(TS_FULL, n1_own, i) - n1_0;
+            const int w = __shfl_sync(TS_FULL, own, i), l = ts_l(w), n = ts_n(w);
+            const int run = s0 + ts_s(w) + d - max(l, 1) + gs[i], depth1 = n1_at0 + ts_n1(w) - n1_0;
             const int later = ts_f_of(gs[i], lane);
             const int kids = later + (d < n ? 1 : 0);
             const bool opens = d > l && d <= n;
