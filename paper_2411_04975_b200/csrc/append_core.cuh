@@ -51,6 +51,35 @@ __device__ int insert_child_warp(int4* ent, int parent, int cb, int n, int pos, 
     return idx;
 }
 
+// The same for up to four lanes at once, by eight lanes each: `src` is the lane that a group works for (-1: none), the
+// other arguments are every lane's own.  Returns the new child's entry to the lanes of src's group.
+__device__ int insert_child_groups(int4* ent, int src, int parent, int cb, int n, int pos, int x, int fresh, bool moves, int lane) {
+    const unsigned FULL = 0xffffffffu;
+    const int l = lane & 7, from = max(src, 0);
+    parent = __shfl_sync(FULL, parent, from); cb = __shfl_sync(FULL, cb, from); n = __shfl_sync(FULL, n, from);
+    pos = __shfl_sync(FULL, pos, from); fresh = __shfl_sync(FULL, fresh, from);
+    moves = __shfl_sync(FULL, moves ? 1 : 0, from) != 0;
+    const bool on = src >= 0;
+    if (on && moves)
+        for (int i = l; i < n; i += 8) ent[fresh + i + (i >= pos ? 1 : 0)] = ent[cb + i];
+    for (int hi = on && !moves ? n : 0; __any_sync(FULL, hi > pos); hi -= 8) {
+        const int i = max(pos, hi - 8) + l;
+        int4 e = make_int4(0, 0, 0, 0);
+        if (i < hi) e = ent[cb + i];
+        __syncwarp();
+        if (i < hi) ent[cb + i + 1] = e;
+        __syncwarp();
+    }
+    const int idx = moves ? fresh + pos : cb + pos;
+    if (on && l == 0) {
+        ent[idx] = make_int4(x, 1, 0, 0);
+        if (moves) *word(&ent[parent], 2) = fresh;
+        *word(&ent[parent], 3) = n + 1;
+    }
+    __syncwarp();
+    return idx;
+}
+
 // ---------------------------------------------------------------------------------------------
 // Append to a request's tree: one warp, a lane per active node.
 //
@@ -67,6 +96,8 @@ __device__ int insert_child_warp(int4* ent, int parent, int cb, int n, int pos, 
 constexpr int APP_AHEAD = 28;                 // tokens looked up ahead
 constexpr int APP_SHALLOW = 4;                // depths looked up ahead
 constexpr int APP_LANES = 8;                  // lanes per search
+constexpr int APP_OPEN = 3;                   // long runs to search from which on every lane searches its own
+constexpr int APP_BIG = 64;                   // entries to move from which on the whole warp does it
 constexpr unsigned ROOM_SHIFT = 24, ROOM_MASK = 31u;            // room behind a node, kept in the spare bits of its w field while appending
 
 struct AppendShared {
@@ -254,6 +285,26 @@ __device__ __forceinline__ void append_tokens(AppendShared& sh, const sd_store& 
                 if (h >= 0) { lo = min(max(h - 1, 0), n - 4); m = 4; }
             }
         }
+        if (__popc(__ballot_sync(FULL, n > 4 && m == 0)) >= APP_OPEN) {
+            // eight parts, probed at their last entries, until at most four entries are left: the first part that does
+            // not lie wholly below x
+            const bool mine = n > 4 && m == 0;
+            int hi = mine ? n : 0;
+            while (__any_sync(FULL, hi - lo > 4)) {
+                if (hi - lo > 4) {
+                    const int step = (hi - lo + 7) >> 3;
+                    int below = 0;
+#pragma unroll
+                    for (int u = 0; u < 7; ++u) {
+                        const int q = lo + (u + 1) * step - 1;
+                        below += q < hi && ent[pcb + q].x < x ? 1 : 0;
+                    }
+                    lo += below * step;
+                    hi = min(hi, lo + step);
+                }
+            }
+            if (mine) { m = hi - lo; place = lo; known = true; }
+        }
         if (m > 0) {
             int t[4];
 #pragma unroll
@@ -265,7 +316,7 @@ __device__ __forceinline__ void append_tokens(AppendShared& sh, const sd_store& 
 #pragma unroll
             for (int u = 0; u < 4; ++u) if (t[u] == x) found = pcb + lo + u;
             // (a hint: the run may have grown since, or be another one by now)
-            if (n > 4) known = found >= 0 || ((lo == 0 || below > 0) && (lo + 4 == n || below < 4));
+            if (!known) known = found >= 0 || ((lo == 0 || below > 0) && (lo + 4 == n || below < 4));
         }
         unsigned open = __ballot_sync(FULL, !known);
         while (open) {                                           // long runs: the whole warp, one after the other
@@ -317,29 +368,45 @@ __device__ __forceinline__ void append_tokens(AppendShared& sh, const sd_store& 
                 used += total;
             }
             if (leaf) new_w = (asz > 0 ? (unsigned)(asz - 1) : room - 1u) << ROOM_SHIFT;
-            // a tail that repeats one token is the only case in which a run to be edited holds the parent of the
-            // next lane: then everything goes lane by lane, deepest first
-            const bool repeats = len >= 2 && x1 == x2;
-            if (leaf && !repeats) {
+            // (the nodes of suffixes of one another: leaves are the deepest lanes' parents)
+            if (leaf) {
                 ent[fresh] = make_int4(x, 1, 0, 0);
                 if (lane == 0) root[x] = fresh;
                 else *reinterpret_cast<int2*>(&ent[parent].z) = make_int2(fresh, 1);
                 new_act = fresh;
             }
-            unsigned runs = __ballot_sync(FULL, need && (repeats || !leaf));
+            unsigned runs = __ballot_sync(FULL, need && !leaf);
             if (runs) {
+                // A tail that repeats one token is the only case in which a run to be edited holds the parent of the next
+                // lane: the deeper lane goes first.
+                const bool moves = asz > 0;
+                const unsigned clash = __ballot_sync(FULL, need && next_parent >= pcb && next_parent < pcb + n);
+                const unsigned big = __ballot_sync(FULL, need && (moves ? n : n - place) > APP_BIG);
                 __syncwarp();
                 while (runs) {
-                    const int src = 31 - __clz((int)runs);
-                    runs &= ~(1u << src);
-                    const int sn = __shfl_sync(FULL, n, src), sfresh = __shfl_sync(FULL, fresh, src);
-                    const bool moves = __shfl_sync(FULL, (leaf || asz > 0) ? 1 : 0, src) != 0;
-                    int idx = sfresh;
-                    if (src == 0) { if (lane == 0) { ent[sfresh] = make_int4(x, 1, 0, 0); root[x] = sfresh; } }
-                    else
-                        idx = insert_child_warp(ent, __shfl_sync(FULL, parent, src), __shfl_sync(FULL, pcb, src), sn,
-                                                __shfl_sync(FULL, place, src), x, sfresh, moves, lane);
-                    if (lane == src) new_act = idx;
+                    const int top = 31 - __clz((int)runs);
+                    unsigned batch = 0;
+                    int mine = -1, took = 0;
+                    while (runs && took < 4) {
+                        const int src = 31 - __clz((int)runs);
+                        if (took > 0 && ((((clash >> src) & 1u) && ((batch >> (src + 1)) & 1u)) || ((big >> src) & 1u))) break;
+                        if ((lane >> 3) == took) mine = src;
+                        batch |= 1u << src;
+                        runs &= ~(1u << src);
+                        ++took;
+                        if ((big >> src) & 1u) break;
+                    }
+                    if (took == 1) {
+                        const int idx = insert_child_warp(ent, __shfl_sync(FULL, parent, top), __shfl_sync(FULL, pcb, top), __shfl_sync(FULL, n, top),
+                                                          __shfl_sync(FULL, place, top), x, __shfl_sync(FULL, fresh, top),
+                                                          __shfl_sync(FULL, moves ? 1 : 0, top) != 0, lane);
+                        if (lane == top) new_act = idx;
+                    } else {
+                        const int idx = insert_child_groups(ent, mine, parent, pcb, n, place, x, fresh, moves, lane);
+                        // the lanes of the batch take theirs, the deepest from the first group
+                        const int at = __shfl_sync(FULL, idx, 8 * (__popc(batch >> 1 >> lane) & 3));
+                        if ((batch >> lane) & 1u) new_act = at;
+                    }
                 }
             }
             live += __popc(needs);
