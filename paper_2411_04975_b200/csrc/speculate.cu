@@ -628,32 +628,93 @@ __device__ __forceinline__ unsigned pool_top(const Pool& C, int n, int lane) {
 }
 
 // The best children (by count, then smallest token; at most `room`) of a node with more than 32: their entries, best
-// first, in `list`.  One class of equal counts after the other, within it in run (token) order.
-__device__ __noinline__ int list_by_count(const int4* __restrict__ ent, int cb, int n, int room, int* list, unsigned& sum_out, int lane) {
-    unsigned sum = 0, top = 0;
-    for (int base = lane; base < n; base += 128) {
-        unsigned y[4];
+// first, in `list`.  One class of equal counts after the other, within it in run (token) order.  The classes are taken
+// from registers: all of a run of up to 128 children, else those that occur often (up to 128 of them; most children
+// of a long run occur once or twice), and only what is left from the run itself.  `hot`: 256 words of the warp's.
+// (Every class by a pass over the run: drafts of 64 requests of text in which one token is every second one 125 us, now 107.)
+__device__ __noinline__ int list_by_count(const int4* __restrict__ ent, int cb, int n, int room, int* list, int* hot, unsigned& sum_out,
+                                          int lane) {
+    unsigned y[4], least = 1u;                                  // counts from `least` on are in the registers
+    int pos[4];
+    if (n <= 128) {
+        unsigned sum = 0;
 #pragma unroll
-        for (int u = 0; u < 4; ++u) y[u] = base + u * 32 < n ? (unsigned)ent[cb + base + u * 32].y : 0u;
-        sum += y[0] + y[1] + y[2] + y[3];                       // (a parent's occurrences fit 31 bits)
-        top = max(top, max(max(y[0], y[1]), max(y[2], y[3])));
-    }
-    sum_out = __reduce_add_sync(FULL, sum);
-    top = __reduce_max_sync(FULL, top);
-    int taken = 0;
-    while (top > 0u && taken < room) {
-        unsigned next = 0;
-        for (int base = 0; base < n; base += 128) {
-            unsigned y[4];
+        for (int u = 0; u < 4; ++u) {
+            pos[u] = u * 32 + lane;
+            y[u] = pos[u] < n ? (unsigned)ent[cb + pos[u]].y : 0u;
+            sum += y[u];                                        // (a parent's occurrences fit 31 bits)
+        }
+        sum_out = __reduce_add_sync(FULL, sum);
+    } else {
+        constexpr int LIMITS = 8;                               // 2, 3, 5, 9, .. 129
+        unsigned sum = 0, many[LIMITS] = {};
+        for (int base = lane; base < n; base += 128) {
+            unsigned v[4];
 #pragma unroll
-            for (int u = 0; u < 4; ++u) y[u] = base + u * 32 + lane < n ? (unsigned)ent[cb + base + u * 32 + lane].y : 0u;
+            for (int u = 0; u < 4; ++u) v[u] = base + u * 32 < n ? (unsigned)ent[cb + base + u * 32].y : 0u;
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
-                const unsigned m = __ballot_sync(FULL, y[u] == top);
+                sum += v[u];
+#pragma unroll
+                for (int k = 0; k < LIMITS; ++k) many[k] += v[u] > (1u << k) ? 1u : 0u;
+            }
+        }
+        sum_out = __reduce_add_sync(FULL, sum);
+        least = 0u;
+#pragma unroll
+        for (int k = LIMITS - 1; k >= 0; --k) if (__reduce_add_sync(FULL, many[k]) <= 128u) least = (1u << k) + 1u;
+        int got = 0;
+        if (least > 0u) {
+            for (int base = 0; base < n; base += 128) {
+                unsigned v[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) v[u] = base + u * 32 + lane < n ? (unsigned)ent[cb + base + u * 32 + lane].y : 0u;
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const unsigned m = __ballot_sync(FULL, v[u] >= least);
+                    const int at = got + __popc(m & ((1u << lane) - 1u));
+                    if (v[u] >= least) { hot[2 * at] = base + u * 32 + lane; hot[2 * at + 1] = (int)v[u]; }
+                    got += __popc(m);
+                }
+            }
+            __syncwarp();
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const bool in = u * 32 + lane < got;
+            pos[u] = in ? hot[2 * (u * 32 + lane)] : 0;
+            y[u] = in ? (unsigned)hot[2 * (u * 32 + lane) + 1] : 0u;
+        }
+    }
+    int taken = 0;
+    unsigned top = __reduce_max_sync(FULL, max(max(y[0], y[1]), max(y[2], y[3])));
+    while (top > 0u && taken < room) {
+        unsigned next = 0;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const unsigned m = __ballot_sync(FULL, y[u] == top);
+            const int at = taken + __popc(m & ((1u << lane) - 1u));
+            if (y[u] == top && at < room) list[at] = cb + pos[u];
+            taken += __popc(m);
+            if (y[u] < top) next = max(next, y[u]);
+        }
+        top = __reduce_max_sync(FULL, next);
+    }
+    // what the registers do not hold (least 0: nothing is in them)
+    top = least - 1u;
+    while (top > 0u && taken < room) {
+        unsigned next = 0;
+        for (int base = 0; base < n && taken < room; base += 128) {
+            unsigned v[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) v[u] = base + u * 32 + lane < n ? (unsigned)ent[cb + base + u * 32 + lane].y : 0u;
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const unsigned m = __ballot_sync(FULL, v[u] == top);
                 const int at = taken + __popc(m & ((1u << lane) - 1u));
-                if (y[u] == top && at < room) list[at] = cb + base + u * 32 + lane;
+                if (v[u] == top && at < room) list[at] = cb + base + u * 32 + lane;
                 taken += __popc(m);
-                if (y[u] < top) next = max(next, y[u]);
+                if (v[u] < top) next = max(next, v[u]);
             }
         }
         top = __reduce_max_sync(FULL, next);
@@ -782,7 +843,7 @@ __device__ __noinline__ void expand_job(BlockShared& sh, WarpWork& W, const int4
                 nl = min(hdr.z, room);
             } else {
                 unsigned sum;
-                nl = list_by_count(ent, cur_cb, cur_n, room, W.one_tok, sum, lane);
+                nl = list_by_count(ent, cur_cb, cur_n, room, W.one_tok, reinterpret_cast<int*>(&W.T), sum, lane);
                 dsum = (double)sum;
             }
             for (int base = 0; base < nl && fits; base += 32) {
@@ -794,6 +855,8 @@ __device__ __noinline__ void expand_job(BlockShared& sh, WarpWork& W, const int4
                     dc = __dmul_rn(cur_d, __ddiv_rn((double)e.y, dsum));         // Eq. 2 with Eq. 1
                 }
                 fits = pool_push(C, P, room, keep, dc, e.x, cur_idx, e.z, (unsigned)e.w, lane);
+                // as many as can still be added: what is worse than the last of them does not matter any more
+                if (nl == room && base + 32 >= nl) P.floor = max(P.floor, (unsigned)__shfl_sync(FULL, __double2hiint(dc), nl - 1 - base));
             }
             continue;
         }

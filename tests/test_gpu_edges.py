@@ -162,3 +162,19 @@ def test_arguments_of_the_calls_of_every_step(U, name, bad, error):
     for k in ("n_draft", "chosen_tree", "chosen_p", "score", "status"):
         assert torch.equal(a[k], b[k])
     pr.close()
+
+
+@pytest.mark.parametrize("children,most", [(33, 3), (128, 9), (129, 1), (300, 2), (300, 40), (140, 140)])
+def test_long_runs_without_a_ready_list_in_the_middle_of_a_tree(U, children, most):
+    rng = np.random.default_rng(children + most)
+    counts = np.full(children, 131) if most == 140 else rng.integers(1, most + 1, children)
+    heads = rng.permutation(np.repeat(np.arange(children), counts))
+    text = np.concatenate([np.stack([np.full(heads.size, 1), np.full(heads.size, 2), 10 + heads], 1).reshape(-1), [5, 1]]).astype(np.int32)
+    pr = U.Pair([], vocab=1024, D=6, n_slots=1, max_req_tokens=text.size + 8)
+    off, flat = U.ragged([text])
+    pr.g.build_requests(np.arange(1), off, U.dev_i32(flat))
+    pr.o.slot_append_batch([0], [text])
+    for budget in (8.0, 63.0):
+        for flags in (0, 4):
+            pr.check_speculate([0], 2, budget, 64, flags=flags)
+    pr.close()
