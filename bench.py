@@ -36,7 +36,7 @@ UNIT = "trees/s"
 OUT_BYTES_PER_REQ = 4 * 64 * 3 + 64 * 8 + 4 * 3 + 8          # tokens, parents, positions, mask, scalars
 FLUSH_BYTES = 256 << 20
 APPEND_BYTES_PER_UPDATE = 32                                   # a node's 16-byte entry read and written back
-STEP_KERNEL = "speculate_fused_kernel<true, 10, 2, 4> (all of sd_step)"
+STEP_KERNEL = "speculate_fused_kernel<true, 14, 2> (all of sd_step)"
 # dram__bytes_read + dram__bytes_write of one launch of that kernel on the full-size large_batch
 # workload, from an ncu capture; it is reported only while the kernel source still has the
 # digest the capture was taken at (profiles/ holds the summary), else as null

@@ -280,13 +280,13 @@ __global__ void select_emit_kernel(sd_store sv, int n, const int32_t* __restrict
 
 // ---------------------------------------------------------------------------------------------
 // Fused path: one block of W warps per request (the kernel itself is described where it is
-// defined).  Two blocks per SM is the usual shape.  A batch
-// of at most one request per SM gets bigger blocks (W = 24 / 16), a batch of more than two
-// requests per SM smaller ones (W = 8 / 5, four per SM) to stay in one wave.
+// defined).  Two blocks per SM is the usual shape.  A batch of at most one request per SM gets blocks with
+// more registers, a batch of more than two requests per SM smaller ones (four per SM) to stay in one wave.
 constexpr int CTA_WARPS = 14;                  // the usual block; 256 requests: 44.2 us (10 warps 51.5, 12 52.1, 13 45.6, 15 48.9, 16 49.3)
 constexpr int CTA_WARPS_STEP = 14;             // of sd_step: 58.6 us per step (8 warps 63.1, 10 60.1, 12 59.2, 16 58.6)
-constexpr int CTA_WARPS_WIDE = 24;             // small batches (one block per SM at most): the block has the SM's
-constexpr int CTA_WARPS_WIDE_STEP = 16;        // registers to itself (80 per thread; sd_step: 128)
+// one block per SM at most, 128 registers per thread: nothing is spilled.  Drafts of 64 requests with long runs 95 us (24 warps of 80
+// registers 107, 20 106, 12 108), of one request 7.3 (8.0, 7.6, 7.1); steps of 64 requests 47.4 (12 warps 49.2, 20 48.7)
+constexpr int CTA_WARPS_WIDE = 16;
 constexpr int CTA_WARPS_NARROW = 8;            // batches of more than two requests per SM: four blocks per SM
 constexpr int CTA_WARPS_NARROW_STEP = 5;       // (sd_step: 96 registers)
 
@@ -1337,7 +1337,7 @@ int device_setup(int dev, int* sm_count) {
     std::lock_guard<std::mutex> lock(g_dev_mutex);
     if (!g_dev[dev].ready) {
         if (raise_smem_limit<false, CTA_WARPS, 2>() != SD_OK || raise_smem_limit<true, CTA_WARPS_STEP, 2>() != SD_OK ||
-            raise_smem_limit<false, CTA_WARPS_WIDE, 1>() != SD_OK || raise_smem_limit<true, CTA_WARPS_WIDE_STEP, 1>() != SD_OK ||
+            raise_smem_limit<false, CTA_WARPS_WIDE, 1>() != SD_OK || raise_smem_limit<true, CTA_WARPS_WIDE, 1>() != SD_OK ||
             raise_smem_limit<false, CTA_WARPS_NARROW, 4>() != SD_OK ||
             raise_smem_limit<true, CTA_WARPS_NARROW_STEP, 4>() != SD_OK)
             return SD_ERR_CUDA;
@@ -1370,18 +1370,16 @@ static int launch_fused(sd_store* s, int32_t n, const int32_t* d_slot, const sd_
     int sms = 0;
     const int rc = device_setup(s->device, &sms);
     if (rc != SD_OK) return rc;
-    // one block per SM is all a small batch can use: sd_speculate then takes more warps if a
-    // request has more jobs (two trees, Pe pattern lengths each) than 16 warps start at once,
-    // sd_step takes more registers
-    const bool wide = n <= sms && (step || 2 * Pe > 2 * CTA_WARPS);
-    // more requests than two 16-warp blocks per SM hold at once: smaller blocks, one wave
+    // one block per SM is all a small batch can use: it takes more registers
+    const bool wide = n <= sms;
+    // more requests than two blocks per SM hold at once: smaller blocks, one wave
     const bool narrow = n > 2 * sms;
 #define SD_LAUNCH_FUSED(STEP, WARPS, MINB, OFF, TOK)                                                                     \
     SD_CUDA_OK(sd_launch(speculate_fused_kernel<STEP, WARPS, MINB>, (unsigned)n, WARPS * 32, sizeof(BlockSharedT<WARPS>), st, \
                          *s, n, d_slot, Pe, prm->alpha, prm->max_spec, prm->flags, prm->tau, d_budget_cap, d_n_draft, d_tokens, \
                          d_parents, d_positions, d_mask, d_chosen_tree, d_chosen_p, d_score, d_status, OFF, TOK))
     if (step) {
-        if (wide) SD_LAUNCH_FUSED(true, CTA_WARPS_WIDE_STEP, 1, d_app_off, d_app_tok);
+        if (wide) SD_LAUNCH_FUSED(true, CTA_WARPS_WIDE, 1, d_app_off, d_app_tok);
         else if (narrow) SD_LAUNCH_FUSED(true, CTA_WARPS_NARROW_STEP, 4, d_app_off, d_app_tok);
         else SD_LAUNCH_FUSED(true, CTA_WARPS_STEP, 2, d_app_off, d_app_tok);
     } else {
