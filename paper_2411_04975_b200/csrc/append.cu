@@ -664,7 +664,7 @@ append_kernel(sd_store sv, const int32_t* d_slot, const int64_t* d_offsets, cons
             __syncthreads();
         }
         if (wib == 0) {
-            append_tokens(sh, sv, slot, tok + k, m, 1, lane, act, cb, w, len, used, live, status);
+            append_tokens<true>(sh, sv, slot, tok + k, m, 1, lane, act, cb, w, len, used, live, status);
             if (lane == 0) { sh_len = len; sh_status = status; }
         }
         __syncthreads();

@@ -1085,7 +1085,7 @@ speculate_fused_kernel(sd_store sv, int n, const int32_t* __restrict__ d_slot, i
             if (!(st & (SD_STATUS_POOL_FULL | SD_STATUS_BAD_TOKEN))) {
                 int act = ss->active[lane], cb = ss->run_cb[lane];
                 unsigned w = append_pack(ss->run_w[lane], ss->room[lane]);
-                append_tokens(sh.app, sv, slot, newtok, n_new, GWARPS, lane, act, cb, w, len, used, live, st);
+                append_tokens<(MINB < 4)>(sh.app, sv, slot, newtok, n_new, GWARPS, lane, act, cb, w, len, used, live, st);
                 append_store(ss, lane, act, cb, w);
             }
             if (lane == 0) { ss->len = len; ss->used = used; ss->live = live; ss->status = st; }
