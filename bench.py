@@ -40,7 +40,7 @@ STEP_KERNEL = "speculate_fused_kernel<true, 14, 2> (all of sd_step)"
 # dram__bytes_read + dram__bytes_write of one launch of that kernel on the full-size large_batch
 # workload, from an ncu capture; it is reported only while the kernel source still has the
 # digest the capture was taken at (profiles/ holds the summary), else as null
-DRAM_TRAFFIC = {"bytes": 28.03e6, "speculate_cu_sha1": "7370e8a536030ddfd449f3b9c42399bd02e1033a"}
+DRAM_TRAFFIC = {"bytes": 16.43e6, "speculate_cu_sha1": "5e1498cbddb7d4a17e19560384e9d6655c204530"}
 
 
 def dram_traffic():
