@@ -10,7 +10,7 @@ _ROOT = os.path.dirname(_HERE)
 CSRC = os.path.join(_HERE, "csrc")
 LIB = os.path.join(_HERE, "libsuffixspec.so")
 CALL = os.path.join(_HERE, "_call.so")
-SOURCES = ["build.cu", "append.cu", "speculate.cu", "query.cu"]
+SOURCES = ["build.cu", "append.cu", "speculate.cu", "query.cu", "memory.cpp"]
 
 
 def _newest_source() -> float:
@@ -19,7 +19,7 @@ def _newest_source() -> float:
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
-    """Compile csrc/*.cu into libsuffixspec.so (cross-compiles without a GPU) and csrc/call.cpp into the
+    """Compile SOURCES into libsuffixspec.so (cross-compiles without a GPU) and csrc/call.cpp into the
     module _call.  Returns the library's path."""
     newest = _newest_source()
 

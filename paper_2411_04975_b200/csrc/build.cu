@@ -5,19 +5,16 @@
 // Hand-written LSD radix sort and scans (no CUB / Thrust).
 // Also: sd_build_requests (the trees of a batch of new requests by the same pipeline).
 #include <algorithm>
-#include <chrono>
-#include <mutex>
 #include <new>
 #include <stdio.h>
 #include <string.h>
-
-#include <unordered_map>
 #include <vector>
 
 #include <cooperative_groups.h>
 
 #include "append_core.cuh"
 #include "global_insert.cuh"
+#include "memory.h"
 #include "suffix_order.cuh"
 
 namespace cg = cooperative_groups;
@@ -900,167 +897,6 @@ __global__ void init_global_state_kernel(GlobalState* g, int used, int live, lon
     g->used = used; g->live = live; g->status = 0; g->epoch = 1; g->tokens = tokens;
 }
 
-}  // namespace
-
-// Device memory: blocks that stores and builds have given back are kept for the next ones, up to 1/32 of the
-// device's memory (5.7 GB of a B200's); the oldest go first when there are more, all of them when an allocation
-// fails (which is then tried once more), and those that nobody has wanted for half a minute.  Getting
-// and returning memory is what a build or a short-lived store would otherwise spend its time on: 20
-// cudaMalloc / cudaFree calls took 2.7 ms of the 3.7 ms of a 32,768-token build and up to 70 ms of a
-// 4 M-token one.  (CUDA's own stream-ordered pools cost 6.2 ms per GB whenever they grow or shrink, cudaMalloc
-// 0.3 - 0.8 ms at any of these sizes.)  A block is given back when the work on it has ended, so the next owner may be
-// on any stream or thread.
-//
-// Test hook: the k-th device allocation from now on fails (k = 1: the next one); 0 switches it off.
-// Only the allocation-failure tests use it.  While it is on nothing is kept.
-namespace {
-
-constexpr int CACHE_DEVICES = 64;
-constexpr int CACHE_FRACTION = 32;
-constexpr double CACHE_SECONDS = 30.0;
-constexpr int KEPT_STREAMS = 8;
-
-typedef std::chrono::steady_clock Clock;
-// What a store holds besides device memory: a stream and events, and pinned memory for the arguments of sd_build_requests.
-struct StreamSet { cudaStream_t aux; cudaEvent_t ev_fork, ev_join, ev_check; void* stage; size_t stage_bytes; };
-struct FreeBlock { void* p; size_t bytes; Clock::time_point since; };
-struct DeviceCache {
-    std::vector<FreeBlock> idle;                      // oldest first
-    size_t bytes = 0, most = 0;
-    StreamSet streams[KEPT_STREAMS];                  // of freed stores, for the next ones
-    int n_streams = 0;
-};
-struct OwnedBlock { size_t bytes; int dev; };
-DeviceCache g_cache[CACHE_DEVICES];
-std::unordered_map<void*, OwnedBlock> g_owned;        // blocks in use
-std::mutex g_cache_mutex;
-long long g_fail_alloc_in = 0;
-bool g_fail_alloc_on = false;
-
-// gives back the oldest blocks until at most `bytes` are kept (the mutex is held)
-void cache_trim(DeviceCache& c, size_t bytes) {
-    size_t n = 0;
-    while (n < c.idle.size() && c.bytes > bytes) { cudaFree(c.idle[n].p); c.bytes -= c.idle[n].bytes; ++n; }
-    c.idle.erase(c.idle.begin(), c.idle.begin() + n);
-}
-
-void cache_expire(DeviceCache& c) {
-    const Clock::time_point now = Clock::now();
-    size_t n = 0;
-    while (n < c.idle.size() && std::chrono::duration<double>(now - c.idle[n].since).count() > CACHE_SECONDS) {
-        cudaFree(c.idle[n].p);
-        c.bytes -= c.idle[n].bytes;
-        ++n;
-    }
-    c.idle.erase(c.idle.begin(), c.idle.begin() + n);
-}
-
-void drop_streams(const StreamSet& s) {
-    for (cudaEvent_t e : {s.ev_fork, s.ev_join, s.ev_check}) if (e) cudaEventDestroy(e);
-    if (s.aux) cudaStreamDestroy(s.aux);
-    if (s.stage) cudaFreeHost(s.stage);
-}
-
-// for a store on the current device, with at least `stage_bytes` of pinned memory
-bool take_streams(int dev, size_t stage_bytes, StreamSet* out) {
-    if (dev >= 0 && dev < CACHE_DEVICES) {
-        std::lock_guard<std::mutex> lock(g_cache_mutex);
-        DeviceCache& d = g_cache[dev];
-        for (int k = d.n_streams - 1; k >= 0; --k)
-            if (d.streams[k].stage_bytes >= stage_bytes) {
-                *out = d.streams[k];
-                d.streams[k] = d.streams[--d.n_streams];
-                return true;
-            }
-    }
-    memset(out, 0, sizeof(*out));
-    out->stage_bytes = std::max<size_t>(stage_bytes, 16384);
-    if (cudaStreamCreateWithFlags(&out->aux, cudaStreamNonBlocking) == cudaSuccess &&
-        cudaEventCreateWithFlags(&out->ev_fork, cudaEventDisableTiming) == cudaSuccess &&
-        cudaEventCreateWithFlags(&out->ev_join, cudaEventDisableTiming) == cudaSuccess &&
-        cudaEventCreateWithFlags(&out->ev_check, cudaEventDisableTiming) == cudaSuccess &&
-        cudaHostAlloc(&out->stage, out->stage_bytes, cudaHostAllocPortable | cudaHostAllocMapped) == cudaSuccess)
-        return true;
-    cudaGetLastError();
-    drop_streams(*out);
-    return false;
-}
-
-void give_streams(int dev, const StreamSet& s) {
-    {
-        std::lock_guard<std::mutex> lock(g_cache_mutex);
-        if (dev >= 0 && dev < CACHE_DEVICES && g_cache[dev].n_streams < KEPT_STREAMS) {
-            g_cache[dev].streams[g_cache[dev].n_streams++] = s;
-            return;
-        }
-    }
-    drop_streams(s);
-}
-
-}  // namespace
-
-cudaError_t sd_device_malloc(void** p, size_t bytes) {
-    *p = nullptr;
-    if (g_fail_alloc_in > 0 && --g_fail_alloc_in == 0) return cudaErrorMemoryAllocation;
-    int dev = -1;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    if (dev < 0 || dev >= CACHE_DEVICES) return cudaErrorInvalidDevice;
-    // (up to a multiple of an eighth of the next lower power of two, 32 MB at most, so that sizes that differ a little share blocks)
-    size_t unit = 512;
-    while (unit * 16 <= bytes && unit < (32u << 20)) unit *= 2;
-    bytes = (bytes + unit - 1) / unit * unit;
-    std::lock_guard<std::mutex> lock(g_cache_mutex);
-    DeviceCache& c = g_cache[dev];
-    if (!g_fail_alloc_on) {
-        cache_expire(c);
-        // the smallest kept block that is not much too large
-        size_t best = c.idle.size();
-        for (size_t k = 0; k < c.idle.size(); ++k)
-            if (c.idle[k].bytes >= bytes && c.idle[k].bytes <= bytes + bytes / 4 && (best == c.idle.size() || c.idle[k].bytes < c.idle[best].bytes))
-                best = k;
-        if (best < c.idle.size()) {
-            *p = c.idle[best].p;
-            g_owned[*p] = OwnedBlock{c.idle[best].bytes, dev};
-            c.bytes -= c.idle[best].bytes;
-            c.idle.erase(c.idle.begin() + best);
-            return cudaSuccess;
-        }
-    }
-    e = cudaMalloc(p, bytes);
-    if (e != cudaSuccess && !c.idle.empty()) {
-        cudaGetLastError();
-        cache_trim(c, 0);
-        e = cudaMalloc(p, bytes);
-    }
-    if (e != cudaSuccess) { *p = nullptr; return e; }
-    g_owned[*p] = OwnedBlock{bytes, dev};
-    return cudaSuccess;
-}
-
-void sd_device_free(void* p) {
-    if (!p) return;
-    std::lock_guard<std::mutex> lock(g_cache_mutex);
-    auto it = g_owned.find(p);
-    if (it == g_owned.end()) return;
-    const OwnedBlock b = it->second;
-    g_owned.erase(it);
-    DeviceCache& c = g_cache[b.dev];
-    if (c.most == 0) {
-        size_t free_bytes = 0, total = 0;
-        if (cudaMemGetInfo(&free_bytes, &total) == cudaSuccess) c.most = total / CACHE_FRACTION;
-    }
-    if (g_fail_alloc_on || b.bytes > c.most) { cudaFree(p); return; }
-    cache_expire(c);
-    cache_trim(c, c.most - b.bytes);
-    c.idle.push_back(FreeBlock{p, b.bytes, Clock::now()});
-    c.bytes += b.bytes;
-}
-
-extern "C" void sd_debug_fail_alloc(int64_t k) { g_fail_alloc_in = k; g_fail_alloc_on = k > 0; }
-
-namespace {
-
 struct DeviceArena {          // temporaries of one build: freed together, or kept in a workspace
     void* ptr[48];
     int n = 0;
@@ -1134,20 +970,6 @@ static bool store_alloc(sd_store* s, T** out, long long count) {
     s->device_bytes += count * (long long)sizeof(T);
     *out = (T*)p;
     return true;
-}
-
-// Releases what a store holds, behind the work on `st`: the caller has waited for every other stream that used the store.
-static void store_release(sd_store* s, cudaStream_t st) {
-    if (!s) return;
-    cudaStreamSynchronize(st);
-    void* const own[] = {s->g_ent, s->g_root, s->g_state, s->gi, s->s_ent, s->s_root, s->s_text, s->s_state};
-    for (void* p : own) sd_device_free(p);
-    if (s->ws) {
-        for (int k = 0; k < 48; ++k) sd_device_free(s->ws->ptr[k]);
-        delete s->ws;
-    }
-    if (s->aux) give_streams(s->device, StreamSet{s->aux, s->ev_fork, s->ev_join, s->ev_check, s->stage, s->stage_bytes});
-    delete s;
 }
 
 // Everything up to the writing of the entries, for one array of sequences: suffix order and the sweeps over it.
@@ -1266,15 +1088,15 @@ extern "C" int sd_build(const sd_build_params* p, const int32_t* d_corpus, const
     bool ok = store_alloc(s, &s->g_root, s->V) && store_alloc(s, &s->g_state, 1) && store_alloc(s, &s->gi, 1) &&
               store_alloc(s, &s->s_ent, (i64)s->R * s->spn) && store_alloc(s, &s->s_root, (i64)s->R * s->V) &&
               store_alloc(s, &s->s_text, (i64)s->R * s->T) && store_alloc(s, &s->s_state, s->R);
-    if (!ok) { store_release(s, st); return SD_ERR_NOMEM; }
+    if (!ok) { sd_store_release(s, st); return SD_ERR_NOMEM; }
     StreamSet streams;
-    if (!take_streams(s->device, stage_bytes_for(s->R), &streams)) { store_release(s, st); return SD_ERR_CUDA; }
+    if (!sd_take_streams(s->device, stage_bytes_for(s->R), &streams)) { sd_store_release(s, st); return SD_ERR_CUDA; }
     s->aux = streams.aux; s->ev_fork = streams.ev_fork; s->ev_join = streams.ev_join; s->ev_check = streams.ev_check;
     s->stage = streams.stage; s->stage_bytes = streams.stage_bytes;
     cudaError_t ce = cudaMemsetAsync(s->g_root, 0xFF, sizeof(int32_t) * (size_t)s->V, st);
     if (ce == cudaSuccess) ce = cudaMemsetAsync(s->s_root, 0xFF, sizeof(int32_t) * (size_t)s->R * s->V, st);
     if (ce == cudaSuccess) ce = cudaMemsetAsync(s->s_state, 0, sizeof(SlotState) * (size_t)s->R, st);
-    if (ce != cudaSuccess) { store_release(s, st); return SD_ERR_CUDA; }
+    if (ce != cudaSuccess) { sd_store_release(s, st); return SD_ERR_CUDA; }
 
     Pipeline P(st);
     const int T256 = 256;
@@ -1285,39 +1107,39 @@ extern "C" int sd_build(const sd_build_params* p, const int32_t* d_corpus, const
         {
             int* bad = nullptr;
             int h_bad = 0;
-            if (!P.tmp.get(&bad, 1)) { store_release(s, st); return SD_ERR_NOMEM; }
+            if (!P.tmp.get(&bad, 1)) { sd_store_release(s, st); return SD_ERR_NOMEM; }
             ce = cudaMemsetAsync(bad, 0, sizeof(int), st);
             validate_kernel<<<grid_for(std::max<i64>(N, n_seqs), T256), T256, 0, st>>>(d_corpus, N, s->V, d_seq_offsets,
                                                                                       n_seqs, bad);
             if (ce == cudaSuccess) ce = cudaMemcpyAsync(&h_bad, bad, sizeof(int), cudaMemcpyDeviceToHost, st);
             if (ce == cudaSuccess) ce = cudaStreamSynchronize(st);
-            if (ce != cudaSuccess) { store_release(s, st); return SD_ERR_CUDA; }
-            if (h_bad) { store_release(s, st); return SD_ERR_INVALID_ARG; }
+            if (ce != cudaSuccess) { sd_store_release(s, st); return SD_ERR_CUDA; }
+            if (h_bad) { sd_store_release(s, st); return SD_ERR_INVALID_ARG; }
         }
         const int rc = pipeline_run(P, d_corpus, d_seq_offsets, n_seqs, N, s->V, D, true, st);
-        if (rc != SD_OK) { store_release(s, st); return rc; }
+        if (rc != SD_OK) { sd_store_release(s, st); return rc; }
         int h_s = 0, h_n1 = 0;
         ce = cudaMemcpyAsync(&h_s, P.ts.s + P.ts.tiles, sizeof(int), cudaMemcpyDeviceToHost, st);
         if (ce == cudaSuccess) ce = cudaMemcpyAsync(&h_n1, P.ts.n1 + P.ts.tiles, sizeof(int), cudaMemcpyDeviceToHost, st);
         if (ce == cudaSuccess) ce = cudaMemcpyAsync(h_wide, P.ts.wide, 2 * sizeof(int), cudaMemcpyDeviceToHost, st);
         if (ce == cudaSuccess) ce = cudaStreamSynchronize(st);
-        if (ce != cudaSuccess) { store_release(s, st); return SD_ERR_CUDA; }
+        if (ce != cudaSuccess) { sd_store_release(s, st); return SD_ERR_CUDA; }
         n_nodes = (i64)h_s + h_n1;
         used_entries = n_nodes + h_wide[1];                     // (a long run leaves its first place empty)
-        if (h_wide[0] > 0 && !P.tmp.get(&wide_list, h_wide[0])) { store_release(s, st); return SD_ERR_NOMEM; }
+        if (h_wide[0] > 0 && !P.tmp.get(&wide_list, h_wide[0])) { sd_store_release(s, st); return SD_ERR_NOMEM; }
     }
 
     i64 extra = p->global_extra_nodes >= 0 ? p->global_extra_nodes : std::max<i64>(1ll << 22, n_nodes);
     s->g_cap = used_entries + extra;
-    if (s->g_cap >= (1ll << 31) - 2) { store_release(s, st); return SD_ERR_INVALID_ARG; }
-    if (!store_alloc(s, &s->g_ent, s->g_cap)) { store_release(s, st); return SD_ERR_NOMEM; }
+    if (s->g_cap >= (1ll << 31) - 2) { sd_store_release(s, st); return SD_ERR_INVALID_ARG; }
+    if (!store_alloc(s, &s->g_ent, s->g_cap)) { sd_store_release(s, st); return SD_ERR_NOMEM; }
 
     if (N > 0) {
         TreeOut out;
         memset(&out, 0, sizeof(out));
         out.ent = s->g_ent; out.root = s->g_root; out.wide = wide_list;
         const int erc = emit_entries<false>(P.ts, out, st);
-        if (erc != SD_OK) { store_release(s, st); return erc; }
+        if (erc != SD_OK) { sd_store_release(s, st); return erc; }
         if (h_wide[0] > 0) {
             ts_wide_place_kernel<<<grid_for(h_wide[0], T256), T256, 0, st>>>(P.ts, wide_list, s->g_ent, (int)n_nodes);
             ts_wide_fill_kernel<<<(unsigned)h_wide[0], TOP_THREADS, 0, st>>>(wide_list, s->g_ent);
@@ -1326,15 +1148,9 @@ extern "C" int sd_build(const sd_build_params* p, const int32_t* d_corpus, const
     init_global_state_kernel<<<1, 1, 0, st>>>(s->g_state, (int)used_entries, (int)n_nodes, N);
     ce = cudaStreamSynchronize(st);
     if (ce == cudaSuccess) ce = cudaGetLastError();
-    if (ce != cudaSuccess) { store_release(s, st); return SD_ERR_CUDA; }
+    if (ce != cudaSuccess) { sd_store_release(s, st); return SD_ERR_CUDA; }
     *out = s;
     return SD_OK;
-}
-
-extern "C" void sd_free(sd_store* s) {
-    if (!s) return;
-    cudaDeviceSynchronize();
-    store_release(s, s->aux);
 }
 
 extern "C" const char* sd_strerror(int code) {
