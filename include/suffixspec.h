@@ -300,7 +300,10 @@ int sd_entropy(sd_store* store, int32_t tree, double* h_entropy, void* stream);
 /* sd_stats: store-wide figures into HOST memory.  Synchronises the stream. */
 int sd_stats(sd_store* store, sd_stats_t* out, void* stream);
 
-/* sd_free: release a store (NULL is a no-op).  Synchronises the device. */
+/*
+ * sd_free: release a store (NULL is a no-op).  Synchronises the device that owns the store, which
+ * need not be the current one; the current device stays as it is.
+ */
 void sd_free(sd_store* store);
 
 /* sd_strerror: static description of an SD_* return code. */

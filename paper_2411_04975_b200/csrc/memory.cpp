@@ -178,6 +178,12 @@ void sd_store_release(sd_store* s, cudaStream_t st) {
 
 extern "C" void sd_free(sd_store* s) {
     if (!s) return;
+    // What may still use the store runs on the device that owns it, whichever is current here (a garbage collector frees
+    // where it happens to run), and its memory goes on to the next store of that device as soon as it is released.
+    int current = -1;
+    const bool away = cudaGetDevice(&current) == cudaSuccess && current != s->device;
+    if (away) cudaSetDevice(s->device);
     cudaDeviceSynchronize();
     sd_store_release(s, s->aux);
+    if (away) cudaSetDevice(current);
 }
