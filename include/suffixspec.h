@@ -7,7 +7,10 @@
  * (cudaHostAlloc / cudaHostRegister, unified addressing) is accepted as it is,
  * and the kernels then read the few KB of inputs and write the drafts across
  * the bus themselves, which saves the copies before and after a step.  A store owns all of its device memory from
- * sd_build() until sd_free().  Calls are asynchronous on `stream` (a
+ * sd_build() until sd_free().  The library keeps memory that stores and builds have released for the next ones: at
+ * most 1/32 of a device's memory (and 8 streams with their events and pinned memory per device), for 30 seconds at
+ * most, after which a thread of the library's gives it back; sd_trim() gives it back at once, and so does a device
+ * allocation of the library's that fails.  Before cudaDeviceReset() call sd_trim().  Calls are asynchronous on `stream` (a
  * cudaStream_t passed as void*, NULL = default stream) unless stated; the
  * per-step calls (sd_append, sd_speculate) never allocate device memory.
  *
@@ -305,6 +308,12 @@ int sd_stats(sd_store* store, sd_stats_t* out, void* stream);
  * need not be the current one; the current device stays as it is.
  */
 void sd_free(sd_store* store);
+
+/*
+ * sd_trim: give back to the driver, on every device, what the library keeps of released stores
+ * (see above).  For a process that wants the memory for something else sooner than in 30 seconds.
+ */
+void sd_trim(void);
 
 /* sd_strerror: static description of an SD_* return code. */
 const char* sd_strerror(int code);

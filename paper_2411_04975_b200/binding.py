@@ -20,7 +20,7 @@ FLAG_GLOBAL_ONLY, FLAG_REQUEST_ONLY, FLAG_LINEAR = 1, 2, 4
 STATUS_BAD_SLOT, STATUS_POOL_FULL, STATUS_GLOBAL_FULL, STATUS_BAD_TOKEN = 1, 2, 4, 8
 
 EXPORTS = ["sd_build", "sd_build_requests", "sd_append", "sd_speculate", "sd_step", "sd_speculate_noalloc", "sd_query_counts",
-           "sd_enumerate", "sd_slot_info", "sd_entropy", "sd_stats", "sd_free", "sd_strerror", "sd_debug_fail_alloc"]
+           "sd_enumerate", "sd_slot_info", "sd_entropy", "sd_stats", "sd_free", "sd_trim", "sd_strerror", "sd_debug_fail_alloc"]
 
 
 class SuffixSpecError(RuntimeError):
@@ -84,6 +84,8 @@ def library() -> C.CDLL:
         lib.sd_stats.argtypes = [vp, C.POINTER(_Stats), vp]
         lib.sd_free.restype = None
         lib.sd_free.argtypes = [vp]
+        lib.sd_trim.restype = None
+        lib.sd_trim.argtypes = []
         lib.sd_debug_fail_alloc.restype = None
         lib.sd_debug_fail_alloc.argtypes = [C.c_int64]
         lib.sd_strerror.restype = C.c_char_p
@@ -175,6 +177,11 @@ def sd_speculate_noalloc(store: int, slots: torch.Tensor, P: int, alpha: float, 
 
 def sd_free(store: int) -> None:
     library().sd_free(store)
+
+
+def sd_trim() -> None:
+    """Give back the memory that is kept of freed stores (by itself that takes up to 30 seconds)."""
+    library().sd_trim()
 
 
 # ---- convenience wrapper ---------------------------------------------------------------------

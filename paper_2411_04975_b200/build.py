@@ -30,7 +30,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
         nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
         cmd = [nvcc, "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
                "-shared", "-Xcompiler", "-fPIC", "-I", os.path.join(_ROOT, "include"), "-I", CSRC,
-               "-cudart", "shared", "-o", LIB]
+               "-cudart", "shared", "-Xlinker", "-z", "-Xlinker", "nodelete", "-o", LIB]   # (a thread of memory.cpp outlives dlclose)
         if verbose:
             cmd += ["-Xptxas", "-v"]
         cmd += [os.path.join(CSRC, f) for f in SOURCES]

@@ -3,9 +3,15 @@
 #include <stdio.h>
 #include <stdlib.h>
 #include <string.h>
+#include <sys/wait.h>
+#include <unistd.h>
 
+#include <atomic>
+#include <chrono>
 #include <map>
 #include <mutex>
+#include <thread>
+#include <vector>
 
 #include "memory.h"
 
@@ -18,24 +24,38 @@ std::mutex mutex;
 std::map<void*, Block> blocks;
 bool busy[DEVICES];                                   // kernels of a caller's stream are still at work
 size_t used[DEVICES];
+int streams;                                          // in existence
+bool touched[DEVICES];                                // some thread made a call with this device current: it has a context
+std::atomic<bool> capturing{false}, spoilt{false};    // some thread captures a stream; a call of another thread broke that
 thread_local int current = 0;
+thread_local cudaStreamCaptureMode mode = cudaStreamCaptureModeGlobal;
+
+size_t all_used() {
+    std::lock_guard<std::mutex> l(mutex);
+    size_t n = 0;
+    for (size_t u : used) n += u;
+    return n + (size_t)streams;
+}
 }  // namespace fake
 
 extern "C" {
 cudaError_t cudaGetDevice(int* d) { *d = fake::current; return cudaSuccess; }
-cudaError_t cudaSetDevice(int d) { if (d < 0 || d >= fake::DEVICES) return cudaErrorInvalidDevice; fake::current = d; return cudaSuccess; }
+cudaError_t cudaSetDevice(int d) { if (d < 0 || d >= fake::DEVICES) return cudaErrorInvalidDevice; fake::current = d; fake::touched[d] = true; return cudaSuccess; }
 cudaError_t cudaDeviceSynchronize() { std::lock_guard<std::mutex> l(fake::mutex); fake::busy[fake::current] = false; return cudaSuccess; }
 cudaError_t cudaGetLastError() { return cudaSuccess; }
 cudaError_t cudaMalloc(void** p, size_t n) {
     std::lock_guard<std::mutex> l(fake::mutex);
     if (fake::used[fake::current] + n > fake::TOTAL) return cudaErrorMemoryAllocation;
     *p = malloc(1);
+    fake::touched[fake::current] = true;
     fake::blocks[*p] = fake::Block{fake::current, n};
     fake::used[fake::current] += n;
     return cudaSuccess;
 }
 cudaError_t cudaFree(void* p) {
     std::lock_guard<std::mutex> l(fake::mutex);
+    fake::touched[fake::current] = true;
+    if (fake::capturing && fake::mode == cudaStreamCaptureModeGlobal) fake::spoilt = true;
     auto it = fake::blocks.find(p);
     if (it == fake::blocks.end()) return cudaErrorInvalidValue;
     fake::busy[it->second.dev] = false;               // (it waits for the device that owns the memory)
@@ -46,8 +66,19 @@ cudaError_t cudaFree(void* p) {
 }
 cudaError_t cudaMemGetInfo(size_t* f, size_t* t) { *t = fake::TOTAL; *f = fake::TOTAL - fake::used[fake::current]; return cudaSuccess; }
 cudaError_t cudaStreamSynchronize(cudaStream_t) { return cudaSuccess; }
-cudaError_t cudaStreamCreateWithFlags(cudaStream_t* s, unsigned) { *s = (cudaStream_t)malloc(1); return cudaSuccess; }
-cudaError_t cudaStreamDestroy(cudaStream_t s) { free(s); return cudaSuccess; }
+cudaError_t cudaThreadExchangeStreamCaptureMode(cudaStreamCaptureMode* m) { std::swap(*m, fake::mode); return cudaSuccess; }
+cudaError_t cudaStreamCreateWithFlags(cudaStream_t* s, unsigned) {
+    std::lock_guard<std::mutex> l(fake::mutex);
+    ++fake::streams;
+    *s = (cudaStream_t)malloc(1);
+    return cudaSuccess;
+}
+cudaError_t cudaStreamDestroy(cudaStream_t s) {
+    std::lock_guard<std::mutex> l(fake::mutex);
+    --fake::streams;
+    free(s);
+    return cudaSuccess;
+}
 cudaError_t cudaEventCreateWithFlags(cudaEvent_t* e, unsigned) { *e = (cudaEvent_t)malloc(1); return cudaSuccess; }
 cudaError_t cudaEventDestroy(cudaEvent_t e) { free(e); return cudaSuccess; }
 cudaError_t cudaHostAlloc(void** p, size_t n, unsigned) { *p = malloc(n); return cudaSuccess; }
@@ -91,9 +122,106 @@ int free_waits_for_the_owner() {
     return 0;
 }
 
+bool given_back_within(double seconds) {
+    for (int k = 0; k < (int)(seconds * 100); ++k) {
+        if (fake::all_used() == 0) return true;
+        std::this_thread::sleep_for(std::chrono::milliseconds(10));
+    }
+    return false;
+}
+
+// Nothing is called any more after the last store was freed: what was kept of it goes back all the same, once it has been
+// kept for as long as that (SD_KEEP_SECONDS, here 0.3), with no context made on a device that had none.
+int kept_memory_goes_back_by_itself() {
+    for (int round = 0; round < 2; ++round) {
+        for (int dev = 1; dev < 3; ++dev) {
+            cudaSetDevice(dev);
+            sd_store* s = make_store(3 << 20);
+            EXPECT(s);
+            sd_free(s);
+        }
+        EXPECT(fake::all_used() > (6u << 20));               // (kept for the next store)
+        fake::capturing = true;
+        EXPECT(given_back_within(10));
+        EXPECT(!fake::spoilt);
+        fake::capturing = false;
+    }
+    EXPECT(!fake::touched[0] && fake::touched[1] && fake::touched[2] && !fake::touched[3]);
+    return 0;
+}
+
+// What a store has taken out of what was kept stays, however long it is used.
+int what_is_in_use_stays() {
+    sd_store* s = make_store(1 << 20);
+    sd_free(s);
+    std::this_thread::sleep_for(std::chrono::milliseconds(100));
+    s = make_store(1 << 20);
+    std::this_thread::sleep_for(std::chrono::milliseconds(700));
+    EXPECT(fake::blocks.count(s->g_ent) == 1 && fake::streams == 1);
+    sd_free(s);
+    EXPECT(given_back_within(10));
+    return 0;
+}
+
+int trim_gives_back_at_once() {
+    void* p = nullptr;
+    cudaSetDevice(2);
+    EXPECT(sd_device_malloc(&p, 5000) == cudaSuccess);
+    for (int dev = 0; dev < 3; ++dev) { cudaSetDevice(dev); sd_free(make_store(1 << 20)); }
+    cudaSetDevice(1);
+    const size_t before = fake::all_used();
+    sd_trim();
+    EXPECT(fake::current == 1);
+    EXPECT(before > (3u << 20) && fake::all_used() > 0 && fake::all_used() < 8192);      // (the block in use stays)
+    EXPECT(fake::blocks.count(p) == 1);
+    sd_device_free(p);
+    sd_trim();
+    EXPECT(fake::all_used() == 0);
+    return 0;
+}
+
+int many_threads() {
+    std::vector<std::thread> threads;
+    std::atomic<int> bad{0};
+    for (int t = 0; t < 8; ++t)
+        threads.emplace_back([t, &bad] {
+            unsigned x = 12345u + 777u * t;
+            cudaSetDevice(t & 1);
+            for (int k = 0; k < 4000; ++k) {
+                x = x * 1664525u + 1013904223u;
+                sd_store* s = make_store(1000 + (x >> 12));
+                if (!s) { ++bad; continue; }
+                if ((x & 1023) == 0) std::this_thread::sleep_for(std::chrono::milliseconds(40));
+                { std::lock_guard<std::mutex> l(fake::mutex); if (fake::blocks.count(s->g_ent) != 1 || fake::blocks[s->g_ent].dev != (t & 1)) ++bad; }
+                sd_free(s);
+                if ((x & 255) == 1) sd_trim();
+            }
+        });
+    for (std::thread& t : threads) t.join();
+    EXPECT(bad == 0);
+    EXPECT(given_back_within(10));
+    return 0;
+}
+
+// A forked child has no thread that gives memory back; it must end all the same.
+int a_forked_child_ends() {
+    sd_free(make_store(1 << 20));
+    const pid_t child = fork();
+    if (child == 0) exit(0);
+    int status = 1;
+    EXPECT(waitpid(child, &status, 0) == child && WIFEXITED(status) && WEXITSTATUS(status) == 0);
+    EXPECT(given_back_within(10));
+    return 0;
+}
+
 struct Check { const char* name; int (*run)(); };
 const Check checks[] = {
     {"free_waits_for_the_owner", free_waits_for_the_owner},
+    {"kept_memory_goes_back_by_itself", kept_memory_goes_back_by_itself},
+    {"what_is_in_use_stays", what_is_in_use_stays},
+    {"trim_gives_back_at_once", trim_gives_back_at_once},
+    {"many_threads", many_threads},
+    {"a_forked_child_ends", a_forked_child_ends},
 };
 
 }  // namespace

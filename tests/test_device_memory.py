@@ -13,13 +13,14 @@ ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 def program(tmp_path_factory):
     out = str(tmp_path_factory.mktemp("device_memory") / "check")
     cuda = os.path.dirname(os.path.dirname(os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")))
-    subprocess.check_call(["g++", "-O1", "-g", "-std=c++17", "-I", build.CSRC, "-I", os.path.join(ROOT, "include"), "-isystem",
+    subprocess.check_call(["g++", "-O1", "-g", "-std=c++17", "-DSD_KEEP_SECONDS=0.3", "-I", build.CSRC, "-I", os.path.join(ROOT, "include"), "-isystem",
                            os.path.join(cuda, "include"), os.path.join(ROOT, "tests", "device_memory_check.cpp"),
                            os.path.join(build.CSRC, "memory.cpp"), "-o", out, "-pthread"])
     return out
 
 
-@pytest.mark.parametrize("check", ["free_waits_for_the_owner"])
+@pytest.mark.parametrize("check", ["free_waits_for_the_owner", "kept_memory_goes_back_by_itself", "what_is_in_use_stays",
+                                   "trim_gives_back_at_once", "many_threads", "a_forked_child_ends"])
 def test_device_memory(program, check):
     p = subprocess.run([program, check], capture_output=True, text=True, timeout=60)
     assert p.returncode == 0, p.stderr

@@ -178,3 +178,15 @@ def test_long_runs_without_a_ready_list_in_the_middle_of_a_tree(U, children, mos
         for flags in (0, 4):
             pr.check_speculate([0], 2, budget, 64, flags=flags)
     pr.close()
+
+
+def test_trim_gives_back_what_freed_stores_left():
+    import paper_2411_04975_b200 as sfx
+    sfx.sd_trim()
+    torch.cuda.synchronize()
+    free0 = torch.cuda.mem_get_info()[0]
+    store = sfx.SuffixStore(None, None, vocab=1000, depth_cap=32, max_requests=64, max_req_tokens=4000, max_spec_cap=64)
+    store.free()
+    assert free0 - torch.cuda.mem_get_info()[0] > (100 << 20)            # kept for the next store
+    sfx.sd_trim()
+    assert free0 - torch.cuda.mem_get_info()[0] < (8 << 20)
