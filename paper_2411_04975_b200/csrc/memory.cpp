@@ -9,6 +9,7 @@
 #include <chrono>
 #include <condition_variable>
 #include <mutex>
+#include <new>
 #include <thread>
 #include <unordered_map>
 #include <vector>
@@ -146,6 +147,16 @@ bool watched() {
     return !g.ending;
 }
 
+// a block in use (the mutex is held); false: no host memory for it
+bool take_down(void* p, size_t bytes, int dev) {
+    try {
+        g.owned[p] = OwnedBlock{bytes, dev};
+    } catch (const std::bad_alloc&) {
+        return false;
+    }
+    return true;
+}
+
 void give_streams(int dev, const StreamSet& s) {
     {
         std::lock_guard<std::mutex> lock(g.mutex);
@@ -205,8 +216,8 @@ cudaError_t sd_device_malloc(void** p, size_t bytes) {
             if (c.idle[k].bytes >= bytes && c.idle[k].bytes <= bytes + bytes / 4 && (best == c.idle.size() || c.idle[k].bytes < c.idle[best].bytes))
                 best = k;
         if (best < c.idle.size()) {
+            if (!take_down(c.idle[best].p, c.idle[best].bytes, dev)) return cudaErrorMemoryAllocation;
             *p = c.idle[best].p;
-            g.owned[*p] = OwnedBlock{c.idle[best].bytes, dev};
             c.bytes -= c.idle[best].bytes;
             c.idle.erase(c.idle.begin() + best);
             return cudaSuccess;
@@ -219,7 +230,7 @@ cudaError_t sd_device_malloc(void** p, size_t bytes) {
         e = cudaMalloc(p, bytes);
     }
     if (e != cudaSuccess) { *p = nullptr; return e; }
-    g.owned[*p] = OwnedBlock{bytes, dev};
+    if (!take_down(*p, bytes, dev)) { cudaFree(*p); *p = nullptr; return cudaErrorMemoryAllocation; }
     return cudaSuccess;
 }
 
@@ -237,7 +248,12 @@ void sd_device_free(void* p) {
     }
     if (g_fail_alloc_on || b.bytes > c.most || !watched()) { cudaFree(p); return; }
     cache_trim(c, c.most - b.bytes);
-    c.idle.push_back(FreeBlock{p, b.bytes, Clock::now()});
+    try {
+        c.idle.push_back(FreeBlock{p, b.bytes, Clock::now()});
+    } catch (const std::bad_alloc&) {
+        cudaFree(p);
+        return;
+    }
     c.bytes += b.bytes;
 }
 

@@ -10,6 +10,7 @@
 #include <chrono>
 #include <map>
 #include <mutex>
+#include <new>
 #include <thread>
 #include <vector>
 
@@ -84,6 +85,15 @@ cudaError_t cudaEventDestroy(cudaEvent_t e) { free(e); return cudaSuccess; }
 cudaError_t cudaHostAlloc(void** p, size_t n, unsigned) { *p = malloc(n); return cudaSuccess; }
 cudaError_t cudaFreeHost(void* p) { free(p); return cudaSuccess; }
 }
+
+static thread_local bool no_host_memory = false;
+void* operator new(size_t n) {
+    void* p = no_host_memory ? nullptr : malloc(n ? n : 1);
+    if (!p) throw std::bad_alloc();
+    return p;
+}
+void operator delete(void* p) noexcept { free(p); }
+void operator delete(void* p, size_t) noexcept { free(p); }
 
 #define EXPECT(x) do { if (!(x)) { fprintf(stderr, "line %d: %s\n", __LINE__, #x); return 1; } } while (0)
 
@@ -214,6 +224,29 @@ int a_forked_child_ends() {
     return 0;
 }
 
+// The C entry points report a lack of host memory and throw nothing; no block is lost.
+int no_host_memory_throws_nothing() {
+    void *p = nullptr, *q = nullptr;
+    no_host_memory = true;
+    const cudaError_t fresh = sd_device_malloc(&p, 4096);
+    no_host_memory = false;
+    EXPECT(fresh == cudaErrorMemoryAllocation && !p && fake::all_used() == 0);
+    EXPECT(sd_device_malloc(&p, 4096) == cudaSuccess);
+    no_host_memory = true;
+    sd_device_free(p);
+    no_host_memory = false;
+    EXPECT(fake::all_used() == 0);
+    EXPECT(sd_device_malloc(&p, 4096) == cudaSuccess);
+    sd_device_free(p);
+    no_host_memory = true;
+    const cudaError_t kept = sd_device_malloc(&q, 4096);
+    no_host_memory = false;
+    EXPECT(kept == cudaErrorMemoryAllocation && !q);
+    sd_trim();
+    EXPECT(fake::all_used() == 0);
+    return 0;
+}
+
 struct Check { const char* name; int (*run)(); };
 const Check checks[] = {
     {"free_waits_for_the_owner", free_waits_for_the_owner},
@@ -222,6 +255,7 @@ const Check checks[] = {
     {"trim_gives_back_at_once", trim_gives_back_at_once},
     {"many_threads", many_threads},
     {"a_forked_child_ends", a_forked_child_ends},
+    {"no_host_memory_throws_nothing", no_host_memory_throws_nothing},
 };
 
 }  // namespace
