@@ -16,6 +16,21 @@
 
 #include "memory.h"
 
+static thread_local bool no_host_memory = false;
+void* operator new(size_t n) {
+    void* p = no_host_memory ? nullptr : malloc(n ? n : 1);
+    if (!p) throw std::bad_alloc();
+    return p;
+}
+void operator delete(void* p) noexcept { free(p); }
+void operator delete(void* p, size_t) noexcept { free(p); }
+
+struct HostMemory {                                   // the stand-in itself has some
+    const bool was = no_host_memory;
+    HostMemory() { no_host_memory = false; }
+    ~HostMemory() { no_host_memory = was; }
+};
+
 // ---- the stand-in: devices of 32 GB, work that is queued on a device until something waits for that device
 namespace fake {
 constexpr int DEVICES = 4;
@@ -45,6 +60,7 @@ cudaError_t cudaSetDevice(int d) { if (d < 0 || d >= fake::DEVICES) return cudaE
 cudaError_t cudaDeviceSynchronize() { std::lock_guard<std::mutex> l(fake::mutex); fake::busy[fake::current] = false; return cudaSuccess; }
 cudaError_t cudaGetLastError() { return cudaSuccess; }
 cudaError_t cudaMalloc(void** p, size_t n) {
+    HostMemory m;
     std::lock_guard<std::mutex> l(fake::mutex);
     if (fake::used[fake::current] + n > fake::TOTAL) return cudaErrorMemoryAllocation;
     *p = malloc(1);
@@ -85,15 +101,6 @@ cudaError_t cudaEventDestroy(cudaEvent_t e) { free(e); return cudaSuccess; }
 cudaError_t cudaHostAlloc(void** p, size_t n, unsigned) { *p = malloc(n); return cudaSuccess; }
 cudaError_t cudaFreeHost(void* p) { free(p); return cudaSuccess; }
 }
-
-static thread_local bool no_host_memory = false;
-void* operator new(size_t n) {
-    void* p = no_host_memory ? nullptr : malloc(n ? n : 1);
-    if (!p) throw std::bad_alloc();
-    return p;
-}
-void operator delete(void* p) noexcept { free(p); }
-void operator delete(void* p, size_t) noexcept { free(p); }
 
 #define EXPECT(x) do { if (!(x)) { fprintf(stderr, "line %d: %s\n", __LINE__, #x); return 1; } } while (0)
 
