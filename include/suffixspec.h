@@ -23,6 +23,9 @@
  *
  * Limits: depth_cap <= 32, max_spec_cap <= 64, P <= depth_cap is not required
  * (pattern lengths above depth_cap or above the context length never match).
+ * The entries of a tree are found by 32-bit indices: the global pool (nodes, copies of
+ * the best children of long runs, head-room) and a slot's pool hold fewer than 2^31 - 2,
+ * and a corpus or the prompts of one call have at most 2^31 - 65536 tokens.
  */
 #ifndef SUFFIXSPEC_H
 #define SUFFIXSPEC_H
@@ -110,7 +113,8 @@ typedef struct {
  * Also allocates max_requests empty per-request trees.  Synchronises the stream.
  * On success *out is the new store; on failure *out is NULL and nothing leaks.
  * Errors: INVALID_ARG (NULL, limits, a corpus token outside [0, V), offsets not
- * ascending), NOMEM (cudaMalloc failed), CUDA.
+ * ascending, a corpus whose tree with its head-room has 2^31 - 2 entries or more), NOMEM
+ * (cudaMalloc failed), CUDA.
  */
 int sd_build(const sd_build_params* params, const int32_t* d_corpus, const int64_t* d_seq_offsets,
              int32_t n_seqs, void* stream, sd_store** out);
@@ -163,7 +167,9 @@ int sd_append(sd_store* store, int32_t n, const int32_t* d_slot, const int64_t* 
  * call's work.  The workspace is shared by all calls on a store: order calls
  * made on different streams.
  * Errors: INVALID_ARG (bad slot, slot twice, offsets not ascending, token outside [0, V): nothing
- * is changed), CAPACITY (n * vocab or the token total does not fit 31 bits), NOMEM, CUDA.
+ * is changed), CAPACITY (n * vocab, the token total or the nodes of all the prompts' trees together
+ * do not fit 31 bits: nothing is changed; only where the token total times depth_cap does not, the
+ * call waits for these nodes to be counted), NOMEM, CUDA.
  */
 int sd_build_requests(sd_store* store, int32_t n, const int32_t* h_slot, const int64_t* h_offsets,
                       const int32_t* d_tokens, void* stream);

@@ -16,6 +16,7 @@
 #include "global_insert.cuh"
 #include "memory.h"
 #include "suffix_order.cuh"
+#include "tree_limits.h"
 
 namespace cg = cooperative_groups;
 
@@ -72,7 +73,7 @@ struct CorpusSort {
     unsigned key_bits;                            // of a token and one more
     int D;
     uint32_t *key[2], *val[2];
-    int* rank;                                    // [N] rank from 0, times two, + 1: the sequence goes on behind its k tokens
+    int* rank;                                    // [N] rank from 0, times two, + 1: the sequence goes on behind its k tokens (32 bits, unsigned)
     unsigned *flags, *go;                         // [N / 32 + 1] by place: a new rank starts, the sequence goes on
     int* table;                                   // [SG_BINS][blocks]
     int* total;                                   // [SG_BINS]
@@ -307,7 +308,7 @@ corpus_sort_kernel(CorpusSort A) {
                 for (int u = 0; u < SG_BATCH; ++u) {
                     const int p = (w0 + wib * 32 + q0 + u) * 32 + lane;
                     const int o = __shfl_sync(0xffffffffu, off, q0 + u);
-                    if (p < p_end) A.rank[x[u]] = (o + __popc(f[u] & (lt | (1u << lane))) - 1) * 2 + (int)((go[u] >> lane) & 1u);
+                    if (p < p_end) A.rank[x[u]] = (int)((unsigned)(o + __popc(f[u] & (lt | (1u << lane))) - 1) * 2u + ((go[u] >> lane) & 1u));
                 }
             }
             before += n_lot;
@@ -464,7 +465,7 @@ struct TreeScan {
     int* r;                                       // [32][tiles] (2): R left behind (-1: none); carried: R from the front
     int* s;                                       // [tiles + 1] nodes below depth 1, carried: S
     int* n1;                                      // [tiles + 1] nodes of depth 1, carried: before the tile
-    int* wide;                                    // [4]: long runs, entries they take with their top blocks, cursors of both
+    TreeTotals* total;                            // in 64 bits: places are right only if these fit 32, nothing is written before the host knows
 };
 
 __device__ __forceinline__ int ts_scan(int v, int lane) {       // inclusive
@@ -537,15 +538,24 @@ __global__ void __launch_bounds__(TS_CARRY) ts_carry_kernel(TreeScan T) {
     const int per = (T.tiles + TS_CARRY - 1) / TS_CARRY;
     const int k0 = threadIdx.x * per, k1 = min(T.tiles, k0 + per);
     if (blockIdx.x == 32) {
-        int a = 0, b = 0;
+        __shared__ i64 sum[TS_CARRY / 32];
+        int b = 0;
+        i64 a = 0;                                              // (a tile's nodes fit 32 bits, the tree's need not)
         for (int k = k0; k < k1; ++k) { a += T.s[k]; b += T.n1[k]; }
-        const int ia = ts_scan(a, lane), ib = ts_scan(b, lane);
-        if (lane == 31) { p0[w] = ia; p1[w] = ib; }
+        i64 ia = a;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const i64 y = __shfl_up_sync(TS_FULL, ia, o);
+            if (lane >= o) ia += y;
+        }
+        const int ib = ts_scan(b, lane);
+        if (lane == 31) { sum[w] = ia; p1[w] = ib; }
         __syncthreads();
-        int ra = ia - a, rb = ib - b, ta = 0, tb = 0;
-        for (int q = 0; q < TS_CARRY / 32; ++q) { if (q < w) { ra += p0[q]; rb += p1[q]; } ta += p0[q]; tb += p1[q]; }
-        for (int k = k0; k < k1; ++k) { a = T.s[k]; b = T.n1[k]; T.s[k] = ra; T.n1[k] = rb; ra += a; rb += b; }
-        if (threadIdx.x == 0) { T.s[T.tiles] = ta; T.n1[T.tiles] = tb; }
+        i64 ra = ia - a, ta = 0;
+        int rb = ib - b, tb = 0;
+        for (int q = 0; q < TS_CARRY / 32; ++q) { if (q < w) { ra += sum[q]; rb += p1[q]; } ta += sum[q]; tb += p1[q]; }
+        for (int k = k0; k < k1; ++k) { const int x = T.s[k]; b = T.n1[k]; T.s[k] = (int)ra; T.n1[k] = rb; ra += x; rb += b; }
+        if (threadIdx.x == 0) { T.s[T.tiles] = (int)ta; T.n1[T.tiles] = tb; T.total->below = ta; T.total->top = tb; }
         return;
     }
     int* const f = T.f + (i64)blockIdx.x * T.tiles;
@@ -648,7 +658,8 @@ ts_runs_kernel(TreeScan T) {
     if (tile >= T.tiles) return;
     const int t0 = tile * T.tile_len, t1 = min(T.N, t0 + T.tile_len);
     int g = ts_g_in(T, tile, lane);
-    int s_end = T.s[tile + 1], R = -1, n_wide = 0, room = 0;
+    int s_end = T.s[tile + 1], R = -1, n_wide = 0;
+    i64 room = 0;
     for (int jb = t0 + ((t1 - t0 - 1) & ~31); jb >= t0; jb -= 32) {
         const int m = min(32, t1 - jb);
         int l_own = 0, n_own = 0, c = 0;
@@ -672,8 +683,11 @@ ts_runs_kernel(TreeScan T) {
     T.r[(i64)lane * T.tiles + tile] = R;
     if (TOP) {
         n_wide = (int)__reduce_add_sync(TS_FULL, (unsigned)n_wide);
-        room = (int)__reduce_add_sync(TS_FULL, (unsigned)room);
-        if (lane == 0 && n_wide) { atomicAdd(&T.wide[0], n_wide); atomicAdd(&T.wide[1], room); }
+        if (n_wide) {
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) room += __shfl_xor_sync(TS_FULL, room, o);
+            if (lane == 0) { atomicAdd(&T.total->n_wide, n_wide); atomicAdd((u64*)&T.total->wide, (u64)room); }
+        }
     }
 }
 
@@ -795,7 +809,7 @@ ts_emit_kernel(TreeScan T, TreeOut O) {
                 const int pos = lane == 0 ? depth1 : place + shift;
                 ent[pos] = make_int4(x[i] - first_tok, es[i] - j, kids > 0 ? run + shift : 0, kids > 0 ? (int)((unsigned)kids | RUN_STATIC) : 0);
                 if (lane == 0) root[x[i] - first_tok] = pos;
-                if (!REQ && kids > SD_TOP_MIN) O.wide[atomicAdd(&T.wide[2], 1)] = make_int4(pos, run + shift, kids, 0);
+                if (!REQ && kids > SD_TOP_MIN) O.wide[atomicAdd(&T.total->listed, 1)] = make_int4(pos, run + shift, kids, 0);
             }
         }
     }
@@ -806,9 +820,9 @@ ts_emit_kernel(TreeScan T, TreeOut O) {
 __global__ void ts_wide_place_kernel(TreeScan T, int4* wide, int4* ent, int first) {
     sd_chain_begin();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= T.wide[0]) return;
+    if (i >= T.total->n_wide) return;
     int4 w = wide[i];
-    w.w = first + atomicAdd(&T.wide[3], w.z + SD_TOP_BLOCK);
+    w.w = first + atomicAdd(&T.total->placed, w.z + SD_TOP_BLOCK);
     wide[i] = w;
     ent[w.x].z = w.w + SD_TOP_BLOCK;
     ent[w.x].w = (int)((unsigned)w.z | RUN_STATIC | RUN_HAS_TOP);
@@ -1006,7 +1020,7 @@ static int pipeline_run(Pipeline& P, const int32_t* d_tok, const int64_t* d_seq_
     const bool have_ends = end_pos != nullptr;
     uint32_t* sa = nullptr;
     bool ok = tmp.get(&ts.lcp, N) && tmp.get(&ts.len, N) && tmp.get(&ts.f, 32 * (i64)ts.tiles) && tmp.get(&ts.e, 32 * (i64)ts.tiles) &&
-              tmp.get(&ts.r, 32 * (i64)ts.tiles) && tmp.get(&ts.s, ts.tiles + 1) && tmp.get(&ts.n1, ts.tiles + 1) && tmp.get(&ts.wide, 4) &&
+              tmp.get(&ts.r, 32 * (i64)ts.tiles) && tmp.get(&ts.s, ts.tiles + 1) && tmp.get(&ts.n1, ts.tiles + 1) && tmp.get(&ts.total, 1) &&
               (have_ends || tmp.get(&end_pos, N)) && tmp.get(&sa, N);
     if (!ok) return SD_ERR_NOMEM;
     if (!have_ends) SD_CUDA_OK(sd_launch(seq_end_kernel, grid_for(N, T256), T256, 0, st, d_seq_offsets, n_seqs, N, end_pos));
@@ -1040,7 +1054,7 @@ static int pipeline_run(Pipeline& P, const int32_t* d_tok, const int64_t* d_seq_
     ts.sa = sa;
     ts.end_pos = end_pos;
     const unsigned grid = (unsigned)((ts.tiles + TS_WARPS - 1) / TS_WARPS);
-    if (top_blocks && cudaMemsetAsync(ts.wide, 0, 4 * sizeof(int), st) != cudaSuccess) return SD_ERR_CUDA;
+    if (top_blocks && cudaMemsetAsync(ts.total, 0, sizeof(TreeTotals), st) != cudaSuccess) return SD_ERR_CUDA;
     SD_CUDA_OK(sd_launch(ts_tiles_kernel, grid, TS_WARPS * 32, 0, st, ts));
     SD_CUDA_OK(sd_launch(ts_carry_kernel, 33, TS_CARRY, 0, st, ts));
     if (top_blocks) SD_CUDA_OK(sd_launch(ts_runs_kernel<true>, grid, TS_WARPS * 32, 0, st, ts));
@@ -1073,7 +1087,7 @@ extern "C" int sd_build(const sd_build_params* p, const int32_t* d_corpus, const
     if (n_seqs > 0) {
         SD_CUDA_OK(cudaMemcpyAsync(&N, d_seq_offsets + n_seqs, sizeof(i64), cudaMemcpyDeviceToHost, st));
         SD_CUDA_OK(cudaStreamSynchronize(st));
-        if (N < 0 || N >= (1ll << 31) - 2) return SD_ERR_INVALID_ARG;
+        if (N < 0 || N > SD_MAX_TOKENS) return SD_ERR_INVALID_ARG;
     }
 
     sd_store* s = new (std::nothrow) sd_store();
@@ -1083,7 +1097,7 @@ extern "C" int sd_build(const sd_build_params* p, const int32_t* d_corpus, const
     if (cudaGetDevice(&s->device) != cudaSuccess) { delete s; return SD_ERR_CUDA; }
     const int D = s->D;
     s->spn = p->slot_pool_nodes > 0 ? p->slot_pool_nodes : 2ll * s->T * D;
-    if (s->spn >= (1ll << 31) - 2) { delete s; return SD_ERR_INVALID_ARG; }
+    if (s->spn > SD_MAX_ENTRIES) { delete s; return SD_ERR_INVALID_ARG; }
 
     bool ok = store_alloc(s, &s->g_root, s->V) && store_alloc(s, &s->g_state, 1) && store_alloc(s, &s->gi, 1) &&
               store_alloc(s, &s->s_ent, (i64)s->R * s->spn) && store_alloc(s, &s->s_root, (i64)s->R * s->V) &&
@@ -1100,8 +1114,7 @@ extern "C" int sd_build(const sd_build_params* p, const int32_t* d_corpus, const
 
     Pipeline P(st);
     const int T256 = 256;
-    i64 n_nodes = 0, used_entries = 0;
-    int h_wide[2] = {0, 0};
+    TreeTotals total = {};
     int4* wide_list = nullptr;
     if (N > 0) {
         {
@@ -1118,20 +1131,14 @@ extern "C" int sd_build(const sd_build_params* p, const int32_t* d_corpus, const
         }
         const int rc = pipeline_run(P, d_corpus, d_seq_offsets, n_seqs, N, s->V, D, true, st);
         if (rc != SD_OK) { sd_store_release(s, st); return rc; }
-        int h_s = 0, h_n1 = 0;
-        ce = cudaMemcpyAsync(&h_s, P.ts.s + P.ts.tiles, sizeof(int), cudaMemcpyDeviceToHost, st);
-        if (ce == cudaSuccess) ce = cudaMemcpyAsync(&h_n1, P.ts.n1 + P.ts.tiles, sizeof(int), cudaMemcpyDeviceToHost, st);
-        if (ce == cudaSuccess) ce = cudaMemcpyAsync(h_wide, P.ts.wide, 2 * sizeof(int), cudaMemcpyDeviceToHost, st);
+        ce = cudaMemcpyAsync(&total, P.ts.total, sizeof(total), cudaMemcpyDeviceToHost, st);
         if (ce == cudaSuccess) ce = cudaStreamSynchronize(st);
         if (ce != cudaSuccess) { sd_store_release(s, st); return SD_ERR_CUDA; }
-        n_nodes = (i64)h_s + h_n1;
-        used_entries = n_nodes + h_wide[1];                     // (a long run leaves its first place empty)
-        if (h_wide[0] > 0 && !P.tmp.get(&wide_list, h_wide[0])) { sd_store_release(s, st); return SD_ERR_NOMEM; }
     }
-
-    i64 extra = p->global_extra_nodes >= 0 ? p->global_extra_nodes : std::max<i64>(1ll << 22, n_nodes);
-    s->g_cap = used_entries + extra;
-    if (s->g_cap >= (1ll << 31) - 2) { sd_store_release(s, st); return SD_ERR_INVALID_ARG; }
+    s->g_cap = sd_pool_entries(total, p->global_extra_nodes);
+    if (s->g_cap < 0) { sd_store_release(s, st); return SD_ERR_INVALID_ARG; }
+    const i64 n_nodes = total.below + total.top, used_entries = n_nodes + total.wide;
+    if (total.n_wide > 0 && !P.tmp.get(&wide_list, total.n_wide)) { sd_store_release(s, st); return SD_ERR_NOMEM; }
     if (!store_alloc(s, &s->g_ent, s->g_cap)) { sd_store_release(s, st); return SD_ERR_NOMEM; }
 
     if (N > 0) {
@@ -1140,9 +1147,9 @@ extern "C" int sd_build(const sd_build_params* p, const int32_t* d_corpus, const
         out.ent = s->g_ent; out.root = s->g_root; out.wide = wide_list;
         const int erc = emit_entries<false>(P.ts, out, st);
         if (erc != SD_OK) { sd_store_release(s, st); return erc; }
-        if (h_wide[0] > 0) {
-            ts_wide_place_kernel<<<grid_for(h_wide[0], T256), T256, 0, st>>>(P.ts, wide_list, s->g_ent, (int)n_nodes);
-            ts_wide_fill_kernel<<<(unsigned)h_wide[0], TOP_THREADS, 0, st>>>(wide_list, s->g_ent);
+        if (total.n_wide > 0) {
+            ts_wide_place_kernel<<<grid_for(total.n_wide, T256), T256, 0, st>>>(P.ts, wide_list, s->g_ent, (int)n_nodes);
+            ts_wide_fill_kernel<<<(unsigned)total.n_wide, TOP_THREADS, 0, st>>>(wide_list, s->g_ent);
         }
     }
     init_global_state_kernel<<<1, 1, 0, st>>>(s->g_state, (int)used_entries, (int)n_nodes, N);
@@ -1272,7 +1279,7 @@ extern "C" int sd_build_requests(sd_store* s, int32_t n, const int32_t* h_slot, 
     }
     const i64 N = h_offsets[n];
     if (N > 0 && !d_tokens) return SD_ERR_INVALID_ARG;
-    if ((i64)n * s->V >= (1ll << 31) - 2 || N >= (1ll << 31) - 2) return SD_ERR_CAPACITY;
+    if ((i64)n * s->V >= (1ll << 31) - 2 || N > SD_MAX_TOKENS) return SD_ERR_CAPACITY;
     cudaStream_t st = (cudaStream_t)stream;
     const int T256 = 256, D = s->D;
 
@@ -1310,6 +1317,12 @@ extern "C" int sd_build_requests(sd_store* s, int32_t n, const int32_t* h_slot, 
         i64 max_len = 0;
         for (int q = 0; q < n; ++q) max_len = std::max<i64>(max_len, h_offsets[q + 1] - h_offsets[q]);
         rc = pipeline_run(P, mtok, d_off, n, N, (i64)n * s->V, D, false, st, max_len, end_pos, RequestBounds{n, d_off, s_req, n1_req});
+        if (rc == SD_OK && N * D > SD_MAX_ENTRIES) {             // the trees' nodes may not fit 32 bits (up to then nothing has changed)
+            TreeTotals total = {};
+            if (cudaMemcpyAsync(&total, P.ts.total, sizeof(total), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+                cudaStreamSynchronize(st) != cudaSuccess) rc = SD_ERR_CUDA;
+            else if (total.below + total.top > SD_MAX_ENTRIES) rc = SD_ERR_CAPACITY;
+        }
     }
     if (rc == SD_OK) SD_CUDA_OK(sd_launch(requests_prepare_kernel, (unsigned)n, PREP_THREADS, 0, st, *s, n, d_slot, d_off, d_tokens, bad));
     if (rc == SD_OK && N > 0) {
