@@ -10,7 +10,7 @@ _ROOT = os.path.dirname(_HERE)
 CSRC = os.path.join(_HERE, "csrc")
 LIB = os.path.join(_HERE, "libsuffixspec.so")
 CALL = os.path.join(_HERE, "_call.so")
-SOURCES = ["build.cu", "append.cu", "speculate.cu", "query.cu", "memory.cpp"]
+SOURCES = ["build.cu", "append.cu", "speculate.cu", "query.cu", "device_memory.cpp"]
 
 
 def _newest_source() -> float:
@@ -30,7 +30,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
         nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
         cmd = [nvcc, "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
                "-shared", "-Xcompiler", "-fPIC", "-I", os.path.join(_ROOT, "include"), "-I", CSRC,
-               "-cudart", "shared", "-Xlinker", "-z", "-Xlinker", "nodelete", "-o", LIB]   # (a thread of memory.cpp outlives dlclose)
+               "-cudart", "shared", "-Xlinker", "-z", "-Xlinker", "nodelete", "-o", LIB]   # (a thread of device_memory.cpp outlives dlclose)
         if verbose:
             cmd += ["-Xptxas", "-v"]
         cmd += [os.path.join(CSRC, f) for f in SOURCES]

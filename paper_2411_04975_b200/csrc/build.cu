@@ -13,8 +13,8 @@
 #include <cooperative_groups.h>
 
 #include "append_core.cuh"
+#include "device_memory.h"
 #include "global_insert.cuh"
-#include "memory.h"
 #include "suffix_order.cuh"
 #include "tree_limits.h"
 

@@ -141,7 +141,7 @@ inline cudaError_t sd_launch(void (*kernel)(K...), unsigned grid, unsigned block
         if (_e != cudaSuccess) return SD_ERR_CUDA;         \
     } while (0)
 
-// Device memory of the library (memory.cpp), and back when the work on it has ended.
+// Device memory of the library (device_memory.cpp), and back when the work on it has ended.
 cudaError_t sd_device_malloc(void** p, size_t bytes);
 void sd_device_free(void* p);
 

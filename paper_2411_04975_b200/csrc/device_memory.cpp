@@ -14,7 +14,7 @@
 #include <unordered_map>
 #include <vector>
 
-#include "memory.h"
+#include "device_memory.h"
 
 // Blocks that stores and builds have given back are kept for the next ones, up to 1/32 of the device's memory (5.7 GB
 // of a B200's).  The oldest go first when there are more, all of them when an allocation fails (which is then tried once

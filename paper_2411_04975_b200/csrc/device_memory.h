@@ -1,4 +1,4 @@
-// Device memory, streams and pinned memory of the library (memory.cpp): kept from store to store.
+// Device memory, streams and pinned memory of the library (device_memory.cpp): kept from store to store.
 #pragma once
 
 #include "common.cuh"

@@ -1,4 +1,4 @@
-// Checks of csrc/memory.cpp on the CPU, linked with the stand-in for the CUDA runtime below: what is kept between stores, when
+// Checks of csrc/device_memory.cpp on the CPU, linked with the stand-in for the CUDA runtime below: what is kept between stores, when
 // it is given back, and what a store's release waits for.  `device_memory_check NAME` runs one check; 0 = it holds.
 #include <stdio.h>
 #include <stdlib.h>
@@ -14,7 +14,7 @@
 #include <thread>
 #include <vector>
 
-#include "memory.h"
+#include "device_memory.h"
 
 static thread_local bool no_host_memory = false;
 void* operator new(size_t n) {

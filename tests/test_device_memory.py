@@ -1,4 +1,4 @@
-"""The memory kept between stores and a store's release (csrc/memory.cpp), on the CPU against a stand-in for the CUDA runtime."""
+"""The memory kept between stores and a store's release (csrc/device_memory.cpp), on the CPU against a stand-in for the CUDA runtime."""
 import os
 import subprocess
 
@@ -15,7 +15,7 @@ def program(tmp_path_factory):
     cuda = os.path.dirname(os.path.dirname(os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")))
     subprocess.check_call(["g++", "-O1", "-g", "-std=c++17", "-DSD_KEEP_SECONDS=0.3", "-I", build.CSRC, "-I", os.path.join(ROOT, "include"), "-isystem",
                            os.path.join(cuda, "include"), os.path.join(ROOT, "tests", "device_memory_check.cpp"),
-                           os.path.join(build.CSRC, "memory.cpp"), "-o", out, "-pthread"])
+                           os.path.join(build.CSRC, "device_memory.cpp"), "-o", out, "-pthread"])
     return out
 
 
