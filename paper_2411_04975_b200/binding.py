@@ -9,7 +9,10 @@ wraps them with output allocation.
 from __future__ import annotations
 
 import ctypes as C
+import importlib.util
 import os
+import subprocess
+import warnings
 from typing import Dict, Optional
 
 import torch
@@ -56,7 +59,7 @@ def library() -> C.CDLL:
     global _lib, _call
     if _lib is None:
         path = _build.LIB
-        if not (os.path.exists(path) and os.path.exists(_build.CALL)) or os.environ.get("SUFFIXSPEC_REBUILD"):
+        if not os.path.exists(path) or os.environ.get("SUFFIXSPEC_REBUILD"):
             path = _build.build()
         lib = C.CDLL(path)
         vp = C.c_void_p
@@ -90,10 +93,49 @@ def library() -> C.CDLL:
         lib.sd_debug_fail_alloc.argtypes = [C.c_int64]
         lib.sd_strerror.restype = C.c_char_p
         lib.sd_strerror.argtypes = [C.c_int]
-        from . import _call as call
-        call.setup(*(C.cast(f, vp).value for f in (lib.sd_speculate, lib.sd_step, lib.sd_append)), _ptr)
-        _lib, _call = lib, call
+        _lib, _call = lib, _load_call(lib)
     return _lib
+
+
+def _load_call(lib):
+    """The native module of the per-step calls, built if this torch has none yet; if it cannot be had (no compiler), the
+    same calls with their arguments converted here."""
+    try:
+        path = _build.call_path()
+        if not os.path.exists(path):
+            path = _build.build_call()
+        spec = importlib.util.spec_from_file_location(__package__ + "._call", path)
+        call = importlib.util.module_from_spec(spec)
+        spec.loader.exec_module(call)
+        call.setup(*(C.cast(f, C.c_void_p).value for f in (lib.sd_speculate, lib.sd_step, lib.sd_append)), _ptr)
+        return call
+    except (ImportError, OSError, subprocess.CalledProcessError) as e:
+        warnings.warn(f"the native module of the per-step calls could not be had ({e}): each call takes the host some 6 us longer",
+                      RuntimeWarning)
+        return _PlainCall(lib)
+
+
+class _PlainCall:
+    """speculate, step and append of the module _call through ctypes."""
+
+    def __init__(self, lib):
+        self._lib = lib
+
+    def speculate(self, store, slots, P, alpha, max_spec, flags, tau, budget_cap, out) -> int:
+        return self._lib.sd_speculate(
+            store, int(slots.numel()), _ptr(slots, torch.int32, "slots"), C.byref(_SpecParams(P, alpha, max_spec, flags, tau)),
+            _ptr(budget_cap, torch.int32, "budget_cap"), *_out_ptrs(out), _stream())
+
+    def step(self, store, slots, offsets, new_tokens, P, alpha, max_spec, flags, tau, budget_cap, out) -> int:
+        return self._lib.sd_step(
+            store, int(slots.numel()), _ptr(slots, torch.int32, "slots"), _ptr(offsets, torch.int64, "offsets"),
+            _ptr(new_tokens, torch.int32, "new_tokens"), C.byref(_SpecParams(P, alpha, max_spec, flags, tau)),
+            _ptr(budget_cap, torch.int32, "budget_cap"), *_out_ptrs(out), _stream())
+
+    def append(self, store, slots, offsets, tokens, reset) -> int:
+        return self._lib.sd_append(
+            store, int(slots.numel()), _ptr(slots, torch.int32, "slots"), _ptr(offsets, torch.int64, "offsets"),
+            _ptr(tokens, torch.int32, "tokens"), _ptr(reset, torch.uint8, "reset"), _stream())
 
 
 def _ptr(t: Optional[torch.Tensor], dtype: torch.dtype, name: str) -> Optional[int]:

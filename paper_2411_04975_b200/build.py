@@ -3,14 +3,21 @@ from __future__ import annotations
 
 import os
 import subprocess
+import sys
 import sysconfig
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 _ROOT = os.path.dirname(_HERE)
 CSRC = os.path.join(_HERE, "csrc")
 LIB = os.path.join(_HERE, "libsuffixspec.so")
-CALL = os.path.join(_HERE, "_call.so")
 SOURCES = ["build.cu", "append.cu", "speculate.cu", "query.cu", "device_memory.cpp"]
+
+
+def call_path() -> str:
+    """The module _call.  It is built against private headers of torch, so its name says for which torch (and Python):
+    behind an upgrade of either the one that is there is not taken for the one that is needed."""
+    import torch
+    return os.path.join(_HERE, f"_call.{sys.implementation.cache_tag}-torch-{torch.__version__}.so")
 
 
 def _newest_source() -> float:
@@ -35,12 +42,13 @@ def build(force: bool = False, verbose: bool = False) -> str:
             cmd += ["-Xptxas", "-v"]
         cmd += [os.path.join(CSRC, f) for f in SOURCES]
         subprocess.check_call(cmd)
-    if not fresh(CALL):
-        _build_call()
+    if not fresh(call_path()):
+        build_call()
     return LIB
 
 
-def _build_call() -> None:
+def build_call() -> str:
+    """Compile csrc/call.cpp into the module _call (host code, no nvcc).  Returns its path."""
     import torch
     from torch.utils.cpp_extension import include_paths
     cuda = os.path.dirname(os.path.dirname(os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")))
@@ -50,10 +58,10 @@ def _build_call() -> None:
     cmd = ["g++", "-O2", "-std=c++17", "-shared", "-fPIC", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}"]
     for path in includes:
         cmd += ["-isystem", path]
-    cmd += [os.path.join(CSRC, "call.cpp"), "-L", lib, "-ltorch_python", "-ltorch_cpu", "-lc10", "-lc10_cuda", "-o", CALL]
+    cmd += [os.path.join(CSRC, "call.cpp"), "-L", lib, "-ltorch_python", "-ltorch_cpu", "-lc10", "-lc10_cuda", "-o", call_path()]
     subprocess.check_call(cmd)
+    return call_path()
 
 
 if __name__ == "__main__":
-    import sys
     print(build(force=True, verbose="-v" in sys.argv))
