@@ -695,10 +695,9 @@ extern "C" int sd_append(sd_store* s, int32_t n, const int32_t* d_slot, const in
     void* args[] = {(void*)s, (void*)&n, (void*)&d_slot, (void*)&d_offsets, (void*)&d_tokens, (void*)&tok_bits};
     SD_CUDA_OK(cudaFuncSetAttribute(global_insert_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(GiShared)));
     SD_CUDA_OK(cudaLaunchCooperativeKernel((void*)global_insert_kernel, dim3(GI_BLOCKS), dim3(GI_THREADS), args, sizeof(GiShared), s->aux));
-    SD_CUDA_OK(cudaEventRecord(s->ev_join, s->aux));
+    // (joined whatever becomes of the launch: the insert reads buffers that the caller may free behind this call on its stream)
+    const cudaError_t record = cudaEventRecord(s->ev_join, s->aux);
     append_kernel<<<(unsigned)n, APPEND_THREADS, 0, st>>>(*s, d_slot, d_offsets, d_tokens, d_reset);
-    SD_CUDA_OK(cudaGetLastError());
-    SD_CUDA_OK(cudaStreamWaitEvent(st, s->ev_join, 0));
-    SD_CUDA_OK(cudaGetLastError());
-    return SD_OK;
+    const cudaError_t launch = cudaGetLastError(), join = cudaStreamWaitEvent(st, s->ev_join, 0);
+    return record == cudaSuccess && launch == cudaSuccess && join == cudaSuccess ? SD_OK : SD_ERR_CUDA;
 }
