@@ -231,6 +231,31 @@ int a_forked_child_ends() {
     return 0;
 }
 
+// 1/32 of a device's 32 GB: the oldest go first, what is larger than that is not kept at all, and what is kept of other devices
+// does not count.
+int kept_memory_is_bounded() {
+    const size_t most = fake::TOTAL / 32, half = most / 2;
+    void* p[6];
+    cudaSetDevice(1);
+    EXPECT(sd_device_malloc(&p[5], half) == cudaSuccess);
+    sd_device_free(p[5]);
+    cudaSetDevice(0);
+    for (int k = 0; k < 5; ++k) EXPECT(sd_device_malloc(&p[k], half - (size_t)k * (80u << 20)) == cudaSuccess);
+    for (int k = 0; k < 5; ++k) {
+        sd_device_free(p[k]);
+        size_t in_use = 0;
+        for (int q = k + 1; q < 5; ++q) in_use += fake::blocks[p[q]].bytes;
+        EXPECT(fake::used[0] - in_use <= most);
+        EXPECT(fake::blocks.count(p[k]) == 1);
+    }
+    EXPECT(fake::blocks.count(p[0]) == 0 && fake::blocks.count(p[5]) == 1);
+    EXPECT(sd_device_malloc(&p[0], most + (64u << 20)) == cudaSuccess);
+    sd_device_free(p[0]);
+    EXPECT(fake::blocks.count(p[0]) == 0 && fake::blocks.count(p[4]) == 1);
+    sd_trim();
+    return 0;
+}
+
 // The C entry points report a lack of host memory and throw nothing; no block is lost.
 int no_host_memory_throws_nothing() {
     void *p = nullptr, *q = nullptr;
@@ -262,6 +287,7 @@ const Check checks[] = {
     {"trim_gives_back_at_once", trim_gives_back_at_once},
     {"many_threads", many_threads},
     {"a_forked_child_ends", a_forked_child_ends},
+    {"kept_memory_is_bounded", kept_memory_is_bounded},
     {"no_host_memory_throws_nothing", no_host_memory_throws_nothing},
 };
 

@@ -21,7 +21,7 @@ def program(tmp_path_factory):
 
 @pytest.mark.parametrize("check", ["free_waits_for_the_owner", "kept_memory_goes_back_by_itself", "what_is_in_use_stays",
                                    "trim_gives_back_at_once", "many_threads", "a_forked_child_ends",
-                                   "no_host_memory_throws_nothing"])
+                                   "kept_memory_is_bounded", "no_host_memory_throws_nothing"])
 def test_device_memory(program, check):
     p = subprocess.run([program, check], capture_output=True, text=True, timeout=60)
     assert p.returncode == 0, p.stderr
