@@ -139,7 +139,9 @@ int sd_build(const sd_build_params* params, const int32_t* d_corpus, const int64
  * call are not affected).  When the global pool cannot hold the new nodes
  * SD_STATUS_GLOBAL_FULL is set: strings whose nodes found no room are missing
  * or counted short, the tree stays consistent and usable, and later calls
- * insert nothing more into it.  n == 0 is a no-op.
+ * insert nothing more into it.  A call's sequences are taken in lots of up to 2,016
+ * start positions; the first lot that does not fit adds no node at all, only the
+ * counts of its strings that exist, and the lots behind it nothing.  n == 0 is a no-op.
  * Stream order: for the caller everything is ordered on `stream`.  Inside the
  * call the insert into the global tree runs on a stream the store owns, which
  * starts behind the work `stream` holds at the call and which `stream` waits
