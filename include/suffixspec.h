@@ -25,7 +25,8 @@
  * (pattern lengths above depth_cap or above the context length never match).
  * The entries of a tree are found by 32-bit indices: the global pool (nodes, copies of
  * the best children of long runs, head-room) and a slot's pool hold fewer than 2^31 - 2,
- * and a corpus or the prompts of one call have at most 2^31 - 65536 tokens.
+ * and a corpus or the prompts of one call have at most 2^31 - 65536 tokens.  A node has
+ * at most 2^24 - 1 children (a vocab of up to 2^24 - 1 cannot exceed that).
  */
 #ifndef SUFFIXSPEC_H
 #define SUFFIXSPEC_H

@@ -19,8 +19,8 @@
 // Blocks that stores and builds have given back are kept for the next ones, up to 1/32 of the device's memory (5.7 GB
 // of a B200's).  The oldest go first when there are more, all of them when an allocation fails (which is then tried once
 // more) or sd_trim is called, and a thread of the library's own gives back what nobody has wanted for half a minute, so
-// that a process that only ever frees its last store does not sit on it.  Getting
-// and returning memory is what a build or a short-lived store would otherwise spend its time on: 20
+// that a process that only ever frees its last store does not sit on it (1 GB given back beside a loop of drafts held up one
+// of its calls, by 2 ms).  Getting and returning memory is what a build or a short-lived store would otherwise spend its time on: 20
 // cudaMalloc / cudaFree calls took 2.7 ms of the 3.7 ms of a 32,768-token build and up to 70 ms of a
 // 4 M-token one.  (CUDA's own stream-ordered pools cost 6.2 ms per GB whenever they grow or shrink, cudaMalloc
 // 0.3 - 0.8 ms at any of these sizes.)  A block is given back when the work on it has ended, so the next owner may be
