@@ -1309,11 +1309,12 @@ extern "C" int sd_build_requests(sd_store* s, int32_t n, const int32_t* h_slot, 
     memcpy(h_args, h_offsets, 8 * ((size_t)n + 1));
     memcpy(h_args + 8 * ((size_t)n + 1), h_slot, 4 * (size_t)n);
     memset(h_args + arg_bytes - 4, 0, 4);
-    SD_CUDA_OK(cudaMemcpyAsync(d_args, h_args, arg_bytes, cudaMemcpyHostToDevice, st));
-    if (N > 0) SD_CUDA_OK(sd_launch(map_tokens_kernel, grid_for(N, T256), T256, 0, st, d_tokens, d_off, n, N, s->V, mtok, end_pos, bad, (int*)s->stage));
-    SD_CUDA_OK(cudaEventRecord(s->ev_check, st));
-    int rc = SD_OK;
-    if (N > 0) {
+    // (from here on the pinned memory is in use: whatever fails, the call waits for it before it returns)
+    cudaError_t ce = cudaMemcpyAsync(d_args, h_args, arg_bytes, cudaMemcpyHostToDevice, st);
+    if (ce == cudaSuccess && N > 0) ce = sd_launch(map_tokens_kernel, grid_for(N, T256), T256, 0, st, d_tokens, d_off, n, N, s->V, mtok, end_pos, bad, (int*)s->stage);
+    const cudaError_t record = cudaEventRecord(s->ev_check, st);
+    int rc = ce == cudaSuccess && record == cudaSuccess ? SD_OK : SD_ERR_CUDA;
+    if (rc == SD_OK && N > 0) {
         i64 max_len = 0;
         for (int q = 0; q < n; ++q) max_len = std::max<i64>(max_len, h_offsets[q + 1] - h_offsets[q]);
         rc = pipeline_run(P, mtok, d_off, n, N, (i64)n * s->V, D, false, st, max_len, end_pos, RequestBounds{n, d_off, s_req, n1_req});
@@ -1324,16 +1325,17 @@ extern "C" int sd_build_requests(sd_store* s, int32_t n, const int32_t* h_slot, 
             else if (total.below + total.top > SD_MAX_ENTRIES) rc = SD_ERR_CAPACITY;
         }
     }
-    if (rc == SD_OK) SD_CUDA_OK(sd_launch(requests_prepare_kernel, (unsigned)n, PREP_THREADS, 0, st, *s, n, d_slot, d_off, d_tokens, bad));
+    if (rc == SD_OK && sd_launch(requests_prepare_kernel, (unsigned)n, PREP_THREADS, 0, st, *s, n, d_slot, d_off, d_tokens, bad) != cudaSuccess) rc = SD_ERR_CUDA;
     if (rc == SD_OK && N > 0) {
         TreeOut out;
         memset(&out, 0, sizeof(out));
         out.sv = *s; out.n_req = n; out.slot = d_slot; out.off = d_off; out.s_req = s_req; out.n1_req = n1_req; out.bad = bad;
         rc = emit_entries<true>(P.ts, out, st);
     }
-    if (rc == SD_OK)
-        SD_CUDA_OK(sd_launch(requests_finalize_kernel, (unsigned)n, 256, 0, st, *s, n, d_slot, d_off, N > 0 ? s_req : nullptr, N > 0 ? n1_req : nullptr, bad));
-    const cudaError_t checked = cudaEventSynchronize(s->ev_check);               // (the pinned memory is free again, too)
+    if (rc == SD_OK && sd_launch(requests_finalize_kernel, (unsigned)n, 256, 0, st, *s, n, d_slot, d_off, N > 0 ? s_req : nullptr,
+                                 N > 0 ? n1_req : nullptr, bad) != cudaSuccess) rc = SD_ERR_CUDA;
+    // (the pinned memory is free again, too)
+    const cudaError_t checked = record == cudaSuccess ? cudaEventSynchronize(s->ev_check) : cudaStreamSynchronize(st);
     if (rc != SD_OK) return rc;
     if (checked != cudaSuccess) return SD_ERR_CUDA;
     if (*h_bad) return SD_ERR_INVALID_ARG;
