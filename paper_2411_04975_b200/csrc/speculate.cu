@@ -290,17 +290,46 @@ constexpr int CTA_WARPS_WIDE = 16;
 constexpr int CTA_WARPS_NARROW = 8;            // batches of more than two requests per SM: four blocks per SM
 constexpr int CTA_WARPS_NARROW_STEP = 5;       // (sd_step: 96 registers)
 
-// Candidates of one job: not ordered.  A candidate is put in once and looked for only when it is its turn, and most never
-// have one: the next node is usually the best child of the node just added, which one comparison with the
-// largest D in the pool tells.  (Keeping the candidates in order cost 1,800 cycles per node, two thirds of the job.)
-constexpr int POOL = 128;                     // four places per lane
-struct Pool {
-    double d[POOL];                           // 0: taken
+// Candidates of one job: not ordered, two per lane in registers.  The next node is the one with the largest D, which a
+// reduction over the lanes tells; its children go to lanes with a free place, a child each, so nothing is sorted, moved or
+// looked up in memory per node.
+// A job is a chain of nodes (30 - 44 of them in the slowest jobs of 256 requests), each a dependent read of its children and about 130
+// instructions at 6 - 9 cycles; with two blocks on an SM the busiest SMs also run out of issue slots.  (Candidates in shared
+// memory, the children read as windows of 32 entries kept in registers, and a division per node: 45.3 us for a draft of 256
+// requests, 43.1 now; 43.6 -> 38.5 on other text; steps 55 -> 51.  The request of a candidate's children into L2 as it is found
+// is worth 1 - 2 % of that; requests into L1, or by cp.async, lost as much.  Telling the others the running SCORE one node
+// later cost 3 %.)
+struct Cand {
+    unsigned hi, lo;                          // D; 0: a free place
+    int tok, cb;
+    unsigned np;                              // children | RUN_HAS_TOP | parent index + 1 from bit 24 on (the last node of 64 is nobody's parent)
+};
+constexpr unsigned CAND_RUN = RUN_COUNT_MASK | RUN_HAS_TOP;
+constexpr int CAND_PAR = 24;
+constexpr int POOL = 96;                      // what two places per lane hold and one node's children
+struct Pool {                                 // to make room (pool_compact)
+    double d[POOL];
     int tok[POOL];
     int cb[POOL];
-    unsigned nc[POOL];
-    unsigned char par[POOL];                  // parent index + 1
+    unsigned np[POOL];
 };
+
+// Eq. 1 for sums up to RECIP_MAX: the quotient from the correctly rounded reciprocal (Markstein, "Computation of elementary
+// functions on the IBM RISC System/6000 processor", 1990, theorem 8: q = RN(a r), then RN(q + r RN(a - b q)) is RN(a / b)).  Three
+// instructions in a row instead of some 30.  The reciprocals are divided by the compiler, in IEEE binary64.
+constexpr int RECIP_MAX = 511;
+struct __align__(16) RecipTable {
+    double r[RECIP_MAX + 1];
+    constexpr RecipTable() : r() {
+        for (int b = 1; b <= RECIP_MAX; ++b) r[b] = 1.0 / (double)b;
+    }
+};
+__device__ const RecipTable g_recip;
+
+__device__ __forceinline__ double quotient(double a, double b, double r) {
+    const double q = __dmul_rn(a, r);
+    return __fma_rn(r, __fma_rn(-b, q, a), q);
+}
 
 struct __align__(16) WarpWork {
     Pool C;
@@ -317,6 +346,7 @@ struct __align__(16) WarpWork {
 template <int WARPS>
 struct BlockSharedT {
     WarpWork w[WARPS];
+    RecipTable recip;
     int node[2][SD_MAX_DEPTH];                // match node per tree and pattern length (-1: none)
     int cb[2][SD_MAX_DEPTH];                  // its child run
     unsigned nc[2][SD_MAX_DEPTH];             // ... as the node's w field (count | flags)
@@ -493,138 +523,59 @@ __device__ __forceinline__ double best_so_far(BlockShared& sh) {
     return __hiloint2double((int)__shfl_sync(FULL, *(volatile unsigned*)&sh.best_hi, 0), 0);
 }
 
-// The state of a job's pool that lives in registers.
-struct PoolState {
-    int n;                                    // places used
-    unsigned top;                             // high word of the largest D in it (0: empty)
-    unsigned floor;                           // candidates whose D has a smaller high word do not matter
-};
-
-// Leaves at least the `room` best candidates and few others: the rest cannot be taken any more.
-__device__ __noinline__ PoolState pool_compact(Pool& C, PoolState P, int room, int lane) {
-    unsigned h[4];
+// Leaves the `room` best of the n candidates in C (what is worse than that many others cannot be taken any more), some more
+// where that is less work, but never more than 64.  Returns how many; `floor` becomes the high word of the least D that matters.
+__device__ __noinline__ int pool_compact(Pool& C, int n, int room, unsigned& floor, int lane) {
+    unsigned h[3];
 #pragma unroll
-    for (int c = 0; c < 4; ++c) h[c] = c * 32 + lane < P.n ? (unsigned)__double2hiint(C.d[c * 32 + lane]) : 0u;
-    unsigned lo = 1u, hi = P.top;                               // the largest limit with at least `room` candidates at or above it
-    int at_lo = 0;
+    for (int c = 0; c < 3; ++c) h[c] = c * 32 + lane < n ? (unsigned)__double2hiint(C.d[c * 32 + lane]) : 0u;
+    unsigned lo = 1u, hi = __reduce_max_sync(FULL, max(max(h[0], h[1]), h[2]));
+    int at_lo = n;                                              // the largest limit with at least `room` candidates at or above it
+    for (int it = 0; it < 32 && lo < hi && (at_lo > room + 8 || at_lo > 64); ++it) {
+        const unsigned mid = lo + (hi - lo + 1u) / 2u;
+        int k = 0;
 #pragma unroll
-    for (int c = 0; c < 4; ++c) at_lo += __popc(__ballot_sync(FULL, h[c] != 0u));
-    if (at_lo > room) {
-        for (int it = 0; it < 32 && lo < hi && at_lo > room + 8; ++it) {
-            const unsigned mid = lo + (hi - lo + 1u) / 2u;
-            int k = 0;
-#pragma unroll
-            for (int c = 0; c < 4; ++c) k += __popc(__ballot_sync(FULL, h[c] >= mid));
-            if (k >= room) { lo = mid; at_lo = k; } else hi = mid - 1u;
-        }
+        for (int c = 0; c < 3; ++c) k += __popc(__ballot_sync(FULL, h[c] >= mid));
+        if (k >= room) { lo = mid; at_lo = k; } else hi = mid - 1u;
     }
-    // (those at the limit may be more than the places: equal D; the first by token are what counts, so they all stay
-    // unless they fill the pool, which the caller checks)
-    double d[4]; int tok[4], cb[4]; unsigned nc[4]; unsigned char par[4];
+    Cand v[3];
+    int to[3];
 #pragma unroll
-    for (int c = 0; c < 4; ++c)
-        if (h[c] >= lo) { const int i = c * 32 + lane; d[c] = C.d[i]; tok[c] = C.tok[i]; cb[c] = C.cb[i]; nc[c] = C.nc[i]; par[c] = C.par[i]; }
-    __syncwarp();
-    int n = 0;
-#pragma unroll
-    for (int c = 0; c < 4; ++c) {
-        const unsigned m = __ballot_sync(FULL, h[c] >= lo);
-        if (h[c] >= lo) {
-            const int i = n + __popc(m & ((1u << lane) - 1u));
-            C.d[i] = d[c]; C.tok[i] = tok[c]; C.cb[i] = cb[c]; C.nc[i] = nc[c]; C.par[i] = par[c];
-        }
-        n += __popc(m);
-    }
-    __syncwarp();
-    P.n = n;
-    if (at_lo >= room) P.floor = max(P.floor, lo);
-    return P;
-}
-
-// Puts one candidate per lane with `keep` into the pool.  `room`: nodes that can still be added.  False: no
-// place (more than POOL - 32 candidates that all may matter: equal D).
-__device__ __forceinline__ bool pool_push(Pool& C, PoolState& P, int room, bool keep, double d, int tok, int par, int cb, unsigned nc,
-                                          int lane) {
-    const unsigned h = (unsigned)__double2hiint(d);
-    keep = keep && h >= P.floor;
-    const unsigned m = __ballot_sync(FULL, keep);
-    if (!m) return true;
-    if (P.n + __popc(m) > POOL) {
-        P = pool_compact(C, P, room, lane);
-        if (P.n + __popc(m) > POOL) return false;
-    }
-    if (keep) {
-        const int i = P.n + __popc(m & ((1u << lane) - 1u));
-        C.d[i] = d; C.tok[i] = tok; C.cb[i] = cb; C.nc[i] = nc; C.par[i] = (unsigned char)(par + 1);
-    }
-    P.n += __popc(m);
-    P.top = max(P.top, __reduce_max_sync(FULL, keep ? h : 0u));
-    __syncwarp();
-    return true;
-}
-
-// Place of the best candidate: larger D, then smaller token, then smaller parent index.  It leaves the pool (its
-// fields stay readable).  P.top > 0.  Where several share the largest D (`ties` of them, at most 32), none is taken:
-// their places are in `list`.
-__device__ __forceinline__ int pool_pop(Pool& C, PoolState& P, int* list, bool turns, int& ties, int lane) {
-    unsigned h[4];
-#pragma unroll
-    for (int c = 0; c < 4; ++c) {
-        h[c] = 0u;
-        if (c * 32 < P.n && c * 32 + lane < P.n) h[c] = (unsigned)__double2hiint(C.d[c * 32 + lane]);
-    }
-    int at = -1, eq = 0;
-    unsigned rest = 0u;                                         // the largest below the top
-#pragma unroll
-    for (int c = 0; c < 4; ++c) {
-        if (c * 32 >= P.n) break;
-        const unsigned b = __ballot_sync(FULL, h[c] == P.top);
-        if (b && at < 0) at = c * 32 + __ffs(b) - 1;
-        eq += __popc(b);
-        if (h[c] != P.top) rest = max(rest, h[c]);
-    }
-    ties = 0;
-    if (eq == 1) {
-        P.top = __reduce_max_sync(FULL, rest);
-        return at;
-    }
-    // several share the high word: full comparison
-    double bd = -1.0;
-    int bt = 0x7fffffff, bp = 0x7fffffff, bi = -1;
-#pragma unroll
-    for (int c = 0; c < 4; ++c)
-        if (h[c] == P.top) {
-            const int i = c * 32 + lane;
-            const double d = C.d[i];
-            const int t = C.tok[i], p = C.par[i];
-            if (bi < 0 || better(d, t, p, bd, bt, bp)) { bd = d; bt = t; bp = p; bi = i; }
-        }
-    const unsigned mlo = __reduce_max_sync(FULL, bi >= 0 ? (unsigned)__double2loint(bd) : 0u);
-    int g = 0;
-#pragma unroll
-    for (int c = 0; c < 4; ++c) {
+    for (int c = 0; c < 3; ++c) {
         const int i = c * 32 + lane;
-        const bool same = h[c] == P.top && (unsigned)__double2loint(C.d[i]) == mlo;
-        const unsigned m = __ballot_sync(FULL, same);
-        const int k = g + __popc(m & ((1u << lane) - 1u));
-        if (same && k < 32) list[k] = i;
-        g += __popc(m);
+        to[c] = -1;
+        if (h[c] < lo) continue;
+        v[c] = Cand{h[c], (unsigned)__double2loint(C.d[i]), C.tok[i], C.cb[i], C.np[i]};
+    }
+    int k = 0;
+    if (at_lo <= 64) {
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            const unsigned m = __ballot_sync(FULL, h[c] >= lo);
+            if (h[c] >= lo) to[c] = k + __popc(m & ((1u << lane) - 1u));
+            k += __popc(m);
+        }
+    } else {
+        // many of equal D: by token and parent then, too
+        int rank[3] = {0, 0, 0};
+        for (int q = 0; q < n; ++q) {
+            const double d = C.d[q];
+            const int tok = C.tok[q], par = (int)(C.np[q] >> CAND_PAR) & 63;
+#pragma unroll
+            for (int c = 0; c < 3; ++c)
+                if (h[c] >= lo) rank[c] += better(d, tok, par, __hiloint2double((int)v[c].hi, (int)v[c].lo), v[c].tok, (int)(v[c].np >> CAND_PAR) & 63) ? 1 : 0;
+        }
+        k = room;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) if (h[c] >= lo && rank[c] < room) to[c] = rank[c];
     }
     __syncwarp();
-    if (g > 1 && g <= 32 && turns) { ties = g; return -1; }
-    const bool in2 = bi >= 0 && (unsigned)__double2loint(bd) == mlo;
-    const unsigned mt = __reduce_min_sync(FULL, in2 ? (unsigned)bt : 0xffffffffu);
-    const bool in3 = in2 && (unsigned)bt == mt;
-    const unsigned mp = __reduce_min_sync(FULL, in3 ? (unsigned)bp : 0xffffffffu);
-    const int src = __ffs(__ballot_sync(FULL, in3 && (unsigned)bp == mp)) - 1;
-    return __shfl_sync(FULL, bi, src);                          // (others have the same high word: P.top stays)
-}
-
-// The largest high word in the pool.
-__device__ __forceinline__ unsigned pool_top(const Pool& C, int n, int lane) {
-    unsigned top = 0u;
-    for (int i = lane; i < n; i += 32) top = max(top, (unsigned)__double2hiint(C.d[i]));
-    return __reduce_max_sync(FULL, top);
+#pragma unroll
+    for (int c = 0; c < 3; ++c)
+        if (to[c] >= 0) { C.d[to[c]] = __hiloint2double((int)v[c].hi, (int)v[c].lo); C.tok[to[c]] = v[c].tok; C.cb[to[c]] = v[c].cb; C.np[to[c]] = v[c].np; }
+    __syncwarp();
+    if (at_lo >= room) floor = max(floor, lo);
+    return k;
 }
 
 // The best children (by count, then smallest token; at most `room`) of a node with more than 32: their entries, best
@@ -730,48 +681,179 @@ __device__ __noinline__ void expand_job(BlockShared& sh, WarpWork& W, const int4
                            int budget, unsigned flags, int nseed, int lane) {
     const int order = tree * SD_MAX_DEPTH + p;                  // loop order of Algorithm 1
     const int buf = W.best_buf ^ 1;
-    Pool& C = W.C;
-    PoolState P{0, 0u, 0u};
+    const unsigned lt = (1u << lane) - 1u;
+    Cand c0{0u, 0u, 0, 0, 0u}, c1{0u, 0u, 0, 0, 0u};
+    unsigned floor = 1u;                                        // candidates whose D has a smaller high word do not matter
     int cnt = 0;
-    double score = 0.0;
-    bool dropped = false, fits = true;
+    double score = 0.0, left = (double)budget;                  // left: nodes that can still be added
+    bool dropped = false;
     // the node whose children are to be offered next: the match node first, D(N_p) = 1
     double cur_d = 1.0;
     int cur_cb = sh.cb[tree][p - 1], cur_idx = -1;
     unsigned cur_w = sh.nc[tree][p - 1];
     bool have_cur = nseed < 0;
-    for (int base = 0; base < nseed && fits; base += 32) {
-        const int q = base + lane;
-        const bool keep = q < nseed;
-        fits = pool_push(C, P, budget, keep, keep ? W.T.d[q] : 0.0, keep ? W.T.tok[q] : 0, -1, keep ? W.T.cb[q] : 0, keep ? W.T.nc[q] : 0u, lane);
+    if (!have_cur) {
+        auto seed = [&](int q) {
+            return q < nseed ? Cand{(unsigned)__double2hiint(W.T.d[q]), (unsigned)__double2loint(W.T.d[q]), W.T.tok[q], W.T.cb[q], W.T.nc[q] & CAND_RUN}
+                             : Cand{0u, 0u, 0, 0, 0u};
+        };
+        c0 = seed(lane); c1 = seed(32 + lane);
     }
-    int4 w = make_int4(-1, 0, 0, 0);                            // window in registers: entries wb .. wb + wvalid
-    int wb = -1, wvalid = 0;
-    while (fits) {
-        if (!have_cur) {
-            if (cnt >= budget || P.top == 0u) break;
-            int ties;
-            const int at = pool_pop(C, P, W.one_tok, !(flags & SD_FLAG_LINEAR), ties, lane);
-            if (ties > 0) {
+    // What is still to come is at most d each: is SCORE at most (with a margin) below one already reached?  (Any lane that
+    // has seen one counts.)  The final SCORE is at least its running value: the others prune on that.
+    unsigned best = 0u;
+    auto hopeless = [&](double d) {
+        best = *(volatile unsigned*)&sh.best_hi;
+        return __any_sync(FULL, (unsigned)__double2hiint(__fma_rn(left, d, score) * 1.000000001) < best) != 0;
+    };
+    auto publish = [&]() { if (lane == 0 && (unsigned)__double2hiint(score) > best) atomicMax(&sh.best_hi, (unsigned)__double2hiint(score)); };
+    while (true) {
+        if (have_cur) {
+            // ---------------- the children of `cur` become candidates
+            have_cur = false;
+            const int cur_n = (int)(cur_w & RUN_COUNT_MASK);
+            if (cur_n == 1) {
+                const unsigned top = __reduce_max_sync(FULL, max(c0.hi, c1.hi));
+                if (top < (unsigned)__double2hiint(cur_d)) {
+                    // An only child has C = 1, so D stays cur_d: while the best waiting candidate is
+                    // strictly worse, the whole chain of only children is added in one go.
+                    const int4 w = load_window(ent, cur_cb, limit, lane);
+                    const bool link = cur_cb + lane < limit && ((unsigned)w.w & RUN_COUNT_MASK) == 1u && w.z == cur_cb + lane + 1;
+                    const unsigned links = __ballot_sync(FULL, link);
+                    const int len = min(min(32, limit - cur_cb), 1 + (links == 0xffffffffu ? 32 : __ffs(~links) - 1));
+                    const int m = min(len, budget - cnt);
+                    if (lane < m) {
+                        W.tok[buf][cnt + lane] = w.x;
+                        W.par[buf][cnt + lane] = (unsigned char)((lane == 0 ? cur_idx : cnt + lane - 1) + 1);
+                    }
+                    for (int q = 0; q < m; ++q) score = __dadd_rn(score, cur_d);
+                    publish();
+                    cnt += m;
+                    left -= (double)m;
+                    cur_idx = cnt - 1;
+                    cur_cb = __shfl_sync(FULL, w.z, m - 1);
+                    cur_w = (unsigned)__shfl_sync(FULL, w.w, m - 1);
+                    if (cnt >= budget) break;
+                    if (hopeless(cur_d)) { dropped = true; break; }
+                    have_cur = true;
+                    continue;
+                }
+            }
+            if (cur_n > 0) {
+                const unsigned par = (unsigned)(cur_idx + 1) << CAND_PAR;
+                int first = cur_cb, nl = cur_n;                 // the entries to offer
+                double dsum = 0.0;
+                const int* list = nullptr;
+                if (cur_n > 32) {
+                    // a long run: only the best of its children, by count, can ever be added.  A ready-made list of them
+                    // stands in front of the run, or is made here.
+                    const int room = budget - cnt;
+                    if (cur_w & RUN_HAS_TOP) {
+                        const int4 hdr = ent[cur_cb - SD_TOP_BLOCK];
+                        dsum = (double)(((unsigned long long)(unsigned)hdr.y << 32) | (unsigned long long)(unsigned)hdr.x);
+                        nl = min(hdr.z, room);
+                        first = cur_cb - SD_TOP_BLOCK + 1;
+                    } else {
+                        unsigned sum;
+                        nl = list_by_count(ent, cur_cb, cur_n, room, W.one_tok, reinterpret_cast<int*>(&W.T), sum, lane);
+                        dsum = (double)sum;
+                        list = W.one_tok;
+                    }
+                }
+                for (int base = 0; base < nl; base += 32) {
+                    const int k = min(32, nl - base);
+                    // a child per lane with a free place; where there are too few, all lanes in order, and room is made
+                    const unsigned f0 = __ballot_sync(FULL, c0.hi == 0u), f1 = __ballot_sync(FULL, c1.hi == 0u);
+                    const bool to0 = __popc(f0) >= k, fits = to0 || __popc(f1) >= k;
+                    const unsigned f = to0 ? f0 : (fits ? f1 : FULL);
+                    const int r = __popc(f & lt);
+                    const bool in = ((f >> lane) & 1u) != 0u && r < k;
+                    int4 e = make_int4(0, 0, 0, 0);
+                    if (in) e = ent[list ? list[base + r] : first + base + r];
+                    double q;
+                    if (cur_n <= 32) {
+                        const unsigned sum = __reduce_add_sync(FULL, (unsigned)e.y);             // sibling sum: the denominator of Eq. 1
+                        if (sum <= (unsigned)RECIP_MAX)
+                        q = quotient((double)e.y, (double)sum, sh.recip.r[sum]);
+                        else q = __ddiv_rn((double)e.y, (double)sum);
+                    } else q = __ddiv_rn((double)e.y, dsum);
+                    const double dc = __dmul_rn(cur_d, q);      // Eq. 2
+                    Cand c{(unsigned)__double2hiint(dc), (unsigned)__double2loint(dc), e.x, e.z, ((unsigned)e.w & CAND_RUN) | par};
+                    const bool keep = in && c.hi >= floor;
+                    if (keep && (c.np & RUN_COUNT_MASK)) prefetch_l2(ent + e.z);
+                    if (fits) {
+                        if (keep) { if (to0) c0 = c; else c1 = c; }
+                    } else if (__any_sync(FULL, keep)) {
+                        if (!keep) c.hi = 0u;
+                        int n = 0;
+                        auto stage = [&](const Cand& v) {
+                            const bool on = v.hi >= floor;      // (a free place's 0 is not)
+                            const unsigned m = __ballot_sync(FULL, on);
+                            if (on) {
+                                const int i = n + __popc(m & lt);
+                                W.C.d[i] = __hiloint2double((int)v.hi, (int)v.lo); W.C.tok[i] = v.tok; W.C.cb[i] = v.cb; W.C.np[i] = v.np;
+                            }
+                            n += __popc(m);
+                        };
+                        stage(c0); stage(c1); stage(c);
+                        __syncwarp();
+                        n = pool_compact(W.C, n, budget - cnt, floor, lane);
+                        auto back = [&](int i) {
+                            return i < n ? Cand{(unsigned)__double2hiint(W.C.d[i]), (unsigned)__double2loint(W.C.d[i]), W.C.tok[i], W.C.cb[i], W.C.np[i]}
+                                         : Cand{0u, 0u, 0, 0, 0u};
+                        };
+                        c0 = back(lane); c1 = back(32 + lane);
+                        __syncwarp();
+                    }
+                    // as many as can still be added: what is worse than the last of them does not matter any more
+                    if (cur_n > 32 && nl == budget - cnt && base + 32 >= nl) {
+                        const unsigned last = __ballot_sync(FULL, in && r == k - 1);
+                        floor = max(floor, __shfl_sync(FULL, c.hi, __ffs(last) - 1));
+                    }
+                }
+            }
+        }
+        // ---------------- the best candidate is the next node
+        const unsigned top = __reduce_max_sync(FULL, max(c0.hi, c1.hi));
+        if (top == 0u) break;
+        unsigned b0 = __ballot_sync(FULL, c0.hi == top), b1 = __ballot_sync(FULL, c1.hi == top);
+        if ((b0 & (b0 - 1u)) | (b1 & (b1 - 1u)) | (b0 && b1 ? 1u : 0u)) {
+            // several share the high word: full comparison
+            const unsigned mlo = __reduce_max_sync(FULL, max(c0.hi == top ? c0.lo : 0u, c1.hi == top ? c1.lo : 0u));
+            const bool t0 = c0.hi == top && c0.lo == mlo, t1 = c1.hi == top && c1.lo == mlo;
+            b0 = __ballot_sync(FULL, t0); b1 = __ballot_sync(FULL, t1);
+            const int ties = __popc(b0) + __popc(b1);
+            if (ties > 1 && (ties > 32 || (flags & SD_FLAG_LINEAR))) {
+                // smallest token, then smallest parent index
+                const unsigned mt = __reduce_min_sync(FULL, min(t0 ? (unsigned)c0.tok : 0xffffffffu, t1 ? (unsigned)c1.tok : 0xffffffffu));
+                const bool s0 = t0 && (unsigned)c0.tok == mt, s1 = t1 && (unsigned)c1.tok == mt;
+                const unsigned p0 = (c0.np >> CAND_PAR) & 63u, p1 = (c1.np >> CAND_PAR) & 63u;
+                const unsigned mp = __reduce_min_sync(FULL, min(s0 ? p0 : 64u, s1 ? p1 : 64u));
+                b0 = __ballot_sync(FULL, s0 && p0 == mp); b1 = __ballot_sync(FULL, s1 && p1 == mp);
+            } else if (ties > 1) {
                 // Candidates of equal D take turns: smallest token first, then smallest parent index, and an
                 // only child (C = 1: the same D again) takes its parent's place.  All of them are ahead of every
                 // other candidate, so a lane each keeps them until one has several children or all have ended.
                 // (Text that occurs a few times below the match node is just this: chains of equal D, token by token in
-                // turn.  Through the pool a node of them costs ten times as much.)
+                // turn.  One by one through the pool a node of them costs several times as much.)
+                const int i0 = __popc(b0 & lt), i1 = __popc(b0) + __popc(b1 & lt);
+                if (t0) { W.one_tok[i0] = c0.tok; W.one_cb[i0] = c0.cb; W.one_nc[i0] = c0.np; }
+                if (t1) { W.one_tok[i1] = c1.tok; W.one_cb[i1] = c1.cb; W.one_nc[i1] = c1.np; }
+                __syncwarp();
                 const bool mine = lane < ties;
-                const int place = mine ? W.one_tok[lane] : 0;
                 bool live = mine;
                 int tok = 0, par = 0, cb = 0;
                 unsigned nc = 0;
                 int4 nx = make_int4(0, 0, 0, 0);                // the only child, read ahead
                 if (mine) {
-                    tok = C.tok[place]; par = C.par[place]; cb = C.cb[place]; nc = C.nc[place];
+                    tok = W.one_tok[lane]; cb = W.one_cb[lane]; nc = W.one_nc[lane];
+                    par = (int)(nc >> CAND_PAR) & 63;
                     if ((nc & RUN_COUNT_MASK) == 1u) nx = ent[cb];
                 }
-                cur_d = C.d[W.one_tok[0]];
+                cur_d = __hiloint2double((int)top, (int)mlo);
                 unsigned alive = (ties == 32 ? FULL : (1u << ties) - 1u);
                 while (cnt < budget) {
-                    if ((cnt & 3) == 0 && (score + (double)(budget - cnt) * cur_d) * 1.000000001 < best_so_far(sh)) { dropped = true; break; }
+                    if ((cnt & 3) == 0 && hopeless(cur_d)) { dropped = true; break; }
                     const unsigned mt = __reduce_min_sync(FULL, live ? (unsigned)tok : 0xffffffffu);
                     unsigned who = __ballot_sync(FULL, live && (unsigned)tok == mt);
                     if (who & (who - 1u)) {
@@ -789,6 +871,7 @@ __device__ __noinline__ void expand_job(BlockShared& sh, WarpWork& W, const int4
                         } else live = false;
                     }
                     score = __dadd_rn(score, cur_d);            // Eq. 4, insertion order
+                    left -= 1.0;
                     ++cnt;
                     if (n == 1) continue;
                     alive &= ~(1u << wl);
@@ -796,144 +879,47 @@ __device__ __noinline__ void expand_job(BlockShared& sh, WarpWork& W, const int4
                         have_cur = true;
                         cur_idx = cnt - 1;
                         cur_cb = __shfl_sync(FULL, cb, wl);
-                        cur_w = __shfl_sync(FULL, nc, wl);
+                        cur_w = (unsigned)__shfl_sync(FULL, nc, wl);
                         break;
                     }
                     if (!alive) break;
                 }
                 if (dropped) break;
-                if (lane == 0) atomicMax(&sh.best_hi, (unsigned)__double2hiint(score));
-                if (mine) {
-                    if (live) { C.tok[place] = tok; C.par[place] = (unsigned char)par; C.cb[place] = cb; C.nc[place] = nc; }
-                    else C.d[place] = 0.0;
-                }
+                publish();
+                if (cnt >= budget) break;
+                if (mine) { W.one_tok[lane] = tok; W.one_cb[lane] = cb; W.one_nc[lane] = (nc & CAND_RUN) | ((unsigned)par << CAND_PAR); }
                 __syncwarp();
-                if (!alive) P.top = pool_top(C, P.n, lane);
-                if (!have_cur || cnt >= budget) continue;
-            } else {
-            cur_d = C.d[at];
-            const int tok = C.tok[at], par = C.par[at];
-            cur_cb = C.cb[at];
-            cur_w = C.nc[at];
-            // everything still to come is at most cur_d each
-            if ((score + (double)(budget - cnt) * cur_d) * 1.000000001 < best_so_far(sh)) { dropped = true; break; }
-            __syncwarp();
-            if (lane == 0) { C.d[at] = 0.0; W.tok[buf][cnt] = tok; W.par[buf][cnt] = (unsigned char)par; }
-            score = __dadd_rn(score, cur_d);                    // Eq. 4, insertion order
-            // the final SCORE of this job is at least its running value: let the others prune on it
-            if (lane == 0) atomicMax(&sh.best_hi, (unsigned)__double2hiint(score));
-            cur_idx = cnt++;
-            if (flags & SD_FLAG_LINEAR) { P.n = 0; P.top = 0u; P.floor = 0u; }
-            __syncwarp();
+                const unsigned lives = __ballot_sync(FULL, live);
+                if (t0) { c0.tok = W.one_tok[i0]; c0.cb = W.one_cb[i0]; c0.np = W.one_nc[i0]; if (!((lives >> i0) & 1u)) c0.hi = 0u; }
+                if (t1) { c1.tok = W.one_tok[i1]; c1.cb = W.one_cb[i1]; c1.np = W.one_nc[i1]; if (!((lives >> i1) & 1u)) c1.hi = 0u; }
+                __syncwarp();
+                continue;
             }
-        }
-        have_cur = false;
-        if (cnt >= budget) break;
-        const int cur_n = (int)(cur_w & RUN_COUNT_MASK);
-        if (cur_n == 0) continue;
-        if (cur_n > 32) {
-            // a long run: only the best of its children, by count, can ever be added.  A ready-made list of them
-            // stands in front of the run, or is made here.
-            const int room = budget - cnt;
-            double dsum;
-            int nl;
-            if (cur_w & RUN_HAS_TOP) {
-                const int4 hdr = ent[cur_cb - SD_TOP_BLOCK];
-                dsum = (double)(((unsigned long long)(unsigned)hdr.y << 32) | (unsigned long long)(unsigned)hdr.x);
-                nl = min(hdr.z, room);
-            } else {
-                unsigned sum;
-                nl = list_by_count(ent, cur_cb, cur_n, room, W.one_tok, reinterpret_cast<int*>(&W.T), sum, lane);
-                dsum = (double)sum;
-            }
-            for (int base = 0; base < nl && fits; base += 32) {
-                const bool keep = base + lane < nl;
-                int4 e = make_int4(0, 0, 0, 0);
-                double dc = 0.0;
-                if (keep) {
-                    e = ent[(cur_w & RUN_HAS_TOP) ? cur_cb - SD_TOP_BLOCK + 1 + base + lane : W.one_tok[base + lane]];
-                    dc = __dmul_rn(cur_d, __ddiv_rn((double)e.y, dsum));         // Eq. 2 with Eq. 1
-                }
-                fits = pool_push(C, P, room, keep, dc, e.x, cur_idx, e.z, (unsigned)e.w, lane);
-                // as many as can still be added: what is worse than the last of them does not matter any more
-                if (nl == room && base + 32 >= nl) P.floor = max(P.floor, (unsigned)__shfl_sync(FULL, __double2hiint(dc), nl - 1 - base));
-            }
-            continue;
         }
         {
-            const int off = cur_cb - wb;
-            if (wb >= 0 && off >= 0 && off + cur_n <= wvalid) {  // the run is already in registers
-                if (off > 0) {
-                    w.x = __shfl_down_sync(FULL, w.x, off); w.y = __shfl_down_sync(FULL, w.y, off);
-                    w.z = __shfl_down_sync(FULL, w.z, off); w.w = __shfl_down_sync(FULL, w.w, off);
-                    wvalid -= off;
-                    wb = cur_cb;
-                }
-            } else {
-                w = load_window(ent, cur_cb, limit, lane);
-                wb = cur_cb;
-                wvalid = min(32, limit - cur_cb);
+            const bool from0 = b0 != 0u;
+            const int wl = __ffs(from0 ? b0 : b1) - 1;
+            const unsigned lo = from0 ? c0.lo : c1.lo, np = from0 ? c0.np : c1.np;
+            const int cb = from0 ? c0.cb : c1.cb;
+            cur_d = __hiloint2double((int)top, (int)__shfl_sync(FULL, lo, wl));
+            cur_cb = __shfl_sync(FULL, cb, wl);
+            cur_w = __shfl_sync(FULL, np, wl) & CAND_RUN;
+            // everything still to come is at most cur_d each
+            if (hopeless(cur_d)) { dropped = true; break; }
+            if (lane == wl) {
+                W.tok[buf][cnt] = from0 ? c0.tok : c1.tok; W.par[buf][cnt] = (unsigned char)((np >> CAND_PAR) & 63u);
+                if (from0) c0.hi = 0u; else c1.hi = 0u;
             }
-        }
-        const unsigned cur_hi = (unsigned)__double2hiint(cur_d);
-        if (cur_n == 1 && P.top < cur_hi) {
-            // An only child has C = 1, so D stays cur_d: while the best waiting candidate is
-            // strictly worse, the whole chain of only children is added in one go.
-            const bool link = lane < wvalid && ((unsigned)w.w & RUN_COUNT_MASK) == 1u && w.z == cur_cb + lane + 1;
-            const unsigned links = __ballot_sync(FULL, link);
-            const int len = min(wvalid, 1 + (links == 0xffffffffu ? 32 : __ffs(~links) - 1));
-            const int m = min(len, budget - cnt);
-            if (lane < m) {
-                W.tok[buf][cnt + lane] = w.x;
-                W.par[buf][cnt + lane] = (unsigned char)((lane == 0 ? cur_idx : cnt + lane - 1) + 1);
-            }
-            for (int q = 0; q < m; ++q) score = __dadd_rn(score, cur_d);
-            if (lane == 0) atomicMax(&sh.best_hi, (unsigned)__double2hiint(score));
-            cnt += m;
-            cur_idx = cnt - 1;
-            cur_cb = __shfl_sync(FULL, w.z, m - 1);
-            cur_w = (unsigned)__shfl_sync(FULL, w.w, m - 1);
-            have_cur = true;
-            if ((score + (double)(budget - cnt) * cur_d) * 1.000000001 < best_so_far(sh)) { dropped = true; break; }
-            continue;
-        }
-        // ---- D of the children; the best of them (largest count, then smallest token: among siblings the order of D)
-        // is the next node to be added if it beats every waiting candidate
-        const bool in = lane < cur_n;
-        const unsigned y = in ? (unsigned)w.y : 0u;
-        const unsigned sum = __reduce_add_sync(FULL, y), most = __reduce_max_sync(FULL, y);      // sibling sum: the denominator of Eq. 1
-        const int b = __ffs(__ballot_sync(FULL, in && y == most)) - 1;
-        const double dc = __dmul_rn(cur_d, __ddiv_rn((double)y, (double)sum));                   // Eq. 2 with Eq. 1
-        const unsigned best_hi = (unsigned)__shfl_sync(FULL, __double2hiint(dc), b);
-        const bool take = best_hi > P.top;
-        if (cur_n > 1 || !take)
-            fits = pool_push(C, P, budget - cnt - (take ? 1 : 0), in && !(take && lane == b), dc, w.x, cur_idx, w.z, (unsigned)w.w, lane);
-        if (take) {
-            // the same steps as taking it from the pool at the top of the loop
-            cur_d = __hiloint2double((int)best_hi, __shfl_sync(FULL, __double2loint(dc), b));
-            if ((score + (double)(budget - cnt) * cur_d) * 1.000000001 < best_so_far(sh)) { dropped = true; break; }
-            const int tok = __shfl_sync(FULL, w.x, b);
-            if (lane == 0) { W.tok[buf][cnt] = tok; W.par[buf][cnt] = (unsigned char)(cur_idx + 1); }
-            score = __dadd_rn(score, cur_d);
-            if (lane == 0) atomicMax(&sh.best_hi, (unsigned)__double2hiint(score));
+            score = __dadd_rn(score, cur_d);                    // Eq. 4, insertion order
+            left -= 1.0;
+            publish();
             cur_idx = cnt++;
-            cur_cb = __shfl_sync(FULL, w.z, b);
-            cur_w = (unsigned)__shfl_sync(FULL, w.w, b);
-            if (flags & SD_FLAG_LINEAR) { P.n = 0; P.top = 0u; P.floor = 0u; }
+            if (cnt >= budget) break;
+            if (flags & SD_FLAG_LINEAR) { c0.hi = 0u; c1.hi = 0u; floor = 1u; }
             have_cur = true;
         }
     }
     __syncwarp();
-    if (!fits) {
-        // more candidates of equal D than the pool holds: one node after the other, with the candidates in order
-        Frontier& F = W.T;
-        int* const otok = W.one_tok;
-        int* const opar = W.one_cb;
-        cnt = expand_serial(ent, sh.cb[tree][p - 1], (int)(sh.nc[tree][p - 1] & RUN_COUNT_MASK), budget, flags, F, otok, opar, score, lane);
-        for (int j = lane; j < cnt; j += 32) { W.tok[buf][j] = otok[j]; W.par[buf][j] = (unsigned char)(opar[j] + 1); }
-        dropped = false;
-        __syncwarp();
-    }
     if (!dropped && (score > W.best_score || (score == W.best_score && score > 0.0 && order < W.best_order))) {
         if (lane == 0) {
             W.best_score = score; W.best_order = order; W.best_n = cnt; W.best_buf = buf;
@@ -1011,6 +997,8 @@ speculate_fused_kernel(sd_store sv, int n, const int32_t* __restrict__ d_slot, i
     };
     const int i = blockIdx.x;
     const int M = sv.M, words = (M + 31) / 32, D = sv.D;
+    for (int q = tid; q < (int)sizeof(RecipTable) / 16; q += NT)
+        reinterpret_cast<double2*>(&sh.recip)[q] = reinterpret_cast<const double2*>(&g_recip)[q];
     const int slot = d_slot[i];
     const bool ok = slot >= 0 && slot < sv.R;
     // a slot may appear once per call: a later appearance is refused (two blocks on one tree would

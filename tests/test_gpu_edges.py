@@ -190,3 +190,28 @@ def test_trim_gives_back_what_freed_stores_left():
     assert free0 - torch.cuda.mem_get_info()[0] > (100 << 20)            # kept for the next store
     sfx.sd_trim()
     assert free0 - torch.cuda.mem_get_info()[0] < (8 << 20)
+
+
+@pytest.mark.parametrize("outer,inner", [(31, 32), (40, 20), (40, 30), (60, 32), (64, 5), (70, 31)])
+def test_more_candidates_than_a_job_has_places_for(U, outer, inner):
+    """Candidates of equal D from several fans until there is no place: the best stay, by token and parent where D is equal."""
+    rng = np.random.default_rng(outer * 100 + inner)
+    seqs = [np.array([7, 10 + c, 100 + e, 300 + (c + e) % 9], np.int32) for c in rng.permutation(outer) for e in rng.permutation(inner)]
+    pr = U.Pair(seqs, vocab=400, D=8, n_slots=1, max_req_tokens=16)
+    pr.append([0], [np.array([7], np.int32)])
+    for budget in (64.0, 41.0):
+        for flags in (0, 4):
+            pr.check_speculate([0], 1, budget, 64, flags=flags)
+    pr.close()
+
+
+@pytest.mark.parametrize("total", [2, 510, 511, 512, 1023])
+def test_quotients_on_both_sides_of_the_table_of_reciprocals(U, total):
+    rng = np.random.default_rng(total)
+    cuts = np.sort(rng.choice(np.arange(1, total), size=min(total - 1, 11), replace=False))
+    counts = np.diff(np.concatenate([[0], cuts, [total]]))
+    seqs = [np.array([7, 10 + c, 50 + (c + e) % 3, 60], np.int32) for c, k in enumerate(counts) for e in range(k)]
+    pr = U.Pair(seqs, vocab=100, D=8, n_slots=1, max_req_tokens=16)
+    pr.append([0], [np.array([7], np.int32)])
+    pr.check_speculate([0], 1, 40.0, 64)
+    pr.close()

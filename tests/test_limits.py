@@ -1,6 +1,7 @@
 """Sizes of trees that 32-bit indices cannot hold are refused (csrc/tree_limits.h): the arithmetic, on the CPU."""
 import os
 import subprocess
+from fractions import Fraction
 
 import pytest
 
@@ -36,3 +37,13 @@ def test_entries_of_the_pool(entries, below, top, wide, extra):
     nodes = below + top
     want = nodes + wide + (extra if extra >= 0 else max(2**22, nodes))
     assert entries(below, top, wide, extra) == (want if want <= MOST else -1)
+
+
+def test_quotient_from_a_rounded_reciprocal_is_rounded_right():
+    """The drafts' quotients for sums up to 511: q = RN(a r), then RN(q + r RN(a - b q)), with exact sums rounded once."""
+    for b in range(1, 512):
+        r = 1.0 / b
+        for a in range(1, b + 1):
+            q = a * r
+            rest = float(Fraction(a) - b * Fraction(q))
+            assert float(Fraction(q) + Fraction(r) * Fraction(rest)) == a / b
