@@ -351,16 +351,16 @@ struct BlockSharedT {
     int cb[2][SD_MAX_DEPTH];                  // its child run
     unsigned nc[2][SD_MAX_DEPTH];             // ... as the node's w field (count | flags)
     unsigned char ordp[SD_MAX_DEPTH];         // pattern lengths - 1 by the number of nodes their jobs can add at most
-    int job[2 * SD_MAX_DEPTH];
     int wide[2 * SD_MAX_DEPTH];               // jobs whose match node has a wide child run
-    int njobs, next, nwide, nwide_kept;
+    int nwide, nwide_kept;
+    unsigned ready[2];                        // per tree: jobs to be taken, a bit per place in ordp
+    int walking, appending;                   // warps whose match nodes are still to come; the request's are
+    int gave_up;                              // a warp waited too long for them
     long long slice_sum[WARPS];
     int slice_fs[WARPS];
     AppendShared app;
     int src_node[SD_MAX_DEPTH];               // where the walk to a global match node starts: node (-1: nowhere) ...
     int src_from[SD_MAX_DEPTH];               // ... and the first token to take
-    int app_done;                             // sd_step: warp 0 has appended the new tokens
-    int nlate, late[SD_MAX_DEPTH];            // per-request jobs whose wait for the append ran out
     unsigned best_hi;                         // high word of the largest SCORE reached so far: a lower
                                               // bound of it (scores are non-negative doubles), which is
                                               // all the pruning needs; 32 bits keep the atomic native
@@ -516,11 +516,6 @@ __device__ void counts_to_d(Frontier& F, int fh, int fs, double d_parent, long l
         F.d[q] = __dmul_rn(d_parent, __ddiv_rn(F.d[q], dsum));
     }
     __syncwarp();
-}
-
-template <class BlockShared>
-__device__ __forceinline__ double best_so_far(BlockShared& sh) {
-    return __hiloint2double((int)__shfl_sync(FULL, *(volatile unsigned*)&sh.best_hi, 0), 0);
 }
 
 // Leaves the `room` best of the n candidates in C (what is worse than that many others cannot be taken any more), some more
@@ -929,50 +924,22 @@ __device__ __noinline__ void expand_job(BlockShared& sh, WarpWork& W, const int4
     __syncwarp();
 }
 
-// A per-request job that goes through the tree's entries: the match node of pattern length p is
-// the slot's active node of depth p (kept current by the append).  Whole warp.
-template <class BlockShared>
-__device__ void request_tree_job(BlockShared& sh, WarpWork& W, const sd_store& sv, const SlotState* ss, const int4* s_ent, int t,
-                                 int p, int budget, unsigned flags, int lane) {
-    // an append that stopped early leaves a context the jobs were not made for
-    if (ss->len != t || (ss->status & (SD_STATUS_POOL_FULL | SD_STATUS_BAD_TOKEN))) return;
-    int node = -1;
-    unsigned rw = 0;
-    if (lane == 0) {
-        node = ss->active[p - 1];
-        int rcb = ss->run_cb[p - 1];
-        rw = ss->run_w[p - 1];
-        if (node >= 0 && rw == RUN_UNKNOWN) { const int4 e = s_ent[node]; rcb = e.z; rw = (unsigned)e.w; }
-        sh.node[1][p - 1] = node; sh.cb[1][p - 1] = rcb; sh.nc[1][p - 1] = rw;
-    }
-    node = __shfl_sync(FULL, node, 0);
-    rw = (unsigned)__shfl_sync(FULL, rw, 0);
-    __syncwarp();
-    const int nch = (int)(rw & RUN_COUNT_MASK);
-    if (node < 0 || nch == 0) return;
-    if (nch > WIDE_RUN && !(rw & RUN_HAS_TOP)) {                 // scanned by all warps together, later
-        if (lane == 0) sh.wide[atomicAdd(&sh.nwide, 1)] = SD_MAX_DEPTH + p - 1;
-        return;
-    }
-    expand_job(sh, W, s_ent, (int)sv.spn, 1, p, budget, flags, -1, lane);
-}
-
 // One block of W warps per request.
 //   1. match.  Global tree: the match nodes are advanced from the nodes cached at the previous
 //      call by descending only the tokens appended since (full walks when the cache is stale).
 //      Per-request tree: the slot's active nodes are the match nodes (sd_step: once the append
 //      is done).
-//   2. expand: the (tree, p) jobs that matched go into a queue, costliest first; a warp per job.
+//   2. expand: a (tree, p) job can be taken as soon as its match node is known, costliest first; a warp per job.
 //      sd_step: warp 0 appends the accepted tokens to the request's tree
-//      meanwhile, exactly as sd_append would, and joins the queue when it is done; the other
-//      warps meet at a barrier of their own until then, and only a warp that has taken a job
-//      through the request's tree waits for the append (a bounded wait on a flag).
+//      meanwhile, exactly as sd_append would; the jobs of that tree can be taken when it is done.  (A warp that finds
+//      nothing to take while something is still to come waits, but not for ever: what is left then is done behind the
+//      block-wide barrier.)
 //   3. jobs of either tree that start at a wide child run without top block are scanned by all
 //      warps together, behind a block-wide barrier.
 //   4. select + emit from shared memory; no global scratch.
 // A job is skipped or dropped, exactly, as soon as an upper bound of its SCORE falls below a
 // score another job of the request has already reached (the running scores are published).
-constexpr int BAR_GROUP = 1, BAR_JOIN = 2;    // hardware barriers beside the block-wide one
+constexpr int WALKERS = 8;                    // warps that walk to global match nodes, four pattern lengths each
 
 template <bool STEP, int WARPS, int MINB>
 __global__ void __launch_bounds__(WARPS * 32, MINB)
@@ -991,10 +958,8 @@ speculate_fused_kernel(sd_store sv, int n, const int32_t* __restrict__ d_slot, i
     BlockShared& sh = *reinterpret_cast<BlockShared*>(smem_raw);
     const int tid = threadIdx.x, lane = tid & 31, wib = tid >> 5;
     const int gtid = tid - GW0 * 32, gw = wib - GW0;             // index inside that group (negative: warp 0 of sd_step)
-    auto group_sync = [&]() {
-        if (STEP) asm volatile("bar.sync %0, %1;" ::"r"(BAR_GROUP), "r"(GT) : "memory");
-        else __syncthreads();
-    };
+    constexpr bool SPLIT = GWARPS > WALKERS;                     // the warps that do not walk look ahead for the append
+    constexpr int WALK = SPLIT ? WALKERS : GWARPS;
     const int i = blockIdx.x;
     const int M = sv.M, words = (M + 31) / 32, D = sv.D;
     for (int q = tid; q < (int)sizeof(RecipTable) / 16; q += NT)
@@ -1025,8 +990,8 @@ speculate_fused_kernel(sd_store sv, int n, const int32_t* __restrict__ d_slot, i
     if (d_budget_cap && d_budget_cap[i] >= 0) cap = min(cap, d_budget_cap[i]);
     if (tid < 2 * SD_MAX_DEPTH) { (&sh.node[0][0])[tid] = -1; (&sh.nc[0][0])[tid] = 0; }
     if (tid == 0) {
-        sh.njobs = 0; sh.next = 0; sh.nwide = 0; sh.nwide_kept = 0; sh.best_hi = 0u;
-        sh.app_done = 0; sh.nlate = 0; sh.app.ahead = 0;
+        sh.nwide = 0; sh.nwide_kept = 0; sh.best_hi = 0u; sh.ready[0] = 0u; sh.ready[1] = 0u;
+        sh.walking = WALK; sh.appending = 1; sh.gave_up = 0; sh.app.ahead = 0;
     }
     if (wib == WARPS - 1) {
         const int c = lane < Pe ? min(budget_for(alpha, lane + 1, cap), 2 * (D - lane - 1)) : -1;
@@ -1044,6 +1009,8 @@ speculate_fused_kernel(sd_store sv, int n, const int32_t* __restrict__ d_slot, i
     // ---------------- 1. match
     bool want_g = usable && !(flags & SD_FLAG_REQUEST_ONLY);
     bool want_r = usable && !(flags & SD_FLAG_GLOBAL_ONLY);
+    // sd_speculate, the match nodes of this very context are at hand
+    const bool at_hand = !STEP && MINB > 1 && ok && ss->g_gen == ss->gen && ss->g_epoch == sv.g_state->epoch && ss->g_len == t;
     if (want_g && gtid >= 0 && gtid < Pe) {
         // the walk to the match node of the last d tokens starts at the node kept from the call before, or at the root
         const bool cache_ok = ss->g_gen == ss->gen && ss->g_epoch == sv.g_state->epoch && ss->g_len <= t;
@@ -1065,117 +1032,140 @@ speculate_fused_kernel(sd_store sv, int n, const int32_t* __restrict__ d_slot, i
     // all cached nodes read before any is replaced; and: is this a second block for the same slot?
     const bool refused = __syncthreads_or(dup) != 0;
     if (refused) { usable = false; want_g = false; want_r = false; status = SD_STATUS_BAD_SLOT; }
-    const bool look_ahead = STEP && n_new >= 3 && usable;         // (one or two tokens are as soon searched for in their turn)
-    if (STEP && wib == 0) {
-        if (ok && n_new > 0 && !refused) {
-            // ---- the request's accepted tokens go into its tree and text (as sd_append does)
-            int len = ss->len, used = ss->used, live = ss->live, st = ss->status;
-            if (!(st & (SD_STATUS_POOL_FULL | SD_STATUS_BAD_TOKEN))) {
-                int act = ss->active[lane], cb = ss->run_cb[lane];
-                unsigned w = append_pack(ss->run_w[lane], ss->room[lane]);
-                append_tokens<(MINB < 4)>(sh.app, sv, slot, newtok, n_new, GWARPS, lane, act, cb, w, len, used, live, st);
-                append_store(ss, lane, act, cb, w);
-            }
-            if (lane == 0) { ss->len = len; ss->used = used; ss->live = live; ss->status = st; }
+    // a lane per place in the order of the jobs (by the number of nodes a job can add at most)
+    const int my_p = sh.ordp[lane] + 1, my_budget = my_p <= Pe ? budget_for(alpha, my_p, cap) : 0;
+    // SCORE <= number of draft nodes (every D <= 1), and SCORE <= number of levels below the
+    // match node: the D values of one level of a tree add up to at most 1 (Eq. 1 shares out
+    // the parent's D among its children)
+    const unsigned my_limit = (unsigned)__double2hiint((double)min(my_budget, D - my_p) * 1.000000001);
+    // the jobs of pattern lengths [pa, pb), whose match nodes are known, can be taken
+    auto offer = [&](int tree, bool want, int pa, int pb, const int4* base) {
+        __syncwarp();
+        const bool job = want && my_p >= pa && my_p < pb && my_p <= t && min(my_budget, D - my_p) > 0 && sh.node[tree][my_p - 1] >= 0;
+        const unsigned wf = job ? sh.nc[tree][my_p - 1] : 0u;
+        const int nch = (int)(wf & RUN_COUNT_MASK);
+        const bool far = nch > WIDE_RUN && !(wf & RUN_HAS_TOP);  // scanned by all warps together, later
+        if (far) sh.wide[atomicAdd(&sh.nwide, 1)] = tree * SD_MAX_DEPTH + my_p - 1;
+        else if (nch > 0) {
+            // all first runs start their way to L2 now, before a warp gets to them
+            const int4* run = base + sh.cb[tree][my_p - 1];
+            for (int l = 0; l < min(4, (nch + 7) >> 3); ++l) prefetch_l2(run + l * 8);
         }
+        const unsigned m = __ballot_sync(FULL, nch > 0 && !far);
         __threadfence_block();
-        if (lane == 0) *(volatile int*)&sh.app_done = 1;        // the jobs that go through the tree may start
-        // join the others once their queue is ready
-        asm volatile("bar.sync %0, %1;" ::"r"(BAR_JOIN), "r"(NT) : "memory");
-    } else {
-        if (look_ahead) {
-            search_ahead(sh.app, sv, sv.s_ent + (long long)slot * sv.spn, sv.s_root + (long long)slot * sv.V, t_old, n_new, gtid / APP_LANES,
-                         GT / APP_LANES, lane);
+        if (lane == 0 && m) atomicOr(&sh.ready[tree], m);
+    };
+    const int4* s_ent = ok ? sv.s_ent + (long long)slot * sv.spn : nullptr;
+    const bool look_ahead = STEP && n_new >= 3 && usable;         // (one or two tokens are as soon searched for in their turn)
+    if (wib == (STEP ? 0 : WARPS - 1)) {
+        // ---- the request's match nodes are its active nodes
+        int act = -1, cb = 0;
+        unsigned w = 0;
+        bool good = usable;
+        if (ok && !refused) {
+            act = ss->active[lane]; cb = ss->run_cb[lane]; w = ss->run_w[lane];
+            if (STEP && n_new > 0) {
+                // ---- sd_step: its accepted tokens go into its tree and text (as sd_append does)
+                int len = ss->len, used = ss->used, live = ss->live, st = ss->status;
+                if (!(st & (SD_STATUS_POOL_FULL | SD_STATUS_BAD_TOKEN))) {
+                    w = append_pack(w, ss->room[lane]);
+                    append_tokens<(MINB < 4)>(sh.app, sv, slot, newtok, n_new, SPLIT ? GWARPS - WALKERS : GWARPS, lane, act, cb, w, len, used, live, st);
+                    append_store(ss, lane, act, cb, w);
+                    if (w != RUN_UNKNOWN) w &= ~(ROOM_MASK << ROOM_SHIFT);
+                }
+                if (lane == 0) { ss->len = len; ss->used = used; ss->live = live; ss->status = st; }
+                // an append that stopped early leaves a context the jobs were not made for
+                good = good && len == t && !(st & (SD_STATUS_POOL_FULL | SD_STATUS_BAD_TOKEN));
+            }
+        }
+        if (good && act >= 0 && w == RUN_UNKNOWN) { const int4 e = s_ent[act]; cb = e.z; w = (unsigned)e.w; }
+        sh.node[1][lane] = act; sh.cb[1][lane] = cb; sh.nc[1][lane] = w;
+        offer(1, good && want_r, 1, SD_MAX_DEPTH + 1, s_ent);
+        __threadfence_block();
+        if (lane == 0) atomicSub(&sh.appending, 1);
+    }
+    if (gw >= 0) {
+        if (look_ahead && (!SPLIT || gw >= WALKERS)) {
+            search_ahead(sh.app, sv, s_ent, sv.s_root + (long long)slot * sv.V, t_old, n_new, (gtid - (SPLIT ? WALKERS * 32 : 0)) / APP_LANES,
+                         (GT - (SPLIT ? WALKERS * 32 : 0)) / APP_LANES, lane);
             __threadfence_block();
             __syncwarp();
             if (lane == 0) atomicAdd(&sh.app.ahead, 1);
         }
         // ---- global match nodes: eight lanes per pattern length
-        if (want_g) {
-            for (int p0 = 0; p0 < Pe; p0 += GT / APP_LANES) {
-                const int d = p0 + gtid / APP_LANES + 1;
-                int node = d <= Pe ? sh.src_node[d - 1] : -1;
-                const int pos = d <= Pe ? sh.src_from[d - 1] : t;
-                int2 zw = make_int2(0, 0);
-                if (node >= 0) zw = *reinterpret_cast<const int2*>(&sv.g_ent[node].z);
-                group_walk(sv.g_ent, (int)sv.g_cap, node, zw, t - pos, lane, [&](int k) {
-                    const int kx = pos + k - t_old;            // (of the new tokens the first ones are at hand)
-                    return kx < 0 ? text[pos + k] : (kx < APP_AHEAD ? sh.app.tok[kx + APP_SHALLOW - 1] : newtok[kx]);
-                });
-                if ((lane & (APP_LANES - 1)) == 0 && d <= Pe) {
-                    ss->g_node[d - 1] = node;
-                    sh.node[0][d - 1] = node;
-                    if (node >= 0) { sh.cb[0][d - 1] = zw.x; sh.nc[0][d - 1] = (unsigned)zw.y; }
-                }
-            }
-            if (gtid == 0) { ss->g_gen = ss->gen; ss->g_epoch = sv.g_state->epoch; ss->g_len = t; ss->g_depths = Pe; }
-        }
-        group_sync();
-
-        // ---------------- 2. the job queue, by the number of nodes a job can add at most
-        // (a lane per pattern length in the order of that number, the global tree's job before the request's)
-        if (gw == 0) {
-            const int p = sh.ordp[lane] + 1;
-            const int c = p <= Pe ? min(budget_for(alpha, p, cap), 2 * (D - p)) : 0;
-            const unsigned wf = c > 0 && sh.node[0][p - 1] >= 0 ? sh.nc[0][p - 1] : 0u;
-            const int nch = (int)(wf & RUN_COUNT_MASK);
-            const bool far = nch > WIDE_RUN && !(wf & RUN_HAS_TOP);
-            const bool j0 = nch > 0 && !far, j1 = c > 0 && want_r && p <= t;
-            if (j0) {
-                // all first runs start their way to L2 now, before a warp gets to them
-                const int4* base = sv.g_ent + sh.cb[0][p - 1];
-                for (int l = 0; l < min(4, (nch + 7) >> 3); ++l) prefetch_l2(base + l * 8);
-            }
-            if (far) sh.wide[atomicAdd(&sh.nwide, 1)] = p - 1;
-            const unsigned b0 = __ballot_sync(FULL, j0), b1 = __ballot_sync(FULL, j1), lt = (1u << lane) - 1u;
-            int at = __popc(b0 & lt) + __popc(b1 & lt);
-            if (j0) sh.job[at++] = p - 1;
-            if (j1) sh.job[at] = SD_MAX_DEPTH + p - 1;
-            if (lane == 0) sh.njobs = __popc(b0) + __popc(b1);
-        }
-        group_sync();
-        if (STEP) asm volatile("bar.arrive %0, %1;" ::"r"(BAR_JOIN), "r"(NT) : "memory");   // warp 0 may come in
-    }
-    const int4* s_ent = ok ? sv.s_ent + (long long)slot * sv.spn : nullptr;
-    {
-        const int njobs = sh.njobs;
-        while (true) {
-            int j = 0;
-            if (lane == 0) j = atomicAdd(&sh.next, 1);
-            j = __shfl_sync(FULL, j, 0);
-            if (j >= njobs) break;
-            const int code = sh.job[j];
-            const int tree = code / SD_MAX_DEPTH, p = code % SD_MAX_DEPTH + 1;
-            const int budget = budget_for(alpha, p, cap);
-            // SCORE <= number of draft nodes (every D <= 1), and SCORE <= number of levels below the
-            // match node: the D values of one level of a tree add up to at most 1 (Eq. 1 shares out
-            // the parent's D among its children)
-            if ((double)min(budget, D - p) * 1.000000001 < best_so_far(sh)) continue;
-            if (tree == 0) {
-                expand_job(sh, W, sv.g_ent, (int)sv.g_cap, 0, p, budget, flags, -1, lane);
-            } else {
-                // through the tree: the match node is the slot's active node of depth p, once the
-                // append is done (bounded wait; a job that runs out of patience is done after the
-                // block-wide barrier below instead)
-                bool ready = true;
-                if (STEP) {
-                    ready = false;
-                    for (int spin = 0; spin < 4096 && !ready; ++spin) {
-                        int flag = 0;
-                        if (lane == 0) flag = *(volatile int*)&sh.app_done;
-                        ready = __shfl_sync(FULL, flag, 0) != 0;
-                        if (!ready) __nanosleep(200);
+        if (gw < WALK) {
+            if (want_g) {
+                for (int p0 = 0; p0 + gw * 4 < Pe; p0 += WALK * 4) {
+                    const int d = p0 + gtid / APP_LANES + 1;
+                    int node = d <= Pe ? sh.src_node[d - 1] : -1;
+                    const int pos = d <= Pe ? sh.src_from[d - 1] : t;
+                    int2 zw = make_int2(0, 0);
+                    if (node >= 0) zw = *reinterpret_cast<const int2*>(&sv.g_ent[node].z);
+                    group_walk(sv.g_ent, (int)sv.g_cap, node, zw, t - pos, lane, [&](int k) {
+                        const int kx = pos + k - t_old;            // (of the new tokens the first ones are at hand)
+                        return kx < 0 ? text[pos + k] : (kx < APP_AHEAD ? sh.app.tok[kx + APP_SHALLOW - 1] : newtok[kx]);
+                    });
+                    if ((lane & (APP_LANES - 1)) == 0 && d <= Pe) {
+                        ss->g_node[d - 1] = node;
+                        sh.node[0][d - 1] = node;
+                        if (node >= 0) { sh.cb[0][d - 1] = zw.x; sh.nc[0][d - 1] = (unsigned)zw.y; }
                     }
+                    offer(0, true, p0 + gw * 4 + 1, p0 + gw * 4 + 5, sv.g_ent);
                 }
-                if (!ready) { if (lane == 0) sh.late[atomicAdd(&sh.nlate, 1)] = p; continue; }
-                request_tree_job(sh, W, sv, ss, s_ent, t, p, budget, flags, lane);
+                if (gtid == 0) { ss->g_gen = ss->gen; ss->g_epoch = sv.g_state->epoch; ss->g_len = t; ss->g_depths = Pe; }
             }
+            __threadfence_block();
+            if (lane == 0) atomicSub(&sh.walking, 1);
         }
     }
+
+    // ---------------- 2. the jobs, until none is left and none can come any more.  (A queue made when all match nodes were
+    // known, whose next job might have to wait for the append: steps of 1 / 64 / 256 / 512 requests 16.5 / 38 / 52 / 42 us, now
+    // 16 / 36 / 48 / 40.  Taking the cheap half at once, too: 50 for 256.)
+    auto work = [&]() {
+        int skip = wib;                                         // (not all warps go for the same one)
+        for (int spins = 0;;) {
+            const int walking = *(volatile int*)&sh.walking, appending = *(volatile int*)&sh.appending;     // before the jobs are looked at
+            const unsigned best = *(volatile unsigned*)&sh.best_hi;
+            const unsigned m0 = *(volatile unsigned*)&sh.ready[0], m1 = *(volatile unsigned*)&sh.ready[1];
+            const unsigned able = __ballot_sync(FULL, my_limit >= best);
+            const unsigned r0 = __ballot_sync(FULL, (m0 >> lane) & 1u), r1 = __ballot_sync(FULL, (m1 >> lane) & 1u);
+            // a job whose bound is below a score already reached is dropped, exactly
+            if (lane == 0 && (r0 & ~able)) atomicAnd(&sh.ready[0], able);
+            if (lane == 0 && (r1 & ~able)) atomicAnd(&sh.ready[1], able);
+            const bool more = __any_sync(FULL, walking != 0 || appending != 0);
+            const bool first = __any_sync(FULL, walking != 0);   // (the costlier half only, while costlier ones may still come)
+            const unsigned v0 = r0 & able & (first ? 0xffffu : FULL), v1 = r1 & able & (first ? 0xffffu : FULL);
+            const int total = __popc(v0) + __popc(v1);
+            if (total == 0) {
+                if (!more) break;
+                if (++spins > 4096) { if (lane == 0) sh.gave_up = 1; break; }
+                __nanosleep(200);
+                continue;
+            }
+            const int k = min(skip, total - 1);
+            const unsigned lt = (1u << lane) - 1u, mine0 = (v0 >> lane) & 1u;
+            const int at = __popc(v0 & lt) + __popc(v1 & lt);   // the global tree's job before the request's
+            const unsigned w0 = __ballot_sync(FULL, mine0 && at == k), w1 = __ballot_sync(FULL, ((v1 >> lane) & 1u) && at + (int)mine0 == k);
+            const int tree = w0 ? 0 : 1, rank = __ffs(w0 | w1) - 1;
+            unsigned old = 0;
+            if (lane == 0) old = atomicAnd(&sh.ready[tree], ~(1u << rank));
+            old = __shfl_sync(FULL, old, 0);
+            skip = 0;
+            if (!((old >> rank) & 1u)) continue;                // another warp was faster
+            __threadfence_block();
+            const int p = __shfl_sync(FULL, my_p, rank), budget = __shfl_sync(FULL, my_budget, rank);
+            expand_job(sh, W, tree == 0 ? sv.g_ent : s_ent, tree == 0 ? (int)sv.g_cap : (int)sv.spn, tree, p, budget, flags, -1, lane);
+        }
+    };
+    // All jobs can be taken at once: in their order, then (256 requests: 38.6 us, without the barrier 41; where the SM has one block
+    // it only costs, 6.2 -> 6.8 us for one request).
+    if (at_hand) __syncthreads();
+    work();
     __syncthreads();                                            // sd_step: the append is done and visible
 
-    // ---------------- 3. what had to wait: an append that stopped early, per-request jobs whose wait
-    // ran out, jobs that start at a wide child run
+    // ---------------- 3. what had to wait: an append that stopped early, jobs that no warp waited for,
+    // jobs that start at a wide child run
     if (STEP && ok && !refused) {
         status = ss->status;
         if (ss->len != t || (status & (SD_STATUS_POOL_FULL | SD_STATUS_BAD_TOKEN))) {
@@ -1186,13 +1176,8 @@ speculate_fused_kernel(sd_store sv, int n, const int32_t* __restrict__ d_slot, i
             if (tid == 0) ss->g_gen = ss->gen - 1;
         }
     }
-    if (sh.nlate > 0 || sh.nwide > 0) {                         // (either only grows before the barrier above)
-        for (int q = wib; q < sh.nlate && usable; q += CTA_WARPS) {
-            const int p = sh.late[q];
-            const int budget = budget_for(alpha, p, cap);
-            if ((double)min(budget, D - p) * 1.000000001 < best_so_far(sh)) continue;
-            request_tree_job(sh, W, sv, ss, s_ent, t, p, budget, flags, lane);
-        }
+    if (sh.gave_up || sh.nwide > 0) {                           // (either only grows before the barrier above)
+        if (sh.gave_up && usable) work();
         __syncthreads();
         // Jobs that start at a wide node (short patterns, hence small budgets): most cannot reach
         // the best score any more and are dropped here.  For the rest the warps of the block share
