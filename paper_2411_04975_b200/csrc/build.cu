@@ -807,7 +807,9 @@ ts_emit_kernel(TreeScan T, TreeOut O) {
             if (opens) R = run + kids;
             if (opens && fits) {
                 const int pos = lane == 0 ? depth1 : place + shift;
-                ent[pos] = make_int4(x[i] - first_tok, es[i] - j, kids > 0 ? run + shift : 0, kids > 0 ? (int)((unsigned)kids | RUN_STATIC) : 0);
+                // (the suffixes that end with a node come first among its own: the one that opens it is one of them, if there are any)
+                const unsigned ends = !REQ && d == n ? RUN_ENDS : 0u;
+                ent[pos] = make_int4(x[i] - first_tok, es[i] - j, kids > 0 ? run + shift : 0, kids > 0 ? (int)((unsigned)kids | RUN_STATIC | ends) : 0);
                 if (lane == 0) root[x[i] - first_tok] = pos;
                 if (!REQ && kids > SD_TOP_MIN) O.wide[atomicAdd(&T.total->listed, 1)] = make_int4(pos, run + shift, kids, 0);
             }
@@ -825,7 +827,7 @@ __global__ void ts_wide_place_kernel(TreeScan T, int4* wide, int4* ent, int firs
     w.w = first + atomicAdd(&T.total->placed, w.z + SD_TOP_BLOCK);
     wide[i] = w;
     ent[w.x].z = w.w + SD_TOP_BLOCK;
-    ent[w.x].w = (int)((unsigned)w.z | RUN_STATIC | RUN_HAS_TOP);
+    ent[w.x].w |= (int)RUN_HAS_TOP;
 }
 
 // One block per long run: the run, and in front of it the sum of its counts and the 64 best children by (count desc, token asc).
@@ -1095,6 +1097,7 @@ extern "C" int sd_build(const sd_build_params* p, const int32_t* d_corpus, const
     memset(s, 0, sizeof(*s));
     s->V = p->vocab; s->D = p->depth_cap; s->R = p->max_requests; s->T = p->max_req_tokens; s->M = p->max_spec_cap;
     if (cudaGetDevice(&s->device) != cudaSuccess) { delete s; return SD_ERR_CUDA; }
+    s->built = N;
     const int D = s->D;
     s->spn = p->slot_pool_nodes > 0 ? p->slot_pool_nodes : 2ll * s->T * D;
     if (s->spn > SD_MAX_ENTRIES) { delete s; return SD_ERR_INVALID_ARG; }

@@ -4,7 +4,7 @@
 // child run:
 //     x = token id          y = count (occurrences of the root-to-node path)
 //     z = index of the first entry of this node's own child run
-//     w = number of children (low 24 bits) | RUN_STATIC (bit 31) | RUN_HAS_TOP (bit 30)
+//     w = number of children (low 24 bits) | RUN_STATIC (bit 31) | RUN_HAS_TOP (bit 30) | RUN_ENDS (bit 29)
 // A child run is a contiguous array of entries sorted by token id, so one
 // 16-byte load per child yields everything Eq. 1 needs (token, count) plus the
 // way down.  A run with n children built online has room for pow2ceil(n)
@@ -30,6 +30,9 @@
 // enter a speculation tree of at most 64 nodes, so expanding such a node reads 1 KB instead
 // of the whole run.  The flag is dropped by the first online update that touches the run.
 #define RUN_HAS_TOP 0x40000000u
+// A node with children laid down by the offline build, in the global tree, with which a sequence ends: its count is more
+// than its children's.  (Means nothing once sequences have been inserted online.)
+#define RUN_ENDS 0x20000000u
 #define SD_TOP_MIN 128            // runs longer than this get a top block
 #define SD_TOP_BLOCK 65           // entries of a top block
 
@@ -71,6 +74,7 @@ struct sd_store {
     // global tree
     int4* g_ent;
     long long g_cap;
+    long long built;          // tokens of the corpus it was built from
     int32_t* g_root;          // [V]
     GlobalState* g_state;
     struct GiScratch* gi;     // of the online insert into the global tree
