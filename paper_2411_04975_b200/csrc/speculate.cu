@@ -353,8 +353,8 @@ struct BlockSharedT {
     unsigned char ordp[SD_MAX_DEPTH];         // pattern lengths - 1 by the number of nodes their jobs can add at most
     int wide[2 * SD_MAX_DEPTH];               // jobs whose match node has a wide child run
     int nwide, nwide_kept;
-    unsigned ready[2];                        // per tree: jobs to be taken, a bit per place in ordp
-    int walking, appending;                   // warps whose match nodes are still to come; the request's are
+    // per tree: jobs to be taken, a bit per place in ordp; warps whose match nodes are still to come; the request's are
+    struct __align__(16) { unsigned ready[2]; int walking, appending; } board;
     int gave_up;                              // a warp waited too long for them
     long long slice_sum[WARPS];
     int slice_fs[WARPS];
@@ -939,6 +939,7 @@ __device__ __noinline__ void expand_job(BlockShared& sh, WarpWork& W, const int4
 //   4. select + emit from shared memory; no global scratch.
 // A job is skipped or dropped, exactly, as soon as an upper bound of its SCORE falls below a
 // score another job of the request has already reached (the running scores are published).
+constexpr int BAR_APPENDED = 1;               // a hardware barrier beside the block-wide one
 constexpr int WALKERS = 8;                    // warps that walk to global match nodes, four pattern lengths each
 
 template <bool STEP, int WARPS, int MINB>
@@ -990,8 +991,8 @@ speculate_fused_kernel(sd_store sv, int n, const int32_t* __restrict__ d_slot, i
     if (d_budget_cap && d_budget_cap[i] >= 0) cap = min(cap, d_budget_cap[i]);
     if (tid < 2 * SD_MAX_DEPTH) { (&sh.node[0][0])[tid] = -1; (&sh.nc[0][0])[tid] = 0; }
     if (tid == 0) {
-        sh.nwide = 0; sh.nwide_kept = 0; sh.best_hi = 0u; sh.ready[0] = 0u; sh.ready[1] = 0u;
-        sh.walking = WALK; sh.appending = 1; sh.gave_up = 0; sh.app.ahead = 0;
+        sh.nwide = 0; sh.nwide_kept = 0; sh.best_hi = 0u; sh.board.ready[0] = 0u; sh.board.ready[1] = 0u;
+        sh.board.walking = WALK; sh.board.appending = 1; sh.gave_up = 0; sh.app.ahead = 0;
     }
     if (wib == WARPS - 1) {
         const int c = lane < Pe ? min(budget_for(alpha, lane + 1, cap), 2 * (D - lane - 1)) : -1;
@@ -1053,7 +1054,7 @@ speculate_fused_kernel(sd_store sv, int n, const int32_t* __restrict__ d_slot, i
         }
         const unsigned m = __ballot_sync(FULL, nch > 0 && !far);
         __threadfence_block();
-        if (lane == 0 && m) atomicOr(&sh.ready[tree], m);
+        if (lane == 0 && m) atomicOr(&sh.board.ready[tree], m);
     };
     const int4* s_ent = ok ? sv.s_ent + (long long)slot * sv.spn : nullptr;
     const bool look_ahead = STEP && n_new >= 3 && usable;         // (one or two tokens are as soon searched for in their turn)
@@ -1082,7 +1083,7 @@ speculate_fused_kernel(sd_store sv, int n, const int32_t* __restrict__ d_slot, i
         sh.node[1][lane] = act; sh.cb[1][lane] = cb; sh.nc[1][lane] = w;
         offer(1, good && want_r, 1, SD_MAX_DEPTH + 1, s_ent);
         __threadfence_block();
-        if (lane == 0) atomicSub(&sh.appending, 1);
+        if (lane == 0) atomicSub(&sh.board.appending, 1);
     }
     if (gw >= 0) {
         if (look_ahead && (!SPLIT || gw >= WALKERS)) {
@@ -1115,7 +1116,7 @@ speculate_fused_kernel(sd_store sv, int n, const int32_t* __restrict__ d_slot, i
                 if (gtid == 0) { ss->g_gen = ss->gen; ss->g_epoch = sv.g_state->epoch; ss->g_len = t; ss->g_depths = Pe; }
             }
             __threadfence_block();
-            if (lane == 0) atomicSub(&sh.walking, 1);
+            if (lane == 0) atomicSub(&sh.board.walking, 1);
         }
     }
 
@@ -1125,22 +1126,28 @@ speculate_fused_kernel(sd_store sv, int n, const int32_t* __restrict__ d_slot, i
     auto work = [&]() {
         int skip = wib;                                         // (not all warps go for the same one)
         for (int spins = 0;;) {
-            const int walking = *(volatile int*)&sh.walking, appending = *(volatile int*)&sh.appending;     // before the jobs are looked at
+            unsigned m0, m1, walking, appending;                // (one access: what is said to have come is there)
+            asm volatile("ld.volatile.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
+                         : "=r"(m0), "=r"(m1), "=r"(walking), "=r"(appending) : "r"((unsigned)__cvta_generic_to_shared(&sh.board)) : "memory");
+            if (__all_sync(FULL, (m0 | m1) == 0u && (walking | appending) != 0u) && ++spins <= 4096) {
+                __nanosleep(400);                               // (200: steps of 512 requests 1 % longer, the append has fewer issue slots)
+                skip = wib;                                     // (what comes next comes all at once)
+                continue;
+            }
             const unsigned best = *(volatile unsigned*)&sh.best_hi;
-            const unsigned m0 = *(volatile unsigned*)&sh.ready[0], m1 = *(volatile unsigned*)&sh.ready[1];
             const unsigned able = __ballot_sync(FULL, my_limit >= best);
             const unsigned r0 = __ballot_sync(FULL, (m0 >> lane) & 1u), r1 = __ballot_sync(FULL, (m1 >> lane) & 1u);
             // a job whose bound is below a score already reached is dropped, exactly
-            if (lane == 0 && (r0 & ~able)) atomicAnd(&sh.ready[0], able);
-            if (lane == 0 && (r1 & ~able)) atomicAnd(&sh.ready[1], able);
-            const bool more = __any_sync(FULL, walking != 0 || appending != 0);
-            const bool first = __any_sync(FULL, walking != 0);   // (the costlier half only, while costlier ones may still come)
+            if (lane == 0 && (r0 & ~able)) atomicAnd(&sh.board.ready[0], able);
+            if (lane == 0 && (r1 & ~able)) atomicAnd(&sh.board.ready[1], able);
+            const bool more = __any_sync(FULL, (walking | appending) != 0u);
+            const bool first = __any_sync(FULL, walking != 0u);   // (the costlier half only, while costlier ones may still come)
             const unsigned v0 = r0 & able & (first ? 0xffffu : FULL), v1 = r1 & able & (first ? 0xffffu : FULL);
             const int total = __popc(v0) + __popc(v1);
             if (total == 0) {
                 if (!more) break;
                 if (++spins > 4096) { if (lane == 0) sh.gave_up = 1; break; }
-                __nanosleep(200);
+                __nanosleep(400);
                 continue;
             }
             const int k = min(skip, total - 1);
@@ -1149,7 +1156,7 @@ speculate_fused_kernel(sd_store sv, int n, const int32_t* __restrict__ d_slot, i
             const unsigned w0 = __ballot_sync(FULL, mine0 && at == k), w1 = __ballot_sync(FULL, ((v1 >> lane) & 1u) && at + (int)mine0 == k);
             const int tree = w0 ? 0 : 1, rank = __ffs(w0 | w1) - 1;
             unsigned old = 0;
-            if (lane == 0) old = atomicAnd(&sh.ready[tree], ~(1u << rank));
+            if (lane == 0) old = atomicAnd(&sh.board.ready[tree], ~(1u << rank));
             old = __shfl_sync(FULL, old, 0);
             skip = 0;
             if (!((old >> rank) & 1u)) continue;                // another warp was faster
@@ -1161,6 +1168,11 @@ speculate_fused_kernel(sd_store sv, int n, const int32_t* __restrict__ d_slot, i
     // All jobs can be taken at once: in their order, then (256 requests: 38.6 us, without the barrier 41; where the SM has one block
     // it only costs, 6.2 -> 6.8 us for one request).
     if (at_hand) __syncthreads();
+    // (nothing to do before the append is done: in a hardware barrier; looking every 200 ns cost such steps 4 %, every 400 ns 2 %)
+    if (STEP && !want_g) {
+        if (wib == 0) asm volatile("bar.arrive %0, %1;" ::"r"(BAR_APPENDED), "r"(NT) : "memory");
+        else asm volatile("bar.sync %0, %1;" ::"r"(BAR_APPENDED), "r"(NT) : "memory");
+    }
     work();
     __syncthreads();                                            // sd_step: the append is done and visible
 
