@@ -5,9 +5,11 @@
 // Hand-written LSD radix sort and scans (no CUB / Thrust).
 // Also: sd_build_requests (the trees of a batch of new requests by the same pipeline).
 #include <algorithm>
+#include <atomic>
 #include <new>
 #include <stdio.h>
 #include <string.h>
+#include <type_traits>
 #include <vector>
 
 #include <cooperative_groups.h>
@@ -399,28 +401,176 @@ int corpus_sort(CorpusSort& A, cudaStream_t st) {
 
 // Suffix order of sequences that are sorted one by one (the trees of different requests share
 // nothing, so no suffix of one request is ever compared with a suffix of another): one block per sequence.
-template <int ITEMS>
-__global__ void __launch_bounds__(BS_THREADS, ITEMS <= 4 ? 2 : 1)
+template <int THREADS, int ITEMS>
+__global__ void __launch_bounds__(THREADS, THREADS == BS_THREADS && ITEMS > 4 ? 1 : 2)
 block_suffix_sort_kernel(const int32_t* tok, const int64_t* seq_off, int V, int tok_bits, int D, uint32_t* sa_out) {
     sd_chain_begin();
     extern __shared__ __align__(16) unsigned char bs_smem[];
-    __shared__ int wsum[BS_THREADS / 32];
+    __shared__ int wsum[THREADS / 32];
     const i64 b = seq_off[blockIdx.x];
     const int n = (int)(seq_off[blockIdx.x + 1] - b), first_tok = (int)blockIdx.x * V;
     if (n <= 0) return;
     const int32_t* const t = tok + b;
-    const unsigned short* const order = block_suffix_order<BS_THREADS, ITEMS>(
+    const unsigned short* const order = block_suffix_order<THREADS, ITEMS>(
         bs_smem, wsum, n, tok_bits, D, [&](int i) { return t[i] - first_tok; }, [](int) { return 0; }, [&](int) { return n; });
-    for (int p = threadIdx.x; p < n; p += BS_THREADS) sa_out[b + p] = (uint32_t)(b + order[p]);
+    for (int p = threadIdx.x; p < n; p += THREADS) sa_out[b + p] = (uint32_t)(b + order[p]);
+}
+
+template <int THREADS, int ITEMS>
+int block_suffix_sort(const int32_t* tok, const int64_t* seq_off, int n_seqs, int V, int tok_bits, int D, uint32_t* sa, cudaStream_t st) {
+    constexpr int smem = block_order_smem<THREADS, ITEMS>();
+    if (smem > 48 * 1024)
+        SD_CUDA_OK(cudaFuncSetAttribute(block_suffix_sort_kernel<THREADS, ITEMS>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    SD_CUDA_OK(sd_launch(block_suffix_sort_kernel<THREADS, ITEMS>, (unsigned)n_seqs, THREADS, smem, st, tok, seq_off, V, tok_bits, D, sa));
+    return SD_OK;
+}
+
+// The same by clusters of blocks: one for a small corpus, or one per prompt.
+constexpr int CC_THREADS = 512, CP_THREADS = 256;                // a corpus of 32,768 tokens 108 us (1,024 threads 113, 256 116), four prompts of 4,096 44 (56, 512 47)
+template <int ITEMS>
+__global__ void __launch_bounds__(CC_THREADS, 1)
+cluster_corpus_sort_kernel(const int32_t* tok, const int64_t* seq_off, int n_seqs, const int* end_pos, int n, int tok_bits, int D, uint32_t* sa_out) {
+    sd_chain_begin();
+    extern __shared__ __align__(16) unsigned char cs_smem[];
+    ClusterOrder<CC_THREADS, ITEMS>& sh = *reinterpret_cast<ClusterOrder<CC_THREADS, ITEMS>*>(cs_smem);
+    const u64* const order = cluster_suffix_order<CC_THREADS, ITEMS>(
+        sh, n, tok_bits, D, [&](int i) { return tok[i]; }, [&](int i) { return i + 1 < end_pos[i]; },
+        [&](int i, int off) {
+            const int e = end_pos[i];
+            if (i >= off && end_pos[i - off] == e) return i - off;
+            int lo = 0, hi = n_seqs;                            // largest q with seq_off[q] <= i
+            while (hi - lo > 1) { const int mid = (lo + hi) >> 1; if (seq_off[mid] <= i) lo = mid; else hi = mid; }
+            const int b = (int)seq_off[lo];
+            return e - min(off, e - b) + (i - b);
+        });
+    const int first = (int)cluster_rank() * CC_THREADS * ITEMS;
+    for (int k = threadIdx.x; k < CC_THREADS * ITEMS && first + k < n; k += CC_THREADS) sa_out[first + k] = (uint32_t)order[k];
+}
+
+// What clusters that have no prompt to sort do meanwhile: a block each, they walk to the global match nodes of the new requests
+// (the last tokens of a prompt are known, the tree is there), which their first draft goes on from as from a draft before.
+struct RequestWalk {
+    sd_store sv;
+    const int32_t* slot;
+    const int32_t* tok;                           // as they came
+    const int* bad;
+};
+
+__device__ __forceinline__ void request_walk(const RequestWalk& R, int q, i64 off, int len) {
+    __shared__ int tail[SD_MAX_DEPTH];                           // the last tokens
+    const int slot = R.slot[q], tid = threadIdx.x, lane = tid & 31, d = tid / APP_LANES + 1;
+    if (*R.bad || slot < 0 || slot >= R.sv.R) return;
+    if (tid < SD_MAX_DEPTH && tid < len) tail[tid] = R.tok[off + len - 1 - tid];
+    __syncthreads();
+    if (d > SD_MAX_DEPTH) return;
+    int node = -1;
+    int2 zw = make_int2(0, 0);
+    if (d <= len && d <= R.sv.D) {
+        node = R.sv.g_root[tail[d - 1]];
+        if (node >= 0) zw = *reinterpret_cast<const int2*>(&R.sv.g_ent[node].z);
+    }
+    group_walk(R.sv.g_ent, (int)R.sv.g_cap, node, zw, d - 1, lane, [&](int k) { return tail[d - 2 - k]; });
+    SlotState* const ss = R.sv.s_state + slot;
+    if ((lane & (APP_LANES - 1)) == 0) ss->g_node[d - 1] = node;
+    // (no good for the request that still has the slot: requests_prepare_kernel makes them the new one's)
+    if (tid == 0) { ss->g_gen = ss->gen - 1; ss->g_epoch = R.sv.g_state->epoch; ss->g_len = len; ss->g_depths = R.sv.D; }
 }
 
 template <int ITEMS>
-int block_suffix_sort(const int32_t* tok, const int64_t* seq_off, int n_seqs, int V, int tok_bits, int D, uint32_t* sa, cudaStream_t st) {
-    constexpr int smem = block_order_smem<BS_THREADS, ITEMS>();
-    if (smem > 48 * 1024)
-        SD_CUDA_OK(cudaFuncSetAttribute(block_suffix_sort_kernel<ITEMS>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    SD_CUDA_OK(sd_launch(block_suffix_sort_kernel<ITEMS>, (unsigned)n_seqs, BS_THREADS, smem, st, tok, seq_off, V, tok_bits, D, sa));
+__global__ void __launch_bounds__(CP_THREADS, 1)
+cluster_prompt_sort_kernel(const int32_t* tok, const int64_t* seq_off, int n_seqs, int V, int tok_bits, int D, uint32_t* sa_out, RequestWalk walk) {
+    sd_chain_begin();
+    extern __shared__ __align__(16) unsigned char cs_smem[];
+    const int c = (int)(blockIdx.x / cluster_blocks());
+    if (c >= n_seqs) {                                           // (whole clusters)
+        const int q = (int)blockIdx.x - n_seqs * (int)cluster_blocks();
+        if (q < n_seqs) request_walk(walk, q, seq_off[q], (int)(seq_off[q + 1] - seq_off[q]));
+        return;
+    }
+    const i64 b = seq_off[c];
+    const int n = (int)(seq_off[c + 1] - b), first_tok = c * V;
+    if (n <= 0) return;
+    const int32_t* const t = tok + b;
+    const u64* const order = cluster_suffix_order<CP_THREADS, ITEMS>(
+        *reinterpret_cast<ClusterOrder<CP_THREADS, ITEMS>*>(cs_smem), n, tok_bits, D, [&](int i) { return t[i] - first_tok; }, [&](int i) { return i + 1 < n; },
+        [&](int i, int off) { return i >= off ? i - off : n - min(off, n) + i; });
+    const int first = (int)cluster_rank() * CP_THREADS * ITEMS;
+    for (int k = threadIdx.x; k < CP_THREADS * ITEMS && first + k < n; k += CP_THREADS) sa_out[b + first + k] = (uint32_t)b + (uint32_t)order[k];
+}
+
+template <class Kernel>
+int allow_clusters(Kernel kernel, size_t smem, unsigned blocks) {
+    SD_CUDA_OK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    if (blocks > 8) SD_CUDA_OK(cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
     return SD_OK;
+}
+
+// f(std::integral_constant<int, ITEMS>) for the least of 1, 2, 4, 8, 16 items that is enough
+constexpr int CP_ITEMS = 16, CC_ITEMS = 8;        // the most
+template <class F>
+int with_items(i64 per_thread, F f) {
+    if (per_thread <= 1) return f(std::integral_constant<int, 1>());
+    if (per_thread <= 2) return f(std::integral_constant<int, 2>());
+    if (per_thread <= 4) return f(std::integral_constant<int, 4>());
+    if (per_thread <= 8) return f(std::integral_constant<int, 8>());
+    return f(std::integral_constant<int, 16>());
+}
+
+unsigned cluster_for(i64 n, unsigned most, int threads) {        // blocks of a cluster for n tokens
+    unsigned blocks = 2;
+    while (blocks < most && (i64)blocks * threads < n) blocks *= 2;
+    return blocks;
+}
+
+int cluster_corpus_sort(const int32_t* tok, const int64_t* seq_off, int n_seqs, const int* end_pos, int n, int tok_bits, int D, unsigned most,
+                        uint32_t* sa, cudaStream_t st) {
+    const unsigned blocks = cluster_for(n, most, CC_THREADS);
+    return with_items((n + (i64)blocks * CC_THREADS - 1) / (blocks * CC_THREADS), [&](auto items) -> int {
+        constexpr int I = decltype(items)::value;
+        const int rc = allow_clusters(cluster_corpus_sort_kernel<I>, sizeof(ClusterOrder<CC_THREADS, I>), blocks);
+        if (rc != SD_OK) return rc;
+        SD_CUDA_OK(sd_launch_clusters(cluster_corpus_sort_kernel<I>, blocks, blocks, CC_THREADS, sizeof(ClusterOrder<CC_THREADS, I>), st, tok, seq_off, n_seqs,
+                                      end_pos, n, tok_bits, D, sa));
+        return SD_OK;
+    });
+}
+
+int cluster_prompt_sort(const int32_t* tok, const int64_t* seq_off, int n_seqs, i64 max_len, int V, int tok_bits, int D, unsigned blocks,
+                        uint32_t* sa, const RequestWalk& walk, cudaStream_t st) {
+    const unsigned grid = ((unsigned)n_seqs + ((unsigned)n_seqs + blocks - 1) / blocks) * blocks;
+    return with_items((max_len + (i64)blocks * CP_THREADS - 1) / (blocks * CP_THREADS), [&](auto items) -> int {
+        constexpr int I = decltype(items)::value;
+        const int rc = allow_clusters(cluster_prompt_sort_kernel<I>, sizeof(ClusterOrder<CP_THREADS, I>), blocks);
+        if (rc != SD_OK) return rc;
+        SD_CUDA_OK(sd_launch_clusters(cluster_prompt_sort_kernel<I>, grid, blocks, CP_THREADS, sizeof(ClusterOrder<CP_THREADS, I>), st, tok, seq_off, n_seqs, V,
+                                      tok_bits, D, sa, walk));
+        return SD_OK;
+    });
+}
+
+// The largest cluster of a device that the sorts can have: 16 blocks where its partitions hold as many, else 8, which is sure.
+unsigned largest_cluster(int dev) {
+    constexpr int MAX_DEVICES = 64;
+    static std::atomic<unsigned> known[MAX_DEVICES];
+    if (dev < 0 || dev >= MAX_DEVICES) return 8;
+    unsigned c = known[dev].load();
+    if (c == 0) {
+        c = 8;
+        constexpr size_t smem = sizeof(ClusterOrder<CC_THREADS, CC_ITEMS>);
+        if (allow_clusters(cluster_corpus_sort_kernel<CC_ITEMS>, smem, CS_MOST) == SD_OK) {
+            cudaLaunchAttribute attr;
+            attr.id = cudaLaunchAttributeClusterDimension;
+            attr.val.clusterDim.x = CS_MOST; attr.val.clusterDim.y = 1; attr.val.clusterDim.z = 1;
+            cudaLaunchConfig_t cfg = {};
+            cfg.gridDim = dim3(CS_MOST); cfg.blockDim = dim3(CC_THREADS); cfg.dynamicSmemBytes = smem;
+            cfg.attrs = &attr; cfg.numAttrs = 1;
+            int n = 0;
+            if (cudaOccupancyMaxActiveClusters(&n, cluster_corpus_sort_kernel<CC_ITEMS>, &cfg) == cudaSuccess && n > 0) c = CS_MOST;
+        }
+        cudaGetLastError();
+        known[dev].store(c);
+    }
+    return c;
 }
 
 // ------------------------------------------------------------------ all depths at once
@@ -704,6 +854,13 @@ struct TreeOut {
     const int* bad;                               // not 0: a token is outside the vocabulary, nothing may change
 };
 
+// A request's active node of depth d is the node of its suffix of d tokens, which comes first among those that begin with it:
+// where that is not all of the tree's depth it is the last node that the suffix opens.
+__device__ __forceinline__ void set_active(SlotState* ss, int d, int node, int run, int kids) {
+    ss->active[d - 1] = node; ss->room[d - 1] = 0;
+    ss->run_cb[d - 1] = kids > 0 ? run : 0; ss->run_w[d - 1] = kids > 0 ? (unsigned)kids | RUN_STATIC : 0u;
+}
+
 // What the lanes need of a suffix in one word, so that one shuffle hands it out: lcp and length (at most 32), S and the
 // depth-1 nodes relative to the first of up to 32 suffixes (at most 31 * 31, 31).  ts_emit_kernel mostly shuffles: 13 -> 8
 // of them per suffix, and the next sub-tile read ahead, 767 -> 569 us for 4.2 M suffixes.  (ts_runs_kernel is bound by
@@ -745,6 +902,7 @@ ts_emit_kernel(TreeScan T, TreeOut O) {
     // the tree this suffix belongs to: entries, root table, what turns S into a place, first token, depth-1 nodes before it
     int4* ent = O.ent;
     int32_t* root = O.root;
+    SlotState* ss = nullptr;
     int shift = 0, first_tok = 0, n1_0 = 0, q = 0, next_req = 0x7fffffff;
     bool fits = true;
     auto enter = [&]() {                                        // request q
@@ -752,6 +910,7 @@ ts_emit_kernel(TreeScan T, TreeOut O) {
         fits = used <= O.sv.spn && O.off[q + 1] - O.off[q] <= O.sv.T && slot >= 0 && slot < O.sv.R;
         ent = O.sv.s_ent + (i64)(fits ? slot : 0) * O.sv.spn;
         root = O.sv.s_root + (i64)(fits ? slot : 0) * O.sv.V;
+        ss = O.sv.s_state + (fits ? slot : 0);
         shift = n1 - O.s_req[q]; n1_0 = O.n1_req[q]; first_tok = q * O.sv.V;
         next_req = (int)O.off[q + 1];
     };
@@ -811,6 +970,7 @@ ts_emit_kernel(TreeScan T, TreeOut O) {
                 const unsigned ends = !REQ && d == n ? RUN_ENDS : 0u;
                 ent[pos] = make_int4(x[i] - first_tok, es[i] - j, kids > 0 ? run + shift : 0, kids > 0 ? (int)((unsigned)kids | RUN_STATIC | ends) : 0);
                 if (lane == 0) root[x[i] - first_tok] = pos;
+                if (REQ && d == n && d < T.D) set_active(ss, d, pos, run + shift, kids);
                 if (!REQ && kids > SD_TOP_MIN) O.wide[atomicAdd(&T.total->listed, 1)] = make_int4(pos, run + shift, kids, 0);
             }
         }
@@ -993,6 +1153,7 @@ struct Pipeline {
     DeviceArena tmp;
     explicit Pipeline(cudaStream_t st) : tmp(st) {}
     TreeScan ts;
+    bool walked = false;                          // the new requests' global match nodes are known
 };
 
 // max_token: largest token value + 1 (sets the number of radix passes; below 2^31).  top_blocks: count the
@@ -1004,10 +1165,10 @@ struct Pipeline {
 // Returns SD_OK, SD_ERR_NOMEM or SD_ERR_CUDA.
 static int pipeline_run(Pipeline& P, const int32_t* d_tok, const int64_t* d_seq_offsets, int n_seqs, i64 N,
                         i64 max_token, int D, bool top_blocks, cudaStream_t st, i64 per_seq_max_len = 0,
-                        int* end_pos = nullptr, RequestBounds bounds = RequestBounds{-1, nullptr, nullptr, nullptr}) {
+                        int* end_pos = nullptr, RequestBounds bounds = RequestBounds{-1, nullptr, nullptr, nullptr},
+                        const RequestWalk* walk = nullptr) {
     const int T256 = 256;
     DeviceArena& tmp = P.tmp;
-    const bool block_sort = per_seq_max_len > 0 && per_seq_max_len <= BS_MAX_LEN;
     TreeScan& ts = P.ts;
     ts.N = (int)N; ts.D = D; ts.tok = d_tok;
     ts.tile_len = TS_SUB;
@@ -1017,7 +1178,18 @@ static int pipeline_run(Pipeline& P, const int32_t* d_tok, const int64_t* d_seq_
     SD_CUDA_OK(cudaGetDevice(&dev));
     SD_CUDA_OK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     const int most_blocks = 2 * sms;
-    if (!block_sort)
+    // Prompts longer than one step of a block are sorted by a cluster of four or eight blocks each while there are at most 128 blocks then
+    // (partitions of 16 multiprocessors and more hold so many at once; with clusters of two, 64 prompts of 8,192 tokens took as long as
+    // by a block each, and their decode 1 % longer), else by a block each.  A corpus of up to 65,536 tokens is sorted by a cluster: whole
+    // builds of 8,000 / 32,768 / 65,536 tokens 329 / 382 / 430 us by the whole device, 222 / 280 / 385 by a cluster, of 100,000 447 and 534.
+    unsigned prompt_cluster = 8;
+    while (prompt_cluster > 1 && (i64)n_seqs * prompt_cluster > 128) prompt_cluster /= 2;
+    if (prompt_cluster > 1) prompt_cluster = cluster_for(per_seq_max_len, prompt_cluster, CP_THREADS);
+    const bool cluster_prompts = prompt_cluster >= 4 && per_seq_max_len > BS_THREADS && per_seq_max_len <= (i64)prompt_cluster * CP_THREADS * CP_ITEMS;
+    const bool block_sort = !cluster_prompts && per_seq_max_len > 0 && per_seq_max_len <= BS_MAX_LEN;
+    const unsigned corpus_cluster = largest_cluster(dev);
+    const bool cluster_corpus = !cluster_prompts && !block_sort && N <= (i64)corpus_cluster * CC_THREADS * CC_ITEMS;
+    if (!block_sort && !cluster_prompts)
         tmp.reserve((long long)N * (16 + 4 + 4 + 4 + 2 + 1) + 4ll * (100 * (i64)ts.tiles + (SG_BINS + 1) * (i64)most_blocks + SG_BINS) + 64 * 256);
     const bool have_ends = end_pos != nullptr;
     uint32_t* sa = nullptr;
@@ -1027,14 +1199,23 @@ static int pipeline_run(Pipeline& P, const int32_t* d_tok, const int64_t* d_seq_
     if (!ok) return SD_ERR_NOMEM;
     if (!have_ends) SD_CUDA_OK(sd_launch(seq_end_kernel, grid_for(N, T256), T256, 0, st, d_seq_offsets, n_seqs, N, end_pos));
     int rc;
-    if (block_sort) {
+    if (cluster_prompts) {
+        const int V = (int)(max_token / n_seqs);                // (as below)
+        rc = cluster_prompt_sort(d_tok, d_seq_offsets, n_seqs, per_seq_max_len, V, bits_for(V), D, prompt_cluster, sa, *walk, st);
+        P.walked = true;
+    } else if (cluster_corpus) {
+        rc = cluster_corpus_sort(d_tok, d_seq_offsets, n_seqs, end_pos, (int)N, bits_for(max_token), D, corpus_cluster, sa, st);
+    } else if (block_sort) {
         const int V = (int)(max_token / n_seqs);                // (a sequence's tokens lie in a range of V of their own)
         const int bits = bits_for(V);
-        if (per_seq_max_len <= BS_THREADS) rc = block_suffix_sort<1>(d_tok, d_seq_offsets, n_seqs, V, bits, D, sa, st);
-        else if (per_seq_max_len <= 2 * BS_THREADS) rc = block_suffix_sort<2>(d_tok, d_seq_offsets, n_seqs, V, bits, D, sa, st);
-        else if (per_seq_max_len <= 4 * BS_THREADS) rc = block_suffix_sort<4>(d_tok, d_seq_offsets, n_seqs, V, bits, D, sa, st);
-        else if (per_seq_max_len <= 8 * BS_THREADS) rc = block_suffix_sort<8>(d_tok, d_seq_offsets, n_seqs, V, bits, D, sa, st);
-        else rc = block_suffix_sort<16>(d_tok, d_seq_offsets, n_seqs, V, bits, D, sa, st);
+        auto sort = [&](auto kernel) { return kernel(d_tok, d_seq_offsets, n_seqs, V, bits, D, sa, st); };
+        if (per_seq_max_len <= BS_SMALL) rc = sort(block_suffix_sort<BS_SMALL, 1>);
+        else if (per_seq_max_len <= 2 * BS_SMALL) rc = sort(block_suffix_sort<BS_SMALL, 2>);
+        else if (per_seq_max_len <= BS_THREADS) rc = sort(block_suffix_sort<BS_SMALL, 4>);
+        else if (per_seq_max_len <= 2 * BS_THREADS) rc = sort(block_suffix_sort<BS_THREADS, 2>);
+        else if (per_seq_max_len <= 4 * BS_THREADS) rc = sort(block_suffix_sort<BS_THREADS, 4>);
+        else if (per_seq_max_len <= 8 * BS_THREADS) rc = sort(block_suffix_sort<BS_THREADS, 8>);
+        else rc = sort(block_suffix_sort<BS_THREADS, 16>);
     } else {
         CorpusSort A;
         A.tok = d_tok; A.seq_off = d_seq_offsets; A.n_seqs = n_seqs; A.end_pos = end_pos; A.N = (int)N; A.D = D; A.sa = sa;
@@ -1205,12 +1386,14 @@ __global__ void map_tokens_kernel(const int32_t* tok, const int64_t* off, int n,
     end_pos[i] = (int)off[q + 1];
 }
 
-// one block per request: forget the slot's old tree and store the new text
+// One block per request: forget the slot's old tree, store the new text, bookkeeping.  The entries and the active nodes are
+// laid down behind this (ts_emit_kernel), but for active nodes that there are none of.
 constexpr int PREP_THREADS = 1024;
 __global__ void __launch_bounds__(PREP_THREADS)
-requests_prepare_kernel(sd_store sv, int n, const int32_t* slot_ids, const int64_t* off, const int32_t* tok, const int* bad) {
+requests_prepare_kernel(sd_store sv, int n, const int32_t* slot_ids, const int64_t* off, const int32_t* tok, const int* s_req,
+                        const int* n1_req, const int* bad, bool walked) {
     sd_chain_begin();
-    const int q = blockIdx.x;
+    const int q = blockIdx.x, tid = threadIdx.x;
     if (q >= n || *bad) return;
     const int slot = slot_ids[q];
     if (slot < 0 || slot >= sv.R) return;
@@ -1218,47 +1401,21 @@ requests_prepare_kernel(sd_store sv, int n, const int32_t* slot_ids, const int64
     int32_t* text = sv.s_text + (i64)slot * sv.T;
     int32_t* root = sv.s_root + (i64)slot * sv.V;
     const int old_len = ss->len;
-    for (int k = threadIdx.x; k < old_len; k += blockDim.x) root[text[k]] = -1;
-    __syncthreads();
     const i64 lo = off[q], hi = off[q + 1];
-    if (hi - lo <= sv.T)
-        for (i64 k = threadIdx.x; k < hi - lo; k += blockDim.x) text[k] = tok[lo + k];
-}
-
-// one block per request: bookkeeping and the active nodes (eight lanes per depth: node of the last d tokens)
-__global__ void __launch_bounds__(256)
-requests_finalize_kernel(sd_store sv, int n, const int32_t* slot_ids, const int64_t* off, const int* s_req, const int* n1_req,
-                         const int* bad) {
-    sd_chain_begin();
-    const int q = blockIdx.x, lane = threadIdx.x & 31, d = threadIdx.x / APP_LANES + 1;
-    if (q >= n || *bad) return;
-    const int slot = slot_ids[q];
-    if (slot < 0 || slot >= sv.R) return;
-    SlotState* ss = sv.s_state + slot;
-    const int n1 = n1_req ? n1_req[q + 1] - n1_req[q] : 0, used = n1_req ? n1 + s_req[q + 1] - s_req[q] : 0;
-    const bool ok = used <= sv.spn && off[q + 1] - off[q] <= sv.T;
-    const int len = ok ? (int)(off[q + 1] - off[q]) : 0;
-    const int4* ent = sv.s_ent + (i64)slot * sv.spn;
-    const int32_t* root = sv.s_root + (i64)slot * sv.V;
-    const int32_t* text = sv.s_text + (i64)slot * sv.T;
-    __shared__ int tail[SD_MAX_DEPTH];                           // the last tokens
-    if (threadIdx.x < SD_MAX_DEPTH && (int)threadIdx.x < len) tail[threadIdx.x] = text[len - 1 - threadIdx.x];
+    const int used = n1_req ? n1_req[q + 1] - n1_req[q] + s_req[q + 1] - s_req[q] : 0;
+    const bool ok = used <= sv.spn && hi - lo <= sv.T;
+    const int len = ok ? (int)(hi - lo) : 0;
+    for (int k = tid; k < old_len; k += PREP_THREADS) root[text[k]] = -1;
     __syncthreads();
-    int node = -1;
-    int2 zw = make_int2(0, 0);
-    if (d <= len && d <= sv.D) {
-        node = root[tail[d - 1]];
-        if (node >= 0) zw = *reinterpret_cast<const int2*>(&ent[node].z);
-    }
-    group_walk(ent, (int)sv.spn, node, zw, d - 1, lane, [&](int k) { return tail[d - 2 - k]; });
-    if ((lane & (APP_LANES - 1)) == 0) {
-        ss->active[d - 1] = node; ss->room[d - 1] = 0;
-        ss->run_cb[d - 1] = node >= 0 ? zw.x : 0; ss->run_w[d - 1] = node >= 0 ? (unsigned)zw.y : 0u;
-    }
-    if (threadIdx.x == 0) {
+    if (hi - lo <= sv.T)
+        for (i64 k = tid; k < hi - lo; k += PREP_THREADS) text[k] = tok[lo + k];
+    // (depth D, too: its node has no children and is asked for by nobody)
+    if (tid < SD_MAX_DEPTH && (tid + 1 > len || tid + 1 >= sv.D)) set_active(ss, tid + 1, -1, 0, 0);
+    if (tid == 0) {
         ss->len = len; ss->used = ok ? used : 0; ss->live = ok ? used : 0;
         ss->status = ok ? 0 : SD_STATUS_POOL_FULL;
         ss->gen += 1;
+        if (walked) ss->g_gen = ss->gen;                         // (request_walk has left the global match nodes)
     }
 }
 
@@ -1320,7 +1477,8 @@ extern "C" int sd_build_requests(sd_store* s, int32_t n, const int32_t* h_slot, 
     if (rc == SD_OK && N > 0) {
         i64 max_len = 0;
         for (int q = 0; q < n; ++q) max_len = std::max<i64>(max_len, h_offsets[q + 1] - h_offsets[q]);
-        rc = pipeline_run(P, mtok, d_off, n, N, (i64)n * s->V, D, false, st, max_len, end_pos, RequestBounds{n, d_off, s_req, n1_req});
+        const RequestWalk walk{*s, d_slot, d_tokens, bad};
+        rc = pipeline_run(P, mtok, d_off, n, N, (i64)n * s->V, D, false, st, max_len, end_pos, RequestBounds{n, d_off, s_req, n1_req}, &walk);
         if (rc == SD_OK && N * D > SD_MAX_ENTRIES) {             // the trees' nodes may not fit 32 bits (up to then nothing has changed)
             TreeTotals total = {};
             if (cudaMemcpyAsync(&total, P.ts.total, sizeof(total), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
@@ -1328,15 +1486,14 @@ extern "C" int sd_build_requests(sd_store* s, int32_t n, const int32_t* h_slot, 
             else if (total.below + total.top > SD_MAX_ENTRIES) rc = SD_ERR_CAPACITY;
         }
     }
-    if (rc == SD_OK && sd_launch(requests_prepare_kernel, (unsigned)n, PREP_THREADS, 0, st, *s, n, d_slot, d_off, d_tokens, bad) != cudaSuccess) rc = SD_ERR_CUDA;
+    if (rc == SD_OK && sd_launch(requests_prepare_kernel, (unsigned)n, PREP_THREADS, 0, st, *s, n, d_slot, d_off, d_tokens, N > 0 ? s_req : nullptr,
+                                 N > 0 ? n1_req : nullptr, bad, P.walked) != cudaSuccess) rc = SD_ERR_CUDA;
     if (rc == SD_OK && N > 0) {
         TreeOut out;
         memset(&out, 0, sizeof(out));
         out.sv = *s; out.n_req = n; out.slot = d_slot; out.off = d_off; out.s_req = s_req; out.n1_req = n1_req; out.bad = bad;
         rc = emit_entries<true>(P.ts, out, st);
     }
-    if (rc == SD_OK && sd_launch(requests_finalize_kernel, (unsigned)n, 256, 0, st, *s, n, d_slot, d_off, N > 0 ? s_req : nullptr,
-                                 N > 0 ? n1_req : nullptr, bad) != cudaSuccess) rc = SD_ERR_CUDA;
     // (the pinned memory is free again, too)
     const cudaError_t checked = record == cudaSuccess ? cudaEventSynchronize(s->ev_check) : cudaStreamSynchronize(st);
     if (rc != SD_OK) return rc;

@@ -139,6 +139,20 @@ inline cudaError_t sd_launch(void (*kernel)(K...), unsigned grid, unsigned block
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<K>(args)...);
 }
 
+// ... in clusters of `blocks` blocks (a divisor of grid).
+template <class... K, class... A>
+inline cudaError_t sd_launch_clusters(void (*kernel)(K...), unsigned grid, unsigned blocks, unsigned block, size_t smem, cudaStream_t st, A... args) {
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = blocks; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid); cfg.blockDim = dim3(block); cfg.dynamicSmemBytes = smem; cfg.stream = st;
+    cfg.attrs = attr; cfg.numAttrs = 2;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<K>(args)...);
+}
+
 #define SD_CUDA_OK(expr)                                   \
     do {                                                   \
         cudaError_t _e = (expr);                           \
