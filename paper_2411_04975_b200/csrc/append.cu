@@ -688,6 +688,7 @@ extern "C" int sd_append(sd_store* s, int32_t n, const int32_t* d_slot, const in
     // beside the appends, on the store's own stream, which starts behind everything the caller's
     // stream holds so far and which the caller's stream waits for before it goes on.
     cudaStream_t st = (cudaStream_t)stream;
+    s->appended = 1;
     SD_CUDA_OK(cudaEventRecord(s->ev_fork, st));
     SD_CUDA_OK(cudaStreamWaitEvent(s->aux, s->ev_fork, 0));
     int tok_bits = 1;

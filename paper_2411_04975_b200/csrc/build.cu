@@ -447,33 +447,49 @@ cluster_corpus_sort_kernel(const int32_t* tok, const int64_t* seq_off, int n_seq
     for (int k = threadIdx.x; k < CC_THREADS * ITEMS && first + k < n; k += CC_THREADS) sa_out[first + k] = (uint32_t)order[k];
 }
 
-// What clusters that have no prompt to sort do meanwhile: a block each, they walk to the global match nodes of the new requests
-// (the last tokens of a prompt are known, the tree is there), which their first draft goes on from as from a draft before.
+// What clusters that have no prompt to sort do meanwhile, on multiprocessors that would be idle: a block per request, they walk to
+// global match nodes, which the request's next draft goes on from as from a draft before.  First the new requests' (the last tokens of a
+// prompt are known, the tree is there), then those of the other slots that an insert into the global tree has made
+// stale: otherwise every one of them walks all the way in its next draft (256 requests as a service: drafts behind an insert
+// 51 us, now 42; the sort beside it 43 -> 47).
+constexpr int MOST_REFRESHED = 1024;
 struct RequestWalk {
     sd_store sv;
+    int n, refreshed;                             // new requests; slots that are looked at (0: there has been no insert)
     const int32_t* slot;
+    const int64_t* off;
     const int32_t* tok;                           // as they came
     const int* bad;
 };
 
-__device__ __forceinline__ void request_walk(const RequestWalk& R, int q, i64 off, int len) {
+__device__ __forceinline__ void request_walk(const RequestWalk& R, int q) {
     __shared__ int tail[SD_MAX_DEPTH];                           // the last tokens
-    const int slot = R.slot[q], tid = threadIdx.x, lane = tid & 31, d = tid / APP_LANES + 1;
+    const int tid = threadIdx.x, lane = tid & 31, d = tid / APP_LANES + 1, D = R.sv.D;
+    const bool fresh = q < R.n;
+    const int slot = fresh ? R.slot[q] : q - R.n;
     if (*R.bad || slot < 0 || slot >= R.sv.R) return;
-    if (tid < SD_MAX_DEPTH && tid < len) tail[tid] = R.tok[off + len - 1 - tid];
+    SlotState* const ss = R.sv.s_state + slot;
+    const int gen = ss->gen, epoch = R.sv.g_state->epoch, len = fresh ? (int)(R.off[q + 1] - R.off[q]) : ss->len;
+    bool leave = false;
+    if (!fresh) {
+        leave = len <= 0 || (ss->status & (SD_STATUS_POOL_FULL | SD_STATUS_BAD_TOKEN)) || (ss->g_gen == gen && ss->g_epoch == epoch && ss->g_len <= len);
+        for (int j = tid; j < R.n; j += CP_THREADS) leave |= R.slot[j] == slot;     // (it is another request's from now on)
+    }
+    if (__syncthreads_or(leave)) return;
+    const int32_t* const end = fresh ? R.tok + R.off[q] + len : R.sv.s_text + (i64)slot * R.sv.T + len;
+    if (tid < SD_MAX_DEPTH && tid < len) tail[tid] = end[-1 - tid];
     __syncthreads();
     if (d > SD_MAX_DEPTH) return;
     int node = -1;
     int2 zw = make_int2(0, 0);
-    if (d <= len && d <= R.sv.D) {
+    if (d <= len && d <= D) {
         node = R.sv.g_root[tail[d - 1]];
         if (node >= 0) zw = *reinterpret_cast<const int2*>(&R.sv.g_ent[node].z);
     }
     group_walk(R.sv.g_ent, (int)R.sv.g_cap, node, zw, d - 1, lane, [&](int k) { return tail[d - 2 - k]; });
-    SlotState* const ss = R.sv.s_state + slot;
     if ((lane & (APP_LANES - 1)) == 0) ss->g_node[d - 1] = node;
-    // (no good for the request that still has the slot: requests_prepare_kernel makes them the new one's)
-    if (tid == 0) { ss->g_gen = ss->gen - 1; ss->g_epoch = R.sv.g_state->epoch; ss->g_len = len; ss->g_depths = R.sv.D; }
+    // (a new request's are no good for the one that still has the slot: requests_prepare_kernel makes them the new one's)
+    if (tid == 0) { ss->g_gen = fresh ? gen - 1 : gen; ss->g_epoch = epoch; ss->g_len = len; ss->g_depths = D; }
 }
 
 template <int ITEMS>
@@ -484,7 +500,7 @@ cluster_prompt_sort_kernel(const int32_t* tok, const int64_t* seq_off, int n_seq
     const int c = (int)(blockIdx.x / cluster_blocks());
     if (c >= n_seqs) {                                           // (whole clusters)
         const int q = (int)blockIdx.x - n_seqs * (int)cluster_blocks();
-        if (q < n_seqs) request_walk(walk, q, seq_off[q], (int)(seq_off[q + 1] - seq_off[q]));
+        if (q < n_seqs + walk.refreshed) request_walk(walk, q);
         return;
     }
     const i64 b = seq_off[c];
@@ -537,7 +553,8 @@ int cluster_corpus_sort(const int32_t* tok, const int64_t* seq_off, int n_seqs, 
 
 int cluster_prompt_sort(const int32_t* tok, const int64_t* seq_off, int n_seqs, i64 max_len, int V, int tok_bits, int D, unsigned blocks,
                         uint32_t* sa, const RequestWalk& walk, cudaStream_t st) {
-    const unsigned grid = ((unsigned)n_seqs + ((unsigned)n_seqs + blocks - 1) / blocks) * blocks;
+    const unsigned walks = (unsigned)n_seqs + (unsigned)walk.refreshed;
+    const unsigned grid = ((unsigned)n_seqs + (walks + blocks - 1) / blocks) * blocks;
     return with_items((max_len + (i64)blocks * CP_THREADS - 1) / (blocks * CP_THREADS), [&](auto items) -> int {
         constexpr int I = decltype(items)::value;
         const int rc = allow_clusters(cluster_prompt_sort_kernel<I>, sizeof(ClusterOrder<CP_THREADS, I>), blocks);
@@ -1477,8 +1494,9 @@ extern "C" int sd_build_requests(sd_store* s, int32_t n, const int32_t* h_slot, 
     if (rc == SD_OK && N > 0) {
         i64 max_len = 0;
         for (int q = 0; q < n; ++q) max_len = std::max<i64>(max_len, h_offsets[q + 1] - h_offsets[q]);
-        const RequestWalk walk{*s, d_slot, d_tokens, bad};
+        const RequestWalk walk{*s, n, s->appended ? std::min(s->R, MOST_REFRESHED) : 0, d_slot, d_off, d_tokens, bad};
         rc = pipeline_run(P, mtok, d_off, n, N, (i64)n * s->V, D, false, st, max_len, end_pos, RequestBounds{n, d_off, s_req, n1_req}, &walk);
+        if (P.walked) s->appended = 0;
         if (rc == SD_OK && N * D > SD_MAX_ENTRIES) {             // the trees' nodes may not fit 32 bits (up to then nothing has changed)
             TreeTotals total = {};
             if (cudaMemcpyAsync(&total, P.ts.total, sizeof(total), cudaMemcpyDeviceToHost, st) != cudaSuccess ||

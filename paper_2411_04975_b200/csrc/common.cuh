@@ -91,6 +91,7 @@ struct sd_store {
     int32_t* j_tok;           // [R*2*D][M]
     int32_t* j_par;           // [R*2*D][M]
     long long device_bytes;
+    int32_t appended;         // HOST: sd_append has been called since stale match nodes were last looked for
     struct sd_workspace* ws;  // HOST: temporaries of sd_build_requests, kept between calls
     // HOST: sd_append runs the insert into the global tree beside the appends to the request trees
     // (they share nothing), on this stream, forked from and joined to the caller's stream

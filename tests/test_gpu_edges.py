@@ -23,7 +23,8 @@ def _text(rng, n, vocab, period=60):
 
 
 @pytest.mark.parametrize("longest,D,vocab", [(1, 1, 2), (33, 32, 3), (1024, 17, 130), (1025, 32, 50), (2049, 2, 7), (4096, 24, 128256),
-                                             (4097, 32, 300), (8193, 31, 65), (16384, 32, 40), (16385, 32, 40)])
+                                             (4097, 32, 300), (8193, 31, 65), (16384, 32, 40), (16385, 32, 40),
+                                             (32768, 32, 40), (32769, 9, 30)])
 def test_prompts_at_the_edges_of_the_block_sort(U, longest, D, vocab):
     rng = np.random.default_rng(longest)
     lens = sorted({1, 2, 15, 16, 17, max(1, longest - 1), longest} & set(range(1, longest + 1)))
@@ -42,7 +43,8 @@ def test_prompts_at_the_edges_of_the_block_sort(U, longest, D, vocab):
     pr.close()
 
 
-@pytest.mark.parametrize("n,D,vocab", [(1, 32, 5), (1023, 32, 9), (1025, 17, 4000), (9000, 24, 60), (303104, 3, 12), (303137, 6, 90)])
+@pytest.mark.parametrize("n,D,vocab", [(1, 32, 5), (1023, 32, 9), (1025, 17, 4000), (9000, 24, 60), (8193, 32, 500), (65536, 32, 700),
+                                       (65537, 31, 700), (303104, 3, 12), (303137, 6, 90)])
 def test_corpora_at_the_edges_of_the_sort(U, n, D, vocab):
     rng = np.random.default_rng(n)
     text = _text(rng, n, vocab, period=200)
@@ -214,4 +216,39 @@ def test_quotients_on_both_sides_of_the_table_of_reciprocals(U, total):
     pr = U.Pair(seqs, vocab=100, D=8, n_slots=1, max_req_tokens=16)
     pr.append([0], [np.array([7], np.int32)])
     pr.check_speculate([0], 1, 40.0, 64)
+    pr.close()
+
+
+@pytest.mark.parametrize("n_slots,new", [(2, 1), (12, 2), (40, 9)])
+def test_match_nodes_found_while_prompts_are_sorted(U, n_slots, new):
+    """New prompts of more than a block's step: their match nodes, and those an insert has made stale, come with the sort."""
+    rng = np.random.default_rng(n_slots)
+    base = [_text(rng, 3000, 60), _text(rng, 500, 60)]
+    pr = U.Pair(base, vocab=60, D=32, n_slots=n_slots, max_req_tokens=1700)
+    every = list(range(n_slots))
+
+    def build(slots, bad=False):
+        prompts = [_text(rng, 1100 + 37 * k, 60, 90) for k in range(len(slots))]
+        off, flat = U.ragged(prompts)
+        if bad:
+            flat[-1] = 60
+            with pytest.raises(Exception):
+                pr.g.build_requests(np.array(slots), off, U.dev_i32(flat))
+            return
+        pr.g.build_requests(np.array(slots), off, U.dev_i32(flat))
+        for k in slots:
+            pr.o.slot_reset(k)
+        pr.o.slot_append_batch(slots, prompts)
+
+    for k in range(0, n_slots, 9):
+        build(every[k:k + 9])
+    for turn in range(3):
+        pr.check_speculate(every, 20, 2.0, 40)
+        pr.append([-1, 0], [_text(rng, 700, 60, 30), base[1][:5]])               # (the drafts' match nodes are stale now)
+        if turn == 1:
+            build(every[:new], bad=True)                                         # a refused call leaves them right, too
+        else:
+            build(every[-new:])
+        pr.append(every, [base[0][k:k + 1 + k % 4] for k in every])
+    pr.check_speculate(every, 20, 2.0, 40)
     pr.close()
