@@ -644,7 +644,8 @@ __device__ __forceinline__ int ts_scan(int v, int lane) {       // inclusive
     return v;
 }
 
-// (1)
+// (1) LONG: tiles of many suffixes.
+template <bool LONG>
 __global__ void __launch_bounds__(TS_WARPS * 32)
 ts_tiles_kernel(TreeScan T) {
     sd_chain_begin();
@@ -658,7 +659,7 @@ ts_tiles_kernel(TreeScan T) {
         if (lane < pl) px = T.tok[q + lane];
     }
     bool seen = false;
-    int cnt = 0, first = T.N, below = 0, top = 0;
+    int cnt = 0, first = T.N, below = 0, top = 0, least = 32;
     for (int jb = t0; jb < t1; jb += 32) {
         const int m = min(32, t1 - jb);
         int q = 0, ln = 0, own = 0;
@@ -677,9 +678,12 @@ ts_tiles_kernel(TreeScan T) {
                 const unsigned ne = __ballot_sync(TS_FULL, x[u] != px || lane >= L[u] || lane >= pl);
                 const int l = ne ? __ffs(ne) - 1 : 32;
                 if (lane == i0 + u) own = l;
-                if (!seen) {
-                    cnt += l == d && L[u] > l ? 1 : 0;
-                    if (l < d) { seen = true; first = jb + i0 + u; }
+                if (!LONG || l <= least) {                               // (else it does nothing to a depth without a reset)
+                    least = l;
+                    if (!seen) {
+                        cnt += l == d && L[u] > l ? 1 : 0;
+                        if (l < d) { seen = true; first = jb + i0 + u; }
+                    }
                 }
                 px = x[u]; pl = L[u];
             }
@@ -826,6 +830,7 @@ ts_runs_kernel(TreeScan T) {
     const int t0 = tile * T.tile_len, t1 = min(T.N, t0 + T.tile_len);
     int g = ts_g_in(T, tile, lane);
     int s_end = T.s[tile + 1], R = -1, n_wide = 0;
+    unsigned open = TS_FULL;                                    // lanes without R
     i64 room = 0;
     for (int jb = t0 + ((t1 - t0 - 1) & ~31); jb >= t0; jb -= 32) {
         const int m = min(32, t1 - jb);
@@ -835,16 +840,23 @@ ts_runs_kernel(TreeScan T) {
         const int all = __shfl_sync(TS_FULL, inc, 31);
         const int s_own = s_end - all + inc - c;
         s_end -= all;
+#pragma unroll 4
         for (int i = m - 1; i >= 0; --i) {
             const int l = __shfl_sync(TS_FULL, l_own, i), n = __shfl_sync(TS_FULL, n_own, i);
-            const bool opens = d > l && d <= n;
-            if (TOP || __any_sync(TS_FULL, opens && R < 0)) {
+            const int gl = __shfl_sync(TS_FULL, g, min(l, 31));
+            // (the depths that it opens: lanes l .. n - 1)
+            if ((((2u << (n - 1)) - 1u) & ~(l < 32 ? (1u << l) - 1u : TS_FULL)) & open) {
                 const int kids = ts_f_of(g, lane) + (d < n ? 1 : 0);
                 const int s = __shfl_sync(TS_FULL, s_own, i);
-                if (opens && R < 0) R = s + d - max(l, 1) + g + kids;
-                if (TOP && opens && kids > SD_TOP_MIN) { ++n_wide; room += kids + SD_TOP_BLOCK; }
+                if (d > l && d <= n && R < 0) R = s + d - max(l, 1) + g + kids;
+                open = __ballot_sync(TS_FULL, R < 0);
             }
-            g = ts_g_step(g, l, n, d);
+            // the nodes that it opens have as many children together, but for their own first ones, as G grows from there on
+            if (TOP && __shfl_sync(TS_FULL, g, 31) - gl >= SD_TOP_MIN) {
+                const int kids = ts_f_of(g, lane) + (d < n ? 1 : 0);
+                if (d > l && d <= n && kids > SD_TOP_MIN) { ++n_wide; room += kids + SD_TOP_BLOCK; }
+            }
+            g = d > l ? (l == 0 ? 0 : gl + (n > l ? 1 : 0)) : g;                    // (ts_g_step)
         }
     }
     T.r[(i64)lane * T.tiles + tile] = R;
@@ -906,6 +918,7 @@ ts_emit_kernel(TreeScan T, TreeOut O) {
             if (c == 0) break;
             const int jb = t0 + c * TS_SUB, m = min(TS_SUB, t1 - jb);
             const int own = lane < m ? ts_pack(T.lcp[jb + lane], T.len[jb + lane], 0, 0) : 0;
+#pragma unroll 8
             for (int i = m - 1; i >= 0; --i) {
                 const int w = __shfl_sync(TS_FULL, own, i), l = ts_l(w);
                 g = ts_g_step(g, l, ts_n(w), d);
@@ -1255,7 +1268,7 @@ static int pipeline_run(Pipeline& P, const int32_t* d_tok, const int64_t* d_seq_
     ts.end_pos = end_pos;
     const unsigned grid = (unsigned)((ts.tiles + TS_WARPS - 1) / TS_WARPS);
     if (top_blocks && cudaMemsetAsync(ts.total, 0, sizeof(TreeTotals), st) != cudaSuccess) return SD_ERR_CUDA;
-    SD_CUDA_OK(sd_launch(ts_tiles_kernel, grid, TS_WARPS * 32, 0, st, ts));
+    SD_CUDA_OK(sd_launch(ts.tile_len >= 256 ? ts_tiles_kernel<true> : ts_tiles_kernel<false>, grid, TS_WARPS * 32, 0, st, ts));
     SD_CUDA_OK(sd_launch(ts_carry_kernel, 33, TS_CARRY, 0, st, ts));
     if (top_blocks) SD_CUDA_OK(sd_launch(ts_runs_kernel<true>, grid, TS_WARPS * 32, 0, st, ts));
     else SD_CUDA_OK(sd_launch(ts_runs_kernel<false>, grid, TS_WARPS * 32, 0, st, ts));
