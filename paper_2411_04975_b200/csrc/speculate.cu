@@ -288,7 +288,7 @@ constexpr int CTA_WARPS_STEP = 14;             // of sd_step: 58.6 us per step (
 // registers 107, 20 106, 12 108), of one request 7.3 (8.0, 7.6, 7.1); steps of 64 requests 47.4 (12 warps 49.2, 20 48.7)
 constexpr int CTA_WARPS_WIDE = 16;
 constexpr int CTA_WARPS_NARROW = 8;            // batches of more than two requests per SM: four blocks per SM
-constexpr int CTA_WARPS_NARROW_STEP = 5;       // (sd_step: 96 registers)
+constexpr int CTA_WARPS_NARROW_STEP = 4;       // (sd_step: 128 registers; with 5 warps of 96 a decode of 512 requests takes 1,925 us, 1,870 now)
 
 // Candidates of one job: not ordered, two per lane in registers.  The next node is the one with the largest D, which a
 // reduction over the lanes tells; its children go to lanes with a free place, a child each, so nothing is sorted, moved or
