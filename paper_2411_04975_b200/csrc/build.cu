@@ -453,13 +453,20 @@ cluster_corpus_sort_kernel(const int32_t* tok, const int64_t* seq_off, int n_seq
 // stale: otherwise every one of them walks all the way in its next draft (256 requests as a service: drafts behind an insert
 // 51 us, now 42; the sort beside it 43 -> 47).
 constexpr int MOST_REFRESHED = 1024;
+// Whether this call of sd_build_requests has been refused for a token outside the vocabulary (in GlobalState, which keeps the last such
+// call: nothing has to be cleared).
+struct BadCall {
+    int32_t* last;
+    int32_t call;
+    __device__ bool operator()() const { return *last == call; }
+};
 struct RequestWalk {
     sd_store sv;
     int n, refreshed;                             // new requests; slots that are looked at (0: there has been no insert)
     const int32_t* slot;
     const int64_t* off;
     const int32_t* tok;                           // as they came
-    const int* bad;
+    BadCall bad;
 };
 
 __device__ __forceinline__ void request_walk(const RequestWalk& R, int q) {
@@ -467,7 +474,7 @@ __device__ __forceinline__ void request_walk(const RequestWalk& R, int q) {
     const int tid = threadIdx.x, lane = tid & 31, d = tid / APP_LANES + 1, D = R.sv.D;
     const bool fresh = q < R.n;
     const int slot = fresh ? R.slot[q] : q - R.n;
-    if (*R.bad || slot < 0 || slot >= R.sv.R) return;
+    if (R.bad() || slot < 0 || slot >= R.sv.R) return;
     SlotState* const ss = R.sv.s_state + slot;
     const int gen = ss->gen, epoch = R.sv.g_state->epoch, len = fresh ? (int)(R.off[q + 1] - R.off[q]) : ss->len;
     bool leave = false;
@@ -880,7 +887,7 @@ struct TreeOut {
     const int32_t* slot;
     const int64_t* off;                           // [n_req + 1]
     const int *s_req, *n1_req;                    // [n_req + 1] S and depth-1 nodes before the request's first suffix
-    const int* bad;                               // not 0: a token is outside the vocabulary, nothing may change
+    BadCall bad;                                  // a token is outside the vocabulary, nothing may change
 };
 
 // A request's active node of depth d is the node of its suffix of d tokens, which comes first among those that begin with it:
@@ -907,7 +914,7 @@ ts_emit_kernel(TreeScan T, TreeOut O) {
     sd_chain_begin();
     extern __shared__ int2 ts_state[];                          // [TS_WARPS][tile_len / TS_SUB][32]: G and end behind each sub-tile
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5, tile = blockIdx.x * TS_WARPS + wib, d = lane + 1;
-    if (tile >= T.tiles || (REQ && *O.bad)) return;
+    if (tile >= T.tiles || (REQ && O.bad())) return;
     const int t0 = tile * T.tile_len, t1 = min(T.N, t0 + T.tile_len);
     const int subs = (t1 - t0 + TS_SUB - 1) / TS_SUB;
     int2* const st = ts_state + (i64)wib * (T.tile_len / TS_SUB) * 32;
@@ -1100,7 +1107,7 @@ ts_wide_fill_kernel(const int4* wide, int4* ent) {
 }
 
 __global__ void init_global_state_kernel(GlobalState* g, int used, int live, long long tokens) {
-    g->used = used; g->live = live; g->status = 0; g->epoch = 1; g->tokens = tokens;
+    g->used = used; g->live = live; g->status = 0; g->epoch = 1; g->tokens = tokens; g->bad_call = 0;
 }
 
 struct DeviceArena {          // temporaries of one build: freed together, or kept in a workspace
@@ -1402,18 +1409,31 @@ __device__ __forceinline__ int seq_rank_of(const int64_t* off, int n, i64 pos) {
     return lo;
 }
 
+// Offsets and slots of a few requests, as arguments of the kernel (a copy of them took 4 us of a refill's 100).
+struct RequestArgs {
+    static constexpr int MOST = 64;
+    int64_t off[MOST + 1];
+    int32_t slot[MOST];
+};
+
 // The tokens in ranges of their own, request by request, and where their request ends.  A token outside the vocabulary
-// sets both flags (the host's one lies in its memory).
-__global__ void map_tokens_kernel(const int32_t* tok, const int64_t* off, int n, i64 N, int V, int32_t* out, int* end_pos, int* bad,
-                                  int* host_bad) {
+// sets both flags (the host's one lies in its memory).  ARGS: also lays down the call's offsets and slots for the kernels behind it.
+template <bool ARGS>
+__global__ void map_tokens_kernel(const int32_t* tok, RequestArgs A, int64_t* off, int32_t* slot, int n, i64 N, int V, int32_t* out, int* end_pos,
+                                  BadCall bad, int* host_bad) {
     sd_chain_begin();
     const i64 i = (i64)blockIdx.x * blockDim.x + threadIdx.x;
+    const int64_t* const o = ARGS ? A.off : off;
+    if (ARGS && i <= n) {
+        off[i] = A.off[i];
+        if (i < n) slot[i] = A.slot[i];
+    }
     if (i >= N) return;
     int t = tok[i];
-    if (t < 0 || t >= V) { *bad = 1; *host_bad = 1; t = 0; }
-    const int q = seq_rank_of(off, n, i);
+    if (t < 0 || t >= V) { *bad.last = bad.call; *host_bad = 1; t = 0; }
+    const int q = seq_rank_of(o, n, i);
     out[i] = q * V + t;
-    end_pos[i] = (int)off[q + 1];
+    end_pos[i] = (int)o[q + 1];
 }
 
 // One block per request: forget the slot's old tree, store the new text, bookkeeping.  The entries and the active nodes are
@@ -1421,10 +1441,10 @@ __global__ void map_tokens_kernel(const int32_t* tok, const int64_t* off, int n,
 constexpr int PREP_THREADS = 1024;
 __global__ void __launch_bounds__(PREP_THREADS)
 requests_prepare_kernel(sd_store sv, int n, const int32_t* slot_ids, const int64_t* off, const int32_t* tok, const int* s_req,
-                        const int* n1_req, const int* bad, bool walked) {
+                        const int* n1_req, BadCall bad, bool walked) {
     sd_chain_begin();
     const int q = blockIdx.x, tid = threadIdx.x;
-    if (q >= n || *bad) return;
+    if (q >= n || bad()) return;
     const int slot = slot_ids[q];
     if (slot < 0 || slot >= sv.R) return;
     SlotState* ss = sv.s_state + slot;
@@ -1480,10 +1500,10 @@ extern "C" int sd_build_requests(sd_store* s, int32_t n, const int32_t* h_slot, 
         memset(s->ws, 0, sizeof(*s->ws));
     }
     P.tmp.keep = s->ws;                                          // temporaries are kept for the next call
-    // Arguments go over in one copy from pinned memory, which ends with a zero: the flag that a bad token sets.  Everything is
+    // Arguments go over with the first kernel, those of many requests in one copy from pinned memory.  Everything is
     // queued behind the check of the tokens and changes nothing if it fails; the host waits for the check alone, so
     // the GPU does not run dry meanwhile (it did, for some 50 us of a 185 us refill).
-    const size_t arg_bytes = 8 * ((size_t)n + 1) + 4 * (size_t)n + 4;
+    const size_t arg_bytes = 8 * ((size_t)n + 1) + 4 * (size_t)n;
     unsigned char* d_args = nullptr;
     int32_t* mtok = nullptr;
     int *end_pos = nullptr, *s_req = nullptr, *n1_req = nullptr;
@@ -1492,16 +1512,26 @@ extern "C" int sd_build_requests(sd_store* s, int32_t n, const int32_t* h_slot, 
     if (!ok) return SD_ERR_NOMEM;
     int64_t* const d_off = reinterpret_cast<int64_t*>(d_args);
     int32_t* const d_slot = reinterpret_cast<int32_t*>(d_off + n + 1);
-    int* const bad = d_slot + n;
-    unsigned char* const h_args = (unsigned char*)s->stage + 16;
+    s->request_calls = s->request_calls == 0x7fffffff ? 1 : s->request_calls + 1;
+    const BadCall bad{&s->g_state->bad_call, s->request_calls};
     volatile int* const h_bad = (volatile int*)s->stage;
     *h_bad = 0;
-    memcpy(h_args, h_offsets, 8 * ((size_t)n + 1));
-    memcpy(h_args + 8 * ((size_t)n + 1), h_slot, 4 * (size_t)n);
-    memset(h_args + arg_bytes - 4, 0, 4);
     // (from here on the pinned memory is in use: whatever fails, the call waits for it before it returns)
-    cudaError_t ce = cudaMemcpyAsync(d_args, h_args, arg_bytes, cudaMemcpyHostToDevice, st);
-    if (ce == cudaSuccess && N > 0) ce = sd_launch(map_tokens_kernel, grid_for(N, T256), T256, 0, st, d_tokens, d_off, n, N, s->V, mtok, end_pos, bad, (int*)s->stage);
+    cudaError_t ce = cudaSuccess;
+    const unsigned map_grid = grid_for(std::max<i64>(N, n + 1), T256);
+    RequestArgs args;
+    if (n <= RequestArgs::MOST && N > 0) {
+        memcpy(args.off, h_offsets, 8 * ((size_t)n + 1));
+        memcpy(args.slot, h_slot, 4 * (size_t)n);
+        ce = sd_launch(map_tokens_kernel<true>, map_grid, T256, 0, st, d_tokens, args, d_off, d_slot, n, N, s->V, mtok, end_pos, bad, (int*)s->stage);
+    } else {
+        unsigned char* const h_args = (unsigned char*)s->stage + 16;
+        memcpy(h_args, h_offsets, 8 * ((size_t)n + 1));
+        memcpy(h_args + 8 * ((size_t)n + 1), h_slot, 4 * (size_t)n);
+        ce = cudaMemcpyAsync(d_args, h_args, arg_bytes, cudaMemcpyHostToDevice, st);
+        if (ce == cudaSuccess && N > 0)
+            ce = sd_launch(map_tokens_kernel<false>, map_grid, T256, 0, st, d_tokens, args, d_off, d_slot, n, N, s->V, mtok, end_pos, bad, (int*)s->stage);
+    }
     const cudaError_t record = cudaEventRecord(s->ev_check, st);
     int rc = ce == cudaSuccess && record == cudaSuccess ? SD_OK : SD_ERR_CUDA;
     if (rc == SD_OK && N > 0) {

@@ -42,6 +42,7 @@ struct GlobalState {          // device-resident bookkeeping of the global tree
     int32_t status;           // SD_STATUS_GLOBAL_FULL or 0
     int32_t epoch;            // grows whenever an online insert changed the tree
     long long tokens;         // tokens inserted
+    int32_t bad_call;         // the last sd_build_requests call with a token outside the vocabulary
 };
 
 struct SlotState {            // device-resident bookkeeping of one request slot
@@ -91,6 +92,7 @@ struct sd_store {
     int32_t* j_tok;           // [R*2*D][M]
     int32_t* j_par;           // [R*2*D][M]
     long long device_bytes;
+    int32_t request_calls;    // HOST: of sd_build_requests
     int32_t appended;         // HOST: sd_append has been called since stale match nodes were last looked for
     struct sd_workspace* ws;  // HOST: temporaries of sd_build_requests, kept between calls
     // HOST: sd_append runs the insert into the global tree beside the appends to the request trees
