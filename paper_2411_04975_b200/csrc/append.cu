@@ -1,5 +1,7 @@
 // sd_append: the batched append kernel for the per-request trees (see append_core.cuh for how one
 // token is appended) and the insert of whole sequences into the global tree.
+#include <atomic>
+
 #include <cooperative_groups.h>
 
 #include "append_core.cuh"
@@ -14,7 +16,7 @@ namespace {
 // Global online insert (a finished request's output goes into the global tree).
 //
 // Inserting a sequence adds one occurrence to every string of at most D tokens that starts at one
-// of its positions: one root-to-depth-D PATH per start position.  Up to GI_REAL positions are taken at once, in one
+// of its positions: one root-to-depth-D PATH per start position.  Up to 1,920 positions are taken at once, in one
 // cooperative launch:
 //   1. every path goes down the tree as far as it exists, eight lanes each, and raises the counts on its way (no path
 //      waits for another: nothing moves yet).  Meanwhile one block sorts the positions' suffixes;
@@ -26,13 +28,15 @@ namespace {
 //   3. events are grouped by parent, and every parent's run is merged once with all its new children (in place, or
 //      into a roomier run), while the rest of the new nodes is written;
 //   4. every parent's entry gets its new run, in the place it has now if its own run was merged, too.
-// Six grid barriers and no rounds: the time is that of the walk (dependent loads) or of the sort, whichever is
+// Six barriers and no rounds: the time is that of the walk (dependent loads) or of the sort, whichever is
 // longer, and of the sweeps over the tiles.  (Level by level with an election per parent and round, by a cluster of 8
 // blocks: 150 us for 352 paths, 58 for 91; now 56 and 42, of which the walk 16 and 12, grouping 8 and 6.)
 // The nodes that a batch adds need the pool to hold them all: a batch that does not fit raises counts only.
-constexpr int GI_BLOCKS = 24;
+// A cluster of 16 blocks, which meet at the hardware's barrier, where the device has room for one; else 24 blocks that meet at a grid
+// barrier (1.5 us each).  Services of 16 / 32 requests 2,651 / 1,975 us with the grid, 2,482 / 1,847 with the cluster; of 256, whose
+// batches its 960 walks at a time often take two rounds for, 11,725 either way.
+constexpr int GI_CLUSTER = 16, GI_GRID = 24;
 constexpr int GI_THREADS = 512;               // (1,024 leave 64 registers: the sweeps spill)
-constexpr int GI_REAL = GI_MAX - SD_MAX_DEPTH;                   // start positions per pass
 constexpr int GI_ITEMS = 256;
 constexpr int GI_CELLS = 2 * GI_MAX;
 constexpr int GI_BIG = 256;                   // runs longer than this are merged by a whole block
@@ -55,16 +59,21 @@ struct GiTable {                              // block 0, while it groups
     int tok[GI_MAX], ev[GI_MAX];
     int n_big;
 };
-constexpr int GI_WARP_TILES = (GI_TILES + GI_BLOCKS - 2) / (GI_BLOCKS - 1);                 // tiles per block, a warp each
+__host__ __device__ constexpr int gi_real(int blocks) {            // start positions per pass: a warp per tile
+    return (blocks - 1) * (GI_THREADS / 32) * GI_TILE < GI_MAX - SD_MAX_DEPTH ? (blocks - 1) * (GI_THREADS / 32) * GI_TILE : GI_MAX - SD_MAX_DEPTH;
+}
+__host__ __device__ constexpr int gi_warp_tiles(int blocks) { return (gi_real(blocks) / GI_TILE + blocks - 2) / (blocks - 1); }  // tiles per block
+template <int BLOCKS>
 struct GiSweep {                              // the other blocks
-    int2 state[GI_WARP_TILES][GI_TILE][32];   // state from behind, by suffix of a tile and depth
+    int2 state[gi_warp_tiles(BLOCKS)][GI_TILE][32];   // state from behind, by suffix of a tile and depth
     int f[GI_TILES][32], e[GI_TILES][32];     // of all tiles; f then r
     int s[GI_TILES], ev[GI_TILES];
 };
+template <int BLOCKS>
 union GiShared {
     GiSort sort;
     GiTable table;
-    GiSweep sweep;
+    GiSweep<BLOCKS> sweep;
 };
 
 // exclusive sum over the block's threads, the total in `all`
@@ -229,7 +238,8 @@ __device__ __forceinline__ void gi_sums(const int* s, const int* ev, int t, int 
 
 // from behind: the events, the end of the last run opened per depth, and the state at every suffix.  s_own: new nodes with a
 // new parent in front of the lane's suffix.
-__device__ __forceinline__ void gi_sweep_runs(GiScratch* X, GiSweep& sw, const GiOwn& o, int wib, int t, int tiles, int m, int lane,
+template <class Sweep>
+__device__ __forceinline__ void gi_sweep_runs(GiScratch* X, Sweep& sw, const GiOwn& o, int wib, int t, int tiles, int m, int lane,
                                               int& s_own) {
     const unsigned FULL = 0xffffffffu;
     const int j0 = t * GI_TILE, mm = min(GI_TILE, m - j0), d = lane + 1;
@@ -277,7 +287,8 @@ __device__ __forceinline__ void gi_sweep_runs(GiScratch* X, GiSweep& sw, const G
 }
 
 // from the front: the new nodes below the events, from entry `used` on (sw.f holds what the tiles left in r)
-__device__ __forceinline__ void gi_sweep_emit(const GiSweep& sw, const GiOwn& o, int4* ent, int used, int wib, int t, int m, int lane,
+template <class Sweep>
+__device__ __forceinline__ void gi_sweep_emit(const Sweep& sw, const GiOwn& o, int4* ent, int used, int wib, int t, int m, int lane,
                                               int s_own) {
     const unsigned FULL = 0xffffffffu;
     const int j0 = t * GI_TILE, mm = min(GI_TILE, m - j0), d = lane + 1;
@@ -442,6 +453,7 @@ __device__ __forceinline__ void gi_merge(const sd_store& sv, const GiScratch* X,
     sync();
 }
 
+template <int GI_BLOCKS>
 __global__ void __launch_bounds__(GI_THREADS, 1)
 global_insert_kernel(sd_store sv, int n, const int32_t* d_slot, const int64_t* d_offsets, const int32_t* d_tokens, int tok_bits) {
     extern __shared__ __align__(16) unsigned char gi_smem[];
@@ -452,13 +464,14 @@ global_insert_kernel(sd_store sv, int n, const int32_t* d_slot, const int64_t* d
     const int D = sv.D;
     int4* const ent = sv.g_ent;
     GiScratch* const X = sv.gi;
-    GiShared& sh = *reinterpret_cast<GiShared*>(gi_smem);
+    GiShared<GI_BLOCKS>& sh = *reinterpret_cast<GiShared<GI_BLOCKS>*>(gi_smem);
+    constexpr int GI_REAL = gi_real(GI_BLOCKS);
+    auto meet = [] { if constexpr (GI_BLOCKS == GI_CLUSTER) cluster_sync(); else cg::this_grid().sync(); };
 
     // (every block looks at all items: all blocks take the same way)
     bool mine = false;
     for (int i = tid; i < n; i += GI_THREADS) mine |= d_slot[i] == -1;
     if (!__syncthreads_or(mine)) return;                         // the usual decode step: nothing for the global tree
-    cg::grid_group grid = cg::this_grid();
     bool full = (sv.g_state->status & SD_STATUS_GLOBAL_FULL) != 0, bad = false, again = false;
     int used = sv.g_state->used, live = 0;
     long long tokens_done = 0;
@@ -502,7 +515,7 @@ global_insert_kernel(sd_store sv, int n, const int32_t* d_slot, const int64_t* d
         const long long total = I.pref[n_items];
 
         for (long long c0 = 0; c0 < total && !full; c0 += GI_REAL) {
-            if (again) grid.sync();                              // the pass before is over
+            if (again) meet();                              // the pass before is over
             again = true;
             const int m = (int)min((long long)GI_REAL, total - c0);
             // ---------------- 1. walk, and sort
@@ -548,7 +561,7 @@ global_insert_kernel(sd_store sv, int n, const int32_t* d_slot, const int64_t* d
                 gi_walk(sv, X, I, d_tokens, c0, m, tid / APP_LANES * (GI_BLOCKS - 1) + blk - 1,
                         (GI_BLOCKS - 1) * GI_THREADS / APP_LANES, lane);
             }
-            grid.sync();
+            meet();
             // ---------------- 2. the sweeps, a warp per tile
             const int tiles = (m + GI_TILE - 1) / GI_TILE, t = (blk - 1) + wib * (GI_BLOCKS - 1);
             const bool sweeps = blk > 0 && t < tiles;
@@ -558,11 +571,11 @@ global_insert_kernel(sd_store sv, int n, const int32_t* d_slot, const int64_t* d
                 gi_own(own, X, t * GI_TILE, min(GI_TILE, m - t * GI_TILE), lane);
                 gi_sweep_tile(X, own, t, m, lane);
             }
-            grid.sync();
+            meet();
             int s_all, ev_all;
             if (blk == 0) gi_sums(X->s, X->ev, tiles, lane, s_all, ev_all);
             else {
-                GiSweep& sw = sh.sweep;
+                auto& sw = sh.sweep;
                 for (int i = tid; i < tiles * 8; i += GI_THREADS) {                 // (four depths at a time)
                     reinterpret_cast<int4*>(sw.f)[i] = reinterpret_cast<const int4*>(X->f)[i];
                     reinterpret_cast<int4*>(sw.e)[i] = reinterpret_cast<const int4*>(X->e)[i];
@@ -572,16 +585,16 @@ global_insert_kernel(sd_store sv, int n, const int32_t* d_slot, const int64_t* d
                 gi_sums(sw.s, sw.ev, tiles, lane, s_all, ev_all);
                 if (sweeps) gi_sweep_runs(X, sw, own, wib, t, tiles, m, lane, s_own);
             }
-            grid.sync();
+            meet();
             // ---------------- 3. grouping (block 0) while the others write the new nodes below the events
             if (blk == 0) gi_group(sv, X, sh.table, wsum, used, s_all, ev_all, tid);
             else {
-                GiSweep& sw = sh.sweep;
+                auto& sw = sh.sweep;
                 for (int i = tid; i < tiles * 8; i += GI_THREADS) reinterpret_cast<int4*>(sw.f)[i] = reinterpret_cast<const int4*>(X->r)[i];
                 __syncthreads();
                 if (sweeps && (long long)used + s_all <= sv.g_cap) gi_sweep_emit(sw, own, ent, used, wib, t, m, lane, s_own);
             }
-            grid.sync();
+            meet();
             // ---------------- merges: a warp per parent, a block per parent with a long run
             const int n_groups = X->n_groups;
             full = X->fits == 0;
@@ -596,7 +609,7 @@ global_insert_kernel(sd_store sv, int n, const int32_t* d_slot, const int64_t* d
                     gi_merge<GI_THREADS>(sv, X, X->m_pos, g, used, tid, [] { __syncthreads(); });
                 }
             }
-            grid.sync();
+            meet();
             // ---------------- 4. the parents' entries
             if (!full) {
                 for (int gi = blk * GI_THREADS + tid; gi < n_groups; gi += GI_BLOCKS * GI_THREADS) {
@@ -678,6 +691,38 @@ append_kernel(sd_store sv, const int32_t* d_slot, const int64_t* d_offsets, cons
 
 }  // namespace
 
+namespace {
+
+// Once per device: the kernels' shared memory, and whether there is room for the cluster.
+int insert_setup(int dev, bool* cluster) {
+    constexpr int MAX_DEVICES = 64;
+    static std::atomic<int> known[MAX_DEVICES];                  // 1: a grid, 2: a cluster
+    if (dev < 0 || dev >= MAX_DEVICES) return SD_ERR_INVALID_ARG;
+    int k = known[dev].load();
+    if (k == 0) {
+        constexpr size_t grid_smem = sizeof(GiShared<GI_GRID>), cluster_smem = sizeof(GiShared<GI_CLUSTER>);
+        SD_CUDA_OK(cudaFuncSetAttribute(global_insert_kernel<GI_GRID>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)grid_smem));
+        k = 1;
+        if (cudaFuncSetAttribute(global_insert_kernel<GI_CLUSTER>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cluster_smem) == cudaSuccess &&
+            cudaFuncSetAttribute(global_insert_kernel<GI_CLUSTER>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) {
+            cudaLaunchAttribute attr;
+            attr.id = cudaLaunchAttributeClusterDimension;
+            attr.val.clusterDim.x = GI_CLUSTER; attr.val.clusterDim.y = 1; attr.val.clusterDim.z = 1;
+            cudaLaunchConfig_t cfg = {};
+            cfg.gridDim = dim3(GI_CLUSTER); cfg.blockDim = dim3(GI_THREADS); cfg.dynamicSmemBytes = cluster_smem;
+            cfg.attrs = &attr; cfg.numAttrs = 1;
+            int n = 0;
+            if (cudaOccupancyMaxActiveClusters(&n, global_insert_kernel<GI_CLUSTER>, &cfg) == cudaSuccess && n > 0) k = 2;
+        }
+        cudaGetLastError();
+        known[dev].store(k);
+    }
+    *cluster = k == 2;
+    return SD_OK;
+}
+
+}  // namespace
+
 extern "C" int sd_append(sd_store* s, int32_t n, const int32_t* d_slot, const int64_t* d_offsets,
                          const int32_t* d_tokens, const uint8_t* d_reset, void* stream) {
     if (!s || n < 0) return SD_ERR_INVALID_ARG;
@@ -694,8 +739,23 @@ extern "C" int sd_append(sd_store* s, int32_t n, const int32_t* d_slot, const in
     int tok_bits = 1;
     while (tok_bits < 31 && (1 << tok_bits) < s->V) ++tok_bits;
     void* args[] = {(void*)s, (void*)&n, (void*)&d_slot, (void*)&d_offsets, (void*)&d_tokens, (void*)&tok_bits};
-    SD_CUDA_OK(cudaFuncSetAttribute(global_insert_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(GiShared)));
-    SD_CUDA_OK(cudaLaunchCooperativeKernel((void*)global_insert_kernel, dim3(GI_BLOCKS), dim3(GI_THREADS), args, sizeof(GiShared), s->aux));
+    bool cluster = false;
+    const int rc = insert_setup(s->device, &cluster);
+    if (rc != SD_OK) return rc;
+    const int gi_blocks = cluster ? GI_CLUSTER : GI_GRID;
+    const void* const gi_kernel = cluster ? (const void*)global_insert_kernel<GI_CLUSTER> : (const void*)global_insert_kernel<GI_GRID>;
+    cudaLaunchAttribute attr;
+    if (cluster) {
+        attr.id = cudaLaunchAttributeClusterDimension;
+        attr.val.clusterDim.x = GI_CLUSTER; attr.val.clusterDim.y = 1; attr.val.clusterDim.z = 1;
+    } else {
+        attr.id = cudaLaunchAttributeCooperative;
+        attr.val.cooperative = 1;
+    }
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)gi_blocks); cfg.blockDim = dim3(GI_THREADS); cfg.stream = s->aux; cfg.attrs = &attr; cfg.numAttrs = 1;
+    cfg.dynamicSmemBytes = cluster ? sizeof(GiShared<GI_CLUSTER>) : sizeof(GiShared<GI_GRID>);
+    SD_CUDA_OK(cudaLaunchKernelExC(&cfg, gi_kernel, args));
     // (joined whatever becomes of the launch: the insert reads buffers that the caller may free behind this call on its stream)
     const cudaError_t record = cudaEventRecord(s->ev_join, s->aux);
     append_kernel<<<(unsigned)n, APPEND_THREADS, 0, st>>>(*s, d_slot, d_offsets, d_tokens, d_reset);
