@@ -164,7 +164,8 @@ int sd_append(sd_store* store, int32_t n, const int32_t* d_slot, const int64_t* 
  * A prompt that does not fit the slot's node pool or text buffer leaves the slot empty with
  * SD_STATUS_POOL_FULL.  Unlike the per-step calls this one may allocate device memory: its
  * temporaries (about 30 bytes per prompt token of the largest batch so far, twice that if one of
- * its prompts has more than 16,384 tokens) are kept by the store and reused.  The host arrays have
+ * its prompts has more than 16,384 tokens, 32,768 in a call of up to 16) are kept by the store and
+ * reused.  The host arrays have
  * been read when the call returns (it waits for the check of the tokens, and so for what `stream`
  * held at the call); the trees themselves are built asynchronously on `stream` like any per-step
  * call's work.  The workspace is shared by all calls on a store: order calls

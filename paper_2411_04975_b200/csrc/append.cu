@@ -17,7 +17,7 @@ namespace {
 //
 // Inserting a sequence adds one occurrence to every string of at most D tokens that starts at one
 // of its positions: one root-to-depth-D PATH per start position.  Up to 1,920 positions are taken at once, in one
-// cooperative launch:
+// launch:
 //   1. every path goes down the tree as far as it exists, eight lanes each, and raises the counts on its way (no path
 //      waits for another: nothing moves yet).  Meanwhile one block sorts the positions' suffixes;
 //   2. the sorted suffixes and their common prefixes are a trie of the whole batch.  Its nodes deeper than the walk
@@ -515,7 +515,7 @@ global_insert_kernel(sd_store sv, int n, const int32_t* d_slot, const int64_t* d
         const long long total = I.pref[n_items];
 
         for (long long c0 = 0; c0 < total && !full; c0 += GI_REAL) {
-            if (again) meet();                              // the pass before is over
+            if (again) meet();                                   // the pass before is over
             again = true;
             const int m = (int)min((long long)GI_REAL, total - c0);
             // ---------------- 1. walk, and sort
@@ -697,8 +697,8 @@ namespace {
 int insert_setup(int dev, bool* cluster) {
     constexpr int MAX_DEVICES = 64;
     static std::atomic<int> known[MAX_DEVICES];                  // 1: a grid, 2: a cluster
-    if (dev < 0 || dev >= MAX_DEVICES) return SD_ERR_INVALID_ARG;
-    int k = known[dev].load();
+    const bool kept = dev >= 0 && dev < MAX_DEVICES;
+    int k = kept ? known[dev].load() : 0;
     if (k == 0) {
         constexpr size_t grid_smem = sizeof(GiShared<GI_GRID>), cluster_smem = sizeof(GiShared<GI_CLUSTER>);
         SD_CUDA_OK(cudaFuncSetAttribute(global_insert_kernel<GI_GRID>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)grid_smem));
@@ -715,7 +715,7 @@ int insert_setup(int dev, bool* cluster) {
             if (cudaOccupancyMaxActiveClusters(&n, global_insert_kernel<GI_CLUSTER>, &cfg) == cudaSuccess && n > 0) k = 2;
         }
         cudaGetLastError();
-        known[dev].store(k);
+        if (kept) known[dev].store(k);
     }
     *cluster = k == 2;
     return SD_OK;

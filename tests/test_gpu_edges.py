@@ -63,7 +63,8 @@ def test_corpora_at_the_edges_of_the_sort(U, n, D, vocab):
 
 @pytest.mark.parametrize("sizes,D,vocab,fresh", [([1], 32, 4, False), ([7, 8, 9], 32, 6, False), ([511, 1, 0, 2], 17, 30, False),
                                                  ([513], 32, 2, False), ([2015], 32, 5, False), ([2016], 8, 700, True),
-                                                 ([2017, 3], 32, 40, False), ([1000, 1000, 1000, 1100], 24, 900, True)])
+                                                 ([2017, 3], 32, 40, False), ([1000, 1000, 1000, 1100], 24, 900, True),
+                                                 ([1920], 32, 50, False), ([1919, 2], 32, 800, True), ([961, 960, 1920], 17, 3, False)])
 def test_global_insert_at_the_edges_of_a_pass(U, sizes, D, vocab, fresh):
     rng = np.random.default_rng(sum(sizes) + D)
     base = [_text(rng, 400, vocab), rng.integers(0, vocab, size=300).astype(np.int32)]
