@@ -298,7 +298,7 @@ constexpr int CTA_WARPS_NARROW_STEP = 4;       // (sd_step: 128 registers; with 
 // memory, the children read as windows of 32 entries kept in registers, and a division per node: 45.3 us for a draft of 256
 // requests, 43.1 now; 43.6 -> 38.5 on other text; steps 55 -> 51.  The request of a candidate's children into L2 as it is found
 // is worth 1 - 2 % of that; requests into L1, or by cp.async, lost as much.  Telling the others the running SCORE one node
-// later cost 3 %.)
+// later cost 3 %.)  Slower on one text: long runs at many depths and a cold L2, where places run out: drafts of 64 requests 94 -> 101.5.
 struct Cand {
     unsigned hi, lo;                          // D; 0: a free place
     int tok, cb;
