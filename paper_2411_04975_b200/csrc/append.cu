@@ -16,7 +16,7 @@ namespace {
 // Global online insert (a finished request's output goes into the global tree).
 //
 // Inserting a sequence adds one occurrence to every string of at most D tokens that starts at one
-// of its positions: one root-to-depth-D PATH per start position.  Up to 1,920 positions are taken at once, in one
+// of its positions: one root-to-depth-D PATH per start position.  Up to 2,016 positions are taken at once, in one
 // launch:
 //   1. every path goes down the tree as far as it exists, eight lanes each, and raises the counts on its way (no path
 //      waits for another: nothing moves yet).  Meanwhile one block sorts the positions' suffixes;
@@ -59,10 +59,8 @@ struct GiTable {                              // block 0, while it groups
     int tok[GI_MAX], ev[GI_MAX];
     int n_big;
 };
-__host__ __device__ constexpr int gi_real(int blocks) {            // start positions per pass: a warp per tile
-    return (blocks - 1) * (GI_THREADS / 32) * GI_TILE < GI_MAX - SD_MAX_DEPTH ? (blocks - 1) * (GI_THREADS / 32) * GI_TILE : GI_MAX - SD_MAX_DEPTH;
-}
-__host__ __device__ constexpr int gi_warp_tiles(int blocks) { return (gi_real(blocks) / GI_TILE + blocks - 2) / (blocks - 1); }  // tiles per block
+__host__ __device__ constexpr int gi_warp_tiles(int blocks) { return ((GI_REAL + GI_TILE - 1) / GI_TILE + blocks - 2) / (blocks - 1); }  // tiles per block
+static_assert(gi_warp_tiles(GI_CLUSTER) <= GI_THREADS / 32 && gi_warp_tiles(GI_GRID) <= GI_THREADS / 32, "a warp per tile");
 template <int BLOCKS>
 struct GiSweep {                              // the other blocks
     int2 state[gi_warp_tiles(BLOCKS)][GI_TILE][32];   // state from behind, by suffix of a tile and depth
@@ -465,7 +463,6 @@ global_insert_kernel(sd_store sv, int n, const int32_t* d_slot, const int64_t* d
     int4* const ent = sv.g_ent;
     GiScratch* const X = sv.gi;
     GiShared<GI_BLOCKS>& sh = *reinterpret_cast<GiShared<GI_BLOCKS>*>(gi_smem);
-    constexpr int GI_REAL = gi_real(GI_BLOCKS);
     auto meet = [] { if constexpr (GI_BLOCKS == GI_CLUSTER) cluster_sync(); else cg::this_grid().sync(); };
 
     // (every block looks at all items: all blocks take the same way)

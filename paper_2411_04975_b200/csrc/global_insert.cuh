@@ -4,8 +4,13 @@
 #include "common.cuh"
 
 constexpr int GI_MAX = 2048;                  // positions of a pass, the tokens looked ahead at included
-constexpr int GI_TILE = 8;                     // suffixes per tile
-constexpr int GI_TILES = GI_MAX / GI_TILE;
+// Start positions of a pass (a lot).  What is in the tree when the pool runs full depends on it: the same for every kernel that inserts.
+constexpr int GI_REAL = GI_MAX - SD_MAX_DEPTH;
+// Suffixes per tile: a tile is a warp's, and the 15 x 16 warps that sweep in a cluster of 16 blocks take 2,016 positions by nines.
+// (By eights, 1,920 a pass, 2,010 positions took two passes: 146 - 148 us, now 116 - 121.  300 sequences of 100 tokens: 1,667 us and, on
+// other text, 1,964; now 1,816 and 1,908, since 960 walks at a time go three times for a full pass.)
+constexpr int GI_TILE = 9;
+constexpr int GI_TILES = (GI_MAX + GI_TILE - 1) / GI_TILE;
 
 // The new children of one node of the tree.
 struct GiGroup {

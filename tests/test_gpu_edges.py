@@ -78,6 +78,24 @@ def test_global_insert_at_the_edges_of_a_pass(U, sizes, D, vocab, fresh):
     pr.close()
 
 
+@pytest.mark.parametrize("n,fits", [(1990, True), (1990, False), (2016, True), (2016, False), (2017, False)])
+def test_what_a_full_pool_takes_goes_by_lots_of_2016(U, n, fits):
+    """New strings throughout, D nodes per start position but for the last ones: a lot that does not fit adds no node, whatever part of it
+    would; the one in front of it stays."""
+    D, vocab = 4, 4096
+    tokens = np.random.default_rng(n).permutation(vocab)[:n].astype(np.int32)
+    nodes = sum(min(D, n - i) for i in range(n))
+    last = sum(min(D, n - i) for i in range(2016)) if n > 2016 else 0    # nodes of the lots in front of the last one
+    pr = U.Pair([], vocab=vocab, D=D, n_slots=1, max_req_tokens=16, global_extra_nodes=nodes if fits else nodes - 1)
+    off, flat = U.ragged([tokens])
+    pr.g.append(U.dev_i32([-1]), torch.as_tensor(off, device=U.DEV), U.dev_i32(flat))
+    st = pr.g.stats()
+    assert st["global_pool_cap"] == (nodes if fits else nodes - 1)
+    assert st["global_status"] == (0 if fits else 4)
+    assert st["global_nodes"] == (nodes if fits else last)
+    pr.close()
+
+
 def test_global_insert_merges_long_runs(U):
     """One token with hundreds of children: runs that move and runs with room, merged by a block, children of which get children."""
     rng = np.random.default_rng(5)
