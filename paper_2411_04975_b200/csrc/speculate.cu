@@ -356,6 +356,7 @@ struct BlockSharedT {
     // per tree: jobs to be taken, a bit per place in ordp; warps whose match nodes are still to come; the request's are
     struct __align__(16) { unsigned ready[2]; int walking, appending; } board;
     int gave_up;                              // a warp waited too long for them
+    int at_hand;                              // all of them are known from the call before
     long long slice_sum[WARPS];
     int slice_fs[WARPS];
     AppendShared app;
@@ -1010,8 +1011,10 @@ speculate_fused_kernel(sd_store sv, int n, const int32_t* __restrict__ d_slot, i
     // ---------------- 1. match
     bool want_g = usable && !(flags & SD_FLAG_REQUEST_ONLY);
     bool want_r = usable && !(flags & SD_FLAG_GLOBAL_ONLY);
-    // sd_speculate, the match nodes of this very context are at hand
-    const bool at_hand = !STEP && MINB > 1 && ok && ss->g_gen == ss->gen && ss->g_epoch == sv.g_state->epoch && ss->g_len == t;
+    // sd_speculate, the match nodes of this very context are at hand?  One thread tells the others: the block of a slot that appears
+    // twice in the call, which is refused, reads these while the slot's first block may be writing them.
+    if (!STEP && MINB > 1 && tid == 0)
+        sh.at_hand = ok && ss->g_gen == ss->gen && ss->g_epoch == sv.g_state->epoch && ss->g_len == t;
     if (want_g && gtid >= 0 && gtid < Pe) {
         // the walk to the match node of the last d tokens starts at the node kept from the call before, or at the root
         const bool cache_ok = ss->g_gen == ss->gen && ss->g_epoch == sv.g_state->epoch && ss->g_len <= t;
@@ -1167,7 +1170,7 @@ speculate_fused_kernel(sd_store sv, int n, const int32_t* __restrict__ d_slot, i
     };
     // All jobs can be taken at once: in their order, then (256 requests: 38.6 us, without the barrier 41; where the SM has one block
     // it only costs, 6.2 -> 6.8 us for one request).
-    if (at_hand) __syncthreads();
+    if (!STEP && MINB > 1 && sh.at_hand) __syncthreads();
     // (nothing to do before the append is done: in a hardware barrier; looking every 200 ns cost such steps 4 %, every 400 ns 2 %)
     if (STEP && !want_g) {
         if (wib == 0) asm volatile("bar.arrive %0, %1;" ::"r"(BAR_APPENDED), "r"(NT) : "memory");

@@ -271,3 +271,24 @@ def test_match_nodes_found_while_prompts_are_sorted(U, n_slots, new):
         pr.append(every, [base[0][k:k + 1 + k % 4] for k in every])
     pr.check_speculate(every, 20, 2.0, 40)
     pr.close()
+
+
+@pytest.mark.parametrize("n", [40, 200, 400])
+def test_slots_that_appear_twice_in_batches_of_every_shape(U, n):
+    """One block per SM, two and four: the later appearances are refused, also while the first ones' match nodes are out of date."""
+    rng = np.random.default_rng(n)
+    pr = U.Pair([_text(rng, 2000, 50)], vocab=50, D=16, n_slots=n, max_req_tokens=100)
+    pr.append(list(range(n)), [_text(rng, int(k), 50) for k in rng.integers(20, 80, n)])
+    call = rng.integers(0, n, n)
+    call[:3] = call[-1]
+    first = np.sort(np.unique(call, return_index=True)[1])
+    again = np.setdiff1d(np.arange(n), first)
+    for turn in range(6):
+        got = {k: v.cpu().numpy() for k, v in pr.g.speculate(U.dev_i32(call), 12, 2.0, 40).items()}
+        got["mask"] = got["mask"].view(np.uint32)
+        assert (got["status"][first] == 0).all() and (got["status"][again] == 1).all()
+        assert (got["n_draft"][again] == 0).all() and (got["chosen_tree"][again] == -1).all()
+        U.assert_same_drafts({k: v[first] for k, v in got.items()}, pr.o.speculate(call[first].tolist(), 12, 2.0, 40, M=64, n_threads=4))
+        some = rng.permutation(n)[:n // 2].tolist()              # every other turn the global tree changes, too
+        pr.append(some + [-1] * (turn % 2), [_text(rng, 2, 50) for _ in some] + [_text(rng, 90, 50)] * (turn % 2))
+    pr.close()
