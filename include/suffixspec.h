@@ -168,8 +168,9 @@ int sd_append(sd_store* store, int32_t n, const int32_t* d_slot, const int64_t* 
  * reused.  The host arrays have
  * been read when the call returns (it waits for the check of the tokens, and so for what `stream`
  * held at the call); the trees themselves are built asynchronously on `stream` like any per-step
- * call's work.  The workspace is shared by all calls on a store: order calls
- * made on different streams.
+ * call's work.  The workspace is shared by all calls of this function on a store: order those
+ * made on different streams.  Calls for other slots (sd_step, sd_speculate, sd_append) and inserts
+ * into the global tree may be at work on other streams meanwhile.
  * Errors: INVALID_ARG (bad slot, slot twice, offsets not ascending, token outside [0, V): nothing
  * is changed), CAPACITY (n * vocab, the token total or the nodes of all the prompts' trees together
  * do not fit 31 bits: nothing is changed; only where the token total times depth_cap does not, the

@@ -628,9 +628,10 @@ global_insert_kernel(sd_store sv, int n, const int32_t* d_slot, const int64_t* d
         }
     }
     bad = __syncthreads_or(bad) != 0;
+    if (again) meet();                               // (who sees the new epoch sees the whole of the new tree; 1 us of an append of 256 requests)
     if (tid == 0 && blk == 0) {
         GlobalState* gs = sv.g_state;
-        gs->epoch += 1;                              // cached match nodes of every slot are stale now
+        sd_release(&gs->epoch, gs->epoch + 1);       // cached match nodes of every slot are stale now
         gs->used = used;
         gs->live += live;
         gs->status |= (full ? SD_STATUS_GLOBAL_FULL : 0) | (bad ? SD_STATUS_BAD_TOKEN : 0);

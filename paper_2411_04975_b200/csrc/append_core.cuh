@@ -148,8 +148,9 @@ __device__ __forceinline__ int group_lookup(RunSearch a, int x, int lane, int& p
 
 // All lanes of the warp call; the eight lanes of a group go `steps` tokens (token(0), ...) down from `node` with child run zw; on
 // return node is the node reached or -1.  The eight entries at hand hold the next levels, too, where they are only
-// children (most of them are): a token then costs no load.  Long runs are searched.
-template <class F>
+// children (most of them are): a token then costs no load.  Long runs are searched.  MOVING: the tree may be changing meanwhile: what
+// is found may be wrong, but nothing outside the `limit` entries is read.
+template <bool MOVING = false, class F>
 __device__ __forceinline__ void group_walk(const int4* ent, int limit, int& node, int2& zw, int steps, int lane, F token) {
     const unsigned FULL = 0xffffffffu;
     const int l = lane & (APP_LANES - 1), gb = lane & ~(APP_LANES - 1);
@@ -159,7 +160,8 @@ __device__ __forceinline__ void group_walk(const int4* ent, int limit, int& node
         bool on = node >= 0 && k < steps;
         if (!__any_sync(FULL, on)) break;
         const int x = on ? token(k) : -1;
-        const int n = on ? (int)((unsigned)zw.y & RUN_COUNT_MASK) : 0;
+        int n = on ? (int)((unsigned)zw.y & RUN_COUNT_MASK) : 0;
+        if (MOVING && (zw.x < 0 || zw.x > limit - n)) { n = 0; zw.x = 0; }
         const bool far = n > APP_LANES;
         if (__any_sync(FULL, far)) {
             int place;

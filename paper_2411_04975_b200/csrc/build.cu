@@ -450,8 +450,8 @@ cluster_corpus_sort_kernel(const int32_t* tok, const int64_t* seq_off, int n_seq
 // What clusters that have no prompt to sort do meanwhile, on multiprocessors that would be idle: a block per request, they walk to
 // global match nodes, which the request's next draft goes on from as from a draft before.  First the new requests' (the last tokens of a
 // prompt are known, the tree is there), then those of the other slots that an insert into the global tree has made
-// stale: otherwise every one of them walks all the way in its next draft (256 requests as a service: drafts behind an insert
-// 51 us, now 42; the sort beside it 43 -> 47).
+// stale, in records of their own (MatchRecord): otherwise every one of them walks all the way in its next draft (256 requests as a
+// service: drafts behind an insert 51 us, now 43, of which 1 to take the record; the sort beside it 43 -> 47).
 constexpr int MOST_REFRESHED = 1024;
 // Whether this call of sd_build_requests has been refused for a token outside the vocabulary (in GlobalState, which keeps the last such
 // call: nothing has to be cleared).
@@ -471,32 +471,53 @@ struct RequestWalk {
 
 __device__ __forceinline__ void request_walk(const RequestWalk& R, int q) {
     __shared__ int tail[SD_MAX_DEPTH];                           // the last tokens
+    __shared__ int sh_epoch, sh_len;
     const int tid = threadIdx.x, lane = tid & 31, d = tid / APP_LANES + 1, D = R.sv.D;
     const bool fresh = q < R.n;
     const int slot = fresh ? R.slot[q] : q - R.n;
     if (R.bad() || slot < 0 || slot >= R.sv.R) return;
     SlotState* const ss = R.sv.s_state + slot;
-    const int gen = ss->gen, epoch = R.sv.g_state->epoch, len = fresh ? (int)(R.off[q + 1] - R.off[q]) : ss->len;
+    MatchRecord* const rec = &ss->record;
+    // An insert may be at work on the tree on another stream (the call itself has nothing to do with that tree): whoever has seen the epoch
+    // of its end sees all that it wrote, and what is found before that carries an epoch that is over by then.
     bool leave = false;
-    if (!fresh) {
-        leave = len <= 0 || (ss->status & (SD_STATUS_POOL_FULL | SD_STATUS_BAD_TOKEN)) || (ss->g_gen == gen && ss->g_epoch == epoch && ss->g_len <= len);
+    if (tid == 0) {
+        sh_epoch = sd_acquire(&R.sv.g_state->epoch);
+        sh_len = fresh ? (int)(R.off[q + 1] - R.off[q]) : sd_relaxed(&ss->len);
+        leave = !fresh && (sh_len <= 0 || sh_len > R.sv.T || (sd_relaxed(&ss->status) & (SD_STATUS_POOL_FULL | SD_STATUS_BAD_TOKEN)) ||
+                           (sd_relaxed(&ss->g_gen) == sd_relaxed(&ss->gen) && sd_relaxed(&ss->g_epoch) == sh_epoch && sd_relaxed(&ss->g_len) <= sh_len));
+    }
+    if (!fresh)
         for (int j = tid; j < R.n; j += CP_THREADS) leave |= R.slot[j] == slot;     // (it is another request's from now on)
+    if (__syncthreads_or(leave)) return;
+    const int epoch = sh_epoch, len = sh_len;
+    const int32_t* const end = fresh ? R.tok + R.off[q] + len : R.sv.s_text + (i64)slot * R.sv.T + len;
+    if (tid < SD_MAX_DEPTH) {
+        tail[tid] = tid < len ? sd_relaxed(&end[-1 - tid]) : -1;
+        leave = tid < len && (tail[tid] < 0 || tail[tid] >= R.sv.V);
     }
     if (__syncthreads_or(leave)) return;
-    const int32_t* const end = fresh ? R.tok + R.off[q] + len : R.sv.s_text + (i64)slot * R.sv.T + len;
-    if (tid < SD_MAX_DEPTH && tid < len) tail[tid] = end[-1 - tid];
-    __syncthreads();
-    if (d > SD_MAX_DEPTH) return;
     int node = -1;
     int2 zw = make_int2(0, 0);
     if (d <= len && d <= D) {
         node = R.sv.g_root[tail[d - 1]];
+        if (node >= (int)R.sv.g_cap) node = -1;
         if (node >= 0) zw = *reinterpret_cast<const int2*>(&R.sv.g_ent[node].z);
     }
-    group_walk(R.sv.g_ent, (int)R.sv.g_cap, node, zw, d - 1, lane, [&](int k) { return tail[d - 2 - k]; });
-    if ((lane & (APP_LANES - 1)) == 0) ss->g_node[d - 1] = node;
-    // (a new request's are no good for the one that still has the slot: requests_prepare_kernel makes them the new one's)
-    if (tid == 0) { ss->g_gen = fresh ? gen - 1 : gen; ss->g_epoch = epoch; ss->g_len = len; ss->g_depths = D; }
+    group_walk<true>(R.sv.g_ent, (int)R.sv.g_cap, node, zw, d - 1, lane, [&](int k) { return tail[d - 2 - k]; });
+    if (fresh) {
+        if ((lane & (APP_LANES - 1)) == 0) ss->g_node[d - 1] = node;
+        // (a new request's are no good for the one that still has the slot: requests_prepare_kernel makes them the new one's)
+        if (tid == 0) { ss->g_gen = ss->gen - 1; ss->g_epoch = epoch; ss->g_len = len; ss->g_depths = D; }
+        return;
+    }
+    if (tid == 0) { rec->version |= 1; sd_fence(); }
+    __syncthreads();
+    if ((lane & (APP_LANES - 1)) == 0) rec->node[d - 1] = node;
+    if (tid < SD_MAX_DEPTH) rec->tail[tid] = tail[tid];
+    if (tid == 0) { rec->epoch = epoch; rec->len = len; }
+    __syncthreads();
+    if (tid == 0) sd_release(&rec->version, rec->version + 1);
 }
 
 template <int ITEMS>

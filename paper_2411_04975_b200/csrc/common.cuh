@@ -45,6 +45,17 @@ struct GlobalState {          // device-resident bookkeeping of the global tree
     int32_t bad_call;         // the last sd_build_requests call with a token outside the vocabulary
 };
 
+// Global match nodes of a slot as sd_build_requests leaves them for requests that are not its own.  Steps and drafts of these may be at
+// work on other streams meanwhile, so nothing of theirs is written, and what is read of them is not relied on: a draft takes the nodes
+// only if they were walked to with the very tokens of its text, in the tree as it is.
+struct MatchRecord {
+    int32_t version;          // odd while it is written
+    int32_t epoch;            // of the global tree
+    int32_t len;              // context length
+    int32_t tail[SD_MAX_DEPTH];     // its last tokens, last first
+    int32_t node[SD_MAX_DEPTH];     // node[d-1]: global node of the last d tokens, -1 none
+};
+
 struct SlotState {            // device-resident bookkeeping of one request slot
     int32_t len;              // context length t
     int32_t used;             // entries handed out of the slot pool
@@ -62,6 +73,7 @@ struct SlotState {            // device-resident bookkeeping of one request slot
     int32_t g_len;            // context length the cache was taken at
     int32_t g_depths;         // depths 1..g_depths are cached
     int32_t g_node[SD_MAX_DEPTH];   // g_node[d-1]: global node of the last d tokens, -1 none
+    MatchRecord record;             // taken where these are out of date
 };
 
 struct sd_workspace {         // grow-only device buffers, reused call after call
@@ -165,6 +177,12 @@ inline cudaError_t sd_launch_clusters(void (*kernel)(K...), unsigned grid, unsig
 // Device memory of the library (device_memory.cpp), and back when the work on it has ended.
 cudaError_t sd_device_malloc(void** p, size_t bytes);
 void sd_device_free(void* p);
+
+// What other kernels may write at the same time.
+__device__ __forceinline__ int sd_acquire(const int32_t* p) { int v; asm volatile("ld.acquire.gpu.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory"); return v; }
+__device__ __forceinline__ int sd_relaxed(const int32_t* p) { int v; asm volatile("ld.relaxed.gpu.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory"); return v; }
+__device__ __forceinline__ void sd_release(int32_t* p, int32_t v) { asm volatile("st.release.gpu.s32 [%0], %1;" ::"l"(p), "r"(v) : "memory"); }
+__device__ __forceinline__ void sd_fence() { asm volatile("fence.acq_rel.gpu;" ::: "memory"); }     // (__threadfence() took 7 us behind an insert)
 
 // Every entry point refuses a store that lives on another device than the current one.
 #define SD_CHECK_DEVICE(s)                                                   \

@@ -993,7 +993,7 @@ speculate_fused_kernel(sd_store sv, int n, const int32_t* __restrict__ d_slot, i
     if (tid < 2 * SD_MAX_DEPTH) { (&sh.node[0][0])[tid] = -1; (&sh.nc[0][0])[tid] = 0; }
     if (tid == 0) {
         sh.nwide = 0; sh.nwide_kept = 0; sh.best_hi = 0u; sh.board.ready[0] = 0u; sh.board.ready[1] = 0u;
-        sh.board.walking = WALK; sh.board.appending = 1; sh.gave_up = 0; sh.app.ahead = 0;
+        sh.board.walking = WALK; sh.board.appending = 1; sh.gave_up = 0; sh.app.ahead = 0; sh.at_hand = 0;
     }
     if (wib == WARPS - 1) {
         const int c = lane < Pe ? min(budget_for(alpha, lane + 1, cap), 2 * (D - lane - 1)) : -1;
@@ -1011,19 +1011,30 @@ speculate_fused_kernel(sd_store sv, int n, const int32_t* __restrict__ d_slot, i
     // ---------------- 1. match
     bool want_g = usable && !(flags & SD_FLAG_REQUEST_ONLY);
     bool want_r = usable && !(flags & SD_FLAG_GLOBAL_ONLY);
-    // sd_speculate, the match nodes of this very context are at hand?  One thread tells the others: the block of a slot that appears
-    // twice in the call, which is refused, reads these while the slot's first block may be writing them.
-    if (!STEP && MINB > 1 && tid == 0)
-        sh.at_hand = ok && ss->g_gen == ss->gen && ss->g_epoch == sv.g_state->epoch && ss->g_len == t;
-    if (want_g && gtid >= 0 && gtid < Pe) {
+    if (want_g && gw == 0) {
         // the walk to the match node of the last d tokens starts at the node kept from the call before, or at the root
-        const bool cache_ok = ss->g_gen == ss->gen && ss->g_epoch == sv.g_state->epoch && ss->g_len <= t;
-        const int k = t - ss->g_len;                            // tokens appended since the cache was taken
-        const int d = gtid + 1;
+        const int d = lane + 1;
+        int len = ss->g_len, depths = ss->g_depths, kept = ss->g_node[lane];
+        bool known = ss->g_gen == ss->gen && ss->g_epoch == sv.g_state->epoch && len <= t;
+        if (!known) {
+            // (a call of sd_build_requests may be writing it)
+            const MatchRecord& rec = ss->record;
+            const int version = sd_acquire(&rec.version);
+            len = sd_relaxed(&rec.len); depths = D; kept = sd_relaxed(&rec.node[lane]);
+            known = version != 0 && (version & 1) == 0 && sd_relaxed(&rec.epoch) == sv.g_state->epoch && len > 0 && len <= t_old;
+            if (known && lane < len && lane < D) known = sd_relaxed(&rec.tail[lane]) == text[len - 1 - lane];
+            sd_fence();
+            known = __all_sync(FULL, known && sd_relaxed(&rec.version) == version);
+        }
+        const int k = t - len;                                  // tokens appended since
+        const int before = __shfl_sync(FULL, kept, max(d - k - 1, 0));
+        // the match nodes of this very context are at hand?  (One warp tells the others: the block of a slot that appears twice in the
+        // call, which is refused, reads all this while the slot's first block may be writing it.)
+        if (!STEP && lane == 0) sh.at_hand = known && k == 0;
         int node = -1, from = t;
-        if (d <= t) {
-            if (cache_ok && d > k && d - k <= ss->g_depths) {
-                node = ss->g_node[d - k - 1];                   // node of the tokens before the new ones
+        if (d <= t && d <= Pe) {
+            if (known && d > k && d - k <= depths) {
+                node = before;                                  // node of the tokens before the new ones
                 from = t - k;
             } else {
                 const int x0 = t - d < t_old ? text[t - d] : newtok[t - d - t_old];
@@ -1031,7 +1042,7 @@ speculate_fused_kernel(sd_store sv, int n, const int32_t* __restrict__ d_slot, i
                 from = t - d + 1;
             }
         }
-        sh.src_node[gtid] = node; sh.src_from[gtid] = from;
+        if (d <= Pe) { sh.src_node[lane] = node; sh.src_from[lane] = from; }
     }
     // all cached nodes read before any is replaced; and: is this a second block for the same slot?
     const bool refused = __syncthreads_or(dup) != 0;

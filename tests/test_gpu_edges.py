@@ -292,3 +292,58 @@ def test_slots_that_appear_twice_in_batches_of_every_shape(U, n):
         some = rng.permutation(n)[:n // 2].tolist()              # every other turn the global tree changes, too
         pr.append(some + [-1] * (turn % 2), [_text(rng, 2, 50) for _ in some] + [_text(rng, 90, 50)] * (turn % 2))
     pr.close()
+
+
+def test_prompts_sorted_beside_steps_and_inserts_on_other_streams(U):
+    """sd_build_requests has nothing to do with the other slots and the global tree: steps of those and inserts into that may be at work on
+    other streams.  What it finds out for them meanwhile is taken for the text that it was found for only."""
+    rng = np.random.default_rng(12)
+    vocab, old, new, D = 40, 100, 4, 24
+    pr = U.Pair([_text(rng, 4000, vocab)], vocab=vocab, D=D, n_slots=old + new, max_req_tokens=2400)
+    every, a, b = list(range(old + new)), torch.cuda.Stream(), torch.cuda.Stream()
+    first = [_text(rng, int(k), vocab) for k in rng.integers(5, 60, old + new)]
+    pr.append(every, first)
+
+    def build():
+        prompts = [_text(rng, 1100 + 200 * k, vocab, 90) for k in range(new)]
+        off, flat = U.ragged(prompts)
+        flat = U.dev_i32(flat)
+        torch.cuda.synchronize()
+
+        def call():
+            with torch.cuda.stream(a):
+                pr.g.build_requests(np.arange(old, old + new), off, flat)
+            torch.cuda.synchronize()
+            for k in range(new):
+                pr.o.slot_reset(old + k)
+            pr.o.slot_append_batch(every[old:], prompts)
+        return call
+
+    for turn in range(8):
+        pr.append([-1], [_text(rng, 300, vocab, 30)])            # the match nodes are stale
+        lists = [_text(rng, 1 + (k + turn) % 7, vocab) for k in range(old)]
+        off, flat = U.ragged(lists)
+        args = (U.dev_i32(every[:old]), torch.as_tensor(off, device=U.DEV), U.dev_i32(flat))
+        call = build()
+        with torch.cuda.stream(b):
+            pr.g.step(*args, 20, 2.0, 40)
+        call()
+        pr.o.slot_append_batch(every[:old], lists, n_threads=4)
+        pr.check_speculate(every, 20, 2.0, 40)
+        seqs = [_text(rng, 700, vocab, 50), _text(rng, 90, vocab)]
+        off, flat = U.ragged(seqs)
+        args = (U.dev_i32([-1, -1]), torch.as_tensor(off, device=U.DEV), U.dev_i32(flat))
+        call = build()
+        with torch.cuda.stream(b):
+            pr.g.append(*args)
+        call()
+        for s in seqs:
+            pr.o.global_insert(s)
+        pr.check_speculate(every[::2], 20, 2.0, 40)
+        pr.append([-1], [_text(rng, 80, vocab)])
+        build()()                                                # leaves match nodes for all ...
+        pr.append(every[:40], [_text(rng, 70, vocab) for _ in range(40)], reset=[1] * 40)       # ... of which some have another text now
+        pr.append(every[30:60], [_text(rng, 3, vocab) for _ in range(30)])
+        pr.check_speculate(every, 20, 2.0, 40)
+    pr.check_tree(-1)
+    pr.close()
