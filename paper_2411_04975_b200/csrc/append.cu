@@ -691,30 +691,32 @@ append_kernel(sd_store sv, const int32_t* d_slot, const int64_t* d_offsets, cons
 
 namespace {
 
-// Once per device: the kernels' shared memory, and whether there is room for the cluster.
+// Whether the device has room for the cluster (asked once), and the limits of the kernel that will be launched, at every call: they are
+// gone after a cudaDeviceReset.
 int insert_setup(int dev, bool* cluster) {
     constexpr int MAX_DEVICES = 64;
     static std::atomic<int> known[MAX_DEVICES];                  // 1: a grid, 2: a cluster
     const bool kept = dev >= 0 && dev < MAX_DEVICES;
     int k = kept ? known[dev].load() : 0;
-    if (k == 0) {
-        constexpr size_t grid_smem = sizeof(GiShared<GI_GRID>), cluster_smem = sizeof(GiShared<GI_CLUSTER>);
-        SD_CUDA_OK(cudaFuncSetAttribute(global_insert_kernel<GI_GRID>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)grid_smem));
-        k = 1;
-        if (cudaFuncSetAttribute(global_insert_kernel<GI_CLUSTER>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cluster_smem) == cudaSuccess &&
-            cudaFuncSetAttribute(global_insert_kernel<GI_CLUSTER>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) {
+    if (k != 1) {
+        constexpr size_t smem = sizeof(GiShared<GI_CLUSTER>);
+        const bool set = cudaFuncSetAttribute(global_insert_kernel<GI_CLUSTER>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) == cudaSuccess &&
+                         cudaFuncSetAttribute(global_insert_kernel<GI_CLUSTER>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
+        if (k == 0) {
             cudaLaunchAttribute attr;
             attr.id = cudaLaunchAttributeClusterDimension;
             attr.val.clusterDim.x = GI_CLUSTER; attr.val.clusterDim.y = 1; attr.val.clusterDim.z = 1;
             cudaLaunchConfig_t cfg = {};
-            cfg.gridDim = dim3(GI_CLUSTER); cfg.blockDim = dim3(GI_THREADS); cfg.dynamicSmemBytes = cluster_smem;
+            cfg.gridDim = dim3(GI_CLUSTER); cfg.blockDim = dim3(GI_THREADS); cfg.dynamicSmemBytes = smem;
             cfg.attrs = &attr; cfg.numAttrs = 1;
             int n = 0;
-            if (cudaOccupancyMaxActiveClusters(&n, global_insert_kernel<GI_CLUSTER>, &cfg) == cudaSuccess && n > 0) k = 2;
-        }
-        cudaGetLastError();
-        if (kept) known[dev].store(k);
+            k = set && cudaOccupancyMaxActiveClusters(&n, global_insert_kernel<GI_CLUSTER>, &cfg) == cudaSuccess && n > 0 ? 2 : 1;
+            cudaGetLastError();
+            if (kept) known[dev].store(k);
+        } else if (!set) return SD_ERR_CUDA;
     }
+    if (k == 1)
+        SD_CUDA_OK(cudaFuncSetAttribute(global_insert_kernel<GI_GRID>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(GiShared<GI_GRID>)));
     *cluster = k == 2;
     return SD_OK;
 }
