@@ -6,6 +6,7 @@
 #include <unistd.h>
 
 #include <algorithm>
+#include <atomic>
 #include <chrono>
 #include <condition_variable>
 #include <mutex>
@@ -257,7 +258,12 @@ void sd_device_free(void* p) {
     c.bytes += b.bytes;
 }
 
+static std::atomic<int> g_trims{0};
+
+int sd_trims() { return g_trims.load(); }
+
 extern "C" void sd_trim(void) {
+    ++g_trims;
     std::lock_guard<std::mutex> lock(g.mutex);
     for (int dev = 0; dev < CACHE_DEVICES; ++dev) cache_expire(dev, g.cache[dev], Clock::time_point::max());
 }

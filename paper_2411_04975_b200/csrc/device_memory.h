@@ -9,5 +9,8 @@ struct StreamSet { cudaStream_t aux; cudaEvent_t ev_fork, ev_join, ev_check; voi
 // For a store on the current device, with at least `stage_bytes` of pinned memory.
 bool sd_take_streams(int dev, size_t stage_bytes, StreamSet* out);
 
+// Calls of sd_trim so far.  What is set up once per device is set up anew behind one: a cudaDeviceReset may have followed.
+int sd_trims();
+
 // Releases what a store holds, behind the work on `st`: the caller has waited for every other stream that used the store.
 void sd_store_release(sd_store* s, cudaStream_t st);

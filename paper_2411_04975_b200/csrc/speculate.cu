@@ -18,6 +18,7 @@
 #include <mutex>
 
 #include "append_core.cuh"
+#include "device_memory.h"
 
 namespace {
 
@@ -1320,7 +1321,7 @@ speculate_fused_kernel(sd_store sv, int n, const int32_t* __restrict__ d_slot, i
 namespace {
 
 constexpr int MAX_DEVICES = 64;
-struct DeviceInfo { bool ready = false; int sm_count = 0; };
+struct DeviceInfo { bool ready = false; int trims = 0, sm_count = 0; };
 DeviceInfo g_dev[MAX_DEVICES];
 std::mutex g_dev_mutex;
 
@@ -1330,17 +1331,19 @@ int raise_smem_limit() {
                                 (int)sizeof(BlockSharedT<WARPS>)) == cudaSuccess ? SD_OK : SD_ERR_CUDA;
 }
 
-// once per device: raise the kernels' dynamic shared memory limit, read the SM count
+// once per device (and behind sd_trim): raise the kernels' dynamic shared memory limit, read the SM count
 int device_setup(int dev, int* sm_count) {
     if (dev < 0 || dev >= MAX_DEVICES) return SD_ERR_INVALID_ARG;
     std::lock_guard<std::mutex> lock(g_dev_mutex);
-    if (!g_dev[dev].ready) {
+    const int trims = sd_trims();
+    if (!g_dev[dev].ready || g_dev[dev].trims != trims) {
         if (raise_smem_limit<false, CTA_WARPS, 2>() != SD_OK || raise_smem_limit<true, CTA_WARPS_STEP, 2>() != SD_OK ||
             raise_smem_limit<false, CTA_WARPS_WIDE, 1>() != SD_OK || raise_smem_limit<true, CTA_WARPS_WIDE, 1>() != SD_OK ||
             raise_smem_limit<false, CTA_WARPS_NARROW, 4>() != SD_OK ||
             raise_smem_limit<true, CTA_WARPS_NARROW_STEP, 4>() != SD_OK)
             return SD_ERR_CUDA;
         SD_CUDA_OK(cudaDeviceGetAttribute(&g_dev[dev].sm_count, cudaDevAttrMultiProcessorCount, dev));
+        g_dev[dev].trims = trims;
         g_dev[dev].ready = true;
     }
     *sm_count = g_dev[dev].sm_count;

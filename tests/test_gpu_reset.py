@@ -31,6 +31,12 @@ for turn in range(2):
     tokens = (np.arange(40) % 7).astype(np.int32)
     rc = lib.sd_append(store, 2, device(np.array([-1, 0], np.int32)), device(np.array([0, 30, 40], np.int64)), device(tokens), None, None)
     assert rc == 0, (turn, rc)
+    spec, M, out = binding._SpecParams(4, 2.0, 8, 0, 0.0), 64, [device(np.zeros(2 * 64, np.int64)) for _ in range(9)]
+    for _ in range(2):
+        rc = lib.sd_speculate(store, 1, device(np.array([0], np.int32)), C.byref(spec), None, *out, None)
+        assert rc == 0, (turn, rc)
+    n_draft = np.zeros(1, np.int32)
+    assert rt.cudaMemcpy(n_draft.ctypes.data, out[0], 4, 2) == 0 and n_draft[0] > 0
     st = binding._Stats()
     assert lib.sd_stats(store, C.byref(st), None) == 0
     assert st.global_tokens == 30 and st.global_nodes == 7 * 8
@@ -41,7 +47,7 @@ print("done")
 """
 
 
-def test_appends_after_a_device_reset():
+def test_appends_and_drafts_after_a_device_reset():
     root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
     r = subprocess.run([sys.executable, "-c", PROGRAM], cwd=root, capture_output=True, text=True, timeout=300)
     assert r.returncode == 0 and r.stdout.endswith("done\n"), r.stderr
