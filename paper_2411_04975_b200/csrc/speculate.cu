@@ -299,7 +299,9 @@ constexpr int CTA_WARPS_NARROW_STEP = 4;       // (sd_step: 128 registers; with 
 // memory, the children read as windows of 32 entries kept in registers, and a division per node: 45.3 us for a draft of 256
 // requests, 43.1 now; 43.6 -> 38.5 on other text; steps 55 -> 51.  The request of a candidate's children into L2 as it is found
 // is worth 1 - 2 % of that; requests into L1, or by cp.async, lost as much.  Telling the others the running SCORE one node
-// later cost 3 %.)  Slower on one text: long runs at many depths and a cold L2, where places run out: drafts of 64 requests 94 -> 101.5.
+// later cost 3 %.)  Slower where branches of few children follow one another all the way (text that copies 19 of 20 spans, of 100
+// tokens each): drafts of 8 / 64 / 256 requests 34 / 38 / 46 -> 39 / 41 / 50; windows there, too, or asking for the children as soon
+// as the node is known brought nothing back with a warm L2.
 struct Cand {
     unsigned hi, lo;                          // D; 0: a free place
     int tok, cb;
@@ -575,11 +577,14 @@ __device__ __noinline__ int pool_compact(Pool& C, int n, int room, unsigned& flo
     return k;
 }
 
-// The best children (by count, then smallest token; at most `room`) of a node with more than 32: their entries, best
-// first, in `list`.  One class of equal counts after the other, within it in run (token) order.  The classes are taken
-// from registers: all of a run of up to 128 children, else those that occur often (up to 128 of them; most children
-// of a long run occur once or twice), and only what is left from the run itself.  `hot`: 256 words of the warp's.
-// (Every class by a pass over the run: drafts of 64 requests of text in which one token is every second one 125 us, now 107.)
+// The best children (by count, then smallest token; at most `room`) of a node with more than 32: their entries in `list`, where `room` are
+// found the last one is the least of them.  They are taken from registers: all of a run of up to 128 children, else those that occur
+// often (up to 128 of them; most children of a long run occur once or twice), and only what is left from the run itself, there
+// one class of equal counts after the other.  `hot`: 256 words of the warp's.
+// Text in which one token is every second one is bound by this: 17 runs of 33 to 128 children in the slowest jobs, with 20 places left on
+// average.  Listed from registers class by class (2,900 to 5,000 cycles a run, a ballot chain per class) drafts of 64 requests took
+// 98.6 us; with the least count found by halves 94.6; with that search begun at 2 and ended at sum / room, the most it can be, 80.7 (1,050
+// to 1,500 cycles).  Every class by a pass over the run took 125.
 __device__ __noinline__ int list_by_count(const int4* __restrict__ ent, int cb, int n, int room, int* list, int* hot, unsigned& sum_out,
                                           int lane) {
     unsigned y[4], least = 1u;                                  // counts from `least` on are in the registers
@@ -634,19 +639,37 @@ __device__ __noinline__ int list_by_count(const int4* __restrict__ ent, int cb, 
             y[u] = in ? (unsigned)hot[2 * (u * 32 + lane) + 1] : 0u;
         }
     }
-    int taken = 0;
-    unsigned top = __reduce_max_sync(FULL, max(max(y[0], y[1]), max(y[2], y[3])));
-    while (top > 0u && taken < room) {
-        unsigned next = 0;
+    // what they hold: those that occur more often than the last one that there is room for, then as many that occur as often, in run order.
+    // `room` of them that occur `cut` times make up room * cut of the sum at least.
+    unsigned cut = 1u, top = min(__reduce_max_sync(FULL, max(max(y[0], y[1]), max(y[2], y[3]))), sum_out / (unsigned)room);
+    while (cut < top) {
+        const unsigned mid = min(2u * cut, cut + (top - cut + 1u) / 2u);
+        unsigned k = 0;
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const unsigned m = __ballot_sync(FULL, y[u] == top);
-            const int at = taken + __popc(m & ((1u << lane) - 1u));
-            if (y[u] == top && at < room) list[at] = cb + pos[u];
-            taken += __popc(m);
-            if (y[u] < top) next = max(next, y[u]);
+        for (int u = 0; u < 4; ++u) k += y[u] >= mid ? 1u : 0u;
+        k = __reduce_add_sync(FULL, k);
+        if (k >= (unsigned)room) cut = mid; else top = mid - 1u;
+        if (k == (unsigned)room) {                              // these are they
+            unsigned fewest = 0xffffffffu;
+#pragma unroll
+            for (int u = 0; u < 4; ++u) if (y[u] >= mid) fewest = min(fewest, y[u]);
+            cut = __reduce_min_sync(FULL, fewest);
+            break;
         }
-        top = __reduce_max_sync(FULL, next);
+    }
+    int taken = 0;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+        const unsigned m = __ballot_sync(FULL, y[u] > cut);
+        if (y[u] > cut) list[taken + __popc(m & ((1u << lane) - 1u))] = cb + pos[u];
+        taken += __popc(m);
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+        const unsigned m = __ballot_sync(FULL, y[u] == cut);
+        const int at = taken + __popc(m & ((1u << lane) - 1u));
+        if (y[u] == cut && at < room) list[at] = cb + pos[u];
+        taken += __popc(m);
     }
     // what the registers do not hold (least 0: nothing is in them)
     top = least - 1u;
@@ -673,7 +696,10 @@ __device__ __noinline__ int list_by_count(const int4* __restrict__ ent, int cb, 
 
 // ExpandSpeculationTree + SCORE for one (tree, p) job by one warp.  nseed >= 0: the match node's best
 // children are in W.T (nseed of them, from ring head 0, with their D).
-template <class BlockShared>
+// ROOMY: candidates that find no lane of their own kind free go into free places of either kind before room is made, through shared memory.
+// On text with long runs at many depths 42 of 54 compactions a request are not needed then (drafts of 64 requests 102.5 -> 98.6 us).
+// Where blocks share an SM the registers that it takes are spilled: drafts of 256 requests 4.5 % longer.
+template <bool ROOMY, class BlockShared>
 __device__ __noinline__ void expand_job(BlockShared& sh, WarpWork& W, const int4* __restrict__ ent, int limit, int tree, int p,
                            int budget, unsigned flags, int nseed, int lane) {
     const int order = tree * SD_MAX_DEPTH + p;                  // loop order of Algorithm 1
@@ -759,7 +785,7 @@ __device__ __noinline__ void expand_job(BlockShared& sh, WarpWork& W, const int4
                 }
                 for (int base = 0; base < nl; base += 32) {
                     const int k = min(32, nl - base);
-                    // a child per lane with a free place; where there are too few, all lanes in order, and room is made
+                    // a child per lane with a free place; where there are too few of a kind, all lanes in order, and a place is found or made
                     const unsigned f0 = __ballot_sync(FULL, c0.hi == 0u), f1 = __ballot_sync(FULL, c1.hi == 0u);
                     const bool to0 = __popc(f0) >= k, fits = to0 || __popc(f1) >= k;
                     const unsigned f = to0 ? f0 : (fits ? f1 : FULL);
@@ -770,8 +796,7 @@ __device__ __noinline__ void expand_job(BlockShared& sh, WarpWork& W, const int4
                     double q;
                     if (cur_n <= 32) {
                         const unsigned sum = __reduce_add_sync(FULL, (unsigned)e.y);             // sibling sum: the denominator of Eq. 1
-                        if (sum <= (unsigned)RECIP_MAX)
-                        q = quotient((double)e.y, (double)sum, sh.recip.r[sum]);
+                        if (sum <= (unsigned)RECIP_MAX) q = quotient((double)e.y, (double)sum, sh.recip.r[sum]);
                         else q = __ddiv_rn((double)e.y, (double)sum);
                     } else q = __ddiv_rn((double)e.y, dsum);
                     const double dc = __dmul_rn(cur_d, q);      // Eq. 2
@@ -792,14 +817,21 @@ __device__ __noinline__ void expand_job(BlockShared& sh, WarpWork& W, const int4
                             }
                             n += __popc(m);
                         };
-                        stage(c0); stage(c1); stage(c);
-                        __syncwarp();
-                        n = pool_compact(W.C, n, budget - cnt, floor, lane);
                         auto back = [&](int i) {
                             return i < n ? Cand{(unsigned)__double2hiint(W.C.d[i]), (unsigned)__double2loint(W.C.d[i]), W.C.tok[i], W.C.cb[i], W.C.np[i]}
                                          : Cand{0u, 0u, 0, 0, 0u};
                         };
-                        c0 = back(lane); c1 = back(32 + lane);
+                        stage(c);
+                        if (ROOMY && n <= __popc(f0) + __popc(f1)) {             // those that matter go into free places of either kind
+                            __syncwarp();
+                            if (c0.hi == 0u) c0 = back(__popc(f0 & lt));
+                            if (c1.hi == 0u) c1 = back(__popc(f0) + __popc(f1 & lt));
+                        } else {
+                            stage(c0); stage(c1);
+                            __syncwarp();
+                            n = pool_compact(W.C, n, budget - cnt, floor, lane);
+                            c0 = back(lane); c1 = back(32 + lane);
+                        }
                         __syncwarp();
                     }
                     // as many as can still be added: what is worse than the last of them does not matter any more
@@ -1177,7 +1209,7 @@ speculate_fused_kernel(sd_store sv, int n, const int32_t* __restrict__ d_slot, i
             if (!((old >> rank) & 1u)) continue;                // another warp was faster
             __threadfence_block();
             const int p = __shfl_sync(FULL, my_p, rank), budget = __shfl_sync(FULL, my_budget, rank);
-            expand_job(sh, W, tree == 0 ? sv.g_ent : s_ent, tree == 0 ? (int)sv.g_cap : (int)sv.spn, tree, p, budget, flags, -1, lane);
+            expand_job<MINB == 1>(sh, W, tree == 0 ? sv.g_ent : s_ent, tree == 0 ? (int)sv.g_cap : (int)sv.spn, tree, p, budget, flags, -1, lane);
         }
     };
     // All jobs can be taken at once: in their order, then (256 requests: 38.6 us, without the barrier 41; where the SM has one block
@@ -1247,7 +1279,7 @@ speculate_fused_kernel(sd_store sv, int n, const int32_t* __restrict__ d_slot, i
                     frontier_merge_list(W.T, 0, fs, budget, O, ofs, -1, lane);
                 }
                 counts_to_d(W.T, 0, fs, 1.0, sum, lane);
-                expand_job(sh, W, ent, tree == 0 ? (int)sv.g_cap : (int)sv.spn, tree, p, budget, flags, fs, lane);
+                expand_job<MINB == 1>(sh, W, ent, tree == 0 ? (int)sv.g_cap : (int)sv.spn, tree, p, budget, flags, fs, lane);
             }
             __syncthreads();
         }

@@ -185,7 +185,8 @@ def test_arguments_of_the_calls_of_every_step(U, name, bad, error):
     pr.close()
 
 
-@pytest.mark.parametrize("children,most", [(33, 3), (128, 9), (129, 1), (300, 2), (300, 40), (140, 140)])
+@pytest.mark.parametrize("children,most", [(33, 3), (128, 9), (129, 1), (300, 2), (300, 40), (140, 140),
+                                           (62, 4), (63, 1), (63, 5), (64, 2), (65, 7), (127, 60)])
 def test_long_runs_without_a_ready_list_in_the_middle_of_a_tree(U, children, most):
     rng = np.random.default_rng(children + most)
     counts = np.full(children, 131) if most == 140 else rng.integers(1, most + 1, children)
@@ -201,6 +202,22 @@ def test_long_runs_without_a_ready_list_in_the_middle_of_a_tree(U, children, mos
     pr.close()
 
 
+@pytest.mark.parametrize("budget", [33, 35, 36, 37, 39, 41, 64])
+def test_the_least_of_a_long_runs_best_children_stays_a_candidate(U, budget):
+    """40 children: the first occurs 50 times, the last 12 times, those between ten times or once.  The first one's children need more places
+    than are left: what goes then goes by the least of the best, wherever it stands in the run."""
+    first = [60] * 20 + list(range(61, 91))
+    seqs = [np.array([7, 10, e, 95], np.int32) for e in first]
+    seqs += [np.array([7, 10 + c, 60 + e, 95], np.int32) for c, k in zip(range(1, 40), [10] * 34 + [1] * 4 + [12]) for e in range(k)]
+    pr = U.Pair(seqs, vocab=100, D=8, n_slots=200, max_req_tokens=16)
+    slots = list(range(200))
+    pr.append(slots, [np.array([7], np.int32)] * 200)
+    for some in (slots[:1], slots):                             # one block per SM, and two
+        for flags in (0, 4):
+            pr.check_speculate(some, 1, float(budget), 64, flags=flags)
+    pr.close()
+
+
 def test_trim_gives_back_what_freed_stores_left():
     import paper_2411_04975_b200 as sfx
     sfx.sd_trim()
@@ -213,7 +230,7 @@ def test_trim_gives_back_what_freed_stores_left():
     assert free0 - torch.cuda.mem_get_info()[0] < (8 << 20)
 
 
-@pytest.mark.parametrize("outer,inner", [(31, 32), (40, 20), (40, 30), (60, 32), (64, 5), (70, 31)])
+@pytest.mark.parametrize("outer,inner", [(31, 32), (40, 20), (40, 30), (60, 32), (64, 5), (70, 31), (31, 3), (31, 5), (28, 17), (32, 9)])
 def test_more_candidates_than_a_job_has_places_for(U, outer, inner):
     """Candidates of equal D from several fans until there is no place: the best stay, by token and parent where D is equal."""
     rng = np.random.default_rng(outer * 100 + inner)
