@@ -257,15 +257,18 @@ entropy_runs_kernel(const int4* __restrict__ ent, const int2* __restrict__ queue
 // the numerator is f(all tokens) - sum of f(count) over the leaves + sum of f(S) - f(count) over the nodes with children; and S is
 // the node's own count unless a sequence ends with the node (RUN_ENDS, one node for every suffix shorter than the tree is deep).  So
 // only these few look at their children, and the others not even at their count.  The values are COUNTED, with their signs, in
-// shared memory (large ones, few, are listed), and the block that ends last takes the logarithms, once per value, and adds up
+// shared memory, and the block that ends last takes the logarithms, once per value, and adds up
 // with the rounding errors carried along: equal values cancel exactly, and no node costs a division or a logarithm in double
 // precision.  (Those of branching nodes' children, 32 at a time: 348 us for 41 M nodes, now 127, 5.1 TB/s.  Error against 80-bit
 // sums over eight corpora: 2.9e-16 to 1.8e-15, now 1.2e-17 to 1.5e-16.)
+// Large values are listed, and every block takes the logarithms of its own: mostly few, but a corpus of short sequences that occur again and
+// again has tens of thousands (28 M tokens, 1,318 sequences of 20: 69 us with all of them left to the block that ends last, now 45).
 constexpr int ENT_SWEEP = 512;                // threads per block
 constexpr int ENT_BLOCKS = 3;                 // per SM
 constexpr int ENT_VALUES = 1024;              // values below are counted, others listed
 constexpr int ENT_AHEAD = 4;                  // loads in flight per lane
-struct EntropySums {
+constexpr int ENT_OWN = 1024;                 // values that a block lists itself; more go to all blocks' list
+struct __align__(16) EntropySums {
     unsigned long long wsum;
     double sum, rest;                         // the numerator in two parts
     int epoch, live;                          // of the tree
@@ -274,8 +277,9 @@ struct EntropySums {
 };
 
 __global__ void __launch_bounds__(ENT_SWEEP, ENT_BLOCKS)
-entropy_sweep_kernel(const int4* __restrict__ ent, const GlobalState* __restrict__ gs, EntropySums* out, int* list) {
+entropy_sweep_kernel(const int4* __restrict__ ent, const GlobalState* __restrict__ gs, EntropySums* out, double2* parts, int* list) {
     __shared__ int net[ENT_VALUES];
+    __shared__ int own[ENT_OWN], n_own;
     __shared__ int2 queue[ENT_SWEEP / 32][32 + 32 * ENT_AHEAD];  // nodes that a sequence ends with
     const unsigned FULL = 0xffffffffu;
     const int tid = threadIdx.x, lane = tid & 31, wib = tid >> 5;
@@ -283,6 +287,7 @@ entropy_sweep_kernel(const int4* __restrict__ ent, const GlobalState* __restrict
     if (blockIdx.x == 0 && tid == 0) { out->epoch = gs->epoch; out->live = n; }
     if (gs->epoch != 1) return;                                  // something was inserted since the build
     for (int v = tid; v < ENT_VALUES; v += ENT_SWEEP) net[v] = 0;
+    if (tid == 0) n_own = 0;
     __syncthreads();
     int2* const q = queue[wib];
     const unsigned lt = (1u << lane) - 1u;
@@ -293,7 +298,9 @@ entropy_sweep_kernel(const int4* __restrict__ ent, const GlobalState* __restrict
         if (v == 2u) twos += k;
         else if (v < (unsigned)ENT_VALUES) atomicAdd(&net[v], k);
         else {
-            list[atomicAdd(&out->n_list, 1)] = k > 0 ? (int)v : -(int)v;
+            const int at = atomicAdd(&n_own, 1), x = k > 0 ? (int)v : -(int)v;
+            if (at < ENT_OWN) own[at] = x;
+            else list[atomicAdd(&out->n_list, 1)] = x;
         }
     };
     auto ended = [&](int2 e) {                                   // children at e.x, e.y as the w field
@@ -338,14 +345,6 @@ entropy_sweep_kernel(const int4* __restrict__ ent, const GlobalState* __restrict
     if (lane == 0 && wt) atomicAdd(&out->wsum, wt);
     __syncthreads();
     for (int v = tid; v < ENT_VALUES; v += ENT_SWEEP) if (net[v]) atomicAdd(&out->net[v], net[v]);
-    // ---- the block that ends last adds up
-    __shared__ bool last;
-    __threadfence();
-    __syncthreads();
-    if (tid == 0) last = atomicAdd(&out->done, 1) == (int)gridDim.x - 1;
-    __syncthreads();
-    if (!last) return;
-    __threadfence();
     double hi = 0.0, lo = 0.0;
     auto plus = [&](double b, double e) {                        // exact sum of hi and b (Knuth), the rest to lo
         const double s = __dadd_rn(hi, b), bb = __dsub_rn(s, hi);
@@ -356,23 +355,42 @@ entropy_sweep_kernel(const int4* __restrict__ ent, const GlobalState* __restrict
         const double f = __dmul_rn(v, log2(v)), p = __dmul_rn(k, f);
         plus(p, __fma_rn(k, f, -p));
     };
-    if (tid == 0 && n > 0) times_f(1.0, (double)gs->tokens);
-    for (int v = tid; v < ENT_VALUES; v += ENT_SWEEP) { const int k = __ldcg(&out->net[v]); if (k) times_f((double)k, (double)v); }
-    const int n_list = __ldcg(&out->n_list);
-    for (int i = tid; i < n_list; i += ENT_SWEEP) { const int v = __ldcg(&list[i]); times_f(v > 0 ? 1.0 : -1.0, fabs((double)v)); }
     __shared__ double shi[ENT_SWEEP / 32], slo[ENT_SWEEP / 32];
     auto over_lanes = [&]() {
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) { const double b = __shfl_xor_sync(FULL, hi, o), e = __shfl_xor_sync(FULL, lo, o); plus(b, e); }
     };
-    over_lanes();
-    if (lane == 0) { shi[wib] = hi; slo[wib] = lo; }
-    __syncthreads();
-    if (wib == 0) {
-        hi = lane < ENT_SWEEP / 32 ? shi[lane] : 0.0; lo = lane < ENT_SWEEP / 32 ? slo[lane] : 0.0;
+    auto over_block = [&]() {                                    // for warp 0
         over_lanes();
-        if (lane == 0) { out->sum = hi; out->rest = lo; }
+        if (lane == 0) { shi[wib] = hi; slo[wib] = lo; }
+        __syncthreads();
+        if (wib == 0) {
+            hi = lane < ENT_SWEEP / 32 ? shi[lane] : 0.0; lo = lane < ENT_SWEEP / 32 ? slo[lane] : 0.0;
+            over_lanes();
+        }
+    };
+    const int mine = min(n_own, ENT_OWN);
+    if (mine > 0) {
+        for (int i = tid; i < mine; i += ENT_SWEEP) { const int v = own[i]; times_f(v > 0 ? 1.0 : -1.0, fabs((double)v)); }
+        over_block();
     }
+    if (tid == 0) parts[blockIdx.x] = make_double2(hi, lo);
+    // ---- the block that ends last adds up
+    __shared__ bool last;
+    __threadfence();
+    __syncthreads();
+    if (tid == 0) last = atomicAdd(&out->done, 1) == (int)gridDim.x - 1;
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    hi = 0.0; lo = 0.0;
+    for (int b = tid; b < (int)gridDim.x; b += ENT_SWEEP) { const double2 x = __ldcg(&parts[b]); plus(x.x, x.y); }
+    if (tid == 0 && n > 0) times_f(1.0, (double)gs->tokens);
+    for (int v = tid; v < ENT_VALUES; v += ENT_SWEEP) { const int k = __ldcg(&out->net[v]); if (k) times_f((double)k, (double)v); }
+    const int n_list = __ldcg(&out->n_list);
+    for (int i = tid; i < n_list; i += ENT_SWEEP) { const int v = __ldcg(&list[i]); times_f(v > 0 ? 1.0 : -1.0, fabs((double)v)); }
+    over_block();
+    if (tid == 0) { out->sum = hi; out->rest = lo; }
 }
 
 }  // namespace
@@ -392,9 +410,14 @@ extern "C" int sd_entropy(sd_store* s, int32_t tree, double* h_entropy, void* st
         const size_t most = (size_t)(s->built / ENT_VALUES) * 2 * (size_t)s->D;
         EntropySums* d = nullptr;
         EntropySums h;
-        if (sd_device_malloc((void**)&d, sizeof(EntropySums) + sizeof(int) * most) != cudaSuccess) { cudaGetLastError(); return SD_ERR_NOMEM; }
+        const unsigned blocks = (unsigned)(sms * ENT_BLOCKS);
+        if (sd_device_malloc((void**)&d, sizeof(EntropySums) + sizeof(double2) * blocks + sizeof(int) * most) != cudaSuccess) {
+            cudaGetLastError();
+            return SD_ERR_NOMEM;
+        }
+        double2* const parts = reinterpret_cast<double2*>(d + 1);
         cudaError_t ce = cudaMemsetAsync(d, 0, sizeof(EntropySums), st);
-        entropy_sweep_kernel<<<(unsigned)(sms * ENT_BLOCKS), ENT_SWEEP, 0, st>>>(ent, s->g_state, d, reinterpret_cast<int*>(d + 1));
+        entropy_sweep_kernel<<<blocks, ENT_SWEEP, 0, st>>>(ent, s->g_state, d, parts, reinterpret_cast<int*>(parts + blocks));
         if (ce == cudaSuccess) ce = cudaMemcpyAsync(&h, d, offsetof(EntropySums, net), cudaMemcpyDeviceToHost, st);
         const cudaError_t done = cudaStreamSynchronize(st);
         if (ce == cudaSuccess) ce = done;

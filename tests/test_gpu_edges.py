@@ -61,6 +61,28 @@ def test_corpora_at_the_edges_of_the_sort(U, n, D, vocab):
     pr.close()
 
 
+@pytest.mark.parametrize("distinct,length,copies,halves", [(40, 40, 1500, False), (4096, 1, 1030, False), (3000, 2, 1030, False),
+                                                           (900, 6, 1100, True), (1500, 2, 1024, True), (700, 1, 1023, False)])
+def test_entropy_of_short_sequences_that_occur_again_and_again(distinct, length, copies, halves):
+    """Every token in one place of one sequence: below the root every child is an only one, so the sum is the root's alone.  Counts on both
+    sides of what is counted in shared memory, and more leaves with large ones than a block lists itself."""
+    import paper_2411_04975_b200 as sfx
+    D = 8
+    seqs = [np.arange(distinct * length, dtype=np.int32).reshape(distinct, length)]
+    if halves:
+        seqs.append(seqs[0][:, :length // 2])                    # sequences end in the middle of others
+    flat = np.concatenate([np.tile(s, (copies, 1)).reshape(-1) for s in seqs])
+    off = np.concatenate([[0], np.cumsum(np.repeat([s.shape[1] for s in seqs], copies * distinct))])
+    st = sfx.SuffixStore(torch.as_tensor(flat, device="cuda:0"), torch.as_tensor(off, device="cuda:0"), vocab=distinct * length, depth_cap=D,
+                         max_requests=1, max_req_tokens=16, max_spec_cap=8, global_extra_nodes=0)
+    counts = np.bincount(flat).astype(np.longdouble)
+    root = counts.sum() * np.log2(counts.sum()) - (counts * np.log2(counts)).sum()
+    nodes = sum(copies * distinct * sum(min(D, s.shape[1] - i) for i in range(s.shape[1])) for s in seqs)     # counts of all nodes
+    want = float(root / nodes)
+    assert abs(st.entropy(-1) - want) <= 1e-13 * want            # (a few roundings of 2^-53)
+    st.free()
+
+
 @pytest.mark.parametrize("sizes,D,vocab,fresh", [([1], 32, 4, False), ([7, 8, 9], 32, 6, False), ([511, 1, 0, 2], 17, 30, False),
                                                  ([513], 32, 2, False), ([2015], 32, 5, False), ([2016], 8, 700, True),
                                                  ([2017, 3], 32, 40, False), ([1000, 1000, 1000, 1100], 24, 900, True),
