@@ -429,7 +429,7 @@ int block_suffix_sort(const int32_t* tok, const int64_t* seq_off, int n_seqs, in
 constexpr int CC_THREADS = 512, CP_THREADS = 256;                // a corpus of 32,768 tokens 108 us (1,024 threads 113, 256 116), four prompts of 4,096 44 (56, 512 47)
 template <int ITEMS>
 __global__ void __launch_bounds__(CC_THREADS, 1)
-cluster_corpus_sort_kernel(const int32_t* tok, const int64_t* seq_off, int n_seqs, const int* end_pos, int n, int tok_bits, int D, uint32_t* sa_out) {
+cluster_corpus_sort_kernel(const int32_t* tok, const int* end_pos, int n, int tok_bits, int D, uint32_t* sa_out) {
     sd_chain_begin();
     extern __shared__ __align__(16) unsigned char cs_smem[];
     ClusterOrder<CC_THREADS, ITEMS>& sh = *reinterpret_cast<ClusterOrder<CC_THREADS, ITEMS>*>(cs_smem);
@@ -438,10 +438,9 @@ cluster_corpus_sort_kernel(const int32_t* tok, const int64_t* seq_off, int n_seq
         [&](int i, int off) {
             const int e = end_pos[i];
             if (i >= off && end_pos[i - off] == e) return i - off;
-            int lo = 0, hi = n_seqs;                            // largest q with seq_off[q] <= i
-            while (hi - lo > 1) { const int mid = (lo + hi) >> 1; if (seq_off[mid] <= i) lo = mid; else hi = mid; }
-            const int b = (int)seq_off[lo];
-            return e - min(off, e - b) + (i - b);
+            int lo = max(i - off, -1), hi = i;                  // the sequence begins behind lo, at hi at the latest
+            while (hi - lo > 1) { const int mid = (lo + hi) >> 1; if (end_pos[mid] == e) hi = mid; else lo = mid; }
+            return e - min(off, e - hi) + (i - hi);
         });
     const int first = (int)cluster_rank() * CC_THREADS * ITEMS;
     for (int k = threadIdx.x; k < CC_THREADS * ITEMS && first + k < n; k += CC_THREADS) sa_out[first + k] = (uint32_t)order[k];
@@ -566,15 +565,14 @@ unsigned cluster_for(i64 n, unsigned most, int threads) {        // blocks of a 
     return blocks;
 }
 
-int cluster_corpus_sort(const int32_t* tok, const int64_t* seq_off, int n_seqs, const int* end_pos, int n, int tok_bits, int D, unsigned most,
-                        uint32_t* sa, cudaStream_t st) {
+int cluster_corpus_sort(const int32_t* tok, const int* end_pos, int n, int tok_bits, int D, unsigned most, uint32_t* sa, cudaStream_t st) {
     const unsigned blocks = cluster_for(n, most, CC_THREADS);
     return with_items((n + (i64)blocks * CC_THREADS - 1) / (blocks * CC_THREADS), [&](auto items) -> int {
         constexpr int I = decltype(items)::value;
         const int rc = allow_clusters(cluster_corpus_sort_kernel<I>, sizeof(ClusterOrder<CC_THREADS, I>), blocks);
         if (rc != SD_OK) return rc;
-        SD_CUDA_OK(sd_launch_clusters(cluster_corpus_sort_kernel<I>, blocks, blocks, CC_THREADS, sizeof(ClusterOrder<CC_THREADS, I>), st, tok, seq_off, n_seqs,
-                                      end_pos, n, tok_bits, D, sa));
+        SD_CUDA_OK(sd_launch_clusters(cluster_corpus_sort_kernel<I>, blocks, blocks, CC_THREADS, sizeof(ClusterOrder<CC_THREADS, I>), st, tok, end_pos, n,
+                                      tok_bits, D, sa));
         return SD_OK;
     });
 }
@@ -1239,7 +1237,9 @@ static int pipeline_run(Pipeline& P, const int32_t* d_tok, const int64_t* d_seq_
     // Prompts longer than one step of a block are sorted by a cluster of four or eight blocks each while there are at most 128 blocks then
     // (partitions of 16 multiprocessors and more hold so many at once; with clusters of two, 64 prompts of 8,192 tokens took as long as
     // by a block each, and their decode 1 % longer), else by a block each.  A corpus of up to 65,536 tokens is sorted by a cluster: whole
-    // builds of 8,000 / 32,768 / 65,536 tokens 329 / 382 / 430 us by the whole device, 222 / 280 / 385 by a cluster, of 100,000 447 and 534.
+    // builds of 8,000 / 32,768 / 65,536 tokens 329 / 382 / 430 us by the whole device, 222 / 280 / 385 by a cluster, of 100,000 447 and 534.  (Where a sequence
+    // begins is looked for among its own positions: by a search over all sequences those of 16 tokens each took longer from 50,000 tokens on
+    // than by the whole device, 65,536 tokens 386 - 400 us, now 333 - 348.)
     unsigned prompt_cluster = 8;
     while (prompt_cluster > 1 && (i64)n_seqs * prompt_cluster > 128) prompt_cluster /= 2;
     if (prompt_cluster > 1) prompt_cluster = cluster_for(per_seq_max_len, prompt_cluster, CP_THREADS);
@@ -1262,7 +1262,7 @@ static int pipeline_run(Pipeline& P, const int32_t* d_tok, const int64_t* d_seq_
         rc = cluster_prompt_sort(d_tok, d_seq_offsets, n_seqs, per_seq_max_len, V, bits_for(V), D, prompt_cluster, sa, *walk, st);
         P.walked = true;
     } else if (cluster_corpus) {
-        rc = cluster_corpus_sort(d_tok, d_seq_offsets, n_seqs, end_pos, (int)N, bits_for(max_token), D, corpus_cluster, sa, st);
+        rc = cluster_corpus_sort(d_tok, end_pos, (int)N, bits_for(max_token), D, corpus_cluster, sa, st);
     } else if (block_sort) {
         const int V = (int)(max_token / n_seqs);                // (a sequence's tokens lie in a range of V of their own)
         const int bits = bits_for(V);
