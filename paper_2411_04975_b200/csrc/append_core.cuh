@@ -402,14 +402,13 @@ __device__ __forceinline__ void append_tokens(AppendShared& sh, const sd_store& 
                 // the others: steps of 512 requests of text without repeats 3 % longer, of one agent 1 %.  Runs of up to four by their lanes: 1 %.)
                 const bool own = need && !leaf && n <= 2 && !((clash >> lane) & 1u);
                 if (own) {
-                    const int base = moves ? fresh : pcb;
-                    const int4 e0 = ent[pcb], e1 = n > 1 ? ent[pcb + 1] : e0;
-                    if (moves || place == 0) ent[base + (place == 0 ? 1 : 0)] = e0;
-                    if (n > 1 && (moves || place <= 1)) ent[base + (place <= 1 ? 2 : 1)] = e1;
-                    ent[base + place] = make_int4(x, 1, 0, 0);
-                    if (moves) *word(&ent[parent], 2) = fresh;
+                    const int4 e0 = ent[pcb], e1 = n > 1 ? ent[pcb + 1] : e0;             // (such a run is always full: it moves)
+                    ent[fresh + (place == 0 ? 1 : 0)] = e0;
+                    if (n > 1) ent[fresh + (place <= 1 ? 2 : 1)] = e1;
+                    ent[fresh + place] = make_int4(x, 1, 0, 0);
+                    *word(&ent[parent], 2) = fresh;
                     *word(&ent[parent], 3) = n + 1;
-                    new_act = base + place;
+                    new_act = fresh + place;
                 }
                 runs = __ballot_sync(FULL, need && !leaf && !own);
                 const unsigned big = __ballot_sync(FULL, need && (moves ? n : n - place) > APP_BIG);
