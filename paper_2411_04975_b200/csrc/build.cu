@@ -548,15 +548,15 @@ int allow_clusters(Kernel kernel, size_t smem, unsigned blocks) {
     return SD_OK;
 }
 
-// f(std::integral_constant<int, ITEMS>) for the least of 1, 2, 4, 8, 16 items that is enough
+// f(std::integral_constant<int, ITEMS>) for the least of 1, 2, 4 .. MOST items that is enough
 constexpr int CP_ITEMS = 16, CC_ITEMS = 8;        // the most
-template <class F>
+template <int MOST, class F>
 int with_items(i64 per_thread, F f) {
     if (per_thread <= 1) return f(std::integral_constant<int, 1>());
     if (per_thread <= 2) return f(std::integral_constant<int, 2>());
     if (per_thread <= 4) return f(std::integral_constant<int, 4>());
-    if (per_thread <= 8) return f(std::integral_constant<int, 8>());
-    return f(std::integral_constant<int, 16>());
+    if (MOST == 8 || per_thread <= 8) return f(std::integral_constant<int, 8>());
+    return f(std::integral_constant<int, MOST>());
 }
 
 unsigned cluster_for(i64 n, unsigned most, int threads) {        // blocks of a cluster for n tokens
@@ -567,7 +567,7 @@ unsigned cluster_for(i64 n, unsigned most, int threads) {        // blocks of a 
 
 int cluster_corpus_sort(const int32_t* tok, const int* end_pos, int n, int tok_bits, int D, unsigned most, uint32_t* sa, cudaStream_t st) {
     const unsigned blocks = cluster_for(n, most, CC_THREADS);
-    return with_items((n + (i64)blocks * CC_THREADS - 1) / (blocks * CC_THREADS), [&](auto items) -> int {
+    return with_items<CC_ITEMS>((n + (i64)blocks * CC_THREADS - 1) / (blocks * CC_THREADS), [&](auto items) -> int {
         constexpr int I = decltype(items)::value;
         const int rc = allow_clusters(cluster_corpus_sort_kernel<I>, sizeof(ClusterOrder<CC_THREADS, I>), blocks);
         if (rc != SD_OK) return rc;
@@ -581,7 +581,7 @@ int cluster_prompt_sort(const int32_t* tok, const int64_t* seq_off, int n_seqs, 
                         uint32_t* sa, const RequestWalk& walk, cudaStream_t st) {
     const unsigned walks = (unsigned)n_seqs + (unsigned)walk.refreshed;
     const unsigned grid = ((unsigned)n_seqs + (walks + blocks - 1) / blocks) * blocks;
-    return with_items((max_len + (i64)blocks * CP_THREADS - 1) / (blocks * CP_THREADS), [&](auto items) -> int {
+    return with_items<CP_ITEMS>((max_len + (i64)blocks * CP_THREADS - 1) / (blocks * CP_THREADS), [&](auto items) -> int {
         constexpr int I = decltype(items)::value;
         const int rc = allow_clusters(cluster_prompt_sort_kernel<I>, sizeof(ClusterOrder<CP_THREADS, I>), blocks);
         if (rc != SD_OK) return rc;
