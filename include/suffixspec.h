@@ -336,6 +336,12 @@ const char* sd_strerror(int code);
  */
 void sd_debug_fail_alloc(int64_t k);
 
+/*
+ * sd_debug_small_clusters: test hook for devices (partitions of one) without room for a cluster of 16 blocks.  From now on (on != 0)
+ * the library does as on such a device, whatever this one has room for; 0 switches it off.  Results are the same.
+ */
+void sd_debug_small_clusters(int32_t on);
+
 #ifdef __cplusplus
 }
 #endif

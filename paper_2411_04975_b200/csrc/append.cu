@@ -5,6 +5,7 @@
 #include <cooperative_groups.h>
 
 #include "append_core.cuh"
+#include "device_memory.h"
 #include "global_insert.cuh"
 #include "suffix_order.cuh"
 
@@ -697,7 +698,7 @@ int insert_setup(int dev, bool* cluster) {
     constexpr int MAX_DEVICES = 64;
     static std::atomic<int> known[MAX_DEVICES];                  // 1: a grid, 2: a cluster
     const bool kept = dev >= 0 && dev < MAX_DEVICES;
-    int k = kept ? known[dev].load() : 0;
+    int k = sd_small_clusters() ? 1 : (kept ? known[dev].load() : 0);
     if (k != 1) {
         constexpr size_t smem = sizeof(GiShared<GI_CLUSTER>);
         const bool set = cudaFuncSetAttribute(global_insert_kernel<GI_CLUSTER>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) == cudaSuccess &&

@@ -595,7 +595,7 @@ int cluster_prompt_sort(const int32_t* tok, const int64_t* seq_off, int n_seqs, 
 unsigned largest_cluster(int dev) {
     constexpr int MAX_DEVICES = 64;
     static std::atomic<unsigned> known[MAX_DEVICES];
-    if (dev < 0 || dev >= MAX_DEVICES) return 8;
+    if (dev < 0 || dev >= MAX_DEVICES || sd_small_clusters()) return 8;
     unsigned c = known[dev].load();
     if (c == 0) {
         c = 8;

@@ -268,6 +268,12 @@ extern "C" void sd_trim(void) {
     for (int dev = 0; dev < CACHE_DEVICES; ++dev) cache_expire(dev, g.cache[dev], Clock::time_point::max());
 }
 
+static std::atomic<bool> g_small_clusters{false};
+
+bool sd_small_clusters() { return g_small_clusters.load(); }
+
+extern "C" void sd_debug_small_clusters(int32_t on) { g_small_clusters = on != 0; }
+
 extern "C" void sd_debug_fail_alloc(int64_t k) { g_fail_alloc_in = k; g_fail_alloc_on = k > 0; }
 
 void sd_store_release(sd_store* s, cudaStream_t st) {

@@ -12,5 +12,8 @@ bool sd_take_streams(int dev, size_t stage_bytes, StreamSet* out);
 // Calls of sd_trim so far.  What is set up once per device is set up anew behind one: a cudaDeviceReset may have followed.
 int sd_trims();
 
+// sd_debug_small_clusters is on.
+bool sd_small_clusters();
+
 // Releases what a store holds, behind the work on `st`: the caller has waited for every other stream that used the store.
 void sd_store_release(sd_store* s, cudaStream_t st);

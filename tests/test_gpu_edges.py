@@ -25,9 +25,43 @@ def _text(rng, n, vocab, period=60):
 @pytest.mark.parametrize("longest,D,vocab", [(1, 1, 2), (33, 32, 3), (1024, 17, 130), (1025, 32, 50), (2049, 2, 7), (4096, 24, 128256),
                                              (4097, 32, 300), (8193, 31, 65), (16384, 32, 40), (16385, 32, 40),
                                              (32768, 32, 40), (32769, 9, 30)])
-def test_prompts_at_the_edges_of_the_block_sort(U, longest, D, vocab):
+def test_prompts_at_the_edges_of_the_sorts(U, longest, D, vocab):
+    """Up to eight prompts in a call: a block each up to 1,024 tokens, then a cluster of eight blocks each, above 32,768 tokens the sort of a
+    whole corpus."""
+    _check_prompts(U, longest, D, vocab, 0)
+
+
+@pytest.mark.parametrize("n,longest,D,vocab", [(33, 1024, 32, 70), (33, 1025, 32, 50), (34, 2048, 24, 90), (33, 2049, 2, 7), (33, 4096, 17, 130),
+                                               (40, 4097, 32, 300), (33, 8192, 9, 128256), (33, 8193, 31, 65), (33, 16384, 32, 40),
+                                               (33, 16385, 8, 40)])
+def test_prompts_at_the_edges_of_the_block_sort(U, n, longest, D, vocab):
+    """More than 32 prompts in a call: a block each up to 16,384 tokens."""
+    _check_prompts(U, longest, D, vocab, n)
+
+
+@pytest.mark.parametrize("n,longest,D,vocab", [(17, 1025, 32, 50), (32, 2049, 24, 128256), (18, 4097, 32, 30), (17, 8193, 17, 300), (32, 16384, 32, 40),
+                                               (17, 16385, 32, 40)])
+def test_prompts_at_the_edges_of_clusters_of_four_blocks(U, n, longest, D, vocab):
+    """17 to 32 prompts in a call: a cluster of four blocks each up to 16,384 tokens."""
+    _check_prompts(U, longest, D, vocab, n)
+
+
+def test_one_long_prompt_is_sorted_as_a_small_corpus(U):
+    rng = np.random.default_rng(40)
+    text = _text(rng, 40000, 90)
+    pr = U.Pair([], vocab=90, D=16, n_slots=1, max_req_tokens=40100)
+    pr.g.build_requests(np.arange(1), np.array([0, text.size]), U.dev_i32(text))
+    pr.o.slot_append_batch([0], [text])
+    pr.check_tree(0)
+    pr.append([0], [text[:9]])
+    pr.check_speculate([0], 12, 2.0, 32)
+    pr.close()
+
+
+def _check_prompts(U, longest, D, vocab, n):
     rng = np.random.default_rng(longest)
     lens = sorted({1, 2, 15, 16, 17, max(1, longest - 1), longest} & set(range(1, longest + 1)))
+    lens += [3 + k for k in range(n - len(lens) - 1)]            # n prompts in all, if that is more
     prompts = [_text(rng, n, vocab) for n in lens] + [np.zeros(0, np.int32)]
     pr = U.Pair([], vocab=vocab, D=D, n_slots=len(prompts), max_req_tokens=longest + 8, M=32)
     off, flat = U.ragged(prompts)
@@ -116,6 +150,30 @@ def test_what_a_full_pool_takes_goes_by_lots_of_2016(U, n, fits):
     assert st["global_status"] == (0 if fits else 4)
     assert st["global_nodes"] == (nodes if fits else last)
     pr.close()
+
+
+@pytest.fixture
+def small_clusters():
+    import paper_2411_04975_b200 as sfx
+    sfx.library().sd_debug_small_clusters(1)
+    yield
+    sfx.library().sd_debug_small_clusters(0)
+
+
+@pytest.mark.parametrize("sizes,D,vocab,fresh", [([7, 8, 9], 32, 6, False), ([513], 32, 2, False), ([2015], 32, 5, False), ([2016], 8, 700, True),
+                                                 ([2017, 3], 32, 40, False), ([1000, 1000, 1000, 1100], 24, 900, True)])
+def test_global_insert_without_a_cluster(U, small_clusters, sizes, D, vocab, fresh):
+    test_global_insert_at_the_edges_of_a_pass(U, sizes, D, vocab, fresh)
+
+
+@pytest.mark.parametrize("n,fits", [(2016, True), (2016, False), (2017, False)])
+def test_what_a_full_pool_takes_without_a_cluster(U, small_clusters, n, fits):
+    test_what_a_full_pool_takes_goes_by_lots_of_2016(U, n, fits)
+
+
+@pytest.mark.parametrize("n,D,vocab", [(1025, 17, 4000), (32768, 32, 500), (32769, 24, 60), (65536, 32, 700)])
+def test_corpora_without_large_clusters(U, small_clusters, n, D, vocab):
+    test_corpora_at_the_edges_of_the_sort(U, n, D, vocab)
 
 
 def test_global_insert_merges_long_runs(U):

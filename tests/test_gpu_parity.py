@@ -582,8 +582,8 @@ def test_build_requests_equals_token_by_token_append(U, D, vocab):
 
 
 def test_build_requests_long_and_short_prompts(U):
-    """Prompts up to 16,384 tokens are sorted by one block each, longer ones by the general
-    pipeline: both must give the tree of the token-by-token append."""
+    """Prompts are sorted by clusters of blocks, by a block each or by the sort of a whole corpus, as
+    their number and the longest one have it: each must give the tree of the token-by-token append."""
     rng = np.random.default_rng(5)
     vocab, D = 300, 12
 
