@@ -1044,11 +1044,12 @@ speculate_fused_kernel(sd_store sv, int n, const int32_t* __restrict__ d_slot, i
     // ---------------- 1. match
     bool want_g = usable && !(flags & SD_FLAG_REQUEST_ONLY);
     bool want_r = usable && !(flags & SD_FLAG_GLOBAL_ONLY);
-    if (want_g && gw == 0) {
+    // (a slot that appears twice is refused below; until then its first block may be writing what this one reads, so the lanes vote)
+    if (gw == 0 && __all_sync(FULL, want_g)) {
         // the walk to the match node of the last d tokens starts at the node kept from the call before, or at the root
         const int d = lane + 1;
         int len = ss->g_len, depths = ss->g_depths, kept = ss->g_node[lane];
-        bool known = ss->g_gen == ss->gen && ss->g_epoch == sv.g_state->epoch && len <= t;
+        bool known = __all_sync(FULL, ss->g_gen == ss->gen && ss->g_epoch == sv.g_state->epoch && len <= t);
         if (!known) {
             // (a call of sd_build_requests may be writing it)
             const MatchRecord& rec = ss->record;
