@@ -1215,7 +1215,7 @@ struct Pipeline {
 // max_token: largest token value + 1 (sets the number of radix passes; below 2^31).  top_blocks: count the
 // long runs.  per_seq_max_len > 0: the sequences are independent
 // (tokens of different sequences never compare equal, sequence k's tokens below sequence k + 1's)
-// and none is longer than that, so each is sorted by a block of its own.
+// and none is longer than that, so each is sorted by a cluster of its own, or a block where there are many or all are short.
 // end_pos: one past the last token of every token's sequence, if that is known already.
 // Nothing is read back to the host.
 // Returns SD_OK, SD_ERR_NOMEM or SD_ERR_CUDA.

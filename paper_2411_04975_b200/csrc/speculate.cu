@@ -6,8 +6,9 @@
 //     nodes are the slot's active nodes, so only jobs through the request's tree wait for it;
 //   - the global match nodes are advanced from the nodes cached at the previous call by
 //     descending only the tokens appended since;
-//   - the (tree, p) jobs go into a queue, costliest first, a warp per job; a job is dropped,
-//     exactly, as soon as an upper bound of its SCORE falls below a score already reached;
+//   - a (tree, p) job can be taken as soon as its match node is known, costliest first, a warp per
+//     job; a job is dropped, exactly, as soon as an upper bound of its SCORE falls below a score
+//     already reached;
 //   - select (Section 3.2: only if SCORE > tau) and emit from shared memory.
 // sd_speculate_noalloc: the two-kernel form, one warp per (request, tree, p) job with the jobs'
 // records in global memory (match_expand_kernel, select_emit_kernel).
@@ -283,8 +284,10 @@ __global__ void select_emit_kernel(sd_store sv, int n, const int32_t* __restrict
 // Fused path: one block of W warps per request (the kernel itself is described where it is
 // defined).  Two blocks per SM is the usual shape.  A batch of at most one request per SM gets blocks with
 // more registers, a batch of more than two requests per SM smaller ones (four per SM) to stay in one wave.
-constexpr int CTA_WARPS = 14;                  // the usual block; 256 requests: 44.2 us (10 warps 51.5, 12 52.1, 13 45.6, 15 48.9, 16 49.3)
-constexpr int CTA_WARPS_STEP = 14;             // of sd_step: 58.6 us per step (8 warps 63.1, 10 60.1, 12 59.2, 16 58.6)
+// (The usual block's size was taken when candidates lay in shared memory: drafts of 256 requests 44.2 us with 14 warps, 51.5 / 52.1 / 45.6 /
+// 48.9 / 49.3 with 10 / 12 / 13 / 15 / 16; steps 58.6, with 8 / 10 / 12 / 16 63.1 / 60.1 / 59.2 / 58.6.  It has not been swept since.)
+constexpr int CTA_WARPS = 14;
+constexpr int CTA_WARPS_STEP = 14;             // of sd_step
 // one block per SM at most, 128 registers per thread: nothing is spilled.  Drafts of 64 requests with long runs 95 us (24 warps of 80
 // registers 107, 20 106, 12 108), of one request 7.3 (8.0, 7.6, 7.1); steps of 64 requests 47.4 (12 warps 49.2, 20 48.7)
 constexpr int CTA_WARPS_WIDE = 16;
